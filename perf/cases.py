@@ -92,19 +92,43 @@ def draw(rng):
 
 
 # ----------------------------------------------------------------------------------------------- what a program keeps
-class _State:
-    """A context, the buffers of its calls, and the inputs of one pass."""
+class _Draws:
+    """The random inputs of one state, drawn in a fixed order from the seed."""
 
-    def __init__(self, case, seed, max_seqs, max_tokens, max_batch, layers=1):
+    def __init__(self, case, seed):
         self.case, self.s = case, SHAPES[case["model"]]
-        s = self.s
         self.code, self.dt = DTYPES[case["dtype"]]
-        self.kdim = s["nkv"] * s["dh"]
+        self.kdim = self.s["nkv"] * self.s["dh"]
         self.g = torch.Generator(device="cuda")
         self.g.manual_seed(seed)
         # residual rows are N(0, 1) with one channel in a hundred twenty times larger, as real residual streams have them
-        self.gain = torch.ones(s["d"], device="cuda")
-        self.gain[torch.randperm(s["d"], generator=self.g, device="cuda")[: s["d"] // 100]] = 20.0
+        self.gain = torch.ones(self.s["d"], device="cuda")
+        self.gain[torch.randperm(self.s["d"], generator=self.g, device="cuda")[: self.s["d"] // 100]] = 20.0
+
+    def normal(self, shape, std=1.0, mean=0.0):
+        return torch.randn(shape, generator=self.g, device="cuda").mul_(std).add_(mean).to(self.dt)
+
+    def rows(self, n):
+        return torch.randn((n, self.s["d"]), generator=self.g, device="cuda").mul_(self.gain).to(self.dt)
+
+    def layer(self):
+        """Norm scale of the input, norm scale of the keys (or None), K and V projection of a layer."""
+        s = self.s
+        gamma_in = self.normal((s["d"],), 0.02, 1.0)
+        gamma_k = self.normal((s["dh"],), 0.02, 1.0) if s["norm"] else None
+        return gamma_in, gamma_k, self.normal((s["d"], 2 * self.kdim), 0.02)
+
+    def lo(self, pos):
+        """First position that a query at `pos` sees."""
+        return max(0, pos - self.s["window"] + 1) if self.s["window"] else 0
+
+
+class _State(_Draws):
+    """A context, the buffers of its calls, and the inputs of one pass."""
+
+    def __init__(self, case, seed, max_seqs, max_tokens, max_batch, layers=1):
+        super().__init__(case, seed)
+        s = self.s
         self.desc = kvd.make_desc(layers, s["d"], s["nq"], s["nkv"], s["dh"], EPS, s["norm"], EPS, kvd.KVD_ROPE_INTERLEAVED,
                                   max_seqs, max_tokens, max_batch)
         self.ctx = kvd.Kvd(self.desc)
@@ -112,17 +136,11 @@ class _State:
             self.ctx.kvd_set_dtype(self.code)
         self.gamma_in = []
         for layer in range(layers):
-            self.gamma_in.append(self.normal((s["d"],), 0.02, 1.0))
-            gamma_k = self.normal((s["dh"],), 0.02, 1.0) if s["norm"] else None
-            self.ctx.kvd_set_layer(layer, self.normal((s["d"], 2 * self.kdim), 0.02), self.gamma_in[-1], gamma_k, s["theta"], s["window"])
+            gamma_in, gamma_k, w = self.layer()
+            self.gamma_in.append(gamma_in)
+            self.ctx.kvd_set_layer(layer, w, gamma_in, gamma_k, s["theta"], s["window"])
         self.ws = torch.empty(kvd.kvd_workspace_bytes(self.desc), dtype=torch.uint8, device="cuda")
         self.ctx.kvd_attach_workspace(self.ws)
-
-    def normal(self, shape, std=1.0, mean=0.0):
-        return torch.randn(shape, generator=self.g, device="cuda").mul_(std).add_(mean).to(self.dt)
-
-    def rows(self, n):
-        return torch.randn((n, self.s["d"]), generator=self.g, device="cuda").mul_(self.gain).to(self.dt)
 
     def kv(self, *shape):
         return (torch.zeros((*shape, self.kdim), dtype=self.dt, device="cuda"), torch.zeros((*shape, self.kdim), dtype=self.dt, device="cuda"))
@@ -134,10 +152,6 @@ class _State:
     def query(self, n):
         self.q = self.normal((n, self.s["nq"], self.s["dh"]))
         self.out = torch.zeros_like(self.q)
-
-    def lo(self, pos):
-        """First position that a query at `pos` sees."""
-        return max(0, pos - self.s["window"] + 1) if self.s["window"] else 0
 
 
 def _ints(values):
@@ -446,3 +460,217 @@ def tolerance(case):
         return {"rel": 0.0016, "max": 0.03 if turn else 0.0064}
     # 2.2e-3 to 3.2e-3, and 1.2e-2 (7.9e-2)
     return {"rel": 0.012, "max": 0.32 if turn else 0.05}
+
+
+# ------------------------------------------------------------------------------------- the same outputs in 64 bits
+def _normed(x, gamma):
+    x = x.double()
+    return x * (x.square().mean(-1, keepdim=True) + EPS).rsqrt() * gamma.double()
+
+
+def _rotate(x, pos, theta):
+    """Rotation of the pairs (2i, 2i + 1) of x [n, heads, d_head] by pos [n]."""
+    dh = x.shape[-1]
+    freq = theta ** (-torch.arange(0, dh, 2, dtype=torch.float64, device=x.device) / dh)
+    angle = (pos.double()[:, None] * freq)[:, None, :]
+    a, b, cos, sin = x[..., 0::2], x[..., 1::2], angle.cos(), angle.sin()
+    return torch.stack((a * cos - b * sin, a * sin + b * cos), -1).flatten(-2)
+
+
+def _heads(x, pos, gamma, theta, dh):
+    """Head norm (where there is one) and rotation of [n, heads * d_head]."""
+    x = x.view(x.shape[0], -1, dh)
+    return _rotate(_normed(x, gamma) if gamma is not None else x, pos, theta).flatten(1)
+
+
+def _project(dr, layer, x, pos, normed=None, w=None):
+    """K and V [n, kdim] of rows x at positions pos (tensor)."""
+    gamma_in, gamma_k, weight = layer
+    w = weight.double() if w is None else w
+    y = torch.cat([(_normed(x[i : i + 8192], gamma_in) if normed is None else normed[i : i + 8192]) @ w for i in range(0, x.shape[0], 8192)])
+    return _heads(y[:, : dr.kdim].contiguous(), pos, gamma_k, dr.s["theta"], dr.s["dh"]), y[:, dr.kdim :].contiguous()
+
+
+def _attend(dr, q, q_pos, k, v, first):
+    """Attention of q [n, nq, dh] at positions q_pos over k, v [m, kdim] at positions first, first + 1, ..."""
+    s = dr.s
+    key = first + torch.arange(k.shape[0], device="cuda")
+    seen = (key[None, :] <= q_pos[:, None]) & ((q_pos[:, None] - key[None, :] < s["window"]) if s["window"] else True)
+    k, v = k.view(-1, s["nkv"], s["dh"]), v.view(-1, s["nkv"], s["dh"])
+    group, out = s["nq"] // s["nkv"], torch.empty(q.shape, dtype=torch.float64, device="cuda")
+    for h in range(s["nq"]):
+        score = (q[:, h].double() @ k[:, h // group].T) / math.sqrt(s["dh"])
+        out[:, h] = score.masked_fill_(~seen, -math.inf).softmax(-1) @ v[:, h // group]
+    return out
+
+
+def _arange(a, b):
+    return torch.arange(a, b, device="cuda")
+
+
+def _exact_step(case, seed):
+    dr, n = _Draws(case, seed), case["ctx"]
+    layer = dr.layer()
+    x = dr.rows(n + 1)
+    q = dr.normal((1, dr.s["nq"], dr.s["dh"]))
+    k, v = _project(dr, layer, x, _arange(0, n + 1))
+    if dr.code == 2:
+        return x[:n].double(), k, v
+    return x[:n].double(), k, v, _attend(dr, q, _arange(n, n + 1), k, v, 0)
+
+
+def _exact_decode(case, seed):
+    dr, b_, live, lens = _Draws(case, seed), case["batch"], case["live"], _lengths(case)
+    layer = dr.layer()
+    rows = [dr.rows(n) for n in lens]
+    x = dr.rows(b_)
+    q = dr.normal((b_, dr.s["nq"], dr.s["dh"]))
+    lo = [dr.lo(n) for n in lens]
+    keep = [min(live, n - a) for n, a in zip(lens, lo)]
+    n_old = [n - p - a for n, p, a in zip(lens, keep, lo)]
+    zeros = lambda room: torch.zeros((b_, room, dr.kdim), dtype=torch.float64, device="cuda")  # noqa: E731
+    old_k, old_v, live_k, live_v = (zeros(room) for room in [max(1, max(n_old))] * 2 + [live + 1] * 2)
+    out, w = torch.zeros(q.shape, dtype=torch.float64, device="cuda"), layer[2].double()
+    for b, n in enumerate(lens):
+        k, v = _project(dr, layer, torch.cat((rows[b][lo[b] :], x[b : b + 1])), _arange(lo[b], n + 1), w=w)
+        rows[b] = None
+        old_k[b, : n_old[b]], old_v[b, : n_old[b]] = k[: n_old[b]], v[: n_old[b]]
+        live_k[b, live - keep[b] :], live_v[b, live - keep[b] :] = k[n_old[b] :], v[n_old[b] :]
+        out[b] = _attend(dr, q[b : b + 1], _arange(n, n + 1), k, v, lo[b])[0]
+    return old_k, old_v, live_k, live_v, out
+
+
+def _exact_cached(case, seed):
+    dr, b_, n, lens = _Draws(case, seed), case["batch"], case["ctx"], _lengths(case)
+    layer = dr.layer()
+    x = dr.rows(b_)
+    k, v = dr.normal((b_, n + 1, dr.kdim)), dr.normal((b_, n + 1, dr.kdim))
+    q = dr.normal((b_, dr.s["nq"], dr.s["dh"]))
+    kn, vn = _project(dr, layer, x, _ints(lens))
+    return kn, vn, _attend_cached(dr, q, lens, k, v, kn, vn)
+
+
+def _attend_cached(dr, q, lens, k, v, kn, vn):
+    """One query per sequence over its cache k, v [b, room, kdim], whose last column are the new tokens' kn, vn."""
+    out = torch.empty(q.shape, dtype=torch.float64, device="cuda")
+    for b, n in enumerate(lens):
+        a = dr.lo(n)
+        at = k.shape[1] - 1 - n + a
+        kb, vb = (torch.cat((t[b, at:-1].double(), new[b : b + 1])) for t, new in ((k, kn), (v, vn)))
+        out[b] = _attend(dr, q[b : b + 1], _arange(n, n + 1), kb, vb, a)[0]
+    return out
+
+
+def _exact_turn(case, seed):
+    dr, new, ctx, live = _Draws(case, seed), case["new"], case["ctx"], case["live"]
+    layer = dr.layer()
+    rows = dr.rows(ctx) if ctx else None
+    x = dr.rows(new)
+    q = dr.normal((new, dr.s["nq"], dr.s["dh"]))
+    lo = dr.lo(ctx)
+    n_old = max(0, ctx - live - lo)
+    start = min(lo, ctx - live)
+    k, v = _project(dr, layer, torch.cat((rows[start:], x)) if ctx else x, _arange(start, ctx + new))
+    out = _attend(dr, q, _arange(ctx, ctx + new), k, v, start)
+    cut = ctx - live - start
+    old = [t[lo - start : lo - start + n_old] if n_old else torch.zeros((1, dr.kdim), dtype=torch.float64, device="cuda") for t in (k, v)]
+    return old[0], old[1], k[cut:], v[cut:], out
+
+
+def _e4m3(x):
+    return x.to(torch.float8_e4m3fn).float()
+
+
+def _fp8_rows(x):
+    """Rows as E4M3 codes and a scale decode (the statistic stays that of the row itself), over the row's rms."""
+    x = x.float()
+    amax = x.abs().amax(-1, keepdim=True).clamp_min(1e-30)
+    decoded = _e4m3(x * (448.0 / amax)).double() * (amax / 448.0).double()
+    return decoded * (x.double().square().mean(-1, keepdim=True) + EPS).rsqrt()
+
+
+def _exact_fp8(case, seed):
+    dr, b_, lens = _Draws(case, seed), case["batch"], _lengths(case)
+    layer = dr.layer()
+    rows = [dr.rows(n) for n in lens]
+    x = dr.rows(b_)
+    q = dr.normal((b_, dr.s["nq"], dr.s["dh"]))
+    w = layer[0].float()[:, None] * layer[2].float()
+    amax = w.abs().max()
+    w = _e4m3(w * (448.0 / amax)).double() * (amax / 448.0).double()
+    new_k, new_v, out = [], [], torch.empty(q.shape, dtype=torch.float64, device="cuda")
+    for b, n in enumerate(lens):
+        every = torch.cat((rows[b], x[b : b + 1]))
+        k, v = _project(dr, layer, every, _arange(0, n + 1), _fp8_rows(every), w)
+        new_k.append(k[n])
+        new_v.append(v[n])
+        out[b] = _attend(dr, q[b : b + 1], _arange(n, n + 1), k, v, 0)[0]
+    return torch.stack(new_k), torch.stack(new_v), out
+
+
+def _fp4_rows(x):
+    """Rows as 4-bit codes under a scale of every 16 channels and one of the row decode, over the row's rms."""
+    xf = x.float()
+    _, ex = torch.frexp(xf.abs().amax(-1, keepdim=True))
+    row = torch.exp2((ex - 11).double()).float()
+    block = xf.view(x.shape[0], -1, 16)
+    scale = _e4m3(block.abs().amax(-1) / 6.0 / row) * row
+    quot = torch.where(scale[..., None] > 0, block / scale[..., None], torch.zeros_like(block))
+    size = quot.abs()
+    step = torch.where(size < 2, 0.5, torch.where(size < 4, 1.0, 2.0))
+    code = (torch.round(size / step) * step).clamp_max(6.0) * quot.sign()
+    decoded = (code * scale[..., None]).view(x.shape).double()
+    return decoded * (x.double().square().mean(-1, keepdim=True) + EPS).rsqrt()
+
+
+def _exact_fp4(case, seed):
+    dr, b_, lens = _Draws(case, seed), case["batch"], _lengths(case)
+    layer = dr.layer()
+    rows = [dr.rows(n) for n in lens]
+    q = dr.normal((b_, dr.s["nq"], dr.s["dh"]))
+    k_out = torch.zeros((b_, max(lens), dr.kdim), dtype=torch.float64, device="cuda")
+    v_out, out = torch.zeros_like(k_out), torch.empty(q.shape, dtype=torch.float64, device="cuda")
+    for b, n in enumerate(lens):
+        k, v = _project(dr, layer, rows[b], _arange(0, n), _fp4_rows(rows[b]) * layer[0].double())
+        k_out[b, :n], v_out[b, :n] = k, v
+        out[b] = _attend(dr, q[b : b + 1], _arange(n - 1, n), k, v, 0)[0]
+    return k_out, v_out, out
+
+
+def _exact_block(case, seed):
+    dr, b_, n, lens = _Draws(case, seed), case["batch"], case["ctx"], _lengths(case)
+    s = dr.s
+    d, width, pos = s["d"], s["nq"] * s["dh"], _ints(lens)
+    layers = [dr.layer() for _ in range(case["layers"])]
+    rest = []
+    for _ in layers:
+        gamma_q = dr.normal((s["dh"],), 0.02, 1.0) if s["norm"] else None
+        wq, wo = dr.normal((d, width), 0.02), dr.normal((width, d), 0.02)
+        w1, gamma = dr.normal((d, 2 * s["mlp"]), 0.02), dr.normal((d,), 0.02, 1.0)
+        w2 = dr.normal((s["mlp"], d), 0.02)
+        rest.append((gamma_q, wq, wo, w1, gamma, w2, dr.normal((b_, n + 1, dr.kdim)), dr.normal((b_, n + 1, dr.kdim))))
+    head, gamma_head = dr.normal((d, s["vocab"]), 0.02), dr.normal((d,), 0.02, 1.0)
+    table = dr.normal((s["vocab"], d))
+    h = table[torch.randint(s["vocab"], (b_,), generator=dr.g, device="cuda")].double()
+    ks, vs = [], []
+    for layer, (gamma_q, wq, wo, w1, gamma, w2, k, v) in zip(layers, rest):
+        x = _normed(h, layer[0])
+        q = _heads(x @ wq.double(), pos, gamma_q, s["theta"], s["dh"]).view(b_, s["nq"], s["dh"])
+        kn, vn = _project(dr, layer, h, pos)
+        h = h + _attend_cached(dr, q, lens, k, v, kn, vn).flatten(1) @ wo.double()
+        gate, up = (_normed(h, gamma) @ w1.double()).chunk(2, -1)
+        act = torch.nn.functional.silu(gate) if case["model"].startswith("qwen") else torch.nn.functional.gelu(gate, approximate="tanh")
+        h = h + (act * up) @ w2.double()
+        ks.append(kn)
+        vs.append(vn)
+    x = _normed(h, gamma_head)
+    logits = torch.cat([x @ head[:, i : i + 32768].double() for i in range(0, s["vocab"], 32768)], -1)
+    return [h, torch.nn.functional.pad(logits, (0, -s["vocab"] % 256))] + ks + vs  # columns up to a whole tile are zeros
+
+
+_EXACT = {"step": _exact_step, "decode": _exact_decode, "cached": _exact_cached, "turn": _exact_turn, "fp8": _exact_fp8,
+          "fp4": _exact_fp4, "block": _exact_block}
+
+
+def exact(case, seed):
+    return _EXACT[case["kind"]](case, seed)
