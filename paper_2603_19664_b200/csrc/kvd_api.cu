@@ -315,6 +315,10 @@ extern "C" kvd_status kvd_set_layer(kvd_ctx *ctx, int layer, const kvd_layer_des
   st = encode_2d(ctx, &ls.tmap_b, ls.wt, d.d_hidden, n_cols, RC_BLOCK_K * 2 / dtype_bytes(ctx->dtype), ctx->block_n / 2,
                  dtype_bytes(ctx->dtype));
   if (st != KVD_OK) return st;
+  if (ctx->dtype != KVD_DTYPE_F32) {
+    st = prepare_rows_map(ctx, ls, d.d_hidden, n_cols, true);
+    if (st != KVD_OK) return st;
+  }
   // the FP8 variant's copy of W' (E4M3 codes and one scale); rows of d_hidden bytes must be TMA-addressable
   if (d.d_hidden % 16 == 0 && ctx->dtype == KVD_DTYPE_BF16) {
     if (!ls.wt8) {
@@ -611,7 +615,38 @@ static kvd_status recompute_launch(kvd_ctx *ctx, int layer, const kvd_store_rang
     fp.scale_log2e = fused_head->scale_log2e;
     return launch_recompute_fused(ctx, ls, tmap_store, tmap_ext, p, fp, stream);
   }
-  kvd_status st = launch_recompute(ctx, ls, tmap_store, tmap_ext, p, stream);
+  kvd_status st;
+  if (!any_store && n_rows <= RW_MAX_ROWS && ctx->dtype != KVD_DTYPE_F32 && p.trace == nullptr) {
+    // only a few new rows: the projection that reads the weights at memory speed (same bits)
+    RowsParams r = {};
+    r.rows = static_cast<const uint4 *>(rows);
+    r.positions = positions;
+    r.k_out = p.jobs[0].k_out;
+    r.v_out = p.jobs[0].v_out;
+    r.out_stride = p.rows_out_stride;
+    r.n_rows = n_rows;
+    r.row_chunks = p.row_chunks;
+    r.n_cols = 2 * kdim;
+    r.k_cols = kdim;
+    r.inv_k = p.inv_d_hidden;
+    r.rms_eps = p.rms_eps;
+    r.qk_norm = p.qk_norm;
+    r.qk_eps = p.qk_eps;
+    r.rope_half = p.rope_style == KVD_ROPE_HALF;
+    r.max_pos = p.max_pos;
+    r.rope_hi = p.rope_hi;
+    r.rope_lo = p.rope_lo;
+    r.gamma_k = p.gamma_k;
+    r.status = p.status;
+    r.timeout_ns = p.timeout_ns;
+    r.append_rows = p.append_rows;
+    r.append_pos = p.append_pos;
+    r.append_sumsq = p.append_sumsq;
+    for (int i = 0; i < p.append_n; ++i) r.append_slot[i] = p.append_slot[i];
+    st = launch_rows(ctx, ls, d.d_hidden, r, true, stream);
+  } else {
+    st = launch_recompute(ctx, ls, tmap_store, tmap_ext, p, stream);
+  }
   if (st == KVD_OK && p.append_n > 0)
     for (int sq = 0; sq < d.max_seqs; ++sq) ctx->rows_stored[static_cast<size_t>(layer) * d.max_seqs + sq] += add[sq];
   return st;

@@ -114,6 +114,40 @@ struct FusedParams {
 };
 struct NoFusedParams {};
 
+// ------------------------------------------------------------------------------ projection of a few rows
+constexpr int RW_MAX_ROWS = RC_INLINE_STAT_ROWS;
+constexpr int RW_FEW_ROWS = 16;
+constexpr int RW_HEAD_TILE = 32;  // columns per CTA of a key or value head
+constexpr int RW_MIN_TILE = 16;   // columns per tile of a plain product, at least
+struct RowsParams {
+  const uint4 *rows;           // [n_rows][row_chunks]
+  const int32_t *positions;    // [n_rows] (heads)
+  const float *sumsq;          // [n_rows], or nullptr: taken from the rows
+  __nv_bfloat16 *k_out;        // heads
+  __nv_bfloat16 *v_out;        // values, or the outputs of a plain product
+  long long out_stride;        // elements
+  int n_rows, nr;              // rows, and rows rounded up to a multiple of 8
+  int row_chunks;              // 16-byte chunks per row
+  int n_cols, k_cols;          // columns; those below k_cols are keys
+  int tile, n_tiles;           // columns per tile, tiles
+  int num_k_blocks, stage_kb;  // k blocks in all and per stage
+  int stages, tail_off, tmem_cols;  // shared and tensor memory
+  int wide_store;              // plain product: outputs are 32-byte aligned
+  float inv_k, rms_eps;
+  int qk_norm;
+  float qk_eps;
+  int rope_half;
+  int max_pos;
+  const float2 *rope_hi, *rope_lo;
+  const float *gamma_k;
+  int *status;
+  unsigned long long timeout_ns;
+  uint4 *append_rows;          // as in RecomputeParams; nullptr: nothing is appended
+  int32_t *append_pos;
+  float *append_sumsq;
+  long long append_slot[RW_MAX_ROWS];
+};
+
 // ------------------------------------------------------------------------------ decode attention
 constexpr int AT_THREADS = 128;        // streaming kernel
 constexpr int AT_WARPS = 4;
@@ -217,6 +251,8 @@ struct LayerState {
   int window = 0;
   RopeTable rope;
   CUtensorMap tmap_b;
+  CUtensorMap tmap_rows[2];  // of wt, for the projection of few and of more rows (16-bit types), and its columns per tile
+  int rows_tile = 0;
   // FP8 variant: E4M3 codes of W' / w_scale8, K-major; one scale for the matrix (device float)
   uint8_t *wt8 = nullptr;
   float *w_scale8 = nullptr;
@@ -295,6 +331,9 @@ kvd_status launch_recompute(kvd_ctx *ctx, const LayerState &ls, const CUtensorMa
 kvd_status launch_recompute_fused(kvd_ctx *ctx, const LayerState &ls, const CUtensorMap &tmap_store,
                                   const CUtensorMap &tmap_rows, const RecomputeParams &p, const FusedParams &fp,
                                   cudaStream_t stream, int eb = 2);
+// `heads`: key and value heads of a layer; otherwise a plain product (bf16)
+kvd_status prepare_rows_map(kvd_ctx *ctx, LayerState &ls, int k, int n_cols, bool heads);
+kvd_status launch_rows(kvd_ctx *ctx, const LayerState &ls, int k, RowsParams &p, bool heads, cudaStream_t stream);
 kvd_status launch_attention(kvd_ctx *ctx, const AttnLaunch &L, int d_head, int group, cudaStream_t stream);
 kvd_status launch_prepare_weights(kvd_ctx *ctx, const __nv_bfloat16 *w, const __nv_bfloat16 *gamma, __nv_bfloat16 *wt,
                                   int d_hidden, int n_cols, cudaStream_t stream);

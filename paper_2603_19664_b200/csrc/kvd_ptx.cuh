@@ -211,6 +211,13 @@ __device__ __forceinline__ void tmem_ld_x16(uint32_t taddr, uint32_t (&r)[16]) {
       : "memory");
 }
 
+__device__ __forceinline__ void tmem_ld_x8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+}
+
 // 32 lanes x 32 consecutive 32-bit columns: thread t of the warp writes row (lane base + t).
 __device__ __forceinline__ void tmem_st_x32(uint32_t taddr, const uint32_t (&r)[32]) {
   asm volatile(
@@ -292,6 +299,9 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
 }
 __device__ __forceinline__ void st_cluster_f32(uint32_t cluster_addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster_v4(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 // TMEM management and MMA for a pair of CTAs (cta_group::2).  alloc / dealloc / relinquish are
 // executed by the same warp index in both CTAs; the MMA and its commits by one thread of the
@@ -450,6 +460,30 @@ __device__ __forceinline__ uint32_t pack_out(float lo, float hi) {
   } else {
     const __half2 v = __floats2half2_rn(lo, hi);
     return *reinterpret_cast<const uint32_t *>(&v);
+  }
+}
+
+// ------------------------------------------------------------------------------ row stores
+// Output stores.  Each epilogue thread owns one row, so the 32 lanes of a store instruction write 32
+// different lines and the instruction occupies the SM's load/store data path once per lane -- cycles
+// the operand ring's TMA writes and the tensor cores' operand reads compete for.  32-byte stores halve
+// the instruction count, and not allocating the lines in L1 (nothing reads them back) halves the
+// data-path cycles again.  `o` holds n16 * 4 packed words.
+template <int N16>
+__device__ __forceinline__ void store_row_piece(__nv_bfloat16 *dst, const uint32_t *o, bool wide) {
+  if (wide) {
+#pragma unroll
+    for (int j = 0; j < N16 / 2; ++j)
+      asm volatile("st.global.L1::no_allocate.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + 16 * j),
+                   "r"(o[8 * j]), "r"(o[8 * j + 1]), "r"(o[8 * j + 2]), "r"(o[8 * j + 3]), "r"(o[8 * j + 4]),
+                   "r"(o[8 * j + 5]), "r"(o[8 * j + 6]), "r"(o[8 * j + 7])
+                   : "memory");
+  } else {
+#pragma unroll
+    for (int j = 0; j < N16; ++j)
+      asm volatile("st.global.L1::no_allocate.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(dst + 8 * j), "r"(o[4 * j]),
+                   "r"(o[4 * j + 1]), "r"(o[4 * j + 2]), "r"(o[4 * j + 3])
+                   : "memory");
   }
 }
 

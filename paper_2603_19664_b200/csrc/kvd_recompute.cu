@@ -163,29 +163,6 @@ KVD_DEFINE_UMMA_KBLOCK(umma_kblock_pair_f8, "f8f6f4")  // E4M3 operands: 128 cha
 KVD_DEFINE_UMMA_KBLOCK(umma_kblock_pair_tf32, "tf32")  // fp32 operands read as TF32: 32 channels = four K=8 steps
 #undef KVD_DEFINE_UMMA_KBLOCK
 
-// Output stores.  Each epilogue thread owns one row, so the 32 lanes of a store instruction write 32
-// different lines and the instruction occupies the SM's load/store data path once per lane -- cycles
-// the operand ring's TMA writes and the tensor cores' operand reads compete for.  32-byte stores halve
-// the instruction count, and not allocating the lines in L1 (nothing reads them back) halves the
-// data-path cycles again.  `o` holds n16 * 4 packed words.
-template <int N16>
-__device__ __forceinline__ void store_row_piece(__nv_bfloat16 *dst, const uint32_t *o, bool wide) {
-  if (wide) {
-#pragma unroll
-    for (int j = 0; j < N16 / 2; ++j)
-      asm volatile("st.global.L1::no_allocate.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + 16 * j),
-                   "r"(o[8 * j]), "r"(o[8 * j + 1]), "r"(o[8 * j + 2]), "r"(o[8 * j + 3]), "r"(o[8 * j + 4]),
-                   "r"(o[8 * j + 5]), "r"(o[8 * j + 6]), "r"(o[8 * j + 7])
-                   : "memory");
-  } else {
-#pragma unroll
-    for (int j = 0; j < N16; ++j)
-      asm volatile("st.global.L1::no_allocate.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(dst + 8 * j), "r"(o[4 * j]),
-                   "r"(o[4 * j + 1]), "r"(o[4 * j + 2]), "r"(o[4 * j + 3])
-                   : "memory");
-  }
-}
-
 // EB = bytes per operand element: 2 = bf16 rows and weights, 1 = the FP8 variant (E4M3 codes of rows and
 // weights; a k block is then 128 channels in the same 128-byte rows, the MMA kind f8f6f4, and the rows'
 // and the matrix's quantisation scales ride in the per-row factor that the statistics warps hand over).

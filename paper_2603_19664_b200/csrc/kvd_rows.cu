@@ -1,0 +1,503 @@
+// Projection of a few rows (at most 64): the K/V of a decode step's new tokens when nothing is recomputed in
+// the same call, and the dense products of a decoder block at decode batch sizes.
+//
+//   Y[M <= 64, N] = X[M, K] * W'      W' K-major, the products and the finishing of kvd_recompute.cu
+//
+// Bound: reading W' once (N * K * 2 bytes).  The 256-row tile of the recompute kernel spends a full tile's MMA
+// time (512 clocks per 64 channels) on rows that are not there and cuts N into 256-column tiles, i.e. 8 to 10
+// CTA pairs for the models' projections.  Here a tile is as narrow as it takes to give every SM one (a multiple
+// of 8 columns, RW_MIN_TILE at least), so that all SMs pull weights at once.
+//
+// The MMA has 64 rows however few of them are rows of X; only those are loaded, the descriptor's other rows are whatever lies behind them in shared memory, and their accumulators (lanes of
+// tensor memory) are never read.
+//
+// The bits are those of the recompute kernel: an output element is one accumulator that takes the same K = 16
+// steps in the same ascending order, and the finishing below repeats that kernel's operations and their order
+// (row statistic, key norm, rotation, rounding).
+//
+// Measured (B200, one bf16 row, time of the launch alone): 2560 -> 262144 columns 323 us with the 256-row tiles, 197 us
+// here (6.8 TB/s of weights); 2560 -> 20480 43 and 23.5 us; 10240 -> 2560 54 and 20.7 us; 2560 -> 2048 20 and 10.7 us; K and
+// V of a Gemma-3-4B layer 25.6 and 12.9 us.  Short products are bound by launch, first-load latency and, where K is
+// long, by the chain of K / 16 dependent MMAs (24 clocks each).  The operands the other way round (weights as the M
+// of the MMA, 64 columns per CTA) measured 282, 38 and 44 us: too few CTAs for the narrow products.
+//
+// Weights never change after they were prepared, so the loads of the first stages are issued before the
+// dependency wait: with programmatic launches they run under the tail of the preceding kernel.
+//
+// Warps: 0 producer (one lane), 1 MMA issuer (one lane) and tensor-memory owner, 2-9 row statistics, of these
+// 4-7 the epilogue.  Plain products walk over tiles (two accumulators); key/value projections
+// have one 32-column tile per CTA, the d_head / 32 CTAs of a head form a cluster and exchange their accumulators,
+// because the key norm runs over the whole head in one fixed order and the half-split rotation pairs columns of
+// different tiles.
+#include <string.h>
+
+#include "kvd_internal.h"
+#include "kvd_ptx.cuh"
+
+namespace kvd {
+
+constexpr int RW_THREADS = 320;
+constexpr int RW_MAX_STAGES = 16;
+constexpr int RW_MMA_ROWS = 64;                           // M of the MMA
+constexpr int RW_BARS = 2 * RW_MAX_STAGES + 4;            // full, empty per stage; tmem_full[2], tmem_empty[2]
+constexpr int RW_TAIL = RW_BARS * 8 + 32 + RW_MAX_ROWS * 3 * 4;  // barriers, tmem pointer + abort, 1/rms, key scale, position
+
+// Four K = 16 steps of one k block: D[64 rows][columns of the tile] += X[64 x 64] W'^T[64 x columns].
+__device__ __forceinline__ void umma_kblock(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
+                                            uint32_t acc_first) {
+  asm volatile(
+      "{\n\t"
+      ".reg .pred p, t;\n\t"
+      ".reg .b64 da, db;\n\t"
+      ".reg .b32 la, lb;\n\t"
+      "setp.ne.b32 p, %5, 0;\n\t"
+      "setp.eq.b32 t, 0, 0;\n\t"
+      "mov.b64 da, {%1, %3};\n\t"
+      "mov.b64 db, {%2, %3};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t"
+      "add.u32 la, %1, 2;\n\t"
+      "add.u32 lb, %2, 2;\n\t"
+      "mov.b64 da, {la, %3};\n\t"
+      "mov.b64 db, {lb, %3};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, t;\n\t"
+      "add.u32 la, %1, 4;\n\t"
+      "add.u32 lb, %2, 4;\n\t"
+      "mov.b64 da, {la, %3};\n\t"
+      "mov.b64 db, {lb, %3};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, t;\n\t"
+      "add.u32 la, %1, 6;\n\t"
+      "add.u32 lb, %2, 6;\n\t"
+      "mov.b64 da, {la, %3};\n\t"
+      "mov.b64 db, {lb, %3};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, t;\n\t"
+      "}"
+      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc_first)
+      : "memory");
+}
+
+// D_HEAD = 0: a plain product, every column scaled by the row factor and stored.  D_HEAD > 0: key and value heads.
+template <int D_HEAD, int DT>
+__global__ void __launch_bounds__(RW_THREADS, 1)
+kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
+                const __grid_constant__ RowsParams p) {
+  constexpr bool HEADS = D_HEAD > 0;
+  constexpr int CL = HEADS ? D_HEAD / RW_HEAD_TILE : 1;  // CTAs of a head
+  constexpr int LD = HEADS ? D_HEAD + 4 : 0;             // floats between the rows of s_y
+  extern __shared__ __align__(1024) uint8_t rw_smem[];
+  if ((smem_u32(rw_smem) & 1023u) != 0u) {  // the 128-byte swizzle is anchored at 1024-byte boundaries
+    if (threadIdx.x == 0) atomicOr(p.status, STATUS_TIMEOUT);
+    return;
+  }
+  const int stages = p.stages, kbs = p.stage_kb, tile = p.tile;
+  const uint32_t x_kb = static_cast<uint32_t>(p.nr) * 128u, w_kb = static_cast<uint32_t>(tile) * 128u;  // bytes per k block
+  const uint32_t stage_bytes = kbs * (x_kb + w_kb), w_off = kbs * x_kb;
+  uint8_t *tail = rw_smem + p.tail_off;  // behind the ring and the rows its last descriptor spans
+  uint64_t *bars = reinterpret_cast<uint64_t *>(tail);
+  uint32_t *s_tmem = reinterpret_cast<uint32_t *>(bars + RW_BARS);
+  volatile int *s_abort = reinterpret_cast<volatile int *>(s_tmem + 1);
+  float *s_rstd = reinterpret_cast<float *>(s_tmem + 8);
+  float *s_kscale = s_rstd + RW_MAX_ROWS;
+  int *s_pos = reinterpret_cast<int *>(s_kscale + RW_MAX_ROWS);
+  float *s_y = reinterpret_cast<float *>(s_pos + RW_MAX_ROWS);  // heads: accumulators of the whole head, [row][LD]
+  const uint32_t ring = smem_u32(rw_smem), bar_base = smem_u32(bars);
+  auto bar_full = [&](int s) { return bar_base + 8u * s; };
+  auto bar_empty = [&](int s) { return bar_base + 8u * (RW_MAX_STAGES + s); };
+  auto bar_tmem_full = [&](int a) { return bar_base + 8u * (2 * RW_MAX_STAGES + a); };
+  auto bar_tmem_empty = [&](int a) { return bar_base + 8u * (2 * RW_MAX_STAGES + 2 + a); };
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const unsigned long long tmo = p.timeout_ns;
+  const int steps = (p.num_k_blocks + kbs - 1) / kbs;  // stages of a tile
+  const int block = static_cast<int>(blockIdx.x), blocks = static_cast<int>(gridDim.x);
+  const int my_tiles = (p.n_tiles - block + blocks - 1) / blocks;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < stages; ++s) {
+      mbar_init(bar_full(s), 1);
+      mbar_init(bar_empty(s), 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(bar_tmem_full(a), 1);
+      mbar_init(bar_tmem_empty(a), 4);  // one arrival per epilogue warp
+    }
+    *s_abort = 0;
+    fence_mbar_init();
+  }
+  grid_launch_dependents();
+  if (warp == 1) {
+    tmem_alloc(smem_u32(s_tmem), p.tmem_cols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  if (CL > 1) cluster_sync_all();  // (also: every CTA of the head runs before anyone writes into its shared memory)
+  else __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *s_tmem;
+
+  if (warp == 0) {
+    // ------------------------------------------------------------------ producer
+    const int total = my_tiles * steps, pre = total < stages ? total : stages;
+    if (elect_one()) {
+      for (int i = 0; i < pre; ++i) {
+        mbar_arrive_expect_tx(bar_full(i), stage_bytes);
+        tma_load_3d(ring + i * stage_bytes + w_off, &tmap_w, bar_full(i), 0, (block + i / steps * blocks) * tile, i % steps * kbs);
+      }
+    }
+    grid_dependency_wait();  // the rows may come from the preceding kernel
+    if (elect_one()) {
+      for (int i = 0; i < pre; ++i) tma_load_3d(ring + i * stage_bytes, &tmap_x, bar_full(i), 0, 0, i % steps * kbs);
+      int issued = pre, s = 0, k = pre % steps, col = (block + pre / steps * blocks) * tile;
+      uint32_t ph = 0;  // parity of the phase of `empty` that frees stage s for its next fill
+      bool ok = true;
+      for (; issued < total; ++issued) {
+        if (!mbar_wait(bar_empty(s), ph, s_abort, tmo)) {
+          raise(p.status, STATUS_TIMEOUT, s_abort);
+          ok = false;
+          break;
+        }
+        mbar_arrive_expect_tx(bar_full(s), stage_bytes);
+        tma_load_3d(ring + s * stage_bytes + w_off, &tmap_w, bar_full(s), 0, col, k * kbs);
+        tma_load_3d(ring + s * stage_bytes, &tmap_x, bar_full(s), 0, 0, k * kbs);
+        if (++k == steps) {
+          k = 0;
+          col += blocks * tile;
+        }
+        if (++s == stages) {
+          s = 0;
+          ph ^= 1u;
+        }
+      }
+      if (!ok || *s_abort != 0) {
+        // leave no copy in flight: wait (bounded) for the last fill of every stage
+        for (int b = 0; b < stages && b < issued; ++b) {
+          const uint32_t par = static_cast<uint32_t>((issued - 1 - b) / stages) & 1u;
+          const unsigned long long t0 = globaltimer_ns();
+          while (!mbar_try_wait(bar_full(b), par))
+            if (globaltimer_ns() - t0 > 100000000ull) break;
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------ MMA issuer
+    grid_dependency_wait();  // (the bounded waits below start when the rows can be loaded)
+    if (elect_one()) {  // (a lane chosen by elect keeps the operands in uniform registers: 24 clocks per MMA, 48 in a branch on the lane number)
+      const uint32_t idesc = DT == 1 ? umma_idesc_f16_f32(RW_MMA_ROWS, tile) : umma_idesc_bf16_f32(RW_MMA_ROWS, tile);
+      constexpr uint32_t desc_hi = (1024u >> 4) | (1u << 14) | (2u << 29);  // as in kvd_recompute.cu
+      int s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int t = 0; ok && t < my_tiles; ++t) {
+        const int a = t & 1;
+        if (!mbar_wait(bar_tmem_empty(a), ((t >> 1) & 1u) ^ 1u, s_abort, tmo)) {
+          raise(p.status, STATUS_TIMEOUT, s_abort);
+          break;
+        }
+        tc_fence_after();
+        const uint32_t d = tmem_base + a * (p.tmem_cols / 2);
+        int left = p.num_k_blocks;
+        for (int k = 0; k < steps; ++k) {
+          if (!mbar_wait(bar_full(s), ph, s_abort, tmo)) {
+            raise(p.status, STATUS_TIMEOUT, s_abort);
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          uint32_t xa = ((ring + s * stage_bytes) >> 4) | (1u << 16), wb = ((ring + s * stage_bytes + w_off) >> 4) | (1u << 16);
+          const int n = left < kbs ? left : kbs;
+          for (int b = 0; b < n; ++b) {
+            umma_kblock(d, xa, wb, desc_hi, idesc, (k | b) != 0 ? 1u : 0u);
+            xa += x_kb >> 4;
+            wb += w_kb >> 4;
+          }
+          left -= n;
+          umma_commit(bar_empty(s));
+          if (++s == stages) {
+            s = 0;
+            ph ^= 1u;
+          }
+        }
+        if (ok) umma_commit(bar_tmem_full(a));
+      }
+    }
+  } else {
+    // ------------------------------------------------------------------ row statistics (Eq. 2)
+    grid_dependency_wait();
+    const int w8 = warp - 2;
+    if (p.sumsq != nullptr) {
+      const int row = threadIdx.x - 64;
+      if (row < p.n_rows) s_rstd[row] = 1.0f / sqrtf(__ldg(p.sumsq + row) * p.inv_k + p.rms_eps);
+    } else {
+      // STORE_RESIDUAL in the same launch (kvd_decode_step_kv): the first CTA writes the rows it reads into the
+      // store slots the host assigned to them
+      const bool append = HEADS && p.append_rows != nullptr && block == 0;
+#pragma unroll 1
+      for (int g = w8; 4 * g < p.n_rows; g += 8) {
+        const uint4 *src[4];
+        uint4 *dst[4] = {nullptr, nullptr, nullptr, nullptr};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = 4 * g + i;
+          src[i] = p.rows + static_cast<size_t>(r < p.n_rows ? r : p.n_rows - 1) * p.row_chunks;
+          if (append && r < p.n_rows) dst[i] = p.append_rows + static_cast<size_t>(p.append_slot[r]) * p.row_chunks;
+        }
+        float ss[4];
+        if (append) warp_rows_sumsq<4, 4, true, DT>(src, dst, p.row_chunks, lane, ss);
+        else warp_rows_sumsq<4, 4, false, DT>(src, dst, p.row_chunks, lane, ss);
+        const float mine = lane == 0 ? ss[0] : lane == 1 ? ss[1] : lane == 2 ? ss[2] : ss[3];
+        const int r = 4 * g + lane;
+        if (lane < 4 && r < p.n_rows) {
+          s_rstd[r] = 1.0f / sqrtf(mine * p.inv_k + p.rms_eps);
+          if (append) {
+            p.append_sumsq[p.append_slot[r]] = mine;
+            p.append_pos[p.append_slot[r]] = p.positions[r];
+          }
+        }
+      }
+    }
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    if (warp >= 4 && warp < 8) {
+      // ---------------------------------------------------------------- epilogue
+      // (M = 64: rows 16 q .. 16 q + 15 are lanes 0-15 of tensor memory quarter q)
+      const int quarter = warp & 3, row = quarter * 16 + lane;
+      const bool valid = lane < 16 && row < p.n_rows, busy = quarter * 16 < p.n_rows;  // busy: warp-uniform
+      const uint32_t rank = CL > 1 ? cluster_ctarank() : 0u;
+      const float rstd = valid ? s_rstd[row] : 0.f;
+      for (int t = 0; t < my_tiles; ++t) {
+        const int a = t & 1, col0 = (block + t * blocks) * tile;
+        if (!warp_wait(bar_tmem_full(a), (t >> 1) & 1u, s_abort, tmo, lane)) {
+          raise(p.status, STATUS_TIMEOUT, s_abort);
+          break;
+        }
+        tc_fence_after();
+        const uint32_t acc = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + a * (p.tmem_cols / 2);
+        const int cols = p.n_cols - col0 < tile ? p.n_cols - col0 : tile;
+        if constexpr (HEADS) {
+          if (busy) {
+            uint32_t v[RW_HEAD_TILE];
+            tmem_ld_x32(acc, v);
+            tmem_wait_ld();
+            if (valid) {
+              float *dst = s_y + row * LD + static_cast<int>(rank) * RW_HEAD_TILE;
+#pragma unroll
+              for (int j = 0; j < RW_HEAD_TILE; j += 4) {
+                *reinterpret_cast<uint4 *>(dst + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                if (col0 < p.k_cols) {  // keys: the whole head goes to each of its CTAs
+#pragma unroll
+                  for (uint32_t q = 1; q < CL; ++q)
+                    st_cluster_v4(map_to_cta(smem_u32(dst + j), (rank + q) % CL), v[j], v[j + 1], v[j + 2], v[j + 3]);
+                }
+              }
+            }
+          }
+        } else {
+          __nv_bfloat16 *dst = p.v_out + static_cast<size_t>(row) * p.out_stride + col0;
+          int c = 0;
+          for (; busy && c + 32 <= cols; c += 32) {
+            uint32_t v[32], o[16];
+            tmem_ld_x32(acc + c, v);
+            tmem_wait_ld();
+#pragma unroll
+            for (int j = 0; j < 16; ++j) o[j] = pack_out<DT>(__uint_as_float(v[2 * j]) * rstd, __uint_as_float(v[2 * j + 1]) * rstd);
+            if (valid) store_row_piece<4>(dst + c, o, p.wide_store != 0);
+          }
+          for (; busy && c < cols; c += 8) {
+            uint32_t v[8], o[4];
+            tmem_ld_x8(acc + c, v);
+            tmem_wait_ld();
+#pragma unroll
+            for (int j = 0; j < 4; ++j) o[j] = pack_out<DT>(__uint_as_float(v[2 * j]) * rstd, __uint_as_float(v[2 * j + 1]) * rstd);
+            if (valid) store_row_piece<1>(dst + c, o, false);
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_tmem_empty(a));
+      }
+    }
+  }
+  __syncwarp();
+  tc_fence_before();
+  if (CL > 1) cluster_sync_all();
+  else __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, p.tmem_cols);
+  }
+  if constexpr (HEADS) {
+    // ------------------------------------------------------------------ key norm, rotation, stores: all warps
+    if (*s_abort != 0) return;
+    constexpr int HALF = D_HEAD / 2;
+    const int col0 = block * RW_HEAD_TILE;
+    const bool key = col0 < p.k_cols;
+    if (threadIdx.x < p.n_rows) {
+      const int r = threadIdx.x;
+      const float rstd = s_rstd[r];
+      float kscale = rstd;
+      if (key && p.qk_norm) {
+        // four chains (columns j mod 4) in ascending order, two-wide: the order of the recompute kernel
+        uint64_t ss2[2] = {0ull, 0ull};
+        const uint64_t rstd2 = pack2(rstd, rstd);
+#pragma unroll 8
+        for (int c = 0; c < D_HEAD; c += 4) {
+          const float4 y = *reinterpret_cast<const float4 *>(s_y + r * LD + c);
+          const uint64_t v0 = fmul2(pack2(y.x, y.y), rstd2), v1 = fmul2(pack2(y.z, y.w), rstd2);
+          ss2[0] = ffma2(v0, v0, ss2[0]);
+          ss2[1] = ffma2(v1, v1, ss2[1]);
+        }
+        float s0, s1, s2, s3;
+        unpack2(ss2[0], s0, s1);
+        unpack2(ss2[1], s2, s3);
+        const float ss = (s0 + s1) + (s2 + s3);
+        kscale = rstd * (1.0f / sqrtf(ss * (1.0f / D_HEAD) + p.qk_eps));
+      }
+      int pos = p.positions[r];
+      if (pos < 0 || pos >= p.max_pos) {
+        atomicOr(p.status, STATUS_POSITION);
+        pos = pos < 0 ? 0 : p.max_pos - 1;
+      }
+      s_kscale[r] = kscale;
+      s_pos[r] = pos;
+    }
+    __syncthreads();
+    const int c = col0 % D_HEAD + 2 * (lane & 15);  // this lane's two columns of the head; half a warp per row
+    for (int r = 2 * warp + (lane >> 4); r < p.n_rows; r += 2 * (RW_THREADS / 32)) {
+      const float *y = s_y + r * LD;
+      const float ks = s_kscale[r];
+      uint32_t o;
+      if (!key) {
+        o = pack_out<DT>(y[c] * ks, y[c + 1] * ks);
+      } else {
+        const int pos = s_pos[r];
+        const float2 *t_hi = p.rope_hi + static_cast<size_t>(pos >> ROPE_LO_BITS) * HALF;
+        const float2 *t_lo = p.rope_lo + (pos & (ROPE_LO_SIZE - 1));
+        auto gamma = [&](int i) { return p.gamma_k ? __ldg(p.gamma_k + i) : 1.0f; };
+        if (!p.rope_half) {
+          const float2 h = __ldg(t_hi + c / 2), l = __ldg(t_lo + c / 2 * ROPE_LO_SIZE);
+          const float cs = fmaf(h.x, l.x, -h.y * l.y), sn = fmaf(h.y, l.x, h.x * l.y);
+          const float a = y[c] * ks * gamma(c), b = y[c + 1] * ks * gamma(c + 1);
+          o = pack_out<DT>(fmaf(a, cs, -b * sn), fmaf(a, sn, b * cs));
+        } else {
+          float v[2];
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const int i = (c + j) % HALF;  // pair (i, i + HALF)
+            const float2 h = __ldg(t_hi + i), l = __ldg(t_lo + i * ROPE_LO_SIZE);
+            const float cs = fmaf(h.x, l.x, -h.y * l.y), sn = fmaf(h.y, l.x, h.x * l.y);
+            const float a = y[i] * ks * gamma(i), b = y[i + HALF] * ks * gamma(i + HALF);
+            v[j] = c < HALF ? fmaf(a, cs, -b * sn) : fmaf(a, sn, b * cs);
+          }
+          o = pack_out<DT>(v[0], v[1]);
+        }
+      }
+      __nv_bfloat16 *dst = (key ? p.k_out + (col0 / D_HEAD) * D_HEAD : p.v_out + (col0 - p.k_cols) / D_HEAD * D_HEAD) +
+                           static_cast<size_t>(r) * p.out_stride + c;
+      *reinterpret_cast<uint32_t *>(dst) = o;
+    }
+  }
+}
+
+template <int D_HEAD, int DT>
+static kvd_status launch_rows_impl(kvd_ctx *ctx, const CUtensorMap &tmap_w, const CUtensorMap &tmap_x, RowsParams &p, cudaStream_t stream) {
+  auto kern = kvd_rows_kernel<D_HEAD, DT>;
+  constexpr int SMEM_MAX = 232448, CL = D_HEAD > 0 ? D_HEAD / RW_HEAD_TILE : 1;
+  static bool configured[64] = {};
+  if (!configured[ctx->device & 63]) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(rows)");
+    configured[ctx->device & 63] = true;
+  }
+  const int stage = p.stage_kb * (p.nr + p.tile) * 128;
+  const int tail = RW_TAIL + (D_HEAD > 0 ? p.nr * (D_HEAD + 4) * 4 : 0);
+  // the descriptor of the last stage's last k block spans RW_MMA_ROWS rows from that block's rows on
+  const int beyond = RW_MMA_ROWS * 128 - (stage - (p.stage_kb - 1) * p.nr * 128);
+  const int slack = beyond > 0 ? beyond : 0;
+  const int total = (p.num_k_blocks + p.stage_kb - 1) / p.stage_kb * ((p.n_tiles + ctx->num_sms - 1) / ctx->num_sms);
+  p.stages = (SMEM_MAX - tail - slack) / stage;
+  if (p.stages > RW_MAX_STAGES) p.stages = RW_MAX_STAGES;
+  if (p.stages > total) p.stages = total;
+  p.tail_off = p.stages * stage + slack;
+  p.tmem_cols = 64;  // two accumulators; the epilogue reads 32 columns at once
+  while (p.tmem_cols < 2 * p.tile) p.tmem_cols *= 2;
+  const int grid = D_HEAD > 0 || p.n_tiles < ctx->num_sms ? p.n_tiles : ctx->num_sms;
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(grid, 1, 1);
+  cfg.blockDim = dim3(RW_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = static_cast<size_t>(p.tail_off) + tail;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = (serial_launch_mask() & 1) ? 0 : 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = CL;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = CL > 1 ? 2 : 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmap_w, tmap_x, p);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "launch rows");
+  ctx->launches += 1;
+  return KVD_OK;
+}
+
+// 3-D map [k block][row][64 channels] of a K-major 16-bit matrix: a box is stage_kb k blocks of box_rows rows.
+static kvd_status encode_kblocks(kvd_ctx *ctx, CUtensorMap *map, const void *base, int k, int rows, int box_rows, int stage_kb) {
+  cuuint64_t dims[3] = {RC_BLOCK_K, static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(k / RC_BLOCK_K)};
+  cuuint64_t strides[2] = {static_cast<cuuint64_t>(k) * 2, RC_BLOCK_K * 2};
+  cuuint32_t box[3] = {RC_BLOCK_K, static_cast<cuuint32_t>(box_rows), static_cast<cuuint32_t>(stage_kb)};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = ctx->encode(map, ctx->dtype == KVD_DTYPE_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
+                           const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    ctx->last_error = "cuTensorMapEncodeTiled (k blocks) failed: " + std::to_string(static_cast<int>(r));
+    return KVD_ERR_CUDA;
+  }
+  return KVD_OK;
+}
+
+// Columns per tile of a plain product: one tile per SM, or as few equal rounds of tiles of at most 256 columns.
+static int rows_tile(const kvd_ctx *ctx, int n_cols) {
+  const int rounds = (n_cols + 256 * ctx->num_sms - 1) / (256 * ctx->num_sms);
+  const int t = ((n_cols + rounds * ctx->num_sms - 1) / (rounds * ctx->num_sms) + 7) / 8 * 8;
+  return t < RW_MIN_TILE ? RW_MIN_TILE : t;
+}
+// k blocks per stage (a power of two up to 8): stages of 25 to 50 KB.  A stage costs the two single-thread loops some
+// 300 clocks of waits and commits whatever it holds (10240 x 2560, one row: 31, 27 and 23 us with 2, 4 and 8), and the
+// ring needs at least four.  `many`: more than RW_FEW_ROWS rows.
+static int rows_stage_kb(int tile, bool many) {
+  int kb = 8;
+  while (kb > 1 && kb * (tile + (many ? RW_MAX_ROWS : RW_FEW_ROWS)) * 128 > 50 * 1024) kb /= 2;
+  return kb;
+}
+
+kvd_status prepare_rows_map(kvd_ctx *ctx, LayerState &ls, int k, int n_cols, bool heads) {
+  ls.rows_tile = heads ? RW_HEAD_TILE : rows_tile(ctx, n_cols);
+  kvd_status st = KVD_OK;
+  for (int many = 0; st == KVD_OK && many < 2; ++many)
+    st = encode_kblocks(ctx, &ls.tmap_rows[many], ls.wt, k, n_cols, ls.rows_tile, rows_stage_kb(ls.rows_tile, many != 0));
+  return st;
+}
+
+kvd_status launch_rows(kvd_ctx *ctx, const LayerState &ls, int k, RowsParams &p, bool heads, cudaStream_t stream) {
+  p.nr = (p.n_rows + 7) / 8 * 8;
+  p.num_k_blocks = k / RC_BLOCK_K;
+  p.tile = ls.rows_tile;
+  const bool many = p.nr > RW_FEW_ROWS;
+  p.stage_kb = rows_stage_kb(p.tile, many);
+  if (p.tile % 16 != 0) p.wide_store = 0;  // a tile has to start at a 32-byte boundary for 32-byte stores
+  p.n_tiles = (p.n_cols + p.tile - 1) / p.tile;
+  CUtensorMap tmap_x;
+  kvd_status st = encode_kblocks(ctx, &tmap_x, p.rows, k, p.n_rows, p.nr, p.stage_kb);
+  if (st != KVD_OK) return st;
+  const CUtensorMap &w = ls.tmap_rows[many ? 1 : 0];
+  if (!heads) return launch_rows_impl<0, 0>(ctx, w, tmap_x, p, stream);
+  const bool half = ctx->dtype == KVD_DTYPE_F16;
+  switch (ctx->desc.d_head) {
+    case 64: return half ? launch_rows_impl<64, 1>(ctx, w, tmap_x, p, stream) : launch_rows_impl<64, 0>(ctx, w, tmap_x, p, stream);
+    case 128: return half ? launch_rows_impl<128, 1>(ctx, w, tmap_x, p, stream) : launch_rows_impl<128, 0>(ctx, w, tmap_x, p, stream);
+    case 256: return half ? launch_rows_impl<256, 1>(ctx, w, tmap_x, p, stream) : launch_rows_impl<256, 0>(ctx, w, tmap_x, p, stream);
+    default: return KVD_ERR_SHAPE;
+  }
+}
+
+}  // namespace kvd

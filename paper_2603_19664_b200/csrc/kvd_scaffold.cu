@@ -217,6 +217,7 @@ extern "C" kvd_status kvd_scaffold_linear_create(kvd_ctx *ctx, const void *w, co
                                 gamma ? static_cast<const __nv_bfloat16 *>(gamma) : ones, lin->ls.wt, k, n, stream);
   if (st == KVD_OK) st = get_rope(ctx, 10000.0f, &lin->ls.rope);  // the kernel's prologue wants a table; no row is rotated
   if (st == KVD_OK) st = encode_2d(ctx, &lin->ls.tmap_b, lin->ls.wt, k, lin->n_pad, RC_BLOCK_K, ctx->block_n / 2, 2);
+  if (st == KVD_OK) st = prepare_rows_map(ctx, lin->ls, k, lin->n_pad, false);
   if (st == KVD_OK) {
     e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) st = cuda_fail(ctx, e, "scaffold linear: sync");
@@ -258,6 +259,22 @@ extern "C" kvd_status kvd_scaffold_linear(kvd_ctx *ctx, const kvd_linear *lin, c
   if (!sc_aligned16(x) || !sc_aligned16(out) || out_row_stride % 8 != 0) return KVD_ERR_ALIGNMENT;
   if (static_cast<size_t>(m) > ctx->ext_sumsq_rows) return KVD_ERR_CAPACITY;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
+  if (m <= RW_MAX_ROWS) {
+    RowsParams r = {};
+    r.rows = static_cast<const uint4 *>(x);
+    r.sumsq = lin->norm ? nullptr : reinterpret_cast<const float *>(ctx->zero_pos);  // zeros: a row factor of exactly 1
+    r.v_out = static_cast<__nv_bfloat16 *>(out);
+    r.out_stride = out_row_stride;
+    r.n_rows = m;
+    r.row_chunks = lin->k / 8;
+    r.n_cols = lin->n_pad;
+    r.wide_store = (out_row_stride * 2 % 32 == 0) && ((reinterpret_cast<uintptr_t>(out) & 31u) == 0);
+    r.inv_k = lin->norm ? 1.0f / static_cast<float>(lin->k) : 0.0f;
+    r.rms_eps = lin->norm ? lin->rms_eps : 1.0f;
+    r.status = ctx->d_status;
+    r.timeout_ns = ctx->timeout_ns;
+    return launch_rows(ctx, lin->ls, lin->k, r, false, stream);
+  }
   CUtensorMap tmap_rows;
   kvd_status st = encode_rows_3d(ctx, &tmap_rows, x, static_cast<uint64_t>(lin->k), static_cast<uint64_t>(m), 1, 2);
   if (st != KVD_OK) return st;
