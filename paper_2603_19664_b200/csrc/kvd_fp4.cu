@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(256, 2) kvd_checkpoint_fp4_kernel(const uint4 
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   grid_launch_dependents();
+  grid_dependency_wait();
   for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += warps) {
     const size_t off = static_cast<size_t>(r) * row_chunks;
     uint4 v[CPL];
@@ -117,6 +118,7 @@ __global__ void __launch_bounds__(256) kvd_expand_fp4_kernel(const uint32_t *__r
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   grid_launch_dependents();
+  grid_dependency_wait();
   for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < R.total_rows; i += warps) {
     int lo = 0, hi = R.n_ranges;
     while (hi - lo > 1) {
@@ -218,12 +220,12 @@ extern "C" kvd_status kvd_checkpoint_residual_fp4(kvd_ctx *ctx, int seq, int lay
   uint32_t *dc = reinterpret_cast<uint32_t *>(ctx->store4_codes + slot * (d / 2));
   uint8_t *db = ctx->store4_block + slot * (d / FP4_BLOCK);
   const uint4 *src = static_cast<const uint4 *>(rows);
+  cudaError_t e;
   if (row_chunks <= 320)
-    kvd_checkpoint_fp4_kernel<10><<<static_cast<unsigned>(blocks), 256, 0, stream>>>(
+    e = launch_dependent(kvd_checkpoint_fp4_kernel<10>, dim3(static_cast<unsigned>(blocks)), 256, stream,
         src, positions, dc, db, ctx->store4_pos + slot, ctx->store4_sumsq + slot, ctx->store4_scale + slot, row_chunks, n);
   else
     return KVD_ERR_SHAPE;  // rows wider than 2560 channels are not held in registers
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(ctx, e, "launch checkpoint_fp4");
   ctx->launches += 1;
   count += n;
@@ -288,10 +290,9 @@ extern "C" kvd_status kvd_recompute_kv_fp4(kvd_ctx *ctx, int layer, const kvd_st
   long long blocks = (static_cast<long long>(total) + 7) / 8;
   const long long cap = static_cast<long long>(ctx->num_sms) * 8;
   if (blocks > cap) blocks = cap;
-  kvd_expand_fp4_kernel<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(
+  cudaError_t e = launch_dependent(kvd_expand_fp4_kernel, dim3(static_cast<unsigned>(blocks)), 256, stream,
       reinterpret_cast<const uint32_t *>(ctx->store4_codes), ctx->store4_block, ctx->store4_pos, ctx->store4_sumsq,
       ctx->store4_scale, reinterpret_cast<uint4 *>(x), xp, xs, row_chunks, R);
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(ctx, e, "launch expand_fp4");
   ctx->launches += 1;
   CUtensorMap tmap_rows;

@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(256) kvd_checkpoint_kernel(const uint4 *__rest
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   grid_launch_dependents();  // the next kernel's set-up may overlap this copy
+  grid_dependency_wait();
   for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += warps) {
     if (!KVD_BOUNDS_OK(r < capacity, status)) continue;  // checking build: the row fits the sequence's slab
     const size_t off = static_cast<size_t>(r) * row_chunks;
@@ -97,6 +98,7 @@ __global__ void __launch_bounds__(256) kvd_checkpoint_scatter_kernel(const uint4
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   grid_launch_dependents();
+  grid_dependency_wait();
   for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += warps) {
     if (!KVD_BOUNDS_OK(P.slot[r] >= 0 && P.slot[r] < total_slots, status)) continue;  // checking build
     const size_t slot = static_cast<size_t>(P.slot[r]);
@@ -120,6 +122,7 @@ __global__ void __launch_bounds__(256) kvd_rowstats_kernel(const uint4 *__restri
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   grid_launch_dependents();
+  grid_dependency_wait();
   for (int r = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 2; r < n; r += 2 * warps) {
     const int r1 = r + 1 < n ? r + 1 : r;
     const uint4 *const src[2] = {rows + static_cast<size_t>(r) * row_chunks, rows + static_cast<size_t>(r1) * row_chunks};
@@ -155,6 +158,7 @@ __global__ void __launch_bounds__(256) kvd_checkpoint_fp8_kernel(const uint4 *__
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   grid_launch_dependents();
+  grid_dependency_wait();
   auto chunk_amax = [](const uint4 &v, float amax) {
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -341,16 +345,16 @@ kvd_status launch_checkpoint(kvd_ctx *ctx, const __nv_bfloat16 *rows, const int3
   const long long cap = static_cast<long long>(ctx->num_sms) * 8;
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
+  cudaError_t e;
   if (ctx->dtype == 2)
-    kvd_checkpoint_kernel<2><<<static_cast<unsigned>(blocks), 256, 0, stream>>>(
+    e = launch_dependent(kvd_checkpoint_kernel<2>, dim3(static_cast<unsigned>(blocks)), 256, stream,
         reinterpret_cast<const uint4 *>(rows), pos, reinterpret_cast<uint4 *>(dst_rows), dst_pos, dst_sumsq, d_hidden / 4, n, capacity, ctx->d_status);
   else if (ctx->dtype == 1)
-    kvd_checkpoint_kernel<1><<<static_cast<unsigned>(blocks), 256, 0, stream>>>(
+    e = launch_dependent(kvd_checkpoint_kernel<1>, dim3(static_cast<unsigned>(blocks)), 256, stream,
         reinterpret_cast<const uint4 *>(rows), pos, reinterpret_cast<uint4 *>(dst_rows), dst_pos, dst_sumsq, d_hidden / 8, n, capacity, ctx->d_status);
   else
-    kvd_checkpoint_kernel<0><<<static_cast<unsigned>(blocks), 256, 0, stream>>>(
+    e = launch_dependent(kvd_checkpoint_kernel<0>, dim3(static_cast<unsigned>(blocks)), 256, stream,
         reinterpret_cast<const uint4 *>(rows), pos, reinterpret_cast<uint4 *>(dst_rows), dst_pos, dst_sumsq, d_hidden / 8, n, capacity, ctx->d_status);
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(ctx, e, "launch checkpoint");
   ctx->launches += 1;
   return KVD_OK;
@@ -362,13 +366,13 @@ kvd_status launch_checkpoint_scatter(kvd_ctx *ctx, const __nv_bfloat16 *rows, co
   const uint4 *src = reinterpret_cast<const uint4 *>(rows);
   uint4 *dst = reinterpret_cast<uint4 *>(ctx->store_rows);
   const long long total = static_cast<long long>(ctx->layers_stored) * ctx->desc.max_seqs * ctx->desc.max_tokens_per_seq;
+  cudaError_t e;
   if (ctx->dtype == 2)
-    kvd_checkpoint_scatter_kernel<2><<<blocks, 256, 0, stream>>>(src, pos, dst, ctx->store_pos, ctx->store_sumsq, d_hidden / 4, n, total, ctx->d_status, slots);
+    e = launch_dependent(kvd_checkpoint_scatter_kernel<2>, dim3(blocks), 256, stream, src, pos, dst, ctx->store_pos, ctx->store_sumsq, d_hidden / 4, n, total, ctx->d_status, slots);
   else if (ctx->dtype == 1)
-    kvd_checkpoint_scatter_kernel<1><<<blocks, 256, 0, stream>>>(src, pos, dst, ctx->store_pos, ctx->store_sumsq, d_hidden / 8, n, total, ctx->d_status, slots);
+    e = launch_dependent(kvd_checkpoint_scatter_kernel<1>, dim3(blocks), 256, stream, src, pos, dst, ctx->store_pos, ctx->store_sumsq, d_hidden / 8, n, total, ctx->d_status, slots);
   else
-    kvd_checkpoint_scatter_kernel<0><<<blocks, 256, 0, stream>>>(src, pos, dst, ctx->store_pos, ctx->store_sumsq, d_hidden / 8, n, total, ctx->d_status, slots);
-  cudaError_t e = cudaGetLastError();
+    e = launch_dependent(kvd_checkpoint_scatter_kernel<0>, dim3(blocks), 256, stream, src, pos, dst, ctx->store_pos, ctx->store_sumsq, d_hidden / 8, n, total, ctx->d_status, slots);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "launch checkpoint (batch)");
   ctx->launches += 1;
   return KVD_OK;
@@ -380,16 +384,16 @@ kvd_status launch_rowstats(kvd_ctx *ctx, const __nv_bfloat16 *rows, float *sumsq
   const long long cap = static_cast<long long>(ctx->num_sms) * 8;
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
+  cudaError_t e;
   if (ctx->dtype == 2)
-    kvd_rowstats_kernel<2><<<static_cast<unsigned>(blocks), 256, 0, stream>>>(reinterpret_cast<const uint4 *>(rows), sumsq,
+    e = launch_dependent(kvd_rowstats_kernel<2>, dim3(static_cast<unsigned>(blocks)), 256, stream, reinterpret_cast<const uint4 *>(rows), sumsq,
                                                                               d_hidden / 4, n);
   else if (ctx->dtype == 1)
-    kvd_rowstats_kernel<1><<<static_cast<unsigned>(blocks), 256, 0, stream>>>(reinterpret_cast<const uint4 *>(rows), sumsq,
+    e = launch_dependent(kvd_rowstats_kernel<1>, dim3(static_cast<unsigned>(blocks)), 256, stream, reinterpret_cast<const uint4 *>(rows), sumsq,
                                                                               d_hidden / 8, n);
   else
-    kvd_rowstats_kernel<0><<<static_cast<unsigned>(blocks), 256, 0, stream>>>(reinterpret_cast<const uint4 *>(rows), sumsq,
+    e = launch_dependent(kvd_rowstats_kernel<0>, dim3(static_cast<unsigned>(blocks)), 256, stream, reinterpret_cast<const uint4 *>(rows), sumsq,
                                                                               d_hidden / 8, n);
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(ctx, e, "launch rowstats");
   ctx->launches += 1;
   return KVD_OK;
@@ -403,15 +407,15 @@ kvd_status launch_checkpoint_fp8(kvd_ctx *ctx, const __nv_bfloat16 *rows, const 
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
   const int row_chunks = d_hidden / 8;
+  cudaError_t e;
   if (row_chunks <= 320)
-    kvd_checkpoint_fp8_kernel<10><<<static_cast<unsigned>(blocks), 256, 0, stream>>>(
+    e = launch_dependent(kvd_checkpoint_fp8_kernel<10>, dim3(static_cast<unsigned>(blocks)), 256, stream,
         reinterpret_cast<const uint4 *>(rows), pos, reinterpret_cast<uint2 *>(dst_codes), dst_pos, dst_sumsq, dst_scale,
         row_chunks, n);
   else
-    kvd_checkpoint_fp8_kernel<0><<<static_cast<unsigned>(blocks), 256, 0, stream>>>(
+    e = launch_dependent(kvd_checkpoint_fp8_kernel<0>, dim3(static_cast<unsigned>(blocks)), 256, stream,
         reinterpret_cast<const uint4 *>(rows), pos, reinterpret_cast<uint2 *>(dst_codes), dst_pos, dst_sumsq, dst_scale,
         row_chunks, n);
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(ctx, e, "launch checkpoint_fp8");
   ctx->launches += 1;
   return KVD_OK;

@@ -26,15 +26,18 @@ static inline bool sc_aligned16(const void *p) { return (reinterpret_cast<uintpt
 namespace kvd {
 
 // ---------------------------------------------------------------------------------- elementwise kernels
-// One CTA per (row, query head), one thread per rotation pair.  The sum of squares over the head is
+// One CTA per (row, query head), one thread per rotation pair.  (The rows and positions are not __restrict__: their
+// loads stay behind the dependency wait.)  The sum of squares over the head is
 // reduced in a fixed order (shuffle tree inside a warp, warps added in index order).
-__global__ void __launch_bounds__(128) kvd_query_finish_kernel(const __nv_bfloat16 *__restrict__ q_in, long long in_stride,
-                                                               const int32_t *__restrict__ positions,
+__global__ void __launch_bounds__(128) kvd_query_finish_kernel(const __nv_bfloat16 *q_in, long long in_stride,
+                                                               const int32_t *positions,
                                                                const __nv_bfloat16 *__restrict__ gamma_q, float eps,
                                                                const float2 *__restrict__ rope_hi,
                                                                const float2 *__restrict__ rope_lo, int max_pos,
                                                                int d_head, int n_q, int half_style,
                                                                __nv_bfloat16 *__restrict__ q_out, int *status) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   __shared__ float s_part[4];
   const int r = blockIdx.x / n_q, h = blockIdx.x % n_q;
   const int i = threadIdx.x, half = d_head / 2;
@@ -69,6 +72,8 @@ __global__ void __launch_bounds__(128) kvd_query_finish_kernel(const __nv_bfloat
 
 __global__ void __launch_bounds__(256) kvd_add_rows_kernel(uint4 *__restrict__ h, const uint4 *__restrict__ y,
                                                            long long y_stride_chunks, int m, int chunks) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   const long long total = static_cast<long long>(m) * chunks;
   for (long long idx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; idx < total;
        idx += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -92,6 +97,8 @@ __device__ __forceinline__ float act_apply(float v, int activation) {
 __global__ void __launch_bounds__(256) kvd_gated_act_kernel(const uint4 *__restrict__ gate_up, long long stride_chunks,
                                                             int m, int width_chunks, int activation,
                                                             uint4 *__restrict__ out) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   const long long total = static_cast<long long>(m) * width_chunks;
   for (long long idx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; idx < total;
        idx += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -113,6 +120,8 @@ __global__ void __launch_bounds__(256) kvd_gated_act_kernel(const uint4 *__restr
 __global__ void __launch_bounds__(256) kvd_embed_kernel(const uint4 *__restrict__ table, const int32_t *__restrict__ tokens,
                                                         int m, int chunks, int vocab, uint4 *__restrict__ out,
                                                         int *status) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   const long long total = static_cast<long long>(m) * chunks;
   for (long long idx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; idx < total;
        idx += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -176,8 +185,7 @@ static unsigned grid_for(long long items, int per_block, int num_sms) {
 
 }  // namespace kvd
 
-static kvd_status sc_launched(kvd_ctx *ctx, const char *what) {
-  cudaError_t e = cudaGetLastError();
+static kvd_status sc_launched(kvd_ctx *ctx, cudaError_t e, const char *what) {
   if (e != cudaSuccess) return cuda_fail(ctx, e, what);
   ctx->launches += 1;
   return KVD_OK;
@@ -340,11 +348,11 @@ extern "C" kvd_status kvd_scaffold_query_finish(kvd_ctx *ctx, int layer, const v
   const kvd_model_desc &d = ctx->desc;
   if (!q_in || !positions || !q_out || in_row_stride < static_cast<int64_t>(d.n_q_heads) * d.d_head) return KVD_ERR_INVALID_ARG;
   const int max_pos = ls.rope.n_hi * ROPE_LO_SIZE < d.max_tokens_per_seq ? ls.rope.n_hi * ROPE_LO_SIZE : d.max_tokens_per_seq;
-  kvd_query_finish_kernel<<<static_cast<unsigned>(m) * d.n_q_heads, d.d_head / 2, 0, static_cast<cudaStream_t>(stream_)>>>(
+  cudaError_t e = launch_dependent(kvd_query_finish_kernel, dim3(static_cast<unsigned>(m) * d.n_q_heads), d.d_head / 2, static_cast<cudaStream_t>(stream_),
       static_cast<const __nv_bfloat16 *>(q_in), in_row_stride, positions, static_cast<const __nv_bfloat16 *>(gamma_q),
       d.qk_norm_eps, ls.rope.hi, ls.rope.lo, max_pos, d.d_head, d.n_q_heads, d.rope_style == KVD_ROPE_HALF ? 1 : 0,
       static_cast<__nv_bfloat16 *>(q_out), ctx->d_status);
-  return sc_launched(ctx, "launch query_finish");
+  return sc_launched(ctx, e, "launch query_finish");
 }
 
 extern "C" kvd_status kvd_scaffold_add_rows(kvd_ctx *ctx, void *h, const void *y, int64_t y_row_stride, int m, int d,
@@ -354,9 +362,9 @@ extern "C" kvd_status kvd_scaffold_add_rows(kvd_ctx *ctx, void *h, const void *y
   if (!h || !y || y_row_stride < d) return KVD_ERR_INVALID_ARG;
   if (d % 8 != 0 || y_row_stride % 8 != 0 || !sc_aligned16(h) || !sc_aligned16(y)) return KVD_ERR_ALIGNMENT;
   const int chunks = d / 8;
-  kvd_add_rows_kernel<<<grid_for(static_cast<long long>(m) * chunks, 256, ctx->num_sms), 256, 0, static_cast<cudaStream_t>(stream_)>>>(
+  cudaError_t e = launch_dependent(kvd_add_rows_kernel, dim3(grid_for(static_cast<long long>(m) * chunks, 256, ctx->num_sms)), 256, static_cast<cudaStream_t>(stream_),
       static_cast<uint4 *>(h), static_cast<const uint4 *>(y), y_row_stride / 8, m, chunks);
-  return sc_launched(ctx, "launch add_rows");
+  return sc_launched(ctx, e, "launch add_rows");
 }
 
 extern "C" kvd_status kvd_scaffold_gated_act(kvd_ctx *ctx, const void *gate_up, int64_t row_stride, int m, int width,
@@ -367,9 +375,9 @@ extern "C" kvd_status kvd_scaffold_gated_act(kvd_ctx *ctx, const void *gate_up, 
   if (!gate_up || !out || row_stride < 2 * static_cast<int64_t>(width)) return KVD_ERR_INVALID_ARG;
   if (width % 8 != 0 || row_stride % 8 != 0 || !sc_aligned16(gate_up) || !sc_aligned16(out)) return KVD_ERR_ALIGNMENT;
   const int wc = width / 8;
-  kvd_gated_act_kernel<<<grid_for(static_cast<long long>(m) * wc, 256, ctx->num_sms), 256, 0, static_cast<cudaStream_t>(stream_)>>>(
+  cudaError_t e = launch_dependent(kvd_gated_act_kernel, dim3(grid_for(static_cast<long long>(m) * wc, 256, ctx->num_sms)), 256, static_cast<cudaStream_t>(stream_),
       static_cast<const uint4 *>(gate_up), row_stride / 8, m, wc, activation, static_cast<uint4 *>(out));
-  return sc_launched(ctx, "launch gated_act");
+  return sc_launched(ctx, e, "launch gated_act");
 }
 
 extern "C" kvd_status kvd_scaffold_embed(kvd_ctx *ctx, const void *table, const int32_t *tokens, int m, int d, int vocab,
@@ -379,9 +387,9 @@ extern "C" kvd_status kvd_scaffold_embed(kvd_ctx *ctx, const void *table, const 
   if (!table || !tokens || !out) return KVD_ERR_INVALID_ARG;
   if (d % 8 != 0 || !sc_aligned16(table) || !sc_aligned16(out)) return KVD_ERR_ALIGNMENT;
   const int chunks = d / 8;
-  kvd_embed_kernel<<<grid_for(static_cast<long long>(m) * chunks, 256, ctx->num_sms), 256, 0, static_cast<cudaStream_t>(stream_)>>>(
+  cudaError_t e = launch_dependent(kvd_embed_kernel, dim3(grid_for(static_cast<long long>(m) * chunks, 256, ctx->num_sms)), 256, static_cast<cudaStream_t>(stream_),
       static_cast<const uint4 *>(table), tokens, m, chunks, vocab, static_cast<uint4 *>(out), ctx->d_status);
-  return sc_launched(ctx, "launch embed");
+  return sc_launched(ctx, e, "launch embed");
 }
 
 extern "C" kvd_status kvd_scaffold_argmax(kvd_ctx *ctx, const void *logits, int64_t row_stride, int m, int n,
@@ -405,8 +413,8 @@ extern "C" kvd_status kvd_scaffold_argmax(kvd_ctx *ctx, const void *logits, int6
   if (e != cudaSuccess) return cuda_fail(ctx, e, "scaffold argmax: clear");
   dim3 grid((n + ARGMAX_SLICE - 1) / ARGMAX_SLICE, m, 1);
   kvd_argmax_slices_kernel<<<grid, 256, 0, stream>>>(static_cast<const __nv_bfloat16 *>(logits), row_stride, n, ctx->argmax_keys);
-  kvd_status st = sc_launched(ctx, "launch argmax (slices)");
+  kvd_status st = sc_launched(ctx, cudaGetLastError(), "launch argmax (slices)");
   if (st != KVD_OK) return st;
   kvd_argmax_finish_kernel<<<(m + 127) / 128, 128, 0, stream>>>(ctx->argmax_keys, m, tokens_out);
-  return sc_launched(ctx, "launch argmax (finish)");
+  return sc_launched(ctx, cudaGetLastError(), "launch argmax (finish)");
 }
