@@ -314,6 +314,9 @@ extern "C" kvd_status kvd_set_layer(kvd_ctx *ctx, int layer, const kvd_layer_des
   // half tile per CTA, 128 bytes of channels per k block
   st = encode_2d(ctx, &ls.tmap_b, ls.wt, d.d_hidden, n_cols, RC_BLOCK_K * 2 / dtype_bytes(ctx->dtype), ctx->block_n / 2,
                  dtype_bytes(ctx->dtype));
+  for (int i = 0; st == KVD_OK && i < 2; ++i)
+    st = encode_2d(ctx, &ls.tmap_b_part[i], ls.wt, d.d_hidden, n_cols, RC_BLOCK_K * 2 / dtype_bytes(ctx->dtype), ctx->block_n >> (i + 2),
+                   dtype_bytes(ctx->dtype));
   if (st != KVD_OK) return st;
   if (ctx->dtype != KVD_DTYPE_F32) {
     st = prepare_rows_map(ctx, ls, d.d_hidden, n_cols, true);

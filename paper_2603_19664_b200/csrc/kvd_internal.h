@@ -67,6 +67,7 @@ struct RecomputeParams {
   int num_k_blocks;  // d_hidden / 64
   int num_m_blocks;  // over all jobs
   int num_n_blocks;
+  int unit_tiles, whole_tiles, parts;  // schedule of the plain kernel (rc_schedule)
   int k_cols;  // n_kv * d_head: fused columns below this index are keys, the rest values
   long long out_row_stride;
   float inv_d_hidden;
@@ -252,6 +253,7 @@ struct LayerState {
   int window = 0;
   RopeTable rope;
   CUtensorMap tmap_b;
+  CUtensorMap tmap_b_part[2];  // the same with boxes of a half and of a quarter of a tile's columns
   CUtensorMap tmap_rows[2];  // of wt, for the projection of few and of more rows (16-bit types), and its columns per tile
   int rows_tile = 0;
   // FP8 variant: E4M3 codes of W' / w_scale8, K-major; one scale for the matrix (device float)
@@ -348,7 +350,7 @@ inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, unsigned thre
 
 // launchers implemented next to their kernels
 kvd_status launch_recompute(kvd_ctx *ctx, const LayerState &ls, const CUtensorMap &tmap_store,
-                            const CUtensorMap &tmap_rows, const RecomputeParams &p, cudaStream_t stream);
+                            const CUtensorMap &tmap_rows, RecomputeParams &p, cudaStream_t stream);
 kvd_status launch_recompute_fused(kvd_ctx *ctx, const LayerState &ls, const CUtensorMap &tmap_store,
                                   const CUtensorMap &tmap_rows, const RecomputeParams &p, const FusedParams &fp,
                                   cudaStream_t stream, int eb = 2);
@@ -368,7 +370,7 @@ kvd_status launch_prepare_weights_fp8(kvd_ctx *ctx, const __nv_bfloat16 *w, cons
                                       int d_hidden, int n_cols, unsigned *amax_scratch, float *scale_out,
                                       cudaStream_t stream);
 kvd_status launch_recompute_fp8(kvd_ctx *ctx, const LayerState &ls, const CUtensorMap &tmap_store,
-                                const CUtensorMap &tmap_rows, const RecomputeParams &p, cudaStream_t stream);
+                                const CUtensorMap &tmap_rows, RecomputeParams &p, cudaStream_t stream);
 kvd_status launch_checkpoint(kvd_ctx *ctx, const __nv_bfloat16 *rows, const int32_t *pos, __nv_bfloat16 *dst_rows,
                              int32_t *dst_pos, float *dst_sumsq, int n, int d_hidden, cudaStream_t stream);
 kvd_status launch_selftest_bounds(kvd_ctx *ctx, cudaStream_t stream);

@@ -173,7 +173,8 @@ KVD_DEFINE_UMMA_KBLOCK(umma_kblock_pair_tf32, "tf32")  // fp32 operands read as 
 template <int BLOCK_N, int D_HEAD, bool TRACE, int FG, int EB = 2, bool LOSM = (FG > 0), int DT = 0>
 __global__ void __launch_bounds__(RC_THREADS, 1)
 kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __grid_constant__ CUtensorMap tmap_rows,
-                     const __grid_constant__ CUtensorMap tmap_b, const __grid_constant__ RecomputeParams p,
+                     const __grid_constant__ CUtensorMap tmap_b, const __grid_constant__ CUtensorMap tmap_b_part,
+                     const __grid_constant__ RecomputeParams p,
                      const __grid_constant__ std::conditional_t<(FG > 0), FusedParams, NoFusedParams> f) {
   using Cfg = RcCfg<BLOCK_N, D_HEAD, FG, LOSM>;
   constexpr int STAGES = Cfg::STAGES;
@@ -220,23 +221,30 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
   const int lane = threadIdx.x & 31;
   const int num_tiles = p.num_m_blocks * p.num_n_blocks;
-  // Tile order.  With more tiles than clusters a cluster works through "units" of two consecutive
-  // tiles that share a row block -- the key tile and the value tile of one head column -- so that the
-  // row statistics are fetched once per unit and reused; key first, so that the last tile of a CTA,
-  // whose epilogue nothing overlaps, is a cheap value tile.  (Units of
-  // all tiles of a row block measured slower: the units are then too few to balance the clusters.)
-  // With no more tiles than clusters every tile is its own unit, all key tiles first.  Falls back to
-  // row-major single tiles when a tile mixes key and value heads.
+  // Tile order (chosen by the host, rc_schedule).  Units of two consecutive tiles that share a row block -- the key
+  // tile and the value tile of one head column, so that the row statistics are fetched once per unit and X is read
+  // once; key first, so that the last tile of a CTA, whose epilogue nothing overlaps, is a cheap value tile -- or
+  // single tiles, all key tiles first, of which the last ones (a round that would leave most clusters idle) are cut
+  // into `parts` column ranges.  (Units of all tiles of a row block measured slower: the units are then too few to
+  // balance the clusters.)  Row-major single tiles when a tile mixes key and value heads.
   const int nk_tiles = (p.k_cols % BLOCK_N == 0) ? p.k_cols / BLOCK_N : 0;
   // (the fused variant always pairs the key tile with the value tile: the scores of the one weight the other)
-  const int unit_tiles = (nk_tiles != 0 && (FUSED || num_tiles > num_clusters)) ? 2 : 1;
-  const int n_units = num_tiles / unit_tiles;
+  const int unit_tiles = FUSED ? 2 : p.unit_tiles;
+  const int whole = FUSED ? num_tiles : p.whole_tiles, parts = FUSED ? 1 : p.parts;  // tiles that are not cut; cuts of the others
+  const int n_units = unit_tiles == 2 ? num_tiles / 2 : whole + (num_tiles - whole) * parts;
   // i-th tile of this cluster -> (job, first row of this CTA's 128 rows within the job, first fused
-  // column, whether it opens a unit); false when the cluster has no i-th tile
-  auto tile_at = [&](int i, int &job, int &m0, int &n0, bool &first) -> bool {
-    const int unit = cluster_id + (i / unit_tiles) * num_clusters, j = i % unit_tiles;
+  // column, columns, whether it opens a unit); false when the cluster has no i-th tile
+  auto tile_at = [&](int i, int &job, int &m0, int &n0, int &width, bool &first) -> bool {
+    int unit = cluster_id + (i / unit_tiles) * num_clusters, sub = 0;
+    const int j = i % unit_tiles;
     if (unit >= n_units) return false;
     first = j == 0;
+    width = BLOCK_N;
+    if (unit_tiles == 1 && unit >= whole) {
+      width = BLOCK_N / parts;
+      sub = (unit - whole) % parts * width;
+      unit = whole + (unit - whole) / parts;
+    }
     int mb;
     if (nk_tiles == 0) {
       mb = unit / p.num_n_blocks;
@@ -254,6 +262,7 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
       mb = unit / nk_tiles;
       n0 = (unit % nk_tiles + (j == 0 ? 0 : nk_tiles)) * BLOCK_N;
     }
+    n0 += sub;
     // jobs own consecutive runs of 256-row blocks: the last job whose first block is <= mb
     int lo = 0, hi = p.n_jobs;
     while (hi - lo > 1) {
@@ -265,7 +274,7 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
     m0 = (mb - p.jobs[lo].mb_start) * (2 * RC_BLOCK_M) + static_cast<int>(cta_rank) * RC_BLOCK_M;
     // checking build: the tile lies inside the job table, its job's row blocks and (for store ranges) the
     // sequence's slab; a tile that does not is not processed by any role
-    if (!KVD_BOUNDS_OK(mb >= 0 && mb < p.num_m_blocks && lo >= 0 && lo < p.n_jobs && n0 >= 0 && n0 < p.num_n_blocks * BLOCK_N &&
+    if (!KVD_BOUNDS_OK(mb >= 0 && mb < p.num_m_blocks && lo >= 0 && lo < p.n_jobs && n0 >= 0 && n0 + width <= p.num_n_blocks * BLOCK_N &&
                            m0 - static_cast<int>(cta_rank) * RC_BLOCK_M < p.jobs[lo].n &&
                            (p.jobs[lo].slab < 0 || p.jobs[lo].row0 + p.jobs[lo].n <= p.store_rows),
                        p.status))
@@ -296,6 +305,7 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
     prefetch_tensormap(&tmap_store);
     prefetch_tensormap(&tmap_rows);
     prefetch_tensormap(&tmap_b);
+    prefetch_tensormap(&tmap_b_part);
   }
   if (threadIdx.x < D_HEAD) s_gamma_k[threadIdx.x] = p.gamma_k ? p.gamma_k[threadIdx.x] : 1.0f;
   if constexpr (LOSM) {
@@ -329,12 +339,13 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
       // the stage barrier lives in the even CTA; `full` is its address as seen from this CTA
       const uint32_t full0 = map_to_cta(bar_full(0), 0);
       uint32_t full = full0, empty = bar_empty(0), dst = smem_base;
-      const int b_row_off = static_cast<int>(cta_rank) * Cfg::B_ROWS;
       bool ok = true;
-      int job, m0, n0;
+      int job, m0, n0, width;
       bool first_of_unit;
-      for (int ti = 0; ok && tile_at(ti, job, m0, n0, first_of_unit); ++ti) {
-        n0 += b_row_off;
+      for (int ti = 0; ok && tile_at(ti, job, m0, n0, width, first_of_unit); ++ti) {
+        n0 += static_cast<int>(cta_rank) * (width / 2);  // this CTA's half of the columns
+        const CUtensorMap *tmap_w = width == BLOCK_N ? &tmap_b : &tmap_b_part;
+        const uint32_t pair_bytes = 2 * (Cfg::A_BYTES + width / 2 * RC_BLOCK_K * 2);
         // rows come from a slab of the residual store or from the caller's buffer (slab 0 of its map)
         const int slab = p.jobs[job].slab;
         const CUtensorMap *tmap_a = slab < 0 ? &tmap_rows : &tmap_store;
@@ -350,9 +361,9 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
             break;
           }
           if (TRACE) waited += clock64() - w0;
-          if (cta_rank == 0) mbar_arrive_expect_tx(bar_full(s), 2 * Cfg::STAGE_BYTES);
+          if (cta_rank == 0) mbar_arrive_expect_tx(bar_full(s), pair_bytes);
           tma_load_3d_pair(dst, tmap_a, full, k0, m0, a_slab);
-          tma_load_2d_pair(dst + Cfg::A_BYTES, &tmap_b, full, k0, n0);
+          tma_load_2d_pair(dst + Cfg::A_BYTES, tmap_w, full, k0, n0);
           ++n_issued;
           full += 8u;
           empty += 8u;
@@ -393,7 +404,7 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
   } else if (warp == 3) {
     if (cta_rank == 0 && elect_one()) {
       // ---------------------------------------------------------------- MMA issuer (even CTA)
-      constexpr uint32_t idesc = EB == 1   ? umma_idesc_e4m3_f32(2 * RC_BLOCK_M, BLOCK_N)
+      constexpr uint32_t idesc_whole = EB == 1   ? umma_idesc_e4m3_f32(2 * RC_BLOCK_M, BLOCK_N)
                                  : EB == 4 ? umma_idesc_tf32_f32(2 * RC_BLOCK_M, BLOCK_N)
                                  : DT == 1 ? umma_idesc_f16_f32(2 * RC_BLOCK_M, BLOCK_N)
                                            : umma_idesc_bf16_f32(2 * RC_BLOCK_M, BLOCK_N);
@@ -406,9 +417,10 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
       uint32_t ph = 0, aph = 0;
       uint32_t full = bar_full(0), empty = bar_empty(0), a_lo = a_lo0;
       bool ok = true;
-      int job_, m0_, n0_;
+      int job_, m0_, n0_, width;
       bool first_;
-      for (int ti = 0; ok && tile_at(ti, job_, m0_, n0_, first_); ++ti) {
+      for (int ti = 0; ok && tile_at(ti, job_, m0_, n0_, width, first_); ++ti) {
+        const uint32_t idesc = idesc_whole - (static_cast<uint32_t>((BLOCK_N - width) >> 3) << 17);  // N = width
         // both CTAs' epilogues have drained accumulator a
         if (!mbar_wait(bar_tmem_empty(a), aph ^ 1u, s_abort, tmo)) {
           raise(p.status, STATUS_TIMEOUT, s_abort);
@@ -466,11 +478,11 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
     const int row = w4 * 32 + lane;
     int a = 0;
     uint32_t aph = 0;
-    int job, m0, n0_;
+    int job, m0, n0_, width_;
     bool first_of_unit;
     float rstd_row = 0.f;  // of this thread's row, kept for the other tiles of the unit
     uint32_t xph = 0;      // phase of the statistics warps' own barrier
-    for (int ti = 0; tile_at(ti, job, m0, n0_, first_of_unit); ++ti) {
+    for (int ti = 0; tile_at(ti, job, m0, n0_, width_, first_of_unit); ++ti) {
       const long long st0 = TRACE ? clock64() : 0;
       // s_rstd[a] is free once the local epilogue that read it has finished with accumulator a
       // the whole warp takes the same branch: aligned instructions follow
@@ -551,9 +563,9 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
     int a = 0;
     uint32_t aph = 0;
     uint32_t sph[2] = {0u, 0u}, eph = 0;  // fused: phases of the score barriers and of the epilogue warps' barrier
-    int job, m0, n0;
+    int job, m0, n0, width;
     bool first_of_unit;
-    for (int ti = 0; tile_at(ti, job, m0, n0, first_of_unit); ++ti) {
+    for (int ti = 0; tile_at(ti, job, m0, n0, width, first_of_unit); ++ti) {
       const RcJob &J = p.jobs[job];
       // fused: does this tile's job attend (K and V are consumed here) or is it a plain job?
       bool attend = false;
@@ -698,14 +710,14 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
       } else {
 
 #pragma unroll 1
-      for (int hh = 0; hh < BLOCK_N / D_HEAD; ++hh) {
-        const int col0 = n0 + hh * D_HEAD;  // first fused column of this head
+      for (int hh = 0; hh * D_HEAD < width; ++hh) {
+        const int col0 = n0 + hh * D_HEAD;  // first fused column of this head (or of this part of a value head)
         const uint32_t tcol = acc + hh * D_HEAD;
         if (col0 >= p.k_cols) {
           // ---- value head (Eq. 14): scale by 1/rms and store
           __nv_bfloat16 *dst = J.v_out + (static_cast<size_t>(m) * out_stride + (col0 - p.k_cols)) * EW;
 #pragma unroll 1
-          for (int c = 0; c < D_HEAD / 32; ++c) {
+          for (int c = 0; c < (width < D_HEAD ? width : D_HEAD) / 32; ++c) {
             uint32_t r[32];
             tmem_ld_x32(tcol + c * 32, r);
             tmem_wait_ld();
@@ -908,14 +920,16 @@ static kvd_status launch_impl(kvd_ctx *ctx, const LayerState &ls, const CUtensor
   using Cfg = RcCfg<BLOCK_N, D_HEAD, FG, LOSM>;
   auto kern = kvd_recompute_kernel<BLOCK_N, D_HEAD, TRACE, FG, EB, LOSM, DT>;
   const CUtensorMap &tmap_b = EB == 1 ? ls.tmap_b8 : ls.tmap_b;
+  const CUtensorMap &tmap_b_part = EB == 1 || p.parts <= 1 ? tmap_b : ls.tmap_b_part[p.parts == 2 ? 0 : 1];
   static bool configured[64] = {};
   if (!configured[ctx->device & 63]) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(recompute)");
     configured[ctx->device & 63] = true;
   }
-  // plain: one cluster per tile at most; fused: per unit of a key tile and a value tile
-  const int work = FG > 0 ? p.num_m_blocks * p.num_n_blocks / 2 : p.num_m_blocks * p.num_n_blocks;
+  // plain: one cluster per tile (or part of one) at most; fused: per unit of a key tile and a value tile
+  const int tiles = p.num_m_blocks * p.num_n_blocks;
+  const int work = FG > 0 || p.unit_tiles == 2 ? tiles / 2 : p.whole_tiles + (tiles - p.whole_tiles) * p.parts;
   const int max_clusters = ctx->num_sms / 2;
   const int clusters = work < max_clusters ? work : max_clusters;
   cudaLaunchConfig_t cfg;
@@ -934,8 +948,8 @@ static kvd_status launch_impl(kvd_ctx *ctx, const LayerState &ls, const CUtensor
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   cudaError_t le;
-  if constexpr (FG > 0) le = cudaLaunchKernelEx(&cfg, kern, tmap_store, tmap_rows, tmap_b, p, *fp);
-  else le = cudaLaunchKernelEx(&cfg, kern, tmap_store, tmap_rows, tmap_b, p, NoFusedParams());
+  if constexpr (FG > 0) le = cudaLaunchKernelEx(&cfg, kern, tmap_store, tmap_rows, tmap_b, tmap_b_part, p, *fp);
+  else le = cudaLaunchKernelEx(&cfg, kern, tmap_store, tmap_rows, tmap_b, tmap_b_part, p, NoFusedParams());
   if (le != cudaSuccess) return cuda_fail(ctx, le, "launch recompute");
   ctx->launches += 1;
   return KVD_OK;
@@ -951,7 +965,7 @@ static kvd_status launch_sel(kvd_ctx *ctx, const LayerState &ls, const CUtensorM
     if (ctx->dtype == 2) return launch_impl<BLOCK_N, D_HEAD, false, 0, 4, true, 2>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
     if (p.trace != nullptr) return launch_impl<BLOCK_N, D_HEAD, true, 0>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
     // one tile per cluster at most: every key tile's epilogue is exposed -> the low table from shared memory
-    if (p.num_m_blocks * p.num_n_blocks <= ctx->num_sms / 2)
+    if (p.whole_tiles + (p.num_m_blocks * p.num_n_blocks - p.whole_tiles) * p.parts <= ctx->num_sms / 2)
       return launch_impl<BLOCK_N, D_HEAD, false, 0, 2, true>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
   }
   // the fused variant on fp16 rows, weights, queries and outputs (same tiles, MMA kind f16 with fp16 operands)
@@ -961,9 +975,46 @@ static kvd_status launch_sel(kvd_ctx *ctx, const LayerState &ls, const CUtensorM
   return launch_impl<BLOCK_N, D_HEAD, false, FG>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
 }
 
+// The plain kernel's schedule: units of two tiles or single tiles, and how the last round of single tiles is cut when it
+// would leave half of the clusters idle or more.  Cost estimate in tiles per cluster, from launches of 128 to 32768
+// rows of the Gemma-3-4B and Qwen3-4B layers (units / single / halves / quarters, us): 88 tiles on 74 clusters 31.1 /
+// 29.5 / 26.6 / 26.3, 160 52.8 / 42.3 / 40.2 / 40.2, 192 54 / 45.9 / 49.3 / 53, 224 61 / 61 / 55.5 / 54.3, 512 125 / 114 / 126 / 144, 1024
+// 254 / 254 / 256 / 277.  Single tiles read X at two distant times: beyond 8 rounds, where it no longer stays in the
+// L2 (64 x 767 rows: 415 us in units, 422 single), units it is.  With less than one round (Qwen, 8 tiles 31 -> 20, 72
+// tiles 23.9 -> 21.7) halves shorten every CTA's exposed epilogue, if a half still holds whole heads: the key norm
+// runs over a head in one thread.
+static void rc_schedule(const kvd_ctx *ctx, RecomputeParams &p, int eb) {
+  const int tiles = p.num_m_blocks * p.num_n_blocks, clusters = ctx->num_sms / 2, bn = ctx->block_n, dh = ctx->desc.d_head;
+  const int nk = p.k_cols % bn == 0 ? p.k_cols / bn : 0;  // 0 also where a tile mixes key and value heads
+  const int rounds = tiles / clusters, last = tiles % clusters;
+  p.unit_tiles = 1;
+  p.whole_tiles = tiles;
+  p.parts = 1;
+  float single = static_cast<float>(rounds + (last > 0 ? 1 : 0));
+  if (eb != 1 && bn == 256 && (nk != 0 || p.k_cols == 0) && last > 0 && rounds <= 8) {
+    int parts = rounds == 0 ? 2 : 4 * last <= clusters ? 4 : 2 * last <= clusters ? 2 : 1;
+    const bool keys = last > p.num_m_blocks * (p.num_n_blocks - nk);  // key tiles among those to be cut
+    if (keys && bn / parts < dh) parts = 1;
+    if (parts > 1) {
+      p.whole_tiles = tiles - last;
+      p.parts = parts;
+      single = static_cast<float>(rounds) + (parts == 2 ? 0.62f : 0.53f);
+    }
+  }
+  if (nk != 0 && p.num_n_blocks == 2 * nk && tiles > clusters) {
+    const float units = 2.f * static_cast<float>((tiles / 2 + clusters - 1) / clusters);
+    if (eb == 1 || rounds > 8 || units <= single) {
+      p.unit_tiles = 2;
+      p.whole_tiles = tiles;
+      p.parts = 1;
+    }
+  }
+}
+
 kvd_status launch_recompute(kvd_ctx *ctx, const LayerState &ls, const CUtensorMap &tmap_store,
-                            const CUtensorMap &tmap_rows, const RecomputeParams &p, cudaStream_t stream) {
+                            const CUtensorMap &tmap_rows, RecomputeParams &p, cudaStream_t stream) {
   const int dh = ctx->desc.d_head;
+  rc_schedule(ctx, p, 2);
   if (ctx->block_n == 256) {
     if (dh == 256) return launch_sel<256, 256>(ctx, ls, tmap_store, tmap_rows, p, nullptr, stream);
     if (dh == 128) return launch_sel<256, 128>(ctx, ls, tmap_store, tmap_rows, p, nullptr, stream);
@@ -1003,8 +1054,9 @@ kvd_status launch_recompute_fused(kvd_ctx *ctx, const LayerState &ls, const CUte
 // The FP8 variant: rows and weights as E4M3 codes (tmap_store is the FP8 store's map, tmap_rows the map of
 // the caller's quantised rows, or the store's again).
 kvd_status launch_recompute_fp8(kvd_ctx *ctx, const LayerState &ls, const CUtensorMap &tmap_store,
-                                const CUtensorMap &tmap_rows, const RecomputeParams &p, cudaStream_t stream) {
+                                const CUtensorMap &tmap_rows, RecomputeParams &p, cudaStream_t stream) {
   const int dh = ctx->desc.d_head;
+  rc_schedule(ctx, p, 1);
   if (ctx->block_n == 256) {
     if (dh == 256 && p.trace != nullptr) return launch_impl<256, 256, true, 0, 1, true>(ctx, ls, tmap_store, tmap_rows, p, nullptr, stream);
     if (dh == 256) return launch_impl<256, 256, false, 0, 1, true>(ctx, ls, tmap_store, tmap_rows, p, nullptr, stream);

@@ -225,6 +225,8 @@ extern "C" kvd_status kvd_scaffold_linear_create(kvd_ctx *ctx, const void *w, co
                                 gamma ? static_cast<const __nv_bfloat16 *>(gamma) : ones, lin->ls.wt, k, n, stream);
   if (st == KVD_OK) st = get_rope(ctx, 10000.0f, &lin->ls.rope);  // the kernel's prologue wants a table; no row is rotated
   if (st == KVD_OK) st = encode_2d(ctx, &lin->ls.tmap_b, lin->ls.wt, k, lin->n_pad, RC_BLOCK_K, ctx->block_n / 2, 2);
+  for (int i = 0; st == KVD_OK && i < 2; ++i)
+    st = encode_2d(ctx, &lin->ls.tmap_b_part[i], lin->ls.wt, k, lin->n_pad, RC_BLOCK_K, ctx->block_n >> (i + 2), 2);
   if (st == KVD_OK) st = prepare_rows_map(ctx, lin->ls, k, lin->n_pad, false);
   if (st == KVD_OK) {
     e = cudaStreamSynchronize(stream);
