@@ -53,6 +53,7 @@ constexpr int PT_LAG = 3;        // blocks a loader thread keeps in flight behin
 template <int D_HEAD, bool PAIR>
 struct PtCfg {
   static constexpr int NCTA = PAIR ? 2 : 1;
+  static constexpr int LOADERS = PT_LOADERS;
   static constexpr int K_ROWS = PT_KEYS / NCTA;                   // keys of a block this CTA holds
   static constexpr int V_COLS = D_HEAD / NCTA;                    // channels of a block this CTA holds
   static constexpr int TILE_BYTES = PT_KEYS * D_HEAD * 2 / NCTA;  // this CTA's share of one K or V block
@@ -98,6 +99,234 @@ __device__ __forceinline__ bool polite_warp_wait(uint32_t bar, uint32_t parity, 
 template <bool PAIR>
 __device__ __forceinline__ bool lead_wait(uint32_t bar, uint32_t parity, const volatile int *abort_flag, unsigned long long timeout_ns) {
   return polite_wait<PAIR>(bar, parity, abort_flag, timeout_ns);
+}
+
+// Whether every row of a warp sees every key of a block, without the row's masks (which cost 460 of the 2380 clocks a
+// softmax warp took for a block): the block lies inside one segment and inside the range all the warp's rows see.
+// Rows that are not stored do not count.
+struct PtWhole {
+  int lo, hi;      // the range that every stored row of the warp sees
+  int seg0, seg1;  // [seg0, seg1): the segment the last block was found in
+  __device__ __forceinline__ PtWhole(bool valid, int row_lo, int row_hi) : seg0(0), seg1(0) {
+    lo = __reduce_max_sync(0xffffffffu, valid ? row_lo : INT_MIN);
+    hi = __reduce_min_sync(0xffffffffu, valid ? row_hi : INT_MAX);
+  }
+  __device__ __forceinline__ bool operator()(const PrefillParams &P, int pos0) {
+    if (pos0 < lo || pos0 + PT_KEYS - 1 > hi) return false;
+    if (pos0 < seg0 || pos0 + PT_KEYS > seg1) {
+#pragma unroll
+      for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg)
+        if (P.first[sg] <= pos0 && pos0 < P.first[sg] + P.len[sg]) {
+          seg0 = P.first[sg];
+          seg1 = P.first[sg] + P.len[sg];
+        }
+    }
+    return pos0 >= seg0 && pos0 + PT_KEYS <= seg1;
+  }
+};
+// Which keys of the block at pos0 does a row see: present in a segment, in [lo, qp] (bit k = key pos0 + k).
+__device__ __forceinline__ unsigned long long pt_visible(const PrefillParams &P, int pos0, int lo, int qp) {
+  unsigned long long vis = 0ull;
+#pragma unroll
+  for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg) {
+    int a = P.first[sg] - pos0, b = P.first[sg] + P.len[sg] - pos0;  // [a, b) of the block's key slots
+    a = a < 0 ? 0 : a;
+    b = b > PT_KEYS ? PT_KEYS : b;
+    if (b > a) vis |= (b - a == 64 ? ~0ull : ((1ull << (b - a)) - 1ull) << a);
+  }
+  int a = lo - pos0, b = qp - pos0 + 1;
+  a = a < 0 ? 0 : a;
+  b = b > PT_KEYS ? PT_KEYS : b;
+  return vis & (b > a ? (b - a == 64 ? ~0ull : ((1ull << (b - a)) - 1ull) << a) : 0ull);
+}
+// Scores of invisible keys become -inf; the maximum of the 64 in four chains of three-input maxima.
+__device__ __forceinline__ float pt_mask_max(uint32_t (&s0)[32], uint32_t (&s1)[32], bool whole, unsigned long long vis) {
+  if (!whole) {
+    const uint32_t v0 = static_cast<uint32_t>(vis), v1 = static_cast<uint32_t>(vis >> 32);
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+      if (!((v0 >> k) & 1u)) s0[k] = 0xff800000u;  // -inf
+      if (!((v1 >> k) & 1u)) s1[k] = 0xff800000u;
+    }
+  }
+  float mx[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
+#pragma unroll
+  for (int k = 0; k < 32; k += 8) {
+    mx[0] = fmax3(mx[0], __uint_as_float(s0[k]), __uint_as_float(s0[k + 1]));
+    mx[1] = fmax3(mx[1], __uint_as_float(s0[k + 2]), __uint_as_float(s0[k + 3]));
+    mx[2] = fmax3(mx[2], __uint_as_float(s0[k + 4]), __uint_as_float(s0[k + 5]));
+    mx[3] = fmax3(mx[3], __uint_as_float(s0[k + 6]), __uint_as_float(s0[k + 7]));
+    mx[0] = fmax3(mx[0], __uint_as_float(s1[k]), __uint_as_float(s1[k + 1]));
+    mx[1] = fmax3(mx[1], __uint_as_float(s1[k + 2]), __uint_as_float(s1[k + 3]));
+    mx[2] = fmax3(mx[2], __uint_as_float(s1[k + 4]), __uint_as_float(s1[k + 5]));
+    mx[3] = fmax3(mx[3], __uint_as_float(s1[k + 6]), __uint_as_float(s1[k + 7]));
+  }
+  return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+}
+// Weights 2^(s * scale - m) of 64 scores: two per fused multiply-add; the row sum adds them up in fp32, the product
+// takes them rounded to the element type.
+template <int DT>
+__device__ __forceinline__ void pt_weights(const uint32_t (&s0)[32], const uint32_t (&s1)[32], uint64_t c2, uint64_t nm2, uint64_t (&l2)[2],
+                                           uint32_t (&w)[32]) {
+  const uint64_t one2 = pack2(1.0f, 1.0f);
+#pragma unroll
+  for (int k = 0; k < 32; k += 2) {
+    float e0, e1;
+    unpack2(ffma2(pack2(__uint_as_float(s0[k]), __uint_as_float(s0[k + 1])), c2, nm2), e0, e1);
+    const float p0 = ex2_approx(e0), p1 = ex2_approx(e1);
+    w[k >> 1] = pack_out<DT>(p0, p1);
+    l2[(k >> 1) & 1] = ffma2(pack2(p0, p1), one2, l2[(k >> 1) & 1]);
+  }
+#pragma unroll
+  for (int k = 0; k < 32; k += 2) {
+    float e0, e1;
+    unpack2(ffma2(pack2(__uint_as_float(s1[k]), __uint_as_float(s1[k + 1])), c2, nm2), e0, e1);
+    const float p0 = ex2_approx(e0), p1 = ex2_approx(e1);
+    w[16 + (k >> 1)] = pack_out<DT>(p0, p1);
+    l2[(k >> 1) & 1] = ffma2(pack2(p0, p1), one2, l2[(k >> 1) & 1]);
+  }
+}
+// A part of the row sum, referred to another maximum.  The factor goes to the four chains, as in a further block
+// without a visible key: whether the tile has such blocks behind the row's last one must not show in the row's bits.
+__device__ __forceinline__ float pt_row_sum(const uint64_t (&l2)[2], float factor) {
+  const uint64_t f2 = pack2(factor, factor);
+  float a0, a1, a2, a3;
+  unpack2(fmul2(l2[0], f2), a0, a1);
+  unpack2(fmul2(l2[1], f2), a2, a3);
+  return (a0 + a1) + (a2 + a3);
+}
+// O (D_HEAD columns of this warp's lanes, from column `col`) times a factor per row.
+template <int D_HEAD>
+__device__ __forceinline__ void pt_rescale(uint32_t col, float alpha) {
+#pragma unroll 1
+  for (int c = 0; c < D_HEAD / 32; ++c) {
+    uint32_t r[32];
+    tmem_ld_x32(col + c * 32, r);
+    tmem_wait_ld();
+#pragma unroll
+    for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
+    tmem_st_x32(col + c * 32, r);
+  }
+  tmem_wait_st();
+}
+
+// The loader warps of a CTA: K and V blocks blk0 .. blk0 + n_blk - 1 of KV head kvh into the rings.
+template <class Cfg, int D_HEAD, class Arrive>
+__device__ __forceinline__ void pt_load_blocks(const PrefillParams &P, uint32_t ring, uint32_t ring_v, uint32_t bar_base, int slots, int blk0, int n_blk,
+                                               int kvh, int rank, int ptid, const Arrive &arrive_lead, volatile int *s_abort,
+                                               unsigned long long tmo) {
+  constexpr int SLOTS_K = Cfg::SLOTS_K, SLOTS_V = Cfg::SLOTS_V;
+  const int lane = ptid & 31;
+  auto bar_full = [&](int v, int sl) { return bar_base + 8u * (v * SLOTS_K + sl); };
+  auto bar_empty = [&](int v, int sl) { return bar_base + 8u * (slots + v * SLOTS_K + sl); };
+  // ------------------------------------------------------------------ K/V blocks into the rings
+  // issue order = the order the products want them, the keys three blocks ahead: K_0 K_1 K_2 | K_3 V_0 | K_4 V_1 | ...
+  // This CTA's share of a block: K_ROWS keys of all channels (K), all 64 keys of V_COLS channels (V).
+  // blocks issued and not yet published to the MMA threads, oldest first.  A block is published once PT_LAG younger
+  // ones have been issued -- or at once, all of them, when the next block would have to wait for a free slot (the
+  // slot is freed by a product that may itself be waiting for one of these blocks).
+  uint32_t pend[PT_LAG + 1] = {};
+  int n_pend = 0;
+  bool ok = true;
+  auto publish_all = [&]() {
+    cp_async_wait_all();
+    fence_proxy_async_smem();
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i <= PT_LAG; ++i)
+      if (i < n_pend && lane == 0) arrive_lead(pend[i]);
+    n_pend = 0;
+  };
+  // rows [row_first, row_first + ROWS) of the block, CPR 16-byte pieces of each starting at element col_first
+  auto gather = [&](auto rows_c, auto cpr_c, uint32_t base, int slab_bytes, int pos_first, int col_first, bool is_v) {
+    constexpr int ROWS = decltype(rows_c)::value, CPR = decltype(cpr_c)::value;
+    constexpr int RSTEP = Cfg::LOADERS / CPR;  // rows one pass of the loader threads covers
+    const int c = ptid % CPR, r0 = ptid / CPR;
+    const uint32_t dst = base + static_cast<uint32_t>(c >> 3) * slab_bytes;
+    // the usual case: one segment holds all the rows -> one base pointer, one stride
+    int whole = -1;
+#pragma unroll
+    for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg)
+      if (P.first[sg] <= pos_first && pos_first + ROWS <= P.first[sg] + P.len[sg]) whole = sg;
+    if (whole >= 0) {
+      const long long stride = P.stride[whole];
+      const __nv_bfloat16 *src = (is_v ? P.v[whole] : P.k[whole]) + static_cast<size_t>(pos_first - P.first[whole] + r0) * stride +
+                                 static_cast<size_t>(kvh) * D_HEAD + col_first + c * 8;
+#pragma unroll
+      for (int pass = 0; pass < ROWS / RSTEP; ++pass) {
+        const int r = r0 + pass * RSTEP;
+        cp_async16(dst + r * 128 + (((c & 7) ^ (r & 7)) << 4), src, true);
+        src += RSTEP * stride;
+      }
+    } else {
+#pragma unroll 1
+      for (int pass = 0; pass < ROWS / RSTEP; ++pass) {
+        const int r = r0 + pass * RSTEP, pos = pos_first + r;
+        const __nv_bfloat16 *src = P.q;
+        bool have = false;
+#pragma unroll
+        for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg) {
+          const int rr = pos - P.first[sg];
+          if (rr >= 0 && rr < P.len[sg]) {
+            src = (is_v ? P.v[sg] : P.k[sg]) + static_cast<size_t>(rr) * P.stride[sg] + static_cast<size_t>(kvh) * D_HEAD + col_first + c * 8;
+            have = true;
+          }
+        }
+        cp_async16(dst + r * 128 + (((c & 7) ^ (r & 7)) << 4), src, have);
+      }
+    }
+  };
+  auto emit = [&](int is_v, int j) -> bool {
+    const int n_slots = is_v ? SLOTS_V : SLOTS_K, slot = j % n_slots;
+    if (j >= n_slots) {
+      const uint32_t par = ((j / n_slots) - 1) & 1;
+      int free_now = lane == 0 ? (mbar_try_wait(bar_empty(is_v, slot), par) ? 1 : 0) : 0;
+      free_now = __shfl_sync(0xffffffffu, free_now, 0);
+      if (!free_now) {
+        publish_all();
+        int got = lane == 0 ? (polite_wait<false>(bar_empty(is_v, slot), par, s_abort, tmo) ? 1 : 0) : 0;
+        got = __shfl_sync(0xffffffffu, got, 0);
+        if (!got) return false;
+      }
+    }
+    const int pos0 = (blk0 + j) * PT_KEYS;
+    if (is_v)
+      gather(std::integral_constant<int, PT_KEYS>(), std::integral_constant<int, Cfg::V_COLS / 8>(), ring_v + slot * Cfg::TILE_BYTES,
+             Cfg::SLAB_V, pos0, static_cast<int>(rank) * Cfg::V_COLS, true);
+    else
+      gather(std::integral_constant<int, Cfg::K_ROWS>(), std::integral_constant<int, D_HEAD / 8>(), ring + slot * Cfg::TILE_BYTES,
+             Cfg::SLAB_K, pos0 + static_cast<int>(rank) * Cfg::K_ROWS, 0, false);
+    cp_async_commit();
+#pragma unroll
+    for (int i = 0; i <= PT_LAG; ++i)
+      if (i == n_pend) pend[i] = bar_full(is_v, slot);
+    ++n_pend;
+    if (n_pend > PT_LAG) {
+      // the oldest block has PT_LAG younger ones behind it: it has landed by now, or nearly
+      cp_async_wait_group<PT_LAG>();
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) arrive_lead(pend[0]);
+#pragma unroll
+      for (int i = 0; i < PT_LAG; ++i) pend[i] = pend[i + 1];
+      --n_pend;
+    }
+    return true;
+  };
+  if (n_blk > 0) {
+    ok = emit(0, 0);
+    if (ok && n_blk > 1) ok = emit(0, 1);
+    if (ok && n_blk > 2) ok = emit(0, 2);
+    for (int j = 0; ok && j < n_blk; ++j) {
+      if (j + 3 < n_blk) ok = emit(0, j + 3);
+      if (ok) ok = emit(1, j);
+    }
+    if (ok) publish_all();
+    else {
+      cp_async_wait_all();
+      raise(P.status, STATUS_TIMEOUT, s_abort);
+    }
+  }
 }
 
 template <int D_HEAD, int G, int DT, bool PAIR>
@@ -237,7 +466,8 @@ __global__ void __launch_bounds__(PT_THREADS, 1) kvd_prefill_attn_tc_kernel(cons
     float m_own = -CUDART_INF_F;    // the maximum this group's part of the row sum refers to
     uint64_t l2[2] = {0ull, 0ull};  // that part, in four chains (two packed pairs)
     bool ok = true;
-    const uint64_t c2 = pack2(P.scale_log2e, P.scale_log2e), one2 = pack2(1.0f, 1.0f);
+    const uint64_t c2 = pack2(P.scale_log2e, P.scale_log2e);
+    PtWhole whole_block(valid, lo, qp);
     const int buf = wg;
     for (int j = wg; j < n_blk; j += 2) {
       const uint32_t ph = (j >> 1) & 1;
@@ -251,49 +481,15 @@ __global__ void __launch_bounds__(PT_THREADS, 1) kvd_prefill_attn_tc_kernel(cons
       uint32_t s0[32], s1[32];
       tmem_ld_x32(s_col, s0);
       tmem_ld_x32(s_col + 32, s1);
-      // which keys of the block does this row see: present in a segment, not after the row's position, inside its window
-      const int pos0 = (blk0 + j) * PT_KEYS;
-      unsigned long long vis = 0ull;
-#pragma unroll
-      for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg) {
-        int a = P.first[sg] - pos0, b = P.first[sg] + P.len[sg] - pos0;  // [a, b) of the block's key slots
-        a = a < 0 ? 0 : a;
-        b = b > PT_KEYS ? PT_KEYS : b;
-        if (b > a) vis |= (b - a == 64 ? ~0ull : ((1ull << (b - a)) - 1ull) << a);
-      }
-      {
-        int a = lo - pos0, b = qp - pos0 + 1;
-        a = a < 0 ? 0 : a;
-        b = b > PT_KEYS ? PT_KEYS : b;
-        vis &= b > a ? (b - a == 64 ? ~0ull : ((1ull << (b - a)) - 1ull) << a) : 0ull;
-      }
+      const bool whole = whole_block(P, (blk0 + j) * PT_KEYS);  // (warp-uniform)
+      unsigned long long vis = ~0ull;
+      if (!whole) vis = pt_visible(P, (blk0 + j) * PT_KEYS, lo, qp);
       tmem_wait_ld();
       // the scores are in registers: their columns may take this group's next block
       tc_fence_before();
       __syncwarp();
       if (lane == 0) arrive_lead(bar_s_free(buf));
-      if (!__all_sync(0xffffffffu, vis == ~0ull)) {
-        const uint32_t v0 = static_cast<uint32_t>(vis), v1 = static_cast<uint32_t>(vis >> 32);
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-          if (!((v0 >> k) & 1u)) s0[k] = 0xff800000u;  // -inf
-          if (!((v1 >> k) & 1u)) s1[k] = 0xff800000u;
-        }
-      }
-      // the block's maximum in four chains of three-input maxima
-      float mx[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
-#pragma unroll
-      for (int k = 0; k < 32; k += 8) {
-        mx[0] = fmax3(mx[0], __uint_as_float(s0[k]), __uint_as_float(s0[k + 1]));
-        mx[1] = fmax3(mx[1], __uint_as_float(s0[k + 2]), __uint_as_float(s0[k + 3]));
-        mx[2] = fmax3(mx[2], __uint_as_float(s0[k + 4]), __uint_as_float(s0[k + 5]));
-        mx[3] = fmax3(mx[3], __uint_as_float(s0[k + 6]), __uint_as_float(s0[k + 7]));
-        mx[0] = fmax3(mx[0], __uint_as_float(s1[k]), __uint_as_float(s1[k + 1]));
-        mx[1] = fmax3(mx[1], __uint_as_float(s1[k + 2]), __uint_as_float(s1[k + 3]));
-        mx[2] = fmax3(mx[2], __uint_as_float(s1[k + 4]), __uint_as_float(s1[k + 5]));
-        mx[3] = fmax3(mx[3], __uint_as_float(s1[k + 6]), __uint_as_float(s1[k + 7]));
-      }
-      const float bm = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * P.scale_log2e;  // log2 units (scale > 0)
+      const float bm = pt_mask_max(s0, s1, whole, vis) * P.scale_log2e;  // log2 units (scale > 0)
       // the row's maximum after block j - 1 comes from the other group; the one after block j goes back to it
       float m_prev = -CUDART_INF_F;
       if (j > 0) {
@@ -317,28 +513,11 @@ __global__ void __launch_bounds__(PT_THREADS, 1) kvd_prefill_attn_tc_kernel(cons
       const float alpha = m_prev == -CUDART_INF_F ? 1.0f : ex2_approx(m_prev - m_use);
       const float alpha_own = m_own == -CUDART_INF_F ? 1.0f : ex2_approx(m_own - m_use);
       m_own = m_new;
-      // weights 2^(s * scale - m): two per fused multiply-add; the row sum adds them up in fp32, the product takes
-      // them rounded to the element type
       uint32_t w[32];
-      const uint64_t nm2 = pack2(-m_use, -m_use), al2 = pack2(alpha_own, alpha_own);
+      const uint64_t al2 = pack2(alpha_own, alpha_own);
       l2[0] = fmul2(l2[0], al2);
       l2[1] = fmul2(l2[1], al2);
-#pragma unroll
-      for (int k = 0; k < 32; k += 2) {
-        float e0, e1;
-        unpack2(ffma2(pack2(__uint_as_float(s0[k]), __uint_as_float(s0[k + 1])), c2, nm2), e0, e1);
-        const float p0 = ex2_approx(e0), p1 = ex2_approx(e1);
-        w[k >> 1] = pack_out<DT>(p0, p1);
-        l2[(k >> 1) & 1] = ffma2(pack2(p0, p1), one2, l2[(k >> 1) & 1]);
-      }
-#pragma unroll
-      for (int k = 0; k < 32; k += 2) {
-        float e0, e1;
-        unpack2(ffma2(pack2(__uint_as_float(s1[k]), __uint_as_float(s1[k + 1])), c2, nm2), e0, e1);
-        const float p0 = ex2_approx(e0), p1 = ex2_approx(e1);
-        w[16 + (k >> 1)] = pack_out<DT>(p0, p1);
-        l2[(k >> 1) & 1] = ffma2(pack2(p0, p1), one2, l2[(k >> 1) & 1]);
-      }
+      pt_weights<DT>(s0, s1, c2, pack2(-m_use, -m_use), l2, w);
       // P_j into shared memory as a K-major A operand (row = MMA row, 128 bytes = 64 keys, 128-byte swizzle); the
       // product that read this buffer two blocks ago has long finished
       if (j >= 2 && !polite_warp_wait(bar_pv_done(buf), ((j - 2) >> 1) & 1, s_abort, tmo, lane)) {
@@ -365,16 +544,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1) kvd_prefill_attn_tc_kernel(cons
           break;
         }
         tc_fence_after();
-#pragma unroll 1
-        for (int c = 0; c < D_HEAD / 32; ++c) {
-          uint32_t r[32];
-          tmem_ld_x32(tmem_base + lane_field + Cfg::COL_O + c * 32, r);
-          tmem_wait_ld();
-#pragma unroll
-          for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
-          tmem_st_x32(tmem_base + lane_field + Cfg::COL_O + c * 32, r);
-        }
-        tmem_wait_st();
+        pt_rescale<D_HEAD>(tmem_base + lane_field + Cfg::COL_O, alpha);
         tc_fence_before();
       } else if constexpr (Cfg::P_TMEM) {
         tmem_wait_st();
@@ -397,11 +567,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1) kvd_prefill_attn_tc_kernel(cons
       }
       if (ok) {
         const float m_use = m_fin == -CUDART_INF_F ? 0.f : m_fin;
-        float a0, a1, a2, a3;
-        unpack2(l2[0], a0, a1);
-        unpack2(l2[1], a2, a3);
-        const float mine = ((a0 + a1) + (a2 + a3)) * (m_own == -CUDART_INF_F ? 1.0f : ex2_approx(m_own - m_use));
-        s_lx[wg][row] = mine;
+        s_lx[wg][row] = pt_row_sum(l2, m_own == -CUDART_INF_F ? 1.0f : ex2_approx(m_own - m_use));
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_l(q4));
         if (!polite_warp_wait(bar_l(q4), 0, s_abort, tmo, lane)) {
@@ -506,115 +672,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1) kvd_prefill_attn_tc_kernel(cons
       else raise(P.status, STATUS_TIMEOUT, s_abort);
     }
   } else {
-    // ------------------------------------------------------------------ K/V blocks into the rings
-    // issue order = the order the products want them, the keys three blocks ahead: K_0 K_1 K_2 | K_3 V_0 | K_4 V_1 | ...
-    // This CTA's share of a block: K_ROWS keys of all channels (K), all 64 keys of V_COLS channels (V).
-    const int ptid = tid - 10 * 32;
-    // blocks issued and not yet published to the MMA threads, oldest first.  A block is published once PT_LAG younger
-    // ones have been issued -- or at once, all of them, when the next block would have to wait for a free slot (the
-    // slot is freed by a product that may itself be waiting for one of these blocks).
-    uint32_t pend[PT_LAG + 1] = {};
-    int n_pend = 0;
-    bool ok = true;
-    auto publish_all = [&]() {
-      cp_async_wait_all();
-      fence_proxy_async_smem();
-      __syncwarp();
-#pragma unroll
-      for (int i = 0; i <= PT_LAG; ++i)
-        if (i < n_pend && lane == 0) arrive_lead(pend[i]);
-      n_pend = 0;
-    };
-    // rows [row_first, row_first + ROWS) of the block, CPR 16-byte pieces of each starting at element col_first
-    auto gather = [&](auto rows_c, auto cpr_c, uint32_t base, int slab_bytes, int pos_first, int col_first, bool is_v) {
-      constexpr int ROWS = decltype(rows_c)::value, CPR = decltype(cpr_c)::value;
-      constexpr int RSTEP = PT_LOADERS / CPR;  // rows one pass of the 128 threads covers
-      const int c = ptid % CPR, r0 = ptid / CPR;
-      const uint32_t dst = base + static_cast<uint32_t>(c >> 3) * slab_bytes;
-      // the usual case: one segment holds all the rows -> one base pointer, one stride
-      int whole = -1;
-#pragma unroll
-      for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg)
-        if (P.first[sg] <= pos_first && pos_first + ROWS <= P.first[sg] + P.len[sg]) whole = sg;
-      if (whole >= 0) {
-        const long long stride = P.stride[whole];
-        const __nv_bfloat16 *src = (is_v ? P.v[whole] : P.k[whole]) + static_cast<size_t>(pos_first - P.first[whole] + r0) * stride +
-                                   static_cast<size_t>(kvh) * D_HEAD + col_first + c * 8;
-#pragma unroll
-        for (int pass = 0; pass < ROWS / RSTEP; ++pass) {
-          const int r = r0 + pass * RSTEP;
-          cp_async16(dst + r * 128 + (((c & 7) ^ (r & 7)) << 4), src, true);
-          src += RSTEP * stride;
-        }
-      } else {
-#pragma unroll 1
-        for (int pass = 0; pass < ROWS / RSTEP; ++pass) {
-          const int r = r0 + pass * RSTEP, pos = pos_first + r;
-          const __nv_bfloat16 *src = P.q;
-          bool have = false;
-#pragma unroll
-          for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg) {
-            const int rr = pos - P.first[sg];
-            if (rr >= 0 && rr < P.len[sg]) {
-              src = (is_v ? P.v[sg] : P.k[sg]) + static_cast<size_t>(rr) * P.stride[sg] + static_cast<size_t>(kvh) * D_HEAD + col_first + c * 8;
-              have = true;
-            }
-          }
-          cp_async16(dst + r * 128 + (((c & 7) ^ (r & 7)) << 4), src, have);
-        }
-      }
-    };
-    auto emit = [&](int is_v, int j) -> bool {
-      const int n_slots = is_v ? SLOTS_V : SLOTS_K, slot = j % n_slots;
-      if (j >= n_slots) {
-        const uint32_t par = ((j / n_slots) - 1) & 1;
-        int free_now = lane == 0 ? (mbar_try_wait(bar_empty(is_v, slot), par) ? 1 : 0) : 0;
-        free_now = __shfl_sync(0xffffffffu, free_now, 0);
-        if (!free_now) {
-          publish_all();
-          int got = lane == 0 ? (polite_wait<false>(bar_empty(is_v, slot), par, s_abort, tmo) ? 1 : 0) : 0;
-          got = __shfl_sync(0xffffffffu, got, 0);
-          if (!got) return false;
-        }
-      }
-      const int pos0 = (blk0 + j) * PT_KEYS;
-      if (is_v)
-        gather(std::integral_constant<int, PT_KEYS>(), std::integral_constant<int, Cfg::V_COLS / 8>(), ring_v + slot * Cfg::TILE_BYTES,
-               Cfg::SLAB_V, pos0, static_cast<int>(rank) * Cfg::V_COLS, true);
-      else
-        gather(std::integral_constant<int, Cfg::K_ROWS>(), std::integral_constant<int, D_HEAD / 8>(), ring + slot * Cfg::TILE_BYTES,
-               Cfg::SLAB_K, pos0 + static_cast<int>(rank) * Cfg::K_ROWS, 0, false);
-      cp_async_commit();
-#pragma unroll
-      for (int i = 0; i <= PT_LAG; ++i)
-        if (i == n_pend) pend[i] = bar_full(is_v, slot);
-      ++n_pend;
-      if (n_pend > PT_LAG) {
-        // the oldest block has PT_LAG younger ones behind it: it has landed by now, or nearly
-        cp_async_wait_group<PT_LAG>();
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) arrive_lead(pend[0]);
-#pragma unroll
-        for (int i = 0; i < PT_LAG; ++i) pend[i] = pend[i + 1];
-        --n_pend;
-      }
-      return true;
-    };
-    if (n_blk > 0) {
-      ok = emit(0, 0);
-      if (ok && n_blk > 1) ok = emit(0, 1);
-      if (ok && n_blk > 2) ok = emit(0, 2);
-      for (int j = 0; ok && j < n_blk; ++j) {
-        if (j + 3 < n_blk) ok = emit(0, j + 3);
-        if (ok) ok = emit(1, j);
-      }
-      if (ok) publish_all();
-      else {
-        cp_async_wait_all();
-        raise(P.status, STATUS_TIMEOUT, s_abort);
-      }
-    }
+    pt_load_blocks<Cfg, D_HEAD>(P, ring, ring_v, bar_base, SLOTS, blk0, n_blk, kvh, static_cast<int>(rank), tid - 10 * 32, arrive_lead, s_abort, tmo);
   }
 
   // ---- teardown: every role is done with tensor memory; in a pair nobody leaves while the partner can still signal
@@ -627,6 +685,309 @@ __global__ void __launch_bounds__(PT_THREADS, 1) kvd_prefill_attn_tc_kernel(cons
     if constexpr (PAIR) tmem_dealloc_pair(tmem_base, Cfg::COLS);
     else tmem_dealloc(tmem_base, Cfg::COLS);
   }
+}
+
+// ------------------------------------------------------------------------------------------------
+// Two row tiles per CTA (d_head 128), for launches that fill the GPU.  In the kernel above the two softmax groups
+// take turns on the blocks of one tile, hand the reference maximum to each other in every block and wait for it (and
+// for the scores) about a third of the time.  Here each group has a tile of its own, so nothing is exchanged, a K or V
+// block is loaded once for 256 rows, and each tile's next scores are there before its softmax asks for them.  A CTA
+// takes longer per block than above (1950 against 1550 clocks, for twice the rows), hence only where there are enough
+// of them (prefill_dual_pays).  4096 tokens of a Qwen3-4B layer 207 -> 161 us, 16384 2783 -> 2030 us.
+//   TMEM = [ O_0, O_1 : d_head columns each | S_00, S_01, S_10, S_11 : 64 columns each (tile, block parity) ]; the
+//          weights of a block overwrite the first half of its scores.  The query tiles are in shared memory.
+//   warps = 0-3 tile 0, 4-7 tile 1, 8 and 9 the products of tiles 0 and 1, 10 and 11 loaders: twelve warps leave a
+//          thread 168 registers (with four loader warps 128, and spills: 169 instead of 161 us).
+//   order = per tile S_0 S_1 | PV_0 S_2 | PV_1 S_3 | ...: one thread issues both products; S_{j+2}, which overwrites the
+//          weights of block j, once PV_j has finished.  (Weights in columns of their own next to one score buffer
+//          measured no better: 174 us.)
+// The bits are those of the kernel above: same blocks, same reference maxima, same products, and the row sum is kept
+// in two parts (even and odd blocks), each with the reference it had two blocks ago.
+template <int D_HEAD>
+struct PdCfg {
+  static constexpr int NCTA = 1;
+  static constexpr int LOADERS = 64, THREADS = 384;
+  static constexpr int K_ROWS = PT_KEYS, V_COLS = D_HEAD;
+  static constexpr int TILE_BYTES = PT_KEYS * D_HEAD * 2;
+  static constexpr int SLAB_K = PT_KEYS * 128, SLAB_V = PT_KEYS * 128;
+  static constexpr int SLAB_Q = PT_ROWS * 128;                   // 64 channels of a query tile
+  static constexpr int Q_BYTES = PT_ROWS * D_HEAD * 2;
+  static constexpr int SLOTS_K = 5, SLOTS_V = 5, SLOTS = SLOTS_K + SLOTS_V;
+  static constexpr int COL_S = 2 * D_HEAD, COLS = 512;
+  static constexpr int N_BARS = 2 * SLOTS + 14;                  // + s_full[2][2], p_ready[2][2], pv_done[2], o_full[2], q_ready[2]
+  static constexpr int SMEM_BYTES = 1024 + 2 * Q_BYTES + SLOTS * TILE_BYTES + N_BARS * 8;
+  static_assert(COL_S + 4 * PT_KEYS <= COLS && SMEM_BYTES <= 232448, "does not fit");
+};
+
+template <int D_HEAD, int G, int DT>
+__global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_dual_kernel(const __grid_constant__ PrefillParams P) {
+  using Cfg = PdCfg<D_HEAD>;
+  constexpr int TOK = PT_ROWS / G;
+  constexpr int SLOTS = Cfg::SLOTS, SLOTS_K = Cfg::SLOTS_K, SLOTS_V = Cfg::SLOTS_V;
+  extern __shared__ uint8_t pt_smem_raw[];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_abort_i, s_lo, s_hi;
+  volatile int *s_abort = &s_abort_i;
+  const uint32_t q_smem = (smem_u32(pt_smem_raw) + 1023u) & ~1023u;  // the swizzle is a function of the address
+  const uint32_t ring = q_smem + 2 * Cfg::Q_BYTES, ring_v = ring + SLOTS_K * Cfg::TILE_BYTES;
+  const uint32_t bar_base = ring + SLOTS * Cfg::TILE_BYTES;
+  auto bar_full = [&](int v, int s) { return bar_base + 8u * (v * SLOTS_K + s); };           // a block has landed
+  auto bar_empty = [&](int v, int s) { return bar_base + 8u * (SLOTS + v * SLOTS_K + s); };  // both tiles' products with it are done
+  auto bar_s_full = [&](int t, int b) { return bar_base + 8u * (2 * SLOTS + 2 * t + b); };       // scores of a block
+  auto bar_p_ready = [&](int t, int b) { return bar_base + 8u * (2 * SLOTS + 4 + 2 * t + b); };  // weights in place
+  auto bar_pv_done = [&](int t) { return bar_base + 8u * (2 * SLOTS + 8 + t); };                 // O += P V finished
+  auto bar_o_full = [&](int t) { return bar_base + 8u * (2 * SLOTS + 10 + t); };
+  auto bar_q_ready = [&](int t) { return bar_base + 8u * (2 * SLOTS + 12 + t); };
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  // start order as above: late tokens first, for every pair of tiles all KV heads before the next shorter one
+  const int n_pairs = static_cast<int>(gridDim.x) / P.n_kv;
+  const int kvh = static_cast<int>(blockIdx.x) % P.n_kv;
+  const int cta_tok0 = (n_pairs - 1 - static_cast<int>(blockIdx.x) / P.n_kv) * 2 * TOK;
+  const unsigned long long tmo = P.timeout_ns;
+
+  if (tid == 0) {
+    for (int s = 0; s < SLOTS; ++s) {
+      mbar_init(bar_full(0, s), Cfg::LOADERS / 32);  // one arrival per loader warp
+      mbar_init(bar_empty(0, s), 2);                 // the commits of both tiles
+    }
+    for (int t = 0; t < 2; ++t) {
+      for (int b = 0; b < 2; ++b) {
+        mbar_init(bar_s_full(t, b), 1);
+        mbar_init(bar_p_ready(t, b), 4);  // one arrival per softmax warp of the tile
+      }
+      mbar_init(bar_pv_done(t), 1);
+      mbar_init(bar_o_full(t), 1);
+      mbar_init(bar_q_ready(t), 4);
+    }
+    fence_mbar_init();
+    s_abort_i = 0;
+    s_lo = INT_MAX;
+    s_hi = -1;
+  }
+  if (warp == 8) {
+    tmem_alloc(smem_u32(&s_tmem), Cfg::COLS);
+    tmem_relinquish();
+  }
+  __syncthreads();
+  // ---- key positions the CTA needs: from the smallest first-visible to the largest last-visible of its tokens
+  if (tid < 2 * TOK && cta_tok0 + tid < P.n_rows) {
+    const int qp = P.q_pos[cta_tok0 + tid];
+    int lo = P.window > 0 ? qp - P.window + 1 : 0;
+    lo = lo < P.seg_lo ? P.seg_lo : lo;
+    const int hi = qp < P.seg_hi ? qp : P.seg_hi;
+    if (hi >= lo) {
+      atomicMin(&s_lo, lo);
+      atomicMax(&s_hi, hi);
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = s_tmem;
+  const int blk0 = s_hi >= 0 ? s_lo / PT_KEYS : 0;
+  const int n_blk = s_hi >= 0 ? s_hi / PT_KEYS - blk0 + 1 : 0;
+
+  if (warp < 8) {
+    // ------------------------------------------------------------------ softmax and epilogue: thread = MMA row of tile t
+    const int t = warp >> 2, q4 = warp & 3;
+    const int row = q4 * 32 + lane;
+    const int tok = cta_tok0 + t * TOK + row / G, g = row % G;
+    const bool valid = row / G < TOK && tok < P.n_rows;
+    const int qp = valid ? P.q_pos[tok] : -1;
+    const int lo = P.window > 0 ? qp - P.window + 1 : 0;
+    const uint32_t lane_field = static_cast<uint32_t>(q4 * 32) << 16;
+    const uint32_t o_col = tmem_base + lane_field + t * D_HEAD;
+    const size_t row_off = (static_cast<size_t>(valid ? tok : 0) * P.n_q + kvh * G + (valid ? g : 0)) * D_HEAD;
+    if (n_blk > 0) {
+      // the query row into shared memory, K-major with the 128-byte swizzle (zeros for padding rows)
+      const uint4 *qsrc = reinterpret_cast<const uint4 *>(P.q + row_off);
+      const uint32_t qdst = q_smem + t * Cfg::Q_BYTES + row * 128;
+#pragma unroll
+      for (int c = 0; c < D_HEAD / 8; ++c) {
+        const uint4 w = valid ? __ldg(qsrc + c) : make_uint4(0u, 0u, 0u, 0u);
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(qdst + (c >> 3) * Cfg::SLAB_Q + (((c & 7) ^ (row & 7)) << 4)), "r"(w.x), "r"(w.y),
+                     "r"(w.z), "r"(w.w)
+                     : "memory");
+      }
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_q_ready(t));
+    }
+    // the two parts of the row sum (blocks of this and of the other parity), each with the reference it had last
+    float m_run = -CUDART_INF_F, m_own = -CUDART_INF_F, m_other = -CUDART_INF_F;
+    uint64_t l2[2] = {0ull, 0ull}, l2_other[2] = {0ull, 0ull};
+    bool ok = true;
+    const uint64_t c2 = pack2(P.scale_log2e, P.scale_log2e);
+    PtWhole whole_block(valid, lo, qp);
+    for (int j = 0; j < n_blk; ++j) {
+      const int buf = j & 1;
+      if (!polite_warp_wait(bar_s_full(t, buf), (j >> 1) & 1, s_abort, tmo, lane)) {
+        raise(P.status, STATUS_TIMEOUT, s_abort);
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t s_col = tmem_base + lane_field + Cfg::COL_S + (2 * t + buf) * PT_KEYS;
+      uint32_t s0[32], s1[32];
+      tmem_ld_x32(s_col, s0);
+      tmem_ld_x32(s_col + 32, s1);
+      const bool whole = whole_block(P, (blk0 + j) * PT_KEYS);  // (warp-uniform)
+      unsigned long long vis = ~0ull;
+      if (!whole) vis = pt_visible(P, (blk0 + j) * PT_KEYS, lo, qp);
+      tmem_wait_ld();
+      const float bm = pt_mask_max(s0, s1, whole, vis) * P.scale_log2e;  // log2 units (scale > 0)
+      // the lazy reference of the kernel above
+      const float m_prev = m_run;
+      m_run = m_prev == -CUDART_INF_F ? bm : (bm > m_prev + PT_TAU ? bm : m_prev);
+      const float m_use = m_run == -CUDART_INF_F ? 0.f : m_run;
+      const float alpha = m_prev == -CUDART_INF_F ? 1.0f : ex2_approx(m_prev - m_use);
+      const float alpha_own = m_own == -CUDART_INF_F ? 1.0f : ex2_approx(m_own - m_use);
+      m_own = m_run;
+      uint32_t w[32];
+      const uint64_t al2 = pack2(alpha_own, alpha_own);
+      l2[0] = fmul2(l2[0], al2);
+      l2[1] = fmul2(l2[1], al2);
+      pt_weights<DT>(s0, s1, c2, pack2(-m_use, -m_use), l2, w);
+      tmem_st_x32(s_col, w);  // over the scores, which are in registers
+      if (__any_sync(0xffffffffu, alpha != 1.0f)) {
+        // O holds the blocks before j (j >= 1 here: a maximum exists); the last of those products must have finished
+        if (!polite_warp_wait(bar_pv_done(t), (j - 1) & 1, s_abort, tmo, lane)) {
+          raise(P.status, STATUS_TIMEOUT, s_abort);
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        pt_rescale<D_HEAD>(o_col, alpha);
+      } else {
+        tmem_wait_st();
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_p_ready(t, buf));
+      // the next block belongs to the other part
+      const float mt = m_own;
+      m_own = m_other;
+      m_other = mt;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const uint64_t lt = l2[i];
+        l2[i] = l2_other[i];
+        l2_other[i] = lt;
+      }
+    }
+    // ---- the row sum: both parts referred to the final maximum (a sum of two: the order does not matter)
+    float l_run = 0.f;
+    if (ok && n_blk > 0) {
+      const float m_use = m_run == -CUDART_INF_F ? 0.f : m_run;
+      l_run = pt_row_sum(l2, m_own == -CUDART_INF_F ? 1.0f : ex2_approx(m_own - m_use)) +
+              pt_row_sum(l2_other, m_other == -CUDART_INF_F ? 1.0f : ex2_approx(m_other - m_use));
+      if (!polite_warp_wait(bar_o_full(t), 0, s_abort, tmo, lane)) {
+        raise(P.status, STATUS_TIMEOUT, s_abort);
+        ok = false;
+      }
+    }
+    // ---- normalise and store (a token without a visible key yields zeros)
+    if (ok) {
+      tc_fence_after();
+      const float inv = l_run > 0.f ? 1.0f / l_run : 0.f;
+      uint4 *dst = reinterpret_cast<uint4 *>(P.out + row_off);
+#pragma unroll 1
+      for (int c = 0; c < D_HEAD / 32; ++c) {
+        uint32_t r[32];
+        if (n_blk > 0) {
+          tmem_ld_x32(o_col + c * 32, r);
+          tmem_wait_ld();
+        } else {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) r[i] = 0u;
+        }
+        uint32_t o[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) o[i] = pack_out<DT>(__uint_as_float(r[2 * i]) * inv, __uint_as_float(r[2 * i + 1]) * inv);
+        if (valid) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) dst[c * 4 + i] = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+        }
+      }
+    }
+  } else if (warp < 10) {
+    // ------------------------------------------------------------------ both products of tile t (one thread)
+    constexpr uint32_t IDESC_BASE = (DT == 0 ? umma_idesc_bf16_f32(PT_ROWS, 8) : umma_idesc_f16_f32(PT_ROWS, 8)) & ~(1u << 17);
+    constexpr uint32_t IDESC_S = IDESC_BASE | (static_cast<uint32_t>(PT_KEYS >> 3) << 17);              // N = 64 keys, B K-major
+    constexpr uint32_t IDESC_O = IDESC_BASE | (static_cast<uint32_t>(D_HEAD >> 3) << 17) | (1u << 16);  // N = d_head, B MN-major
+    const int t = warp - 8;
+    if (n_blk > 0 && elect_one()) {
+      bool ok = polite_wait<false>(bar_q_ready(t), 0, s_abort, tmo);
+      auto scores = [&](int j) -> bool {
+        const int slot = j % SLOTS_K;
+        if (!polite_wait<false>(bar_full(0, slot), (j / SLOTS_K) & 1, s_abort, tmo)) return false;
+        tc_fence_after();
+        const uint32_t d = tmem_base + Cfg::COL_S + (2 * t + (j & 1)) * PT_KEYS;
+        const uint64_t qdesc0 = umma_smem_desc_sw128(q_smem + t * Cfg::Q_BYTES), kdesc0 = umma_smem_desc_sw128(ring + slot * Cfg::TILE_BYTES);
+#pragma unroll
+        for (int ks = 0; ks < D_HEAD / 16; ++ks)
+          umma_bf16(d, qdesc0 + (((ks >> 2) * Cfg::SLAB_Q + (ks & 3) * 32) >> 4), kdesc0 + (((ks >> 2) * Cfg::SLAB_K + (ks & 3) * 32) >> 4), IDESC_S,
+                    ks > 0 ? 1u : 0u);
+        umma_commit(bar_empty(0, slot));
+        umma_commit(bar_s_full(t, j & 1));
+        return true;
+      };
+      ok = ok && scores(0);
+      if (ok && n_blk > 1) ok = scores(1);
+      for (int j = 0; ok && j < n_blk; ++j) {
+        const int slot = j % SLOTS_V;
+        // the weights are in place (and O has been rescaled where a reference maximum moved), the V block has landed
+        if (!polite_wait<false>(bar_p_ready(t, j & 1), (j >> 1) & 1, s_abort, tmo) ||
+            !polite_wait<false>(bar_full(1, slot), (j / SLOTS_V) & 1, s_abort, tmo)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint64_t vdesc0 = umma_smem_desc_sw128_mn(ring_v + slot * Cfg::TILE_BYTES, Cfg::SLAB_V);
+        const uint32_t p_col = tmem_base + Cfg::COL_S + (2 * t + (j & 1)) * PT_KEYS;
+#pragma unroll
+        for (int ks = 0; ks < PT_KEYS / 16; ++ks)
+          umma_f16_ts(tmem_base + t * D_HEAD, p_col + ks * 8, vdesc0 + ((ks * 16 * 128) >> 4), IDESC_O, (j > 0 || ks > 0) ? 1u : 0u);
+        umma_commit(bar_empty(1, slot));
+        umma_commit(bar_pv_done(t));
+        // (the next scores of this buffer are not urgent: they wait for the product that reads the weights in it)
+        if (j + 2 < n_blk) ok = polite_wait<false>(bar_pv_done(t), j & 1, s_abort, tmo) && scores(j + 2);
+      }
+      if (ok) umma_commit(bar_o_full(t));
+      else raise(P.status, STATUS_TIMEOUT, s_abort);
+    }
+  } else {
+    auto arrive = [&](uint32_t bar) { mbar_arrive(bar); };
+    pt_load_blocks<Cfg, D_HEAD>(P, ring, ring_v, bar_base, SLOTS, blk0, n_blk, kvh, 0, tid - 10 * 32, arrive, s_abort, tmo);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 8) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, Cfg::COLS);
+  }
+}
+
+template <int D_HEAD, int G>
+static kvd_status prefill_dual_launch(kvd_ctx *ctx, const PrefillParams &P, cudaStream_t stream) {
+  using Cfg = PdCfg<D_HEAD>;
+  auto k0 = kvd_prefill_attn_dual_kernel<D_HEAD, G, 0>;
+  auto k1 = kvd_prefill_attn_dual_kernel<D_HEAD, G, 1>;
+  static bool configured[64] = {};
+  if (!configured[ctx->device & 63]) {
+    cudaError_t e = cudaFuncSetAttribute(k0, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(prefill attention)");
+    configured[ctx->device & 63] = true;
+  }
+  const int tok = 2 * (PT_ROWS / G);
+  const unsigned grid = static_cast<unsigned>((P.n_rows + tok - 1) / tok * P.n_kv);
+  if (ctx->dtype == 1) k1<<<grid, Cfg::THREADS, Cfg::SMEM_BYTES, stream>>>(P);
+  else k0<<<grid, Cfg::THREADS, Cfg::SMEM_BYTES, stream>>>(P);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "launch prefill attention");
+  ctx->launches += 1;
+  return KVD_OK;
 }
 
 template <int D_HEAD, int G, bool PAIR>
@@ -663,6 +1024,16 @@ static kvd_status prefill_tc_launch(kvd_ctx *ctx, const PrefillParams &P, cudaSt
   return KVD_OK;
 }
 
+// Two tiles per CTA once single tiles would be more than one per SM (Qwen3-4B layer, one tile / two tiles per CTA: 56 single
+// tiles 104 / 150 us, 176 113 / 95, 280 170 / 136, 1024 208 / 161).  At d_head 64 the products are too short for it:
+// 294 tiles of a SmolLM2 layer 58 / 72 us.
+static bool prefill_dual_pays(const kvd_ctx *ctx, const PrefillParams &P, int group) {
+  static const char *env = getenv("KVD_PREFILL_DUAL");  // 0/1 overrides, for comparisons
+  if (env) return env[0] == '1';
+  const int tok = PT_ROWS / group;
+  return static_cast<long long>((P.n_rows + tok - 1) / tok) * P.n_kv > ctx->num_sms;
+}
+
 template <int D_HEAD>
 static kvd_status prefill_tc_group(kvd_ctx *ctx, const PrefillParams &P, int group, cudaStream_t stream) {
   // pairs where the K/V bytes per block bound the kernel (d_head = 256); at 128 the softmax does, and the hand-overs
@@ -677,6 +1048,18 @@ static kvd_status prefill_tc_group(kvd_ctx *ctx, const PrefillParams &P, int gro
         case 3: return prefill_tc_launch<D_HEAD, 3, true>(ctx, P, stream);
         case 4: return prefill_tc_launch<D_HEAD, 4, true>(ctx, P, stream);
         case 8: return prefill_tc_launch<D_HEAD, 8, true>(ctx, P, stream);
+        default: return KVD_ERR_SHAPE;
+      }
+    }
+  }
+  if constexpr (D_HEAD == 128) {
+    if (prefill_dual_pays(ctx, P, group)) {
+      switch (group) {
+        case 1: return prefill_dual_launch<D_HEAD, 1>(ctx, P, stream);
+        case 2: return prefill_dual_launch<D_HEAD, 2>(ctx, P, stream);
+        case 3: return prefill_dual_launch<D_HEAD, 3>(ctx, P, stream);
+        case 4: return prefill_dual_launch<D_HEAD, 4>(ctx, P, stream);
+        case 8: return prefill_dual_launch<D_HEAD, 8>(ctx, P, stream);
         default: return KVD_ERR_SHAPE;
       }
     }
