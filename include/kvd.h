@@ -502,9 +502,13 @@ kvd_status kvd_selftest_bounds_check(kvd_ctx *ctx, void *stream);
  *   6/7 epilogue start / end     8 cycles the row-statistics warp waited   9 its total cycles
  *   10 tile index                11 (tile 0 only) kernel start
  *   12/13 (tile 0 only) global timer in ns at kernel start / end    14 (tile 0 only) kernel end
- * A call whose grid does not fit `bytes` records nothing.  No effect on results.  Traced variants: the bf16
- * kernel, and for the Gemma-3-4B head shape (d_head 256, 2 query heads per KV head) kvd_recompute_kv_fp8 and
- * kvd_decode_attention_recompute_fp8; other variants ignore the hook. */
+ * A call whose grid does not fit `bytes` (kvd_trace_bytes) records nothing.  No effect on results.  Traced variants:
+ * the bf16 kernel, and for the Gemma-3-4B head shape (d_head 256, 2 query heads per KV head) kvd_recompute_kv_fp8 and
+ * kvd_decode_attention_recompute_fp8; other variants ignore the hook.
+ * kvd_trace_bytes: what a launch over `row_blocks` blocks of 256 rows (each row source rounded up by itself) needs on a
+ * device of `num_sms` SMs; variant 0 kvd_recompute_kv*, 1 kvd_recompute_kv_fp8*, 2 the fused calls.  0 on bad
+ * arguments.  148 CTAs' worth (148 * 8 * 16 * 8 bytes on a B200) is enough for every launch. */
+size_t kvd_trace_bytes(const kvd_model_desc *d, int row_blocks, int variant, int num_sms);
 kvd_status kvd_set_trace(kvd_ctx *ctx, void *buf, size_t bytes);
 
 /* Number of kernels this context has launched since creation (all entry points). */

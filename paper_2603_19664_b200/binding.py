@@ -43,7 +43,7 @@ EXPORTED_SYMBOLS = (
     "kvd_checkpoint_residual_fp4", "kvd_fp4_scratch_bytes", "kvd_recompute_kv_fp4",
     "kvd_rows_stored", "kvd_workspace_bytes", "kvd_attention_split", "kvd_attach_workspace", "kvd_checkpoint_residual", "kvd_checkpoint_residual_step", "kvd_decode_step_kv", "kvd_recompute_kv",
     "kvd_recompute_kv_step",
-    "kvd_decode_attention", "kvd_decode_attention_rows", "kvd_prefill_attention", "kvd_decode_attention_static", "kvd_memory_stats", "kvd_poll_status", "kvd_selftest_wait_timeout", "kvd_build_has_checks", "kvd_selftest_bounds_check", "kvd_set_trace", "kvd_launch_count", "kvd_last_cuda_error",
+    "kvd_decode_attention", "kvd_decode_attention_rows", "kvd_prefill_attention", "kvd_decode_attention_static", "kvd_memory_stats", "kvd_poll_status", "kvd_selftest_wait_timeout", "kvd_build_has_checks", "kvd_selftest_bounds_check", "kvd_set_trace", "kvd_trace_bytes", "kvd_launch_count", "kvd_last_cuda_error",
     "kvd_status_string", "kvd_version",
     # include/kvd_scaffold.h: the parts of a decoder layer around the hot path, for whole-stack tests and benchmarks
     "kvd_scaffold_linear_create", "kvd_scaffold_linear_destroy", "kvd_scaffold_linear_out_cols", "kvd_scaffold_linear",
@@ -217,6 +217,8 @@ def load() -> ctypes.CDLL:
     lib.kvd_selftest_bounds_check.restype = i32
     lib.kvd_set_trace.argtypes = [vp, vp, sz]
     lib.kvd_set_trace.restype = i32
+    lib.kvd_trace_bytes.argtypes = [ctypes.POINTER(kvd_model_desc), i32, i32, i32]
+    lib.kvd_trace_bytes.restype = sz
     lib.kvd_launch_count.argtypes = [vp]
     lib.kvd_launch_count.restype = ctypes.c_uint64
     lib.kvd_last_cuda_error.argtypes = [vp]
@@ -288,6 +290,10 @@ def kvd_fp4_scratch_bytes(desc: kvd_model_desc, max_rows: int) -> int:
 
 def kvd_workspace_bytes(desc: kvd_model_desc) -> int:
     return int(load().kvd_workspace_bytes(ctypes.byref(desc)))
+
+
+def kvd_trace_bytes(desc: kvd_model_desc, row_blocks: int, variant: int = 0, num_sms: int = 148) -> int:
+    return int(load().kvd_trace_bytes(ctypes.byref(desc), row_blocks, variant, num_sms))
 
 
 def kvd_fused_recompute_pays(desc: kvd_model_desc, total_rows: int, fp8: bool = False) -> bool:

@@ -458,7 +458,7 @@ extern "C" kvd_status kvd_checkpoint_residual_step(kvd_ctx *ctx, int layer, int 
 
 // The launch parameters every variant of the recompute kernel shares (jobs are filled in by the caller).
 static void fill_launch_params(const kvd_ctx *ctx, const LayerState &ls, RecomputeParams &p, int n_jobs, int m_blocks,
-                               int k_blocks, int64_t out_row_stride) {
+                               int k_blocks, int64_t out_row_stride, int eb, bool fused) {
   const kvd_model_desc &d = ctx->desc;
   const int kdim = d.n_kv_heads * d.d_head;
   p.n_jobs = n_jobs;
@@ -478,7 +478,6 @@ static void fill_launch_params(const kvd_ctx *ctx, const LayerState &ls, Recompu
   p.gamma_k = d.qk_norm ? ls.gamma_k : nullptr;
   p.status = ctx->d_status;
   p.timeout_ns = ctx->timeout_ns;
-  p.trace = nullptr;
   p.ext_rows = nullptr;
   p.w_scale = nullptr;
   p.rows_out_stride = out_row_stride;
@@ -487,6 +486,7 @@ static void fill_launch_params(const kvd_ctx *ctx, const LayerState &ls, Recompu
   p.append_pos = nullptr;
   p.append_sumsq = nullptr;
   p.store_rows = d.max_tokens_per_seq;
+  schedule_recompute(ctx, p, eb, fused);
   p.row_chunks = d.d_hidden * dtype_bytes(ctx->dtype) / 16;
   // 32-byte stores need every output row 32-byte aligned
   p.wide_store = out_row_stride * dtype_bytes(ctx->dtype) % 32 == 0;
@@ -577,7 +577,7 @@ static kvd_status recompute_launch(kvd_ctx *ctx, int layer, const kvd_store_rang
   // the kernel is handed both maps; an unused one aliases the other
   const CUtensorMap &tmap_store = any_store ? ctx->store_maps[layer] : tmap_rows;
   const CUtensorMap &tmap_ext = n_rows > 0 ? tmap_rows : ctx->store_maps[layer];
-  fill_launch_params(ctx, ls, p, n_jobs, mb, d.d_hidden * es / (2 * RC_BLOCK_K), out_row_stride);  // 128 bytes per k block
+  fill_launch_params(ctx, ls, p, n_jobs, mb, d.d_hidden * es / (2 * RC_BLOCK_K), out_row_stride, es, fused != nullptr);  // 128 bytes per k block
   p.ext_rows = static_cast<const __nv_bfloat16 *>(rows);
   std::vector<int> add;
   if (step && n_rows > 0) {
@@ -605,11 +605,6 @@ static kvd_status recompute_launch(kvd_ctx *ctx, int layer, const kvd_store_rang
       p.append_pos = ctx->store_pos;
       p.append_sumsq = ctx->store_sumsq;
     }
-  }
-  if (ctx->trace) {
-    const int tiles = p.num_m_blocks * p.num_n_blocks;
-    const size_t ctas = 2 * static_cast<size_t>(tiles < ctx->num_sms / 2 ? tiles : ctx->num_sms / 2);
-    if (ctas * RC_TRACE_TILES * RC_TRACE_FIELDS * sizeof(long long) <= ctx->trace_bytes) p.trace = ctx->trace;
   }
   if (fused) {
     fp.part_o = fused_head->part_o;
@@ -805,13 +800,8 @@ static kvd_status recompute_launch_fp8(kvd_ctx *ctx, int layer, const kvd_store_
   const CUtensorMap &map_store = any_store ? ctx->store8_maps[layer] : tmap_rows;
   const CUtensorMap &map_rows = have_rows ? tmap_rows : ctx->store8_maps[layer];
   // 128 channels per k block; the tail reads zeros
-  fill_launch_params(ctx, ls, p, n_jobs, mb, (d.d_hidden + 2 * RC_BLOCK_K - 1) / (2 * RC_BLOCK_K), out_row_stride);
+  fill_launch_params(ctx, ls, p, n_jobs, mb, (d.d_hidden + 2 * RC_BLOCK_K - 1) / (2 * RC_BLOCK_K), out_row_stride, 1, fused != nullptr);
   p.w_scale = ls.w_scale8;
-  if (ctx->trace) {
-    const int tiles = p.num_m_blocks * p.num_n_blocks;
-    const size_t ctas = 2 * static_cast<size_t>(tiles < ctx->num_sms / 2 ? tiles : ctx->num_sms / 2);
-    if (ctas * RC_TRACE_TILES * RC_TRACE_FIELDS * sizeof(long long) <= ctx->trace_bytes) p.trace = ctx->trace;
-  }
   if (fused) {
     fp.part_o = fused_head->part_o;
     fp.part_ml = fused_head->part_ml;
@@ -1261,6 +1251,12 @@ extern "C" kvd_status kvd_selftest_wait_timeout(kvd_ctx *ctx, int limit_ms, void
   if (!ctx || limit_ms <= 0 || limit_ms > 1000) return KVD_ERR_INVALID_ARG;
   return launch_selftest_timeout(ctx, static_cast<unsigned long long>(limit_ms) * 1000000ull,
                                  static_cast<cudaStream_t>(stream_));
+}
+
+extern "C" size_t kvd_trace_bytes(const kvd_model_desc *d, int row_blocks, int variant, int num_sms) {
+  if (check_desc(d) != KVD_OK || row_blocks <= 0 || variant < 0 || variant > 2 || num_sms < 2) return 0;
+  const int kdim = d->n_kv_heads * d->d_head, bn = pick_block_n(d);
+  return rc_trace_bytes(rc_schedule(num_sms, bn, d->d_head, row_blocks, 2 * kdim / bn, kdim, variant == 0 ? 2 : 1, variant == 2).clusters);
 }
 
 extern "C" kvd_status kvd_set_trace(kvd_ctx *ctx, void *buf, size_t bytes) {

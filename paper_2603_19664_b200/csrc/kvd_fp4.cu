@@ -329,7 +329,6 @@ extern "C" kvd_status kvd_recompute_kv_fp4(kvd_ctx *ctx, int layer, const kvd_st
   p.gamma_k = d.qk_norm ? ls.gamma_k : nullptr;
   p.status = ctx->d_status;
   p.timeout_ns = ctx->timeout_ns;
-  p.trace = nullptr;
   p.ext_rows = x;
   p.row_chunks = row_chunks;
   p.w_scale = nullptr;
@@ -341,5 +340,7 @@ extern "C" kvd_status kvd_recompute_kv_fp4(kvd_ctx *ctx, int layer, const kvd_st
   p.wide_store = out_row_stride * 2 % 32 == 0;
   for (int j = 0; j < n_jobs; ++j)
     if (((reinterpret_cast<uintptr_t>(p.jobs[j].k_out) | reinterpret_cast<uintptr_t>(p.jobs[j].v_out)) & 31u) != 0) p.wide_store = 0;
+  schedule_recompute(ctx, p, 2, false);
+  p.trace = nullptr;
   return launch_recompute(ctx, ls, tmap_rows, tmap_rows, p, stream);
 }

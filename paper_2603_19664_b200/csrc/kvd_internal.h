@@ -67,7 +67,7 @@ struct RecomputeParams {
   int num_k_blocks;  // d_hidden / 64
   int num_m_blocks;  // over all jobs
   int num_n_blocks;
-  int unit_tiles, whole_tiles, parts;  // schedule of the plain kernel (rc_schedule)
+  int unit_tiles, whole_tiles, parts, clusters;  // set by schedule_recompute
   int k_cols;  // n_kv * d_head: fused columns below this index are keys, the rest values
   long long out_row_stride;
   float inv_d_hidden;
@@ -349,8 +349,26 @@ inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, unsigned thre
 }
 
 // launchers implemented next to their kernels
+// Schedule of a launch: its tiles (units of two, single ones, cut ones) and its CTA pairs.  The one place both the launch
+// and the size test of the trace buffer take the grid from.
+struct RcSchedule {
+  int unit_tiles, whole_tiles, parts, clusters;
+};
+RcSchedule rc_schedule(int num_sms, int block_n, int d_head, int m_blocks, int n_blocks, int k_cols, int eb, bool fused);
+inline size_t rc_trace_bytes(int clusters) {
+  return 2 * static_cast<size_t>(clusters) * RC_TRACE_TILES * RC_TRACE_FIELDS * sizeof(long long);
+}
+// After the sizes of `p` are known: its schedule, and the trace buffer if the launch fits it.
+inline void schedule_recompute(const kvd_ctx *ctx, RecomputeParams &p, int eb, bool fused) {
+  const RcSchedule s = rc_schedule(ctx->num_sms, ctx->block_n, ctx->desc.d_head, p.num_m_blocks, p.num_n_blocks, p.k_cols, eb, fused);
+  p.unit_tiles = s.unit_tiles;
+  p.whole_tiles = s.whole_tiles;
+  p.parts = s.parts;
+  p.clusters = s.clusters;
+  p.trace = ctx->trace && rc_trace_bytes(s.clusters) <= ctx->trace_bytes ? ctx->trace : nullptr;
+}
 kvd_status launch_recompute(kvd_ctx *ctx, const LayerState &ls, const CUtensorMap &tmap_store,
-                            const CUtensorMap &tmap_rows, RecomputeParams &p, cudaStream_t stream);
+                            const CUtensorMap &tmap_rows, const RecomputeParams &p, cudaStream_t stream);
 kvd_status launch_recompute_fused(kvd_ctx *ctx, const LayerState &ls, const CUtensorMap &tmap_store,
                                   const CUtensorMap &tmap_rows, const RecomputeParams &p, const FusedParams &fp,
                                   cudaStream_t stream, int eb = 2);
@@ -370,7 +388,7 @@ kvd_status launch_prepare_weights_fp8(kvd_ctx *ctx, const __nv_bfloat16 *w, cons
                                       int d_hidden, int n_cols, unsigned *amax_scratch, float *scale_out,
                                       cudaStream_t stream);
 kvd_status launch_recompute_fp8(kvd_ctx *ctx, const LayerState &ls, const CUtensorMap &tmap_store,
-                                const CUtensorMap &tmap_rows, RecomputeParams &p, cudaStream_t stream);
+                                const CUtensorMap &tmap_rows, const RecomputeParams &p, cudaStream_t stream);
 kvd_status launch_checkpoint(kvd_ctx *ctx, const __nv_bfloat16 *rows, const int32_t *pos, __nv_bfloat16 *dst_rows,
                              int32_t *dst_pos, float *dst_sumsq, int n, int d_hidden, cudaStream_t stream);
 kvd_status launch_selftest_bounds(kvd_ctx *ctx, cudaStream_t stream);

@@ -927,14 +927,9 @@ static kvd_status launch_impl(kvd_ctx *ctx, const LayerState &ls, const CUtensor
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(recompute)");
     configured[ctx->device & 63] = true;
   }
-  // plain: one cluster per tile (or part of one) at most; fused: per unit of a key tile and a value tile
-  const int tiles = p.num_m_blocks * p.num_n_blocks;
-  const int work = FG > 0 || p.unit_tiles == 2 ? tiles / 2 : p.whole_tiles + (tiles - p.whole_tiles) * p.parts;
-  const int max_clusters = ctx->num_sms / 2;
-  const int clusters = work < max_clusters ? work : max_clusters;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3(2 * clusters, 1, 1);
+  cfg.gridDim = dim3(2 * p.clusters, 1, 1);
   cfg.blockDim = dim3(RC_THREADS, 1, 1);
   cfg.dynamicSmemBytes = Cfg::SMEM_BYTES;
   cfg.stream = stream;
@@ -983,38 +978,36 @@ static kvd_status launch_sel(kvd_ctx *ctx, const LayerState &ls, const CUtensorM
 // L2 (64 x 767 rows: 415 us in units, 422 single), units it is.  With less than one round (Qwen, 8 tiles 31 -> 20, 72
 // tiles 23.9 -> 21.7) halves shorten every CTA's exposed epilogue, if a half still holds whole heads: the key norm
 // runs over a head in one thread.
-static void rc_schedule(const kvd_ctx *ctx, RecomputeParams &p, int eb) {
-  const int tiles = p.num_m_blocks * p.num_n_blocks, clusters = ctx->num_sms / 2, bn = ctx->block_n, dh = ctx->desc.d_head;
-  const int nk = p.k_cols % bn == 0 ? p.k_cols / bn : 0;  // 0 also where a tile mixes key and value heads
+RcSchedule rc_schedule(int num_sms, int block_n, int d_head, int m_blocks, int n_blocks, int k_cols, int eb, bool fused) {
+  const int tiles = m_blocks * n_blocks, clusters = num_sms / 2;
+  const int nk = k_cols % block_n == 0 ? k_cols / block_n : 0;  // 0 also where a tile mixes key and value heads
   const int rounds = tiles / clusters, last = tiles % clusters;
-  p.unit_tiles = 1;
-  p.whole_tiles = tiles;
-  p.parts = 1;
+  RcSchedule s = {1, tiles, 1, 0};
   float single = static_cast<float>(rounds + (last > 0 ? 1 : 0));
-  if (eb != 1 && bn == 256 && (nk != 0 || p.k_cols == 0) && last > 0 && rounds <= 8) {
+  if (eb != 1 && block_n == 256 && (nk != 0 || k_cols == 0) && last > 0 && rounds <= 8) {
     int parts = rounds == 0 ? 2 : 4 * last <= clusters ? 4 : 2 * last <= clusters ? 2 : 1;
-    const bool keys = last > p.num_m_blocks * (p.num_n_blocks - nk);  // key tiles among those to be cut
-    if (keys && bn / parts < dh) parts = 1;
+    const bool keys = last > m_blocks * (n_blocks - nk);  // key tiles among those to be cut
+    if (keys && block_n / parts < d_head) parts = 1;
     if (parts > 1) {
-      p.whole_tiles = tiles - last;
-      p.parts = parts;
+      s.whole_tiles = tiles - last;
+      s.parts = parts;
       single = static_cast<float>(rounds) + (parts == 2 ? 0.62f : 0.53f);
     }
   }
-  if (nk != 0 && p.num_n_blocks == 2 * nk && tiles > clusters) {
-    const float units = 2.f * static_cast<float>((tiles / 2 + clusters - 1) / clusters);
-    if (eb == 1 || rounds > 8 || units <= single) {
-      p.unit_tiles = 2;
-      p.whole_tiles = tiles;
-      p.parts = 1;
-    }
+  bool units = fused;
+  if (nk != 0 && n_blocks == 2 * nk && tiles > clusters) {
+    const float cost = 2.f * static_cast<float>((tiles / 2 + clusters - 1) / clusters);
+    units = units || eb == 1 || rounds > 8 || cost <= single;
   }
+  if (units) s = {2, tiles, 1, 0};
+  const int work = units ? tiles / 2 : s.whole_tiles + (tiles - s.whole_tiles) * s.parts;
+  s.clusters = work < clusters ? work : clusters;
+  return s;
 }
 
 kvd_status launch_recompute(kvd_ctx *ctx, const LayerState &ls, const CUtensorMap &tmap_store,
-                            const CUtensorMap &tmap_rows, RecomputeParams &p, cudaStream_t stream) {
+                            const CUtensorMap &tmap_rows, const RecomputeParams &p, cudaStream_t stream) {
   const int dh = ctx->desc.d_head;
-  rc_schedule(ctx, p, 2);
   if (ctx->block_n == 256) {
     if (dh == 256) return launch_sel<256, 256>(ctx, ls, tmap_store, tmap_rows, p, nullptr, stream);
     if (dh == 128) return launch_sel<256, 128>(ctx, ls, tmap_store, tmap_rows, p, nullptr, stream);
@@ -1054,9 +1047,8 @@ kvd_status launch_recompute_fused(kvd_ctx *ctx, const LayerState &ls, const CUte
 // The FP8 variant: rows and weights as E4M3 codes (tmap_store is the FP8 store's map, tmap_rows the map of
 // the caller's quantised rows, or the store's again).
 kvd_status launch_recompute_fp8(kvd_ctx *ctx, const LayerState &ls, const CUtensorMap &tmap_store,
-                                const CUtensorMap &tmap_rows, RecomputeParams &p, cudaStream_t stream) {
+                                const CUtensorMap &tmap_rows, const RecomputeParams &p, cudaStream_t stream) {
   const int dh = ctx->desc.d_head;
-  rc_schedule(ctx, p, 1);
   if (ctx->block_n == 256) {
     if (dh == 256 && p.trace != nullptr) return launch_impl<256, 256, true, 0, 1, true>(ctx, ls, tmap_store, tmap_rows, p, nullptr, stream);
     if (dh == 256) return launch_impl<256, 256, false, 0, 1, true>(ctx, ls, tmap_store, tmap_rows, p, nullptr, stream);

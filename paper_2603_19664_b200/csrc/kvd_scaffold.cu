@@ -324,7 +324,6 @@ extern "C" kvd_status kvd_scaffold_linear(kvd_ctx *ctx, const kvd_linear *lin, c
   p.gamma_k = nullptr;
   p.status = ctx->d_status;
   p.timeout_ns = ctx->timeout_ns;
-  p.trace = nullptr;
   p.ext_rows = static_cast<const __nv_bfloat16 *>(x);
   p.row_chunks = lin->k / 8;
   p.wide_store = (out_row_stride * 2 % 32 == 0) && ((reinterpret_cast<uintptr_t>(out) & 31u) == 0);
@@ -335,6 +334,8 @@ extern "C" kvd_status kvd_scaffold_linear(kvd_ctx *ctx, const kvd_linear *lin, c
   p.append_pos = nullptr;
   p.append_sumsq = nullptr;
   p.store_rows = m;
+  schedule_recompute(ctx, p, 2, false);
+  p.trace = nullptr;
   return launch_recompute(ctx, lin->ls, tmap_rows, tmap_rows, p, stream);
 }
 

@@ -112,3 +112,22 @@ def test_fused_predicate_is_host_only_and_shape_aware():
     assert kvd.kvd_fused_recompute_pays(gemma, 4096, fp8=True) and not kvd.kvd_fused_recompute_pays(gemma, 1024, fp8=True)
     assert not kvd.kvd_fused_recompute_pays(smol, 1 << 20)  # no fused kernel for this shape
     assert not kvd.kvd_fused_recompute_pays(gemma, 0)
+
+
+def test_trace_bytes_cover_the_grid_a_launch_gets():
+    """The trace buffer's size test is taken from the schedule the launch uses: a launch of fewer tiles than clusters is
+    cut into twice as many pieces where a piece still holds whole key heads."""
+    per_cta = 8 * 16 * 8
+    qwen = kvd.make_desc(1, 2560, 32, 8, 128, 1e-6, True, 1e-6)
+    gemma = kvd.make_desc(1, 2560, 8, 4, 256, 1e-6, True, 1e-6)
+    smol = kvd.make_desc(1, 576, 9, 3, 64, 1e-5, False, 1e-5)
+    assert kvd.kvd_trace_bytes(qwen, 1) == 32 * per_cta          # 8 tiles, halved
+    assert kvd.kvd_trace_bytes(qwen, 1, variant=1) == 16 * per_cta
+    assert kvd.kvd_trace_bytes(gemma, 1) == 16 * per_cta         # a half tile would split a key head
+    assert kvd.kvd_trace_bytes(gemma, 1, variant=2) == 8 * per_cta  # units of a key and a value tile
+    assert kvd.kvd_trace_bytes(smol, 1) == 6 * per_cta           # 128-column tiles
+    for desc in (qwen, gemma, smol):
+        for variant in (0, 1, 2):
+            for blocks in (1, 5, 9, 10, 18, 19, 37, 1000):
+                assert 0 < kvd.kvd_trace_bytes(desc, blocks, variant) <= 148 * per_cta
+    assert kvd.kvd_trace_bytes(qwen, 0) == 0 and kvd.kvd_trace_bytes(qwen, 1, variant=3) == 0
