@@ -504,7 +504,9 @@ kvd_status kvd_selftest_bounds_check(kvd_ctx *ctx, void *stream);
  *   12/13 (tile 0 only) global timer in ns at kernel start / end    14 (tile 0 only) kernel end
  * A call whose grid does not fit `bytes` (kvd_trace_bytes) records nothing.  No effect on results.  Traced variants:
  * the bf16 kernel, and for the Gemma-3-4B head shape (d_head 256, 2 query heads per KV head) kvd_recompute_kv_fp8 and
- * kvd_decode_attention_recompute_fp8; other variants ignore the hook.
+ * kvd_decode_attention_recompute_fp8; other variants ignore the hook.  What is traced is always the recompute kernel: a
+ * bf16 call of at most 64 caller rows and no store range, which otherwise runs on the few-row kernel (same bits, other
+ * times), takes the recompute kernel while a buffer that fits it is attached.
  * kvd_trace_bytes: what a launch over `row_blocks` blocks of 256 rows (each row source rounded up by itself) needs on a
  * device of `num_sms` SMs; variant 0 kvd_recompute_kv*, 1 kvd_recompute_kv_fp8*, 2 the fused calls.  0 on bad
  * arguments.  148 CTAs' worth (148 * 8 * 16 * 8 bytes on a B200) is enough for every launch. */

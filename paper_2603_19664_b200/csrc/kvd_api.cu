@@ -615,7 +615,8 @@ static kvd_status recompute_launch(kvd_ctx *ctx, int layer, const kvd_store_rang
   }
   kvd_status st;
   if (!any_store && n_rows <= RW_MAX_ROWS && ctx->dtype != KVD_DTYPE_F32 && p.trace == nullptr) {
-    // only a few new rows: the projection that reads the weights at memory speed (same bits)
+    // only a few new rows: the projection that reads the weights at memory speed (same bits).  A traced call (bf16) stays
+    // on the kernel that records, as kvd_set_trace says.
     RowsParams r = {};
     r.rows = static_cast<const uint4 *>(rows);
     r.positions = positions;

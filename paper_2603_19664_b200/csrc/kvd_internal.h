@@ -365,7 +365,8 @@ inline void schedule_recompute(const kvd_ctx *ctx, RecomputeParams &p, int eb, b
   p.whole_tiles = s.whole_tiles;
   p.parts = s.parts;
   p.clusters = s.clusters;
-  p.trace = ctx->trace && rc_trace_bytes(s.clusters) <= ctx->trace_bytes ? ctx->trace : nullptr;
+  // (fp16 and fp32 kernels record nothing, and the hook must not choose the kernel of a call it cannot trace)
+  p.trace = ctx->trace && ctx->dtype == KVD_DTYPE_BF16 && rc_trace_bytes(s.clusters) <= ctx->trace_bytes ? ctx->trace : nullptr;
 }
 kvd_status launch_recompute(kvd_ctx *ctx, const LayerState &ls, const CUtensorMap &tmap_store,
                             const CUtensorMap &tmap_rows, const RecomputeParams &p, cudaStream_t stream);

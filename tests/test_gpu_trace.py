@@ -40,3 +40,28 @@ def test_trace_stays_inside_its_buffer(shape, n):
     assert (t[:, 0, 7] > t[:, 0, 6]).all()  # every CTA recorded its first tile's epilogue
     assert ctx.kvd_poll_status() == kvd.KVD_OK
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype", [0, 1], ids=["bf16", "f16"])
+def test_a_traced_call_of_few_rows(dtype):
+    """bf16: a call of at most 64 caller rows takes the kernel that records while a buffer is attached, with the bits of
+    the few-row kernel it takes otherwise.  fp16: nothing records, the attached buffer stays untouched."""
+    shape = QWEN3_4B
+    kdim, t = shape.n_kv_heads * shape.d_head, (torch.bfloat16, torch.float16)[dtype]
+    ctx = kvd.Kvd(kvd.make_desc(1, shape.d_hidden, shape.n_q_heads, shape.n_kv_heads, shape.d_head, shape.rms_eps, shape.qk_norm,
+                                shape.rms_eps, shape.rope_style, 1, 256, 1))
+    ctx.kvd_set_dtype(dtype)
+    g = torch.Generator(device="cuda").manual_seed(2)
+    w = (torch.randn((shape.d_hidden, 2 * kdim), generator=g, device="cuda") * 0.02).to(t)
+    ctx.kvd_set_layer(0, w, torch.ones(shape.d_hidden, device="cuda").to(t), torch.ones(shape.d_head, device="cuda").to(t), shape.rope_theta)
+    x, pos = torch.randn((33, shape.d_hidden), generator=g, device="cuda").to(t), torch.arange(33, dtype=torch.int32, device="cuda")
+    k, v, k2, v2 = (torch.empty((33, kdim), dtype=t, device="cuda") for _ in range(4))
+    ctx.kvd_recompute_kv(0, x, pos, 33, k, v, kdim)
+    trace = torch.zeros((148, 8, 16), dtype=torch.int64, device="cuda")
+    ctx.kvd_set_trace(trace)
+    ctx.kvd_recompute_kv(0, x, pos, 33, k2, v2, kdim)
+    ctx.kvd_set_trace(None)
+    assert torch.equal(k, k2) and torch.equal(v, v2)
+    assert bool((trace[0, 0, 7] > trace[0, 0, 6])) == (dtype == 0) and bool((trace[32:] == 0).all())
+    assert ctx.kvd_poll_status() == kvd.KVD_OK
+    ctx.close()
