@@ -122,7 +122,6 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
     *s_abort = 0;
     fence_mbar_init();
   }
-  grid_launch_dependents();
   if (warp == 1) {
     tmem_alloc(smem_u32(s_tmem), p.tmem_cols);
     tmem_relinquish();
@@ -132,6 +131,9 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
   else __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
+  // Only now, with the tensor memory in hand: the allocation is a wait without a limit, and a dependent let in before it
+  // could take the columns this CTA waits for, and then wait for this kernel's end.
+  grid_launch_dependents();
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer

@@ -65,3 +65,22 @@ def test_products_of_few_rows_have_the_bits_of_the_large_call(k, n):
             assert bool((out[:m, lin.out_cols:] == 7).all()) and bool((out[m] == 7).all()), (r0, m, pad)
     assert ctx.kvd_poll_status() == kvd.KVD_OK
     ctx.close()
+
+
+@pytest.mark.parametrize("k,n", [(64, 128), (128, 20480), (256, 20480)])
+def test_successive_products_overlap_without_changing_bits(k, n):
+    """Launches that follow one another directly, each a dependent of the last, with much tensor memory and little shared
+    memory per CTA: every one ends, with the bits of a launch alone."""
+    ctx, _ = open_layer(GEMMA3_4B_GLOBAL, max_tokens=256)
+    g = torch.Generator(device="cuda").manual_seed(k + n)
+    lin = ctx.kvd_scaffold_linear_create((torch.randn((k, n), generator=g, device="cuda") * 0.05).bfloat16(), None, k, n)
+    x = torch.randn((8, 5, k), generator=g, device="cuda").bfloat16()
+    alone, out = (torch.zeros((8, 5, lin.out_cols), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    for i in range(8):
+        ctx.kvd_scaffold_linear(lin, x[i], 5, alone[i], lin.out_cols)
+        torch.cuda.synchronize()
+    for i in range(8):
+        ctx.kvd_scaffold_linear(lin, x[i], 5, out[i], lin.out_cols)
+    assert torch.equal(alone, out)
+    assert ctx.kvd_poll_status() == kvd.KVD_OK
+    ctx.close()

@@ -1,0 +1,42 @@
+"""Source rules of kernels that start before their predecessor has finished (programmatic dependent launches).
+
+They are properties of the source that no run shows reliably: breaking one gives a hang or a stale read only when a
+launch happens to overlap its neighbours in the wrong way.
+"""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2603_19664_b200", "csrc")
+TEXT = {f: re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, f)).read()) for f in sorted(os.listdir(CSRC))}
+ALL = "\n".join(TEXT.values())
+
+
+def _span(start, opening, closing):
+    depth, i = 1, start
+    while depth:
+        depth += {opening: 1, closing: -1}.get(ALL[i], 0)
+        i += 1
+    return i
+
+
+# name -> (arguments, body) of every kernel
+KERNELS = {}
+for m in re.finditer(r"__global__ void\s+(?:__launch_bounds__\((?:[^()]|\([^()]*\))*\)\s*)?(\w+)\s*\(", ALL):
+    args_end = _span(m.end(), "(", ")")
+    body = ALL.index("{", args_end) + 1
+    KERNELS[m.group(1)] = (ALL[m.end():args_end], ALL[body:_span(body, "{", "}")])
+
+
+@pytest.mark.parametrize("name", sorted(k for k, (_, b) in KERNELS.items() if "tmem_alloc" in b and "grid_launch_dependents" in b))
+def test_dependents_start_only_after_tensor_memory_is_allocated(name):
+    """tcgen05.alloc waits without a limit.  A dependent that is let in first can take the columns its predecessor waits
+    for, and then waits for that predecessor's end."""
+    body = KERNELS[name][1]
+    alloc, start = body.index("tmem_alloc"), body.index("grid_launch_dependents")
+    assert alloc < start and re.search(r"__syncthreads\(\)|cluster_sync_all\(\)", body[alloc:start])
+
+
+def test_both_projection_kernels_are_covered():
+    assert all("tmem_alloc" in KERNELS[k][1] and "grid_launch_dependents" in KERNELS[k][1] for k in ("kvd_rows_kernel", "kvd_recompute_kernel"))
