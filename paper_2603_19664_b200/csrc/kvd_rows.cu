@@ -149,11 +149,9 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
       for (int i = 0; i < pre; ++i) tma_load_3d(ring + i * stage_bytes, &tmap_x, bar_full(i), 0, 0, i % steps * kbs);
       int issued = pre, s = 0, k = pre % steps, col = (block + pre / steps * blocks) * tile;
       uint32_t ph = 0;  // parity of the phase of `empty` that frees stage s for its next fill
-      bool ok = true;
       for (; issued < total; ++issued) {
         if (!mbar_wait(bar_empty(s), ph, s_abort, tmo)) {
           raise(p.status, STATUS_TIMEOUT, s_abort);
-          ok = false;
           break;
         }
         mbar_arrive_expect_tx(bar_full(s), stage_bytes);
@@ -168,14 +166,14 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
           ph ^= 1u;
         }
       }
-      if (!ok || *s_abort != 0) {
-        // leave no copy in flight: wait (bounded) for the last fill of every stage
-        for (int b = 0; b < stages && b < issued; ++b) {
-          const uint32_t par = static_cast<uint32_t>((issued - 1 - b) / stages) & 1u;
-          const unsigned long long t0 = globaltimer_ns();
-          while (!mbar_try_wait(bar_full(b), par))
-            if (globaltimer_ns() - t0 > 100000000ull) break;
-        }
+      // Leave no copy in flight: wait (bounded) for the last fill of every stage.  Always, and longer than the MMA issuer
+      // waits: that thread may give up after this one has issued everything, and then nobody else watches the copies.
+      // (In a launch that runs its course the issuer waits for the same fills.)
+      const unsigned long long t0 = globaltimer_ns();
+      for (int b = 0; b < stages && b < issued; ++b) {
+        const uint32_t par = static_cast<uint32_t>((issued - 1 - b) / stages) & 1u;
+        while (!mbar_try_wait(bar_full(b), par))
+          if (globaltimer_ns() - t0 > tmo + 100000000ull) break;
       }
     }
   } else if (warp == 1) {

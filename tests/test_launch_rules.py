@@ -40,3 +40,14 @@ def test_dependents_start_only_after_tensor_memory_is_allocated(name):
 
 def test_both_projection_kernels_are_covered():
     assert all("tmem_alloc" in KERNELS[k][1] and "grid_launch_dependents" in KERNELS[k][1] for k in ("kvd_rows_kernel", "kvd_recompute_kernel"))
+
+
+def test_few_row_producer_waits_for_its_last_copies_on_every_path():
+    """A CTA that ends with a bulk copy in flight lets it land in the next CTA's shared memory."""
+    body = KERNELS["kvd_rows_kernel"][1]
+    drain = body[body.index("int issued"):body.index("umma_kblock")]
+    drain = drain[:drain.index("else if (warp == 1)")]
+    last = drain[drain.rindex("for (int b = 0; b < stages && b < issued"):]
+    assert "mbar_try_wait(bar_full(b), par)" in last and "tmo +" in last
+    between = drain[drain.rindex("ph ^= 1u;"):drain.rindex("for (int b = 0")]
+    assert "if (" not in between  # the wait hangs on no condition
