@@ -41,10 +41,10 @@ __device__ __forceinline__ float e4m3_value(uint32_t code) {
 // One warp per row.  Lane l holds chunks l, l + 32, ... (8 channels each); a block of 16 channels is a pair of
 // neighbouring chunks, i.e. an even lane and its odd neighbour.  Rows of up to 32 * CPL chunks stay in registers.
 template <int CPL>
-__global__ void __launch_bounds__(256, 2) kvd_checkpoint_fp4_kernel(const uint4 *__restrict__ rows, const int32_t *__restrict__ pos,
-                                                                 uint32_t *__restrict__ dst_codes, uint8_t *__restrict__ dst_block,
-                                                                 int32_t *__restrict__ dst_pos, float *__restrict__ dst_sumsq,
-                                                                 float *__restrict__ dst_scale, int row_chunks, int n) {
+__global__ void __launch_bounds__(256, 2) kvd_checkpoint_fp4_kernel(const uint4 *rows, const int32_t *pos,
+                                                                 uint32_t *dst_codes, uint8_t *dst_block,
+                                                                 int32_t *dst_pos, float *dst_sumsq,
+                                                                 float *dst_scale, int row_chunks, int n) {
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   grid_launch_dependents();
@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(256, 2) kvd_checkpoint_fp4_kernel(const uint4 
 #pragma unroll
     for (int i = 0; i < CPL; ++i) {
       const int c = lane + 32 * i;
-      v[i] = c < row_chunks ? __ldg(rows + off + c) : make_uint4(0u, 0u, 0u, 0u);
+      v[i] = c < row_chunks ? rows[off + c] : make_uint4(0u, 0u, 0u, 0u);
     }
 #pragma unroll
     for (int i = 0; i < CPL; ++i) {
@@ -114,10 +114,10 @@ struct Fp4Ranges {
   int dst0[KVD_MAX_STORE_RANGES + 1];      // first scratch row of each range (ascending), then the total
   long long slot0[KVD_MAX_STORE_RANGES];   // first store slot of each range
 };
-__global__ void __launch_bounds__(256) kvd_expand_fp4_kernel(const uint32_t *__restrict__ codes, const uint8_t *__restrict__ block,
-                                                             const int32_t *__restrict__ spos, const float *__restrict__ ssumsq,
-                                                             const float *__restrict__ sscale, uint4 *__restrict__ out_rows,
-                                                             int32_t *__restrict__ out_pos, float *__restrict__ out_sumsq,
+__global__ void __launch_bounds__(256) kvd_expand_fp4_kernel(const uint32_t *codes, const uint8_t *block,
+                                                             const int32_t *spos, const float *ssumsq,
+                                                             const float *sscale, uint4 *out_rows,
+                                                             int32_t *out_pos, float *out_sumsq,
                                                              int row_chunks, const __grid_constant__ Fp4Ranges R) {
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
@@ -131,14 +131,14 @@ __global__ void __launch_bounds__(256) kvd_expand_fp4_kernel(const uint32_t *__r
       else hi = mid;
     }
     const size_t slot = static_cast<size_t>(R.slot0[lo]) + (i - R.dst0[lo]);
-    const float s_row = __ldg(sscale + slot);
+    const float s_row = sscale[slot];
     for (int c0 = lane; c0 < row_chunks; c0 += 32 * FP4_CPL) {
       uint32_t packed[FP4_CPL], scale[FP4_CPL];
 #pragma unroll
       for (int q = 0; q < FP4_CPL; ++q) {
         const int c = c0 + 32 * q < row_chunks ? c0 + 32 * q : row_chunks - 1;
-        packed[q] = __ldg(codes + slot * row_chunks + c);
-        scale[q] = __ldg(block + slot * (row_chunks / 2) + (c >> 1));
+        packed[q] = codes[slot * row_chunks + c];
+        scale[q] = block[slot * (row_chunks / 2) + (c >> 1)];
       }
 #pragma unroll
       for (int q = 0; q < FP4_CPL; ++q) {
@@ -153,8 +153,8 @@ __global__ void __launch_bounds__(256) kvd_expand_fp4_kernel(const uint32_t *__r
       }
     }
     if (lane == 0) {
-      out_pos[i] = __ldg(spos + slot);
-      out_sumsq[i] = __ldg(ssumsq + slot);
+      out_pos[i] = spos[slot];
+      out_sumsq[i] = ssumsq[slot];
     }
   }
 }

@@ -328,6 +328,12 @@ inline int serial_launch_mask() {
   return mask;
 }
 
+// A kernel launched as a programmatic dependent runs while its predecessor does.  What the predecessor may still write
+// (rows, positions, statistics, codes) it therefore reads by plain loads behind grid_dependency_wait(): no __ldg (the
+// non-coherent load is for memory that nobody writes during the kernel), and, in the kernels started by the function
+// below, no __restrict__ on an argument (it permits a load to move above the wait).  __ldg is for tables and weights,
+// which are complete before the first launch that reads them.
+//
 // Launch of a small kernel that calls grid_dependency_wait() before it touches memory: as a programmatic dependent of
 // its predecessor, so that its launch latency and the predecessor's end overlap (three decoder blocks at batch 1, 35
 // launches: 459 -> 421 us) -- if its grid leaves half of the SMs free.  Larger grids are ordered plainly: the next

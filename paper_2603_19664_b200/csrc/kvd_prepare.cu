@@ -62,10 +62,10 @@ __global__ void kvd_convert_gamma_kernel(const typename ElemBits<DT>::type *__re
 // takes the row's sum of squares (the RMSNorm statistic of Eq. 2), which the recompute kernel reads
 // back instead of taking it again for every recomputation.
 template <int DT>
-__global__ void __launch_bounds__(256) kvd_checkpoint_kernel(const uint4 *__restrict__ rows,
-                                                             const int32_t *__restrict__ pos,
-                                                             uint4 *__restrict__ dst_rows, int32_t *__restrict__ dst_pos,
-                                                             float *__restrict__ dst_sumsq, int row_chunks, int n,
+__global__ void __launch_bounds__(256) kvd_checkpoint_kernel(const uint4 *rows,
+                                                             const int32_t *pos,
+                                                             uint4 *dst_rows, int32_t *dst_pos,
+                                                             float *dst_sumsq, int row_chunks, int n,
                                                              int capacity, int *status) {
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
@@ -88,11 +88,11 @@ __global__ void __launch_bounds__(256) kvd_checkpoint_kernel(const uint4 *__rest
 // The same for one new row per sequence of a decode batch: row r goes to slot P.slot[r] of the store
 // (rows, positions and statistics are indexed by slot), so that a whole batch is appended in one launch.
 template <int DT>
-__global__ void __launch_bounds__(256) kvd_checkpoint_scatter_kernel(const uint4 *__restrict__ rows,
-                                                                     const int32_t *__restrict__ pos,
-                                                                     uint4 *__restrict__ store_rows,
-                                                                     int32_t *__restrict__ store_pos,
-                                                                     float *__restrict__ store_sumsq, int row_chunks, int n,
+__global__ void __launch_bounds__(256) kvd_checkpoint_scatter_kernel(const uint4 *rows,
+                                                                     const int32_t *pos,
+                                                                     uint4 *store_rows,
+                                                                     int32_t *store_pos,
+                                                                     float *store_sumsq, int row_chunks, int n,
                                                                      long long total_slots, int *status,
                                                                      const __grid_constant__ CkptSlots P) {
   const int lane = threadIdx.x & 31;
@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(256) kvd_checkpoint_scatter_kernel(const uint4
 // ahead of the main kernel when the caller hands it more rows than that kernel's statistics warps
 // can cover under the main loop.
 template <int DT>
-__global__ void __launch_bounds__(256) kvd_rowstats_kernel(const uint4 *__restrict__ rows, float *__restrict__ sumsq,
+__global__ void __launch_bounds__(256) kvd_rowstats_kernel(const uint4 *rows, float *sumsq,
                                                            int row_chunks, int n) {
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
@@ -149,12 +149,12 @@ __device__ __forceinline__ uint32_t e4m3x4(float a, float b, float c, float d) {
 // CPL > 0: rows of at most 32 * CPL chunks are held in registers (one pass over memory); CPL = 0: any
 // width, the row is read three times (it sits in L1 / L2 after the first).  The arithmetic is the same.
 template <int CPL>
-__global__ void __launch_bounds__(256) kvd_checkpoint_fp8_kernel(const uint4 *__restrict__ rows,
-                                                                 const int32_t *__restrict__ pos,
-                                                                 uint2 *__restrict__ dst_codes,
-                                                                 int32_t *__restrict__ dst_pos,
-                                                                 float *__restrict__ dst_sumsq,
-                                                                 float *__restrict__ dst_scale, int row_chunks, int n) {
+__global__ void __launch_bounds__(256) kvd_checkpoint_fp8_kernel(const uint4 *rows,
+                                                                 const int32_t *pos,
+                                                                 uint2 *dst_codes,
+                                                                 int32_t *dst_pos,
+                                                                 float *dst_sumsq,
+                                                                 float *dst_scale, int row_chunks, int n) {
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   grid_launch_dependents();
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(256) kvd_checkpoint_fp8_kernel(const uint4 *__
 #pragma unroll
       for (int i = 0; i < CPL; ++i) {
         const int c = lane + 32 * i;
-        v[i] = c < row_chunks ? __ldg(rows + off + c) : make_uint4(0u, 0u, 0u, 0u);
+        v[i] = c < row_chunks ? rows[off + c] : make_uint4(0u, 0u, 0u, 0u);
       }
       // the lane's chunks in ascending order, as warp_rows_sumsq takes them (absent chunks add exact zeros)
       uint64_t ps2[4] = {0ull, 0ull, 0ull, 0ull};
@@ -209,12 +209,12 @@ __global__ void __launch_bounds__(256) kvd_checkpoint_fp8_kernel(const uint4 *__
       float s1[1];
       warp_rows_sumsq<1, 10, false>(src, none, row_chunks, lane, s1);
       ss = s1[0];
-      for (int c = lane; c < row_chunks; c += 32) amax = chunk_amax(__ldg(rows + off + c), amax);
+      for (int c = lane; c < row_chunks; c += 32) amax = chunk_amax(rows[off + c], amax);
 #pragma unroll
       for (int k = 16; k >= 1; k >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, k));
       amax = fmaxf(amax, 1e-30f);
       const float scale = __fdiv_rn(amax, 448.0f), recip = __fdiv_rn(448.0f, amax);
-      for (int c = lane; c < row_chunks; c += 32) dst_codes[off + c] = chunk_codes(__ldg(rows + off + c), recip);
+      for (int c = lane; c < row_chunks; c += 32) dst_codes[off + c] = chunk_codes(rows[off + c], recip);
       if (lane == 0) dst_scale[r] = scale;
     }
     if (lane == 0) {

@@ -533,7 +533,7 @@ __device__ __forceinline__ void warp_rows_sumsq(const uint4 *const (&src)[R], ui
 #pragma unroll
     for (int r = 0; r < R; ++r)
 #pragma unroll
-      for (int j = 0; j < B; ++j) v[r][j] = __ldg(src[r] + c + 32 * j);
+      for (int j = 0; j < B; ++j) v[r][j] = src[r][c + 32 * j];
 #pragma unroll
     for (int r = 0; r < R; ++r)
 #pragma unroll
@@ -545,7 +545,7 @@ __device__ __forceinline__ void warp_rows_sumsq(const uint4 *const (&src)[R], ui
   for (; c < n_chunks; c += 32) {
     uint4 v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = __ldg(src[r] + c);
+    for (int r = 0; r < R; ++r) v[r] = src[r][c];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       if (COPY && dst[r] != nullptr) dst[r][c] = v[r];

@@ -496,10 +496,10 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
         if (J.sumsq != nullptr) {
           // checkpointed rows (or caller rows whose statistics a kernel of their own took): the sum of
           // squares is read back
-          const float sum = row < n_here ? __ldg(J.sumsq + m0 + row) : 0.f;
+          const float sum = row < n_here ? J.sumsq[m0 + row] : 0.f;
           rstd_row = 1.0f / sqrtf(sum * p.inv_d_hidden + p.rms_eps);
           // FP8 rows: the accumulator is a sum of code products; row scale and matrix scale go with 1/rms
-          if (EB == 1) rstd_row *= (row < n_here ? __ldg(J.scale + m0 + row) : 0.f) * __ldg(p.w_scale);
+          if (EB == 1) rstd_row *= (row < n_here ? J.scale[m0 + row] : 0.f) * __ldg(p.w_scale);
         } else {
           // a few caller rows: the four warps share them in groups of four rows (group g -> warp g % 4),
           // leave 1/rms in s_rstd[a] and meet on a barrier before every thread picks up its own row.

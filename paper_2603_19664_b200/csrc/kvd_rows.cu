@@ -224,7 +224,7 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
     const int w8 = warp - 2;
     if (p.sumsq != nullptr) {
       const int row = threadIdx.x - 64;
-      if (row < p.n_rows) s_rstd[row] = 1.0f / sqrtf(__ldg(p.sumsq + row) * p.inv_k + p.rms_eps);
+      if (row < p.n_rows) s_rstd[row] = 1.0f / sqrtf(p.sumsq[row] * p.inv_k + p.rms_eps);
     } else {
       // STORE_RESIDUAL in the same launch (kvd_decode_step_kv): the first CTA writes the rows it reads into the
       // store slots the host assigned to them

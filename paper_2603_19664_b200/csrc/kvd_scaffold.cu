@@ -26,16 +26,15 @@ static inline bool sc_aligned16(const void *p) { return (reinterpret_cast<uintpt
 namespace kvd {
 
 // ---------------------------------------------------------------------------------- elementwise kernels
-// One CTA per (row, query head), one thread per rotation pair.  (The rows and positions are not __restrict__: their
-// loads stay behind the dependency wait.)  The sum of squares over the head is
+// One CTA per (row, query head), one thread per rotation pair.  The sum of squares over the head is
 // reduced in a fixed order (shuffle tree inside a warp, warps added in index order).
 __global__ void __launch_bounds__(128) kvd_query_finish_kernel(const __nv_bfloat16 *q_in, long long in_stride,
                                                                const int32_t *positions,
-                                                               const __nv_bfloat16 *__restrict__ gamma_q, float eps,
-                                                               const float2 *__restrict__ rope_hi,
-                                                               const float2 *__restrict__ rope_lo, int max_pos,
+                                                               const __nv_bfloat16 *gamma_q, float eps,
+                                                               const float2 *rope_hi,
+                                                               const float2 *rope_lo, int max_pos,
                                                                int d_head, int n_q, int half_style,
-                                                               __nv_bfloat16 *__restrict__ q_out, int *status) {
+                                                               __nv_bfloat16 *q_out, int *status) {
   grid_launch_dependents();
   grid_dependency_wait();
   __shared__ float s_part[4];
@@ -70,7 +69,7 @@ __global__ void __launch_bounds__(128) kvd_query_finish_kernel(const __nv_bfloat
   dst[ib] = __float2bfloat16_rn(fmaf(a, s, b * c));
 }
 
-__global__ void __launch_bounds__(256) kvd_add_rows_kernel(uint4 *__restrict__ h, const uint4 *__restrict__ y,
+__global__ void __launch_bounds__(256) kvd_add_rows_kernel(uint4 *h, const uint4 *y,
                                                            long long y_stride_chunks, int m, int chunks) {
   grid_launch_dependents();
   grid_dependency_wait();
@@ -94,9 +93,9 @@ __device__ __forceinline__ float act_apply(float v, int activation) {
   return 0.5f * v * (1.0f + tanhf(0.7978845608028654f * (v + 0.044715f * v * v * v)));
 }
 
-__global__ void __launch_bounds__(256) kvd_gated_act_kernel(const uint4 *__restrict__ gate_up, long long stride_chunks,
+__global__ void __launch_bounds__(256) kvd_gated_act_kernel(const uint4 *gate_up, long long stride_chunks,
                                                             int m, int width_chunks, int activation,
-                                                            uint4 *__restrict__ out) {
+                                                            uint4 *out) {
   grid_launch_dependents();
   grid_dependency_wait();
   const long long total = static_cast<long long>(m) * width_chunks;
@@ -117,8 +116,8 @@ __global__ void __launch_bounds__(256) kvd_gated_act_kernel(const uint4 *__restr
   }
 }
 
-__global__ void __launch_bounds__(256) kvd_embed_kernel(const uint4 *__restrict__ table, const int32_t *__restrict__ tokens,
-                                                        int m, int chunks, int vocab, uint4 *__restrict__ out,
+__global__ void __launch_bounds__(256) kvd_embed_kernel(const uint4 *table, const int32_t *tokens,
+                                                        int m, int chunks, int vocab, uint4 *out,
                                                         int *status) {
   grid_launch_dependents();
   grid_dependency_wait();

@@ -51,3 +51,24 @@ def test_few_row_producer_waits_for_its_last_copies_on_every_path():
     assert "mbar_try_wait(bar_full(b), par)" in last and "tmo +" in last
     between = drain[drain.rindex("ph ^= 1u;"):drain.rindex("for (int b = 0")]
     assert "if (" not in between  # the wait hangs on no condition
+
+
+SMALL = sorted(set(re.findall(r"launch_dependent\((?:ctx, )?(kvd_\w+)", ALL)))
+
+
+def test_the_small_dependent_kernels_are_found():
+    assert len(SMALL) == 10 and all(k in KERNELS for k in SMALL), SMALL
+
+
+@pytest.mark.parametrize("name", SMALL)
+def test_inputs_of_a_small_dependent_kernel_are_plain_loads_behind_the_wait(name):
+    args, body = KERNELS[name]
+    assert "__restrict__" not in args and "__ldg" not in body
+    assert "grid_dependency_wait();" in body
+
+
+def test_row_statistics_are_plain_loads():
+    text = TEXT["kvd_ptx.cuh"]
+    assert "__ldg" not in text[text.index("void warp_rows_sumsq("):]
+    for f in ("kvd_recompute.cu", "kvd_rows.cu"):
+        assert not re.search(r"__ldg\([^)]*(sumsq|J\.scale|positions)", TEXT[f]), f
