@@ -35,8 +35,8 @@
  *   - Kernels after the first of a call sequence are launched as programmatic dependents of their
  *     predecessor in the stream (their set-up overlaps its tail; they wait for its completion before
  *     touching its results), which is transparent to callers and to stream capture.  Environment:
- *     KVD_SERIAL_LAUNCH (bit mask: 1 recompute, 2 attention streaming, 4 attention merge) restores
- *     plain stream ordering for those kernels; KVD_SPIN_LIMIT_MS (read by kvd_create) bounds every
+ *     KVD_SERIAL_LAUNCH (bit mask: 1 recompute and few-row projection, 2 attention streaming, 4 attention
+ *     merge, 8 all others) restores plain stream ordering for those kernels; KVD_SPIN_LIMIT_MS (read by kvd_create) bounds every
  *     in-kernel pipeline wait (default 2000 ms).
  */
 #ifndef KVD_H_

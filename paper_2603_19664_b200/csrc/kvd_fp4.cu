@@ -235,7 +235,7 @@ extern "C" kvd_status kvd_checkpoint_residual_fp4(kvd_ctx *ctx, int seq, int lay
   const uint4 *src = static_cast<const uint4 *>(rows);
   cudaError_t e;
   if (row_chunks <= 320)
-    e = launch_dependent(kvd_checkpoint_fp4_kernel<10>, dim3(static_cast<unsigned>(blocks)), 256, stream,
+    e = launch_dependent(ctx, kvd_checkpoint_fp4_kernel<10>, dim3(static_cast<unsigned>(blocks)), 256, stream,
         src, positions, dc, db, ctx->store4_pos + slot, ctx->store4_sumsq + slot, ctx->store4_scale + slot, row_chunks, n);
   else
     return KVD_ERR_SHAPE;  // rows wider than 2560 channels are not held in registers
@@ -303,7 +303,7 @@ extern "C" kvd_status kvd_recompute_kv_fp4(kvd_ctx *ctx, int layer, const kvd_st
   long long blocks = (static_cast<long long>(total) + 7) / 8;
   const long long cap = static_cast<long long>(ctx->num_sms) * 8;
   if (blocks > cap) blocks = cap;
-  cudaError_t e = launch_dependent(kvd_expand_fp4_kernel, dim3(static_cast<unsigned>(blocks)), 256, stream,
+  cudaError_t e = launch_dependent(ctx, kvd_expand_fp4_kernel, dim3(static_cast<unsigned>(blocks)), 256, stream,
       reinterpret_cast<const uint32_t *>(ctx->store4_codes), ctx->store4_block, ctx->store4_pos, ctx->store4_sumsq,
       ctx->store4_scale, reinterpret_cast<uint4 *>(x), xp, xs, row_chunks, R);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "launch expand_fp4");

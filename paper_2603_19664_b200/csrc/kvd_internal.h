@@ -318,7 +318,7 @@ struct kvd_ctx {
 
 namespace kvd {
 // Kernels are launched as programmatic dependents of their predecessor in the stream unless the
-// environment variable KVD_SERIAL_LAUNCH says otherwise: a bit mask, 1 = recompute kernel, 2 = attention
+// environment variable KVD_SERIAL_LAUNCH says otherwise: a bit mask, 1 = recompute and few-row kernels, 2 = attention
 // streaming kernel, 4 = attention merge kernel, 8 = all others get plain stream ordering instead.
 inline int serial_launch_mask() {
   static const int mask = [] {
@@ -332,7 +332,9 @@ inline int serial_launch_mask() {
 // (rows, positions, statistics, codes) it therefore reads by plain loads behind grid_dependency_wait(): no __ldg (the
 // non-coherent load is for memory that nobody writes during the kernel), and, in the kernels started by the function
 // below, no __restrict__ on an argument (it permits a load to move above the wait).  __ldg is for tables and weights,
-// which are complete before the first launch that reads them.
+// which are complete before the first launch that reads them.  (Of older kernels, decode attention still streams K and V,
+// and the fused recompute kernel its queries, by non-coherent loads behind the wait: plain ones measured 80.1 -> 81.0 us
+// for a decode step of 4 x 2048 tokens, 55.0 -> 55.4 for one of 4096.)
 //
 // Launch of a small kernel that calls grid_dependency_wait() before it touches memory: as a programmatic dependent of
 // its predecessor, so that its launch latency and the predecessor's end overlap (three decoder blocks at batch 1, 35
@@ -340,7 +342,7 @@ inline int serial_launch_mask() {
 // kernel's CTAs then wait on SMs this one still needs (decoding 3000 FP4 rows ahead of their projection: 56 -> 66 us
 // for the step with an early start).
 template <typename... P, typename... A>
-inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, unsigned threads, cudaStream_t stream, A &&...args) {
+inline cudaError_t launch_dependent(const kvd_ctx *ctx, void (*kern)(P...), dim3 grid, unsigned threads, cudaStream_t stream, A &&...args) {
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = grid;
@@ -348,13 +350,12 @@ inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, unsigned thre
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = (serial_launch_mask() & 8) || grid.x > 74 ? 0 : 1;
+  attr[0].val.programmaticStreamSerializationAllowed = (serial_launch_mask() & 8) || 2 * grid.x > static_cast<unsigned>(ctx->num_sms) ? 0 : 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
-// launchers implemented next to their kernels
 // Schedule of a launch: its tiles (units of two, single ones, cut ones) and its CTA pairs.  The one place both the launch
 // and the size test of the trace buffer take the grid from.
 struct RcSchedule {
@@ -374,6 +375,7 @@ inline void schedule_recompute(const kvd_ctx *ctx, RecomputeParams &p, int eb, b
   // (fp16 and fp32 kernels record nothing, and the hook must not choose the kernel of a call it cannot trace)
   p.trace = ctx->trace && ctx->dtype == KVD_DTYPE_BF16 && rc_trace_bytes(s.clusters) <= ctx->trace_bytes ? ctx->trace : nullptr;
 }
+// launchers implemented next to their kernels
 kvd_status launch_recompute(kvd_ctx *ctx, const LayerState &ls, const CUtensorMap &tmap_store,
                             const CUtensorMap &tmap_rows, const RecomputeParams &p, cudaStream_t stream);
 kvd_status launch_recompute_fused(kvd_ctx *ctx, const LayerState &ls, const CUtensorMap &tmap_store,

@@ -347,13 +347,13 @@ kvd_status launch_checkpoint(kvd_ctx *ctx, const __nv_bfloat16 *rows, const int3
   if (blocks < 1) blocks = 1;
   cudaError_t e;
   if (ctx->dtype == 2)
-    e = launch_dependent(kvd_checkpoint_kernel<2>, dim3(static_cast<unsigned>(blocks)), 256, stream,
+    e = launch_dependent(ctx, kvd_checkpoint_kernel<2>, dim3(static_cast<unsigned>(blocks)), 256, stream,
         reinterpret_cast<const uint4 *>(rows), pos, reinterpret_cast<uint4 *>(dst_rows), dst_pos, dst_sumsq, d_hidden / 4, n, capacity, ctx->d_status);
   else if (ctx->dtype == 1)
-    e = launch_dependent(kvd_checkpoint_kernel<1>, dim3(static_cast<unsigned>(blocks)), 256, stream,
+    e = launch_dependent(ctx, kvd_checkpoint_kernel<1>, dim3(static_cast<unsigned>(blocks)), 256, stream,
         reinterpret_cast<const uint4 *>(rows), pos, reinterpret_cast<uint4 *>(dst_rows), dst_pos, dst_sumsq, d_hidden / 8, n, capacity, ctx->d_status);
   else
-    e = launch_dependent(kvd_checkpoint_kernel<0>, dim3(static_cast<unsigned>(blocks)), 256, stream,
+    e = launch_dependent(ctx, kvd_checkpoint_kernel<0>, dim3(static_cast<unsigned>(blocks)), 256, stream,
         reinterpret_cast<const uint4 *>(rows), pos, reinterpret_cast<uint4 *>(dst_rows), dst_pos, dst_sumsq, d_hidden / 8, n, capacity, ctx->d_status);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "launch checkpoint");
   ctx->launches += 1;
@@ -368,11 +368,11 @@ kvd_status launch_checkpoint_scatter(kvd_ctx *ctx, const __nv_bfloat16 *rows, co
   const long long total = static_cast<long long>(ctx->layers_stored) * ctx->desc.max_seqs * ctx->desc.max_tokens_per_seq;
   cudaError_t e;
   if (ctx->dtype == 2)
-    e = launch_dependent(kvd_checkpoint_scatter_kernel<2>, dim3(blocks), 256, stream, src, pos, dst, ctx->store_pos, ctx->store_sumsq, d_hidden / 4, n, total, ctx->d_status, slots);
+    e = launch_dependent(ctx, kvd_checkpoint_scatter_kernel<2>, dim3(blocks), 256, stream, src, pos, dst, ctx->store_pos, ctx->store_sumsq, d_hidden / 4, n, total, ctx->d_status, slots);
   else if (ctx->dtype == 1)
-    e = launch_dependent(kvd_checkpoint_scatter_kernel<1>, dim3(blocks), 256, stream, src, pos, dst, ctx->store_pos, ctx->store_sumsq, d_hidden / 8, n, total, ctx->d_status, slots);
+    e = launch_dependent(ctx, kvd_checkpoint_scatter_kernel<1>, dim3(blocks), 256, stream, src, pos, dst, ctx->store_pos, ctx->store_sumsq, d_hidden / 8, n, total, ctx->d_status, slots);
   else
-    e = launch_dependent(kvd_checkpoint_scatter_kernel<0>, dim3(blocks), 256, stream, src, pos, dst, ctx->store_pos, ctx->store_sumsq, d_hidden / 8, n, total, ctx->d_status, slots);
+    e = launch_dependent(ctx, kvd_checkpoint_scatter_kernel<0>, dim3(blocks), 256, stream, src, pos, dst, ctx->store_pos, ctx->store_sumsq, d_hidden / 8, n, total, ctx->d_status, slots);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "launch checkpoint (batch)");
   ctx->launches += 1;
   return KVD_OK;
@@ -386,13 +386,13 @@ kvd_status launch_rowstats(kvd_ctx *ctx, const __nv_bfloat16 *rows, float *sumsq
   if (blocks < 1) blocks = 1;
   cudaError_t e;
   if (ctx->dtype == 2)
-    e = launch_dependent(kvd_rowstats_kernel<2>, dim3(static_cast<unsigned>(blocks)), 256, stream, reinterpret_cast<const uint4 *>(rows), sumsq,
+    e = launch_dependent(ctx, kvd_rowstats_kernel<2>, dim3(static_cast<unsigned>(blocks)), 256, stream, reinterpret_cast<const uint4 *>(rows), sumsq,
                                                                               d_hidden / 4, n);
   else if (ctx->dtype == 1)
-    e = launch_dependent(kvd_rowstats_kernel<1>, dim3(static_cast<unsigned>(blocks)), 256, stream, reinterpret_cast<const uint4 *>(rows), sumsq,
+    e = launch_dependent(ctx, kvd_rowstats_kernel<1>, dim3(static_cast<unsigned>(blocks)), 256, stream, reinterpret_cast<const uint4 *>(rows), sumsq,
                                                                               d_hidden / 8, n);
   else
-    e = launch_dependent(kvd_rowstats_kernel<0>, dim3(static_cast<unsigned>(blocks)), 256, stream, reinterpret_cast<const uint4 *>(rows), sumsq,
+    e = launch_dependent(ctx, kvd_rowstats_kernel<0>, dim3(static_cast<unsigned>(blocks)), 256, stream, reinterpret_cast<const uint4 *>(rows), sumsq,
                                                                               d_hidden / 8, n);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "launch rowstats");
   ctx->launches += 1;
@@ -409,11 +409,11 @@ kvd_status launch_checkpoint_fp8(kvd_ctx *ctx, const __nv_bfloat16 *rows, const 
   const int row_chunks = d_hidden / 8;
   cudaError_t e;
   if (row_chunks <= 320)
-    e = launch_dependent(kvd_checkpoint_fp8_kernel<10>, dim3(static_cast<unsigned>(blocks)), 256, stream,
+    e = launch_dependent(ctx, kvd_checkpoint_fp8_kernel<10>, dim3(static_cast<unsigned>(blocks)), 256, stream,
         reinterpret_cast<const uint4 *>(rows), pos, reinterpret_cast<uint2 *>(dst_codes), dst_pos, dst_sumsq, dst_scale,
         row_chunks, n);
   else
-    e = launch_dependent(kvd_checkpoint_fp8_kernel<0>, dim3(static_cast<unsigned>(blocks)), 256, stream,
+    e = launch_dependent(ctx, kvd_checkpoint_fp8_kernel<0>, dim3(static_cast<unsigned>(blocks)), 256, stream,
         reinterpret_cast<const uint4 *>(rows), pos, reinterpret_cast<uint2 *>(dst_codes), dst_pos, dst_sumsq, dst_scale,
         row_chunks, n);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "launch checkpoint_fp8");

@@ -350,7 +350,7 @@ extern "C" kvd_status kvd_scaffold_query_finish(kvd_ctx *ctx, int layer, const v
   const kvd_model_desc &d = ctx->desc;
   if (!q_in || !positions || !q_out || in_row_stride < static_cast<int64_t>(d.n_q_heads) * d.d_head) return KVD_ERR_INVALID_ARG;
   const int max_pos = ls.rope.n_hi * ROPE_LO_SIZE < d.max_tokens_per_seq ? ls.rope.n_hi * ROPE_LO_SIZE : d.max_tokens_per_seq;
-  cudaError_t e = launch_dependent(kvd_query_finish_kernel, dim3(static_cast<unsigned>(m) * d.n_q_heads), d.d_head / 2, static_cast<cudaStream_t>(stream_),
+  cudaError_t e = launch_dependent(ctx, kvd_query_finish_kernel, dim3(static_cast<unsigned>(m) * d.n_q_heads), d.d_head / 2, static_cast<cudaStream_t>(stream_),
       static_cast<const __nv_bfloat16 *>(q_in), in_row_stride, positions, static_cast<const __nv_bfloat16 *>(gamma_q),
       d.qk_norm_eps, ls.rope.hi, ls.rope.lo, max_pos, d.d_head, d.n_q_heads, d.rope_style == KVD_ROPE_HALF ? 1 : 0,
       static_cast<__nv_bfloat16 *>(q_out), ctx->d_status);
@@ -364,7 +364,7 @@ extern "C" kvd_status kvd_scaffold_add_rows(kvd_ctx *ctx, void *h, const void *y
   if (!h || !y || y_row_stride < d) return KVD_ERR_INVALID_ARG;
   if (d % 8 != 0 || y_row_stride % 8 != 0 || !sc_aligned16(h) || !sc_aligned16(y)) return KVD_ERR_ALIGNMENT;
   const int chunks = d / 8;
-  cudaError_t e = launch_dependent(kvd_add_rows_kernel, dim3(grid_for(static_cast<long long>(m) * chunks, 256, ctx->num_sms)), 256, static_cast<cudaStream_t>(stream_),
+  cudaError_t e = launch_dependent(ctx, kvd_add_rows_kernel, dim3(grid_for(static_cast<long long>(m) * chunks, 256, ctx->num_sms)), 256, static_cast<cudaStream_t>(stream_),
       static_cast<uint4 *>(h), static_cast<const uint4 *>(y), y_row_stride / 8, m, chunks);
   return sc_launched(ctx, e, "launch add_rows");
 }
@@ -377,7 +377,7 @@ extern "C" kvd_status kvd_scaffold_gated_act(kvd_ctx *ctx, const void *gate_up, 
   if (!gate_up || !out || row_stride < 2 * static_cast<int64_t>(width)) return KVD_ERR_INVALID_ARG;
   if (width % 8 != 0 || row_stride % 8 != 0 || !sc_aligned16(gate_up) || !sc_aligned16(out)) return KVD_ERR_ALIGNMENT;
   const int wc = width / 8;
-  cudaError_t e = launch_dependent(kvd_gated_act_kernel, dim3(grid_for(static_cast<long long>(m) * wc, 256, ctx->num_sms)), 256, static_cast<cudaStream_t>(stream_),
+  cudaError_t e = launch_dependent(ctx, kvd_gated_act_kernel, dim3(grid_for(static_cast<long long>(m) * wc, 256, ctx->num_sms)), 256, static_cast<cudaStream_t>(stream_),
       static_cast<const uint4 *>(gate_up), row_stride / 8, m, wc, activation, static_cast<uint4 *>(out));
   return sc_launched(ctx, e, "launch gated_act");
 }
@@ -389,7 +389,7 @@ extern "C" kvd_status kvd_scaffold_embed(kvd_ctx *ctx, const void *table, const 
   if (!table || !tokens || !out) return KVD_ERR_INVALID_ARG;
   if (d % 8 != 0 || !sc_aligned16(table) || !sc_aligned16(out)) return KVD_ERR_ALIGNMENT;
   const int chunks = d / 8;
-  cudaError_t e = launch_dependent(kvd_embed_kernel, dim3(grid_for(static_cast<long long>(m) * chunks, 256, ctx->num_sms)), 256, static_cast<cudaStream_t>(stream_),
+  cudaError_t e = launch_dependent(ctx, kvd_embed_kernel, dim3(grid_for(static_cast<long long>(m) * chunks, 256, ctx->num_sms)), 256, static_cast<cudaStream_t>(stream_),
       static_cast<const uint4 *>(table), tokens, m, chunks, vocab, static_cast<uint4 *>(out), ctx->d_status);
   return sc_launched(ctx, e, "launch embed");
 }

@@ -72,3 +72,11 @@ def test_row_statistics_are_plain_loads():
     assert "__ldg" not in text[text.index("void warp_rows_sumsq("):]
     for f in ("kvd_recompute.cu", "kvd_rows.cu"):
         assert not re.search(r"__ldg\([^)]*(sumsq|J\.scale|positions)", TEXT[f]), f
+
+
+def test_the_early_start_threshold_follows_the_device():
+    """Which grids leave half of the SMs free is a question to the device, not a literal."""
+    text = TEXT["kvd_internal.h"]
+    fn = text[text.index("inline cudaError_t launch_dependent("):]
+    fn = fn[:fn.index("\n}")]
+    assert "ctx->num_sms" in fn and not re.search(r"grid\.x\s*[<>]=?\s*\d", fn)
