@@ -726,7 +726,7 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
   constexpr int SLOTS = Cfg::SLOTS, SLOTS_K = Cfg::SLOTS_K, SLOTS_V = Cfg::SLOTS_V;
   extern __shared__ uint8_t pt_smem_raw[];
   __shared__ uint32_t s_tmem;
-  __shared__ int s_abort_i, s_lo, s_hi;
+  __shared__ int s_abort_i, s_lo[2], s_hi[2];  // first and last key position a tile needs
   volatile int *s_abort = &s_abort_i;
   const uint32_t q_smem = (smem_u32(pt_smem_raw) + 1023u) & ~1023u;  // the swizzle is a function of the address
   const uint32_t ring = q_smem + 2 * Cfg::Q_BYTES, ring_v = ring + SLOTS_K * Cfg::TILE_BYTES;
@@ -761,31 +761,38 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
     }
     fence_mbar_init();
     s_abort_i = 0;
-    s_lo = INT_MAX;
-    s_hi = -1;
+    for (int t = 0; t < 2; ++t) {
+      s_lo[t] = INT_MAX;
+      s_hi[t] = -1;
+    }
   }
   if (warp == 8) {
     tmem_alloc(smem_u32(&s_tmem), Cfg::COLS);
     tmem_relinquish();
   }
   __syncthreads();
-  // ---- key positions the CTA needs: from the smallest first-visible to the largest last-visible of its tokens
+  // ---- key positions a tile needs: from the smallest first-visible to the largest last-visible of its tokens
   if (tid < 2 * TOK && cta_tok0 + tid < P.n_rows) {
     const int qp = P.q_pos[cta_tok0 + tid];
     int lo = P.window > 0 ? qp - P.window + 1 : 0;
     lo = lo < P.seg_lo ? P.seg_lo : lo;
     const int hi = qp < P.seg_hi ? qp : P.seg_hi;
     if (hi >= lo) {
-      atomicMin(&s_lo, lo);
-      atomicMax(&s_hi, hi);
+      atomicMin(&s_lo[tid / TOK], lo);
+      atomicMax(&s_hi[tid / TOK], hi);
     }
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = s_tmem;
-  const int blk0 = s_hi >= 0 ? s_lo / PT_KEYS : 0;
-  const int n_blk = s_hi >= 0 ? s_hi / PT_KEYS - blk0 + 1 : 0;
+  // The blocks the CTA loads, and the ones of these that tile t takes: its own range and no more.  In a block only the
+  // other tile sees, an infinity or a NaN in V would reach this tile's rows as a weight of 0 times it.
+  const int hi_all = s_hi[0] > s_hi[1] ? s_hi[0] : s_hi[1], lo_all = s_lo[0] < s_lo[1] ? s_lo[0] : s_lo[1];
+  const int blk0 = hi_all >= 0 ? lo_all / PT_KEYS : 0;
+  const int n_blk = hi_all >= 0 ? hi_all / PT_KEYS - blk0 + 1 : 0;
+  auto tile_skip = [&](int t) { return s_hi[t] >= 0 ? s_lo[t] / PT_KEYS - blk0 : 0; };                        // blocks before its first
+  auto tile_blocks = [&](int t) { return s_hi[t] >= 0 ? s_hi[t] / PT_KEYS - s_lo[t] / PT_KEYS + 1 : 0; };
 
   if (warp < 8) {
     // ------------------------------------------------------------------ softmax and epilogue: thread = MMA row of tile t
@@ -795,10 +802,11 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
     const bool valid = row / G < TOK && tok < P.n_rows;
     const int qp = valid ? P.q_pos[tok] : -1;
     const int lo = P.window > 0 ? qp - P.window + 1 : 0;
+    const int first_blk = blk0 + tile_skip(t), n = tile_blocks(t);
     const uint32_t lane_field = static_cast<uint32_t>(q4 * 32) << 16;
     const uint32_t o_col = tmem_base + lane_field + t * D_HEAD;
     const size_t row_off = (static_cast<size_t>(valid ? tok : 0) * P.n_q + kvh * G + (valid ? g : 0)) * D_HEAD;
-    if (n_blk > 0) {
+    if (n > 0) {
       // the query row into shared memory, K-major with the 128-byte swizzle (zeros for padding rows)
       const uint4 *qsrc = reinterpret_cast<const uint4 *>(P.q + row_off);
       const uint32_t qdst = q_smem + t * Cfg::Q_BYTES + row * 128;
@@ -819,7 +827,7 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
     bool ok = true;
     const uint64_t c2 = pack2(P.scale_log2e, P.scale_log2e);
     PtWhole whole_block(valid, lo, qp);
-    for (int j = 0; j < n_blk; ++j) {
+    for (int j = 0; j < n; ++j) {
       const int buf = j & 1;
       if (!polite_warp_wait(bar_s_full(t, buf), (j >> 1) & 1, s_abort, tmo, lane)) {
         raise(P.status, STATUS_TIMEOUT, s_abort);
@@ -831,9 +839,9 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
       uint32_t s0[32], s1[32];
       tmem_ld_x32(s_col, s0);
       tmem_ld_x32(s_col + 32, s1);
-      const bool whole = whole_block(P, (blk0 + j) * PT_KEYS);  // (warp-uniform)
+      const bool whole = whole_block(P, (first_blk + j) * PT_KEYS);  // (warp-uniform)
       unsigned long long vis = ~0ull;
-      if (!whole) vis = pt_visible(P, (blk0 + j) * PT_KEYS, lo, qp);
+      if (!whole) vis = pt_visible(P, (first_blk + j) * PT_KEYS, lo, qp);
       tmem_wait_ld();
       const float bm = pt_mask_max(s0, s1, whole, vis) * P.scale_log2e;  // log2 units (scale > 0)
       // the lazy reference of the kernel above
@@ -877,7 +885,7 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
     }
     // ---- the row sum: both parts referred to the final maximum (a sum of two: the order does not matter)
     float l_run = 0.f;
-    if (ok && n_blk > 0) {
+    if (ok && n > 0) {
       const float m_use = m_run == -CUDART_INF_F ? 0.f : m_run;
       l_run = pt_row_sum(l2, m_own == -CUDART_INF_F ? 1.0f : ex2_approx(m_own - m_use)) +
               pt_row_sum(l2_other, m_other == -CUDART_INF_F ? 1.0f : ex2_approx(m_other - m_use));
@@ -894,7 +902,7 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
 #pragma unroll 1
       for (int c = 0; c < D_HEAD / 32; ++c) {
         uint32_t r[32];
-        if (n_blk > 0) {
+        if (n > 0) {
           tmem_ld_x32(o_col + c * 32, r);
           tmem_wait_ld();
         } else {
@@ -917,10 +925,23 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
     constexpr uint32_t IDESC_O = IDESC_BASE | (static_cast<uint32_t>(D_HEAD >> 3) << 17) | (1u << 16);  // N = d_head, B MN-major
     const int t = warp - 8;
     if (n_blk > 0 && elect_one()) {
-      bool ok = polite_wait<false>(bar_q_ready(t), 0, s_abort, tmo);
+      const int skip = tile_skip(t), n = tile_blocks(t);
+      // blocks that only the other tile takes: released when they have landed (not earlier: the next phase of the
+      // slot's barrier must not get this tile's arrival before the other tile's of this phase)
+      auto pass = [&](int from, int to) -> bool {
+        for (int b = from; b < to; ++b)
+          for (int v = 0; v < 2; ++v) {
+            const int slots = v ? SLOTS_V : SLOTS_K, slot = b % slots;
+            if (!polite_wait<false>(bar_full(v, slot), (b / slots) & 1, s_abort, tmo)) return false;
+            mbar_arrive(bar_empty(v, slot));
+          }
+        return true;
+      };
+      bool ok = pass(0, skip);
+      if (ok && n > 0) ok = polite_wait<false>(bar_q_ready(t), 0, s_abort, tmo);
       auto scores = [&](int j) -> bool {
-        const int slot = j % SLOTS_K;
-        if (!polite_wait<false>(bar_full(0, slot), (j / SLOTS_K) & 1, s_abort, tmo)) return false;
+        const int slot = (skip + j) % SLOTS_K;
+        if (!polite_wait<false>(bar_full(0, slot), ((skip + j) / SLOTS_K) & 1, s_abort, tmo)) return false;
         tc_fence_after();
         const uint32_t d = tmem_base + Cfg::COL_S + (2 * t + (j & 1)) * PT_KEYS;
         const uint64_t qdesc0 = umma_smem_desc_sw128(q_smem + t * Cfg::Q_BYTES), kdesc0 = umma_smem_desc_sw128(ring + slot * Cfg::TILE_BYTES);
@@ -932,13 +953,13 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
         umma_commit(bar_s_full(t, j & 1));
         return true;
       };
-      ok = ok && scores(0);
-      if (ok && n_blk > 1) ok = scores(1);
-      for (int j = 0; ok && j < n_blk; ++j) {
-        const int slot = j % SLOTS_V;
+      if (ok && n > 0) ok = scores(0);
+      if (ok && n > 1) ok = scores(1);
+      for (int j = 0; ok && j < n; ++j) {
+        const int slot = (skip + j) % SLOTS_V;
         // the weights are in place (and O has been rescaled where a reference maximum moved), the V block has landed
         if (!polite_wait<false>(bar_p_ready(t, j & 1), (j >> 1) & 1, s_abort, tmo) ||
-            !polite_wait<false>(bar_full(1, slot), (j / SLOTS_V) & 1, s_abort, tmo)) {
+            !polite_wait<false>(bar_full(1, slot), ((skip + j) / SLOTS_V) & 1, s_abort, tmo)) {
           ok = false;
           break;
         }
@@ -951,10 +972,11 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
         umma_commit(bar_empty(1, slot));
         umma_commit(bar_pv_done(t));
         // (the next scores of this buffer are not urgent: they wait for the product that reads the weights in it)
-        if (j + 2 < n_blk) ok = polite_wait<false>(bar_pv_done(t), j & 1, s_abort, tmo) && scores(j + 2);
+        if (j + 2 < n) ok = polite_wait<false>(bar_pv_done(t), j & 1, s_abort, tmo) && scores(j + 2);
       }
       if (ok) umma_commit(bar_o_full(t));
-      else raise(P.status, STATUS_TIMEOUT, s_abort);
+      if (ok) ok = pass(skip + n, n_blk);
+      if (!ok) raise(P.status, STATUS_TIMEOUT, s_abort);
     }
   } else {
     auto arrive = [&](uint32_t bar) { mbar_arrive(bar); };

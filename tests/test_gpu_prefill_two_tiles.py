@@ -53,3 +53,38 @@ def test_rows_of_a_long_call_equal_those_of_short_calls(shape, T, step, dtype):
     assert torch.equal(mixed, out[order])
     assert ctx.kvd_poll_status() == kvd.KVD_OK
     ctx.close()
+
+
+@pytest.mark.parametrize("window", [0, 90])
+@pytest.mark.parametrize("group", [1, 2, 3, 4, 8])
+def test_a_tile_takes_no_block_that_only_its_neighbour_sees(group, window):
+    """A weight of 0 times an infinity in V is a NaN, so an infinity reaches the rows of a 128-row tile through every block
+    the tile walks -- and through no other block: as in a call of that tile alone.  A tile without a visible key is zero."""
+    n_kv, d_head, first = 8, 128, 5
+    shape = LayerShape("inf", 128, group * n_kv, n_kv, d_head, 1e-6, False, 1.0e4, window)
+    tok, kdim = 128 // group, n_kv * d_head
+    T = tok * (148 // n_kv + 4) + tok // 2  # more than one tile per SM, the last one short
+    desc = kvd.make_desc(1, shape.d_hidden, shape.n_q_heads, n_kv, d_head, 1e-6, False, 1e-6, shape.rope_style, 1, T + 512, 1)
+    ctx = kvd.Kvd(desc)
+    w = make_layer_weights(shape)
+    bf16 = [torch.from_numpy(b.astype(np.uint32) << np.uint32(16)).view(torch.float32).bfloat16().cuda() for b in (w.w_kv, w.gamma_in)]
+    ctx.kvd_set_layer(0, bf16[0], bf16[1], None, shape.rope_theta, window)
+    ctx.kvd_attach_workspace(torch.empty(kvd.kvd_workspace_bytes(desc), dtype=torch.uint8, device="cuda"))
+    g = torch.Generator(device="cuda").manual_seed(5)
+    k, v = (torch.randn((T + 200, kdim), generator=g, device="cuda").bfloat16() for _ in range(2))
+    for p in (70, T // 2, T // 2 + 63, T):
+        v[p] = float("inf")
+    q = torch.randn((T, shape.n_q_heads, d_head), generator=g, device="cuda").bfloat16()
+    pos = torch.arange(T, dtype=torch.int32, device="cuda") + 26  # tiles end inside key blocks
+    pos[: 2 * tok] = torch.arange(2 * tok, dtype=torch.int32, device="cuda").flip(0) * 2 + first  # two tiles far apart
+    pos[4 * tok: 5 * tok] = first - 3  # sees nothing, beside a tile that does
+    segs = [(k, v, kdim, first, T + 200)]
+    out, alone = torch.full_like(q, 9.0), torch.full_like(q, 9.0)
+    ctx.kvd_prefill_attention(0, T, q, pos, segs, 0.0, out)
+    for r0 in range(0, T, tok):
+        ctx.kvd_prefill_attention(0, min(tok, T - r0), q[r0:], pos[r0:], segs, 0.0, alone[r0:])
+    assert ctx.kvd_poll_status() == kvd.KVD_OK
+    nan = torch.isnan(alone)
+    assert torch.equal(torch.isnan(out), nan) and torch.equal(out[~nan], alone[~nan])
+    assert bool(nan.any()) and not bool(nan.all()) and bool((out[4 * tok: 5 * tok] == 0).all())
+    ctx.close()
