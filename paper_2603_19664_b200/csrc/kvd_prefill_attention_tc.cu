@@ -1046,14 +1046,44 @@ static kvd_status prefill_tc_launch(kvd_ctx *ctx, const PrefillParams &P, cudaSt
   return KVD_OK;
 }
 
-// Two tiles per CTA once single tiles would be more than one per SM (Qwen3-4B layer, one tile / two tiles per CTA: 56 single
-// tiles 104 / 150 us, 176 113 / 95, 280 170 / 136, 1024 208 / 161).  At d_head 64 the products are too short for it:
-// 294 tiles of a SmolLM2 layer 58 / 72 us.
+// Time a launch of CTAs of `tok` tokens would take: a CTA costs `per_cta` + `per_block` for every key block it walks, the
+// CTAs start longest first, so an SM gets one of the first round, one of the reversed second round, and so on.  The
+// positions are on the device; the host assumes the usual call, whose last row sits at the last key.
+static float prefill_estimate(const kvd_ctx *ctx, const PrefillParams &P, int tok, float per_cta, float per_block) {
+  const int tiles = (P.n_rows + tok - 1) / tok, total = tiles * P.n_kv, sms = ctx->num_sms;
+  auto cost = [&](int i) {
+    const int t0 = (tiles - 1 - i / P.n_kv) * tok, t1 = (t0 + tok < P.n_rows ? t0 + tok : P.n_rows) - 1;
+    const int last = P.seg_hi - (P.n_rows - 1 - t1);
+    int first = P.window > 0 ? P.seg_hi - (P.n_rows - 1 - t0) - P.window + 1 : P.seg_lo;
+    first = first < P.seg_lo ? P.seg_lo : first;
+    return per_cta + per_block * static_cast<float>(last >= first ? last / PT_KEYS - first / PT_KEYS + 1 : 0);
+  };
+  float longest = 0.f;
+  for (int m = 0; m < sms && m < total; ++m) {
+    float sum = 0.f;
+    for (int r = 0; r * sms < total; ++r) {
+      const int i = r * sms + (r % 2 == 0 ? m : sms - 1 - m);
+      if (i < total) sum += cost(i);
+    }
+    longest = sum > longest ? sum : longest;
+  }
+  return longest;
+}
+
+// Two tiles per CTA (d_head 128) or one.  Two serve more rows per clock but walk a block more slowly, so a call whose
+// longest tiles set its time wants one, and one that keeps every SM busy for several rounds wants two.  Up to one round
+// of single tiles: one.  Beyond four rounds: two.  Between: by estimate; the costs (us) are fitted to 102 launches of 1 to
+// 27 rounds with groups of 1 to 8, windows of 0, 128 and 1024 and 0 to 7000 earlier keys (5 % rms).  One / two tiles per
+// CTA, us: 32 query on 8 KV heads, 600 tokens 14.9 / 21.9, 600 on 7000 176 / 140, 1300 36.1 / 34.0, 2500 93 / 81, 4096
+// 206 / 162; 16 on 8, 1300 23.3 / 32.4, 2500 52.0 / 53.5, 4096 104 / 81; 4 on 1, 8000 99 / 145.  Two tiles whenever there is
+// more than one round, as it was before, cost up to 1.5 times the time.  At d_head 64 the products are too short for two
+// tiles: 294 tiles of a SmolLM2 layer 58 / 72 us.
 static bool prefill_dual_pays(const kvd_ctx *ctx, const PrefillParams &P, int group) {
-  static const char *env = getenv("KVD_PREFILL_DUAL");  // 0/1 overrides, for comparisons
-  if (env) return env[0] == '1';
   const int tok = PT_ROWS / group;
-  return static_cast<long long>((P.n_rows + tok - 1) / tok) * P.n_kv > ctx->num_sms;
+  const long long tiles = static_cast<long long>((P.n_rows + tok - 1) / tok) * P.n_kv;
+  if (tiles <= ctx->num_sms) return false;
+  if (tiles > 4 * ctx->num_sms) return true;
+  return prefill_estimate(ctx, P, 2 * tok, 10.4f, 1.07f) < prefill_estimate(ctx, P, tok, 6.0f, 0.74f);
 }
 
 template <int D_HEAD>

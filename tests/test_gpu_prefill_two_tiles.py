@@ -1,4 +1,5 @@
-"""Long calls of kvd_prefill_attention at d_head 128 take two row tiles per CTA; short ones one.
+"""Long calls of kvd_prefill_attention at d_head 128 (more than four 128-row tiles per SM) take two row tiles per CTA,
+short ones (at most one per SM) one, those between whichever is estimated to end sooner.
 
 A token's bits do not depend on the call it is in, so rows of a long call equal the same rows in short calls (which the
 other file compares with the oracle): causal and windowed, across a gap between segments, rows past the last key and
@@ -18,7 +19,7 @@ PAIRS = LayerShape("g2", 128, 16, 8, 128, 1e-6, False, 1.0e4)
 
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16], ids=["bf16", "f16"])
-@pytest.mark.parametrize("shape,T,step", [(QWEN3_4B, 1300, 260), (SMOLLM2_135M, 4300, 700), (WINDOW, 2500, 500), (PAIRS, 1500, 300)], ids=lambda v: getattr(v, "name", str(v)))
+@pytest.mark.parametrize("shape,T,step", [(QWEN3_4B, 1300, 260), (SMOLLM2_135M, 4300, 700), (WINDOW, 2500, 500), (PAIRS, 1500, 300), (WINDOW, 5000, 500), (PAIRS, 5000, 300)], ids=lambda v: getattr(v, "name", str(v)))
 def test_rows_of_a_long_call_equal_those_of_short_calls(shape, T, step, dtype):
     kdim = shape.n_kv_heads * shape.d_head
     desc = kvd.make_desc(1, shape.d_hidden, shape.n_q_heads, shape.n_kv_heads, shape.d_head, shape.rms_eps, shape.qk_norm,
@@ -63,7 +64,7 @@ def test_a_tile_takes_no_block_that_only_its_neighbour_sees(group, window):
     n_kv, d_head, first = 8, 128, 5
     shape = LayerShape("inf", 128, group * n_kv, n_kv, d_head, 1e-6, False, 1.0e4, window)
     tok, kdim = 128 // group, n_kv * d_head
-    T = tok * (148 // n_kv + 4) + tok // 2  # more than one tile per SM, the last one short
+    T = tok * (4 * 148 // n_kv + 4) + tok // 2  # more than four tiles per SM: two per CTA; the last one short
     desc = kvd.make_desc(1, shape.d_hidden, shape.n_q_heads, n_kv, d_head, 1e-6, False, 1e-6, shape.rope_style, 1, T + 512, 1)
     ctx = kvd.Kvd(desc)
     w = make_layer_weights(shape)
