@@ -1257,7 +1257,8 @@ extern "C" kvd_status kvd_selftest_wait_timeout(kvd_ctx *ctx, int limit_ms, void
 extern "C" size_t kvd_trace_bytes(const kvd_model_desc *d, int row_blocks, int variant, int num_sms) {
   if (check_desc(d) != KVD_OK || row_blocks <= 0 || variant < 0 || variant > 2 || num_sms < 2) return 0;
   const int kdim = d->n_kv_heads * d->d_head, bn = pick_block_n(d);
-  return rc_trace_bytes(rc_schedule(num_sms, bn, d->d_head, row_blocks, 2 * kdim / bn, kdim, variant == 0 ? 2 : 1, variant == 2).clusters);
+  const int eb = variant == 0 ? 2 : 1;  // (a fused launch has one schedule whatever its element)
+  return rc_trace_bytes(rc_schedule(num_sms, bn, d->d_head, row_blocks, 2 * kdim / bn, d->d_hidden / RC_BLOCK_K, kdim, eb, variant == 2).clusters);
 }
 
 extern "C" kvd_status kvd_set_trace(kvd_ctx *ctx, void *buf, size_t bytes) {

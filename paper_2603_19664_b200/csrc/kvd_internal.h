@@ -361,13 +361,13 @@ inline cudaError_t launch_dependent(const kvd_ctx *ctx, void (*kern)(P...), dim3
 struct RcSchedule {
   int unit_tiles, whole_tiles, parts, clusters;
 };
-RcSchedule rc_schedule(int num_sms, int block_n, int d_head, int m_blocks, int n_blocks, int k_cols, int eb, bool fused);
+RcSchedule rc_schedule(int num_sms, int block_n, int d_head, int m_blocks, int n_blocks, int k_blocks, int k_cols, int eb, bool fused);
 inline size_t rc_trace_bytes(int clusters) {
   return 2 * static_cast<size_t>(clusters) * RC_TRACE_TILES * RC_TRACE_FIELDS * sizeof(long long);
 }
 // After the sizes of `p` are known: its schedule, and the trace buffer if the launch fits it.
 inline void schedule_recompute(const kvd_ctx *ctx, RecomputeParams &p, int eb, bool fused) {
-  const RcSchedule s = rc_schedule(ctx->num_sms, ctx->block_n, ctx->desc.d_head, p.num_m_blocks, p.num_n_blocks, p.k_cols, eb, fused);
+  const RcSchedule s = rc_schedule(ctx->num_sms, ctx->block_n, ctx->desc.d_head, p.num_m_blocks, p.num_n_blocks, p.num_k_blocks, p.k_cols, eb, fused);
   p.unit_tiles = s.unit_tiles;
   p.whole_tiles = s.whole_tiles;
   p.parts = s.parts;

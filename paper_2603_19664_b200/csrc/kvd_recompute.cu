@@ -978,7 +978,11 @@ static kvd_status launch_sel(kvd_ctx *ctx, const LayerState &ls, const CUtensorM
 // L2 (64 x 767 rows: 415 us in units, 422 single), units it is.  With less than one round (Qwen, 8 tiles 31 -> 20, 72
 // tiles 23.9 -> 21.7) halves shorten every CTA's exposed epilogue, if a half still holds whole heads: the key norm
 // runs over a head in one thread.
-RcSchedule rc_schedule(int num_sms, int block_n, int d_head, int m_blocks, int n_blocks, int k_cols, int eb, bool fused) {
+// Two rounds of halves in place of one of whole tiles: what the shorter epilogue gives is constant, what halves cost per k
+// block is not (products of 2560 columns, whole / halves, us: K 2560, 40 tiles 18.4 / 17.2, 60 tiles 18.9 / 18.5; K 10240,
+// 55.7 / 59.1 and 58.6 / 66.2).
+constexpr int RC_CUT_K_BLOCKS = 64;
+RcSchedule rc_schedule(int num_sms, int block_n, int d_head, int m_blocks, int n_blocks, int k_blocks, int k_cols, int eb, bool fused) {
   const int tiles = m_blocks * n_blocks, clusters = num_sms / 2;
   const int nk = k_cols % block_n == 0 ? k_cols / block_n : 0;  // 0 also where a tile mixes key and value heads
   const int rounds = tiles / clusters, last = tiles % clusters;
@@ -988,6 +992,7 @@ RcSchedule rc_schedule(int num_sms, int block_n, int d_head, int m_blocks, int n
     int parts = rounds == 0 ? 2 : 4 * last <= clusters ? 4 : 2 * last <= clusters ? 2 : 1;
     const bool keys = last > m_blocks * (n_blocks - nk);  // key tiles among those to be cut
     if (keys && block_n / parts < d_head) parts = 1;
+    if (rounds == 0 && 2 * tiles > clusters && k_blocks > RC_CUT_K_BLOCKS) parts = 1;  // two rounds of halves: not with a long K
     if (parts > 1) {
       s.whole_tiles = tiles - last;
       s.parts = parts;

@@ -126,6 +126,10 @@ def test_trace_bytes_cover_the_grid_a_launch_gets():
     assert kvd.kvd_trace_bytes(gemma, 1) == 16 * per_cta         # a half tile would split a key head
     assert kvd.kvd_trace_bytes(gemma, 1, variant=2) == 8 * per_cta  # units of a key and a value tile
     assert kvd.kvd_trace_bytes(smol, 1) == 6 * per_cta           # 128-column tiles
+    # 40 tiles: two rounds of halves (74 clusters) with a short K, one round of whole tiles with a long one
+    wide = kvd.make_desc(1, 8192, 32, 8, 128, 1e-6, True, 1e-6)
+    assert kvd.kvd_trace_bytes(qwen, 5) == 148 * per_cta and kvd.kvd_trace_bytes(wide, 5) == 80 * per_cta
+    assert kvd.kvd_trace_bytes(wide, 1) == 32 * per_cta          # halves in one round: always
     for desc in (qwen, gemma, smol):
         for variant in (0, 1, 2):
             for blocks in (1, 5, 9, 10, 18, 19, 37, 1000):
