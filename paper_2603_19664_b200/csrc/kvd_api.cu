@@ -641,6 +641,7 @@ static kvd_status recompute_launch(kvd_ctx *ctx, int layer, const kvd_store_rang
     r.append_rows = p.append_rows;
     r.append_pos = p.append_pos;
     r.append_sumsq = p.append_sumsq;
+    r.store_slots = static_cast<long long>(ctx->layers_stored) * d.max_seqs * d.max_tokens_per_seq;
     for (int i = 0; i < p.append_n; ++i) r.append_slot[i] = p.append_slot[i];
     st = launch_rows(ctx, ls, d.d_hidden, r, true, stream);
   } else {

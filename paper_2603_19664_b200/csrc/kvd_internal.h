@@ -148,6 +148,7 @@ struct RowsParams {
   int32_t *append_pos;
   float *append_sumsq;
   long long append_slot[RW_MAX_ROWS];
+  long long store_slots;       // slots of the store (checking build)
 };
 
 // ------------------------------------------------------------------------------ decode attention

@@ -237,7 +237,9 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
         for (int i = 0; i < 4; ++i) {
           const int r = 4 * g + i;
           src[i] = p.rows + static_cast<size_t>(r < p.n_rows ? r : p.n_rows - 1) * p.row_chunks;
-          if (append && r < p.n_rows) dst[i] = p.append_rows + static_cast<size_t>(p.append_slot[r]) * p.row_chunks;
+          // (checking build: the slot lies inside the store)
+          if (append && r < p.n_rows && KVD_BOUNDS_OK(p.append_slot[r] >= 0 && p.append_slot[r] < p.store_slots, p.status))
+            dst[i] = p.append_rows + static_cast<size_t>(p.append_slot[r]) * p.row_chunks;
         }
         float ss[4];
         if (append) warp_rows_sumsq<4, 4, true, DT>(src, dst, p.row_chunks, lane, ss);
@@ -246,7 +248,7 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
         const int r = 4 * g + lane;
         if (lane < 4 && r < p.n_rows) {
           s_rstd[r] = 1.0f / sqrtf(mine * p.inv_k + p.rms_eps);
-          if (append) {
+          if (append && KVD_BOUNDS_OK(p.append_slot[r] >= 0 && p.append_slot[r] < p.store_slots, p.status)) {
             p.append_sumsq[p.append_slot[r]] = mine;
             p.append_pos[p.append_slot[r]] = p.positions[r];
           }
@@ -269,7 +271,8 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
         }
         tc_fence_after();
         const uint32_t acc = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + a * (p.tmem_cols / 2);
-        const int cols = p.n_cols - col0 < tile ? p.n_cols - col0 : tile;
+        // (checking build: the tile's columns exist; otherwise none is stored)
+        const int cols = !KVD_BOUNDS_OK(col0 >= 0 && col0 < p.n_cols && col0 % tile == 0, p.status) ? 0 : p.n_cols - col0 < tile ? p.n_cols - col0 : tile;
         if constexpr (HEADS) {
           if (busy) {
             uint32_t v[RW_HEAD_TILE];
@@ -360,6 +363,8 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
     __syncthreads();
     const int c = col0 % D_HEAD + 2 * (lane & 15);  // this lane's two columns of the head; half a warp per row
     for (int r = 2 * warp + (lane >> 4); r < p.n_rows; r += 2 * (RW_THREADS / 32)) {
+      // (checking build: this CTA's columns lie inside the key or the value heads)
+      if (!KVD_BOUNDS_OK(col0 + RW_HEAD_TILE <= (key ? p.k_cols : p.n_cols) && r < RW_MAX_ROWS, p.status)) continue;
       const float *y = s_y + r * LD;
       const float ks = s_kscale[r];
       uint32_t o;

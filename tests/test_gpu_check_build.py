@@ -7,7 +7,7 @@ bit of the status word that kvd_poll_status reports as KVD_ERR_BOUNDS.
 
 This test (1) shows the mechanism reporting, through the self-test entry point whose index is out of range by
 construction and whose guarded access is skipped, and the context staying usable afterwards; (2) runs the
-oracle-parity suites of the recompute, attention, fused and FP8 paths against the checking build in a child
+oracle-parity suites of the recompute, attention, fused, FP8 and few-row paths against the checking build in a child
 process -- every one of those tests ends by polling the status word, so a failed index test anywhere fails it.
 """
 import os
@@ -61,7 +61,7 @@ def test_checking_build_reports_and_passes_the_parity_suites():
     r = subprocess.run([sys.executable, "-c", SELFTEST], cwd=ROOT, env=env, capture_output=True, text=True, timeout=900)
     assert r.returncode == 0 and "checking build ok" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
     files = ["tests/test_gpu_recompute.py", "tests/test_gpu_attention.py", "tests/test_gpu_fused.py", "tests/test_gpu_fp8.py",
-             "tests/test_gpu_scaffold.py"]
+             "tests/test_gpu_scaffold.py", "tests/test_gpu_rows.py"]
     r = subprocess.run([sys.executable, "-m", "pytest", "-x", "-q", "-m", "gpu", "-p", "no:cacheprovider", *files], cwd=ROOT,
                        env=env, capture_output=True, text=True, timeout=1800)
     assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-2000:]

@@ -80,3 +80,9 @@ def test_the_early_start_threshold_follows_the_device():
     fn = text[text.index("inline cudaError_t launch_dependent("):]
     fn = fn[:fn.index("\n}")]
     assert "ctx->num_sms" in fn and not re.search(r"grid\.x\s*[<>]=?\s*\d", fn)
+
+
+def test_kernels_that_derive_store_slots_or_tiles_test_them_in_the_checking_build():
+    body = KERNELS["kvd_rows_kernel"][1]
+    for index in ("append_slot[r]", "col0"):
+        assert re.search(r"KVD_BOUNDS_OK\([^;]*" + re.escape(index), body), index
