@@ -84,3 +84,26 @@ def test_successive_products_overlap_without_changing_bits(k, n):
     assert torch.equal(alone, out)
     assert ctx.kvd_poll_status() == kvd.KVD_OK
     ctx.close()
+
+
+@pytest.mark.parametrize("shape", [GEMMA3_4B_GLOBAL, QWEN3_4B, SMOLLM2_135M], ids=lambda s: s.name)
+def test_few_fp16_rows_have_the_bits_of_the_large_call(shape):
+    kdim, t = shape.n_kv_heads * shape.d_head, torch.float16
+    ctx = kvd.Kvd(kvd.make_desc(1, shape.d_hidden, shape.n_q_heads, shape.n_kv_heads, shape.d_head, shape.rms_eps, shape.qk_norm,
+                                shape.rms_eps, shape.rope_style, 1, 1024, 1))
+    ctx.kvd_set_dtype(1)
+    g = torch.Generator(device="cuda").manual_seed(4)
+    w = (torch.randn((shape.d_hidden, 2 * kdim), generator=g, device="cuda") * 0.02).to(t)
+    gammas = [(1 + 0.1 * torch.randn((n,), generator=g, device="cuda")).to(t) for n in (shape.d_hidden, shape.d_head)]
+    ctx.kvd_set_layer(0, w, gammas[0], gammas[1] if shape.qk_norm else None, shape.rope_theta)
+    x = torch.randn((200, shape.d_hidden), generator=g, device="cuda").to(t)
+    pos = (torch.arange(200, dtype=torch.int32, device="cuda") * 5) % 1024
+    k, v = (torch.empty((200, kdim), dtype=t, device="cuda") for _ in range(2))
+    ctx.kvd_recompute_kv(0, x, pos, 200, k, v, kdim)
+    for r0, n in ((0, 1), (3, 8), (20, 9), (31, 16), (50, 17), (64, 33), (136, 64)):
+        kk, vv = (torch.full((n + 1, kdim + 8), 7.0, dtype=t, device="cuda") for _ in range(2))
+        ctx.kvd_recompute_kv(0, x[r0:], pos[r0:], n, kk, vv, kdim + 8)
+        assert torch.equal(kk[:n, :kdim], k[r0:r0 + n]) and torch.equal(vv[:n, :kdim], v[r0:r0 + n]), (r0, n)
+        assert bool((kk[:n, kdim:] == 7).all()) and bool((kk[n] == 7).all()) and bool((vv[n] == 7).all()), (r0, n)
+    assert ctx.kvd_poll_status() == kvd.KVD_OK
+    ctx.close()
