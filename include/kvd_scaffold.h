@@ -9,9 +9,10 @@
  * on the library's own kernels, so that a whole-stack run uses no third-party GEMM or elementwise library:
  *
  *   kvd_scaffold_linear          out = s (x W'),  W' = diag(gamma) W prepared once; s = 1/rms(x) per row when a
- *                                gamma was given (RMSNorm of Eq. 1-2 folded in), 1 otherwise.  Runs on the
- *                                recompute kernel of kvd.h (same tcgen05 tiles, every column treated as a value
- *                                column), so a row's output bits do not depend on how many rows a call carries.
+ *                                gamma was given (RMSNorm of Eq. 1-2 folded in), 1 otherwise.  At most 64 rows run on
+ *                                a kernel of their own (narrow tcgen05 tiles over all SMs, bound by reading W'), more
+ *                                on the recompute kernel of kvd.h (every column treated as a value column); a row's
+ *                                output bits do not depend on how many rows a call carries.
  *   kvd_scaffold_query_finish    per query head: optional RMS norm over d_head, then the rotation of Eq. 11-12
  *                                at the row's position (the same tables as the keys).
  *   kvd_scaffold_add_rows        h <- h + y (Eq. 8 / Eq. 9 residual adds), rounded to bf16.
@@ -21,8 +22,7 @@
  *
  * Conventions are those of kvd.h: plain C, DEVICE pointers are the caller's bf16 buffers (16-byte aligned),
  * launches are asynchronous on `stream`, argument errors are found on the host before anything is launched,
- * bf16 contexts only (KVD_ERR_UNSUPPORTED after kvd_set_dtype chose another type).  Throughput is not the
- * point of these calls: a product always walks 256-row tiles, whatever the batch.
+ * bf16 contexts only (KVD_ERR_UNSUPPORTED after kvd_set_dtype chose another type).
  */
 #ifndef KVD_SCAFFOLD_H_
 #define KVD_SCAFFOLD_H_

@@ -2,7 +2,7 @@
 //
 //   CTA   = (tile of query tokens, KV head): 128 MMA rows = 128 / G tokens x the G query heads of the head's group (for
 //           G = 3, 42 tokens and two empty rows; empty rows are zeros that are never stored).
-//   pair  = for d_head >= 128 two CTAs with neighbouring tiles of the same KV head form a cluster and run the products
+//   pair  = for d_head 256 two CTAs with neighbouring tiles of the same KV head form a cluster and run the products
 //           as tcgen05.mma.cta_group::2 (M = 256, 128 rows per CTA): a K or V block is shared by the pair, each CTA
 //           loads and holds half of it (K: half the keys, V: half the channels -- the halves the instruction reads from
 //           either shared memory).  Half the bytes per CTA through L2 and shared memory, twice the blocks in flight.
@@ -693,7 +693,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1) kvd_prefill_attn_tc_kernel(cons
 // for the scores) about a third of the time.  Here each group has a tile of its own, so nothing is exchanged, a K or V
 // block is loaded once for 256 rows, and each tile's next scores are there before its softmax asks for them.  A CTA
 // takes longer per block than above (1950 against 1550 clocks, for twice the rows), hence only where there are enough
-// of them (prefill_dual_pays).  4096 tokens of a Qwen3-4B layer 207 -> 161 us, 16384 2783 -> 2030 us.
+// of them (prefill_dual_pays).  4096 tokens of a Qwen3-4B layer 207 -> 162 us, 16384 2783 -> 2030 us.
 //   TMEM = [ O_0, O_1 : d_head columns each | S_00, S_01, S_10, S_11 : 64 columns each (tile, block parity) ]; the
 //          weights of a block overwrite the first half of its scores.  The query tiles are in shared memory.
 //   warps = 0-3 tile 0, 4-7 tile 1, 8 and 9 the products of tiles 0 and 1, 10 and 11 loaders: twelve warps leave a

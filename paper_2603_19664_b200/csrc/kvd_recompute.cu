@@ -28,14 +28,13 @@
 //
 // The producer and the MMA issuer are single threads whose loop must finish well inside the 512
 // clocks a k block of MMAs takes; their loops are therefore kept to a few dozen instructions
-// (incremental addresses, one asm block per k block).  They are chosen by elect.sync in a warp-uniform branch: behind a
-// test of the lane number the compiler moves every operand of an MMA or a load to uniform registers at run time (48 to
-// 65 clocks per MMA, issue alone, against 24).  4096 rows of a Gemma-3-4B layer 39.9 -> 37.9 us, 6757 rows 59.2 -> 56.4 us,
-// 16384 rows of a Qwen3-4B layer 138.6 -> 134.3 us; the two prefill-attention issuers gained nothing from it.  Every wait is bounded; on expiry the kernel
-// records STATUS_TIMEOUT and drains.
+// (incremental addresses, one asm block per k block).  They are chosen by elect.sync in a warp-uniform branch: issue
+// alone measured 24 clocks per MMA that way and 48 to 65 behind a test of the lane number.  Device time of a launch:
+// 4096 rows of a Gemma-3-4B layer 31.3 -> 30.7 us; the two prefill-attention issuers gained nothing from it.  Every wait
+// is bounded; on expiry the kernel records STATUS_TIMEOUT and drains.
 //
-// Bit-reproducibility: the k loop always runs over all of d_hidden in ascending order with one MMA
-// shape, a row's sum of squares is taken by one function in one fixed order wherever it is taken
+// Bit-reproducibility: the k loop always runs over all of d_hidden in ascending order in steps of K = 16 (tiles of 256,
+// 128 and 64 columns give an element the same bits: measured by the tests, not promised by PTX), a row's sum of squares is taken by one function in one fixed order wherever it is taken
 // (warp_rows_sumsq), the key norm is reduced by the single thread that owns the row, and cos/sin
 // depend on (position, channel) only.  A row's output bits are therefore independent of M, of the
 // row's index and of whether it came from the store or from the caller.
@@ -974,9 +973,11 @@ static kvd_status launch_sel(kvd_ctx *ctx, const LayerState &ls, const CUtensorM
 // would leave half of the clusters idle or more.  Cost estimate in tiles per cluster, from launches of 128 to 32768
 // rows of the Gemma-3-4B and Qwen3-4B layers (units / single / halves / quarters, us): 88 tiles on 74 clusters 31.1 /
 // 29.5 / 26.6 / 26.3, 160 52.8 / 42.3 / 40.2 / 40.2, 192 54 / 45.9 / 49.3 / 53, 224 61 / 61 / 55.5 / 54.3, 512 125 / 114 / 126 / 144, 1024
-// 254 / 254 / 256 / 277.  Single tiles read X at two distant times: beyond 8 rounds, where it no longer stays in the
-// L2 (64 x 767 rows: 415 us in units, 422 single), units it is.  With less than one round (Qwen, 8 tiles 31 -> 20, 72
-// tiles 23.9 -> 21.7) halves shorten every CTA's exposed epilogue, if a half still holds whole heads: the key norm
+// 254 / 254 / 256 / 277.  The same rule serves fp16, fp32 (TF32) and the scaffold's products; units and single tiles before
+// it / with it, us: fp16 2600 rows 34.0 / 26.5, 5000 55.8 / 39.4; fp32 2600 rows 60.9 / 43.9, 5000 103 / 77; 2560 x 2560
+// products of 2000 rows 28.9 / 22.9, of 3000 (not cut) 29.9 / 29.9.  Single tiles read X at two distant times: beyond 8 rounds, where it no longer stays in the
+// L2 (64 x 767 rows: 415 us in units, 422 single), units it is.  With less than one round (Qwen, 200 rows = 8 tiles
+// 19.6 -> 12.8, 2304 rows = 72 tiles 21.4 -> 20.1) halves shorten every CTA's exposed epilogue, if a half still holds whole heads: the key norm
 // runs over a head in one thread.
 // Two rounds of halves in place of one of whole tiles: what the shorter epilogue gives is constant, what halves cost per k
 // block is not (products of 2560 columns, whole / halves, us: K 2560, 40 tiles 18.4 / 17.2, 60 tiles 18.9 / 18.5; K 10240,

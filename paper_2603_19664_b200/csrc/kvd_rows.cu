@@ -8,8 +8,8 @@
 // CTA pairs for the models' projections.  Here a tile is as narrow as it takes to give every SM one (a multiple
 // of 8 columns, RW_MIN_TILE at least), so that all SMs pull weights at once.
 //
-// The MMA has 64 rows however few of them are rows of X; only those are loaded, the descriptor's other rows are whatever lies behind them in shared memory, and their accumulators (lanes of
-// tensor memory) are never read.
+// The MMA has 64 rows however few of them are rows of X; only those are loaded, the descriptor's other rows are whatever
+// lies behind them in shared memory, and their accumulators (lanes of tensor memory) are never read.
 //
 // The bits are those of the recompute kernel: an output element is one accumulator that takes the same K = 16
 // steps in the same ascending order, and the finishing below repeats that kernel's operations and their order
@@ -179,7 +179,7 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     grid_dependency_wait();  // (the bounded waits below start when the rows can be loaded)
-    if (elect_one()) {  // (a lane chosen by elect keeps the operands in uniform registers: 24 clocks per MMA, 48 in a branch on the lane number)
+    if (elect_one()) {  // (24 clocks per MMA; 48 in a branch on the lane number)
       const uint32_t idesc = DT == 1 ? umma_idesc_f16_f32(RW_MMA_ROWS, tile) : umma_idesc_bf16_f32(RW_MMA_ROWS, tile);
       constexpr uint32_t desc_hi = (1024u >> 4) | (1u << 14) | (2u << 29);  // as in kvd_recompute.cu
       int s = 0;
