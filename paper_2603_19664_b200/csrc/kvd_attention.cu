@@ -113,11 +113,16 @@ __global__ void __launch_bounds__(AT_THREADS, ALLIN ? 2 : AT_CTAS_PER_SM) kvd_at
   grid_dependency_wait();
   // ---- query of every head of the group, pre-multiplied by scale * log2(e)
   uint64_t qf[G][4];  // channel pairs (2j, 2j+1)
-  auto load_query = [&]() {
+  uint4 q_raw[G];
+  auto fetch_query = [&]() {
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+      q_raw[g] = *reinterpret_cast<const uint4 *>(P.q + (static_cast<size_t>(si) * P.n_q + kvh * G + g) * D_HEAD + lig * 8);
+  };
+  auto scale_query = [&]() {
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      const __nv_bfloat16 *qp = P.q + (static_cast<size_t>(si) * P.n_q + kvh * G + g) * D_HEAD + lig * 8;
-      const uint4 w = *reinterpret_cast<const uint4 *>(qp);
+      const uint4 w = q_raw[g];
       const uint64_t sc2 = pack2(P.scale_log2e, P.scale_log2e);
       qf[g][0] = fmul2(x2_to_f32x2<DT>(w.x), sc2);
       qf[g][1] = fmul2(x2_to_f32x2<DT>(w.y), sc2);
@@ -125,7 +130,9 @@ __global__ void __launch_bounds__(AT_THREADS, ALLIN ? 2 : AT_CTAS_PER_SM) kvd_at
       qf[g][3] = fmul2(x2_to_f32x2<DT>(w.w), sc2);
     }
   };
-  if constexpr (!ALLIN) load_query();
+  constexpr bool LATE_QUERY = !ALLIN && G <= 2;  // (wider groups have no registers left for it)
+  if constexpr (!ALLIN) fetch_query();
+  if constexpr (!ALLIN && !LATE_QUERY) scale_query();
 
   float m_run[G], l_run[G];
   uint64_t acc[G][4];  // channel pairs
@@ -276,7 +283,8 @@ __global__ void __launch_bounds__(AT_THREADS, ALLIN ? 2 : AT_CTAS_PER_SM) kvd_at
     uint32_t ma = 0, mb = 0;
     issue(0, ka, va, ma);
     issue(1, kb, vb, mb);
-    load_query();
+    fetch_query();
+    scale_query();
     step(ka, va, ma);
     step(kb, vb, mb);
   } else {
@@ -285,7 +293,10 @@ __global__ void __launch_bounds__(AT_THREADS, ALLIN ? 2 : AT_CTAS_PER_SM) kvd_at
     // register double buffering or a shared-memory ring at half the occupancy.
     uint4 ka[U], va[U];
     uint32_t ma = 0;
-    for (int it = 0; it < S.iters; ++it) {
+    issue(0, ka, va, ma);
+    if constexpr (LATE_QUERY) scale_query();  // (behind the first loads: the wait for the query is not one of its own)
+    step(ka, va, ma);
+    for (int it = 1; it < S.iters; ++it) {
       issue(it, ka, va, ma);
       step(ka, va, ma);
     }
@@ -742,9 +753,13 @@ static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t str
   // Starting early pays for launches of up to one wave (the set-up hides under the predecessor's tail);
   // a many-wave grid whose first CTAs sit on the SMs waiting slowed a short predecessor down in
   // measurements (11 us lost on a 24 us predecessor), so those are ordered plainly.
-  const bool small = S.total_chunks * S.n_kv <= 148 * AT_CTAS_PER_SM;
+  // Behind the few-row projection every grid does: that kernel's CTAs are resident and few, it leaves room for this one's
+  // beside them (RW_HEADS_SMEM), and it is too short for the waiting CTAs to cost what they save.  Gemma-3-4B layer, one
+  // new token per sequence, ordered plainly / started early, us per step: 16 x 2048 fp16 43.0 / 38.0, window layer 40 x
+  // 3000 56.0 / 54.2, Qwen3-4B 8 x 4000 51.9 / 48.5.
+  const bool early = S.early_start || S.total_chunks * S.n_kv <= 148 * AT_CTAS_PER_SM;
   if (S.total_chunks > 0) {
-    attr[0].val.programmaticStreamSerializationAllowed = (small && !(serial_launch_mask() & 2)) ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = (early && !(serial_launch_mask() & 2)) ? 1 : 0;
     cfg.gridDim = dim3(S.total_chunks * S.n_kv, 1, 1);
     cfg.blockDim = dim3(AT_THREADS, 1, 1);
     if constexpr (G >= 3 && D_HEAD <= 128) {
@@ -764,7 +779,7 @@ static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t str
     }
     if (e != cudaSuccess) return e;
   }
-  attr[0].val.programmaticStreamSerializationAllowed = (small && !(serial_launch_mask() & 4)) ? 1 : 0;
+  attr[0].val.programmaticStreamSerializationAllowed = (early && !(serial_launch_mask() & 4)) ? 1 : 0;
   // as many warps per merge CTA as the longest sequence of the launch has groups of partials
   int max_chunks = 1;
   for (int i = 0; i < S.n_seqs; ++i) max_chunks = S.seq[i].merge_count > max_chunks ? S.seq[i].merge_count : max_chunks;
@@ -782,6 +797,7 @@ static kvd_status launch_attn_impl(kvd_ctx *ctx, const AttnLaunch &L, cudaStream
     static thread_local AttnLaunchT<NSEQ> S;
     static_cast<AttnLaunchHead &>(S) = static_cast<const AttnLaunchHead &>(L);
     for (int i = 0; i < L.n_seqs; ++i) S.seq[i] = L.seq[i];
+    S.early_start = ctx->few_rows_last;
     // fp16 contexts (kvd_set_dtype): the same kernels reading and writing fp16
     cudaError_t e = ctx->dtype == 1 ? attn_launch_pair<D_HEAD, G, NSEQ, 1>(S, stream)
                                     : attn_launch_pair<D_HEAD, G, NSEQ, 0>(S, stream);
@@ -985,6 +1001,7 @@ extern "C" kvd_status kvd_decode_attention_static(int n_q_heads, int n_kv_heads,
   L.part_o = reinterpret_cast<float *>(scratch + ml_bytes);
   L.status = nullptr;
   L.max_parts = parts;
+  L.early_start = false;
   switch (d_head) {
     case 64: return static_launch_d<64>(L, group, stream);
     case 128: return static_launch_d<128>(L, group, stream);

@@ -31,6 +31,8 @@
 // different tiles.
 #include <string.h>
 
+#include <type_traits>
+
 #include "kvd_internal.h"
 #include "kvd_ptx.cuh"
 
@@ -39,6 +41,11 @@ namespace kvd {
 constexpr int RW_THREADS = 320;
 constexpr int RW_MAX_STAGES = 16;
 constexpr int RW_MMA_ROWS = 64;                           // M of the MMA
+// Shared memory of key and value heads of few rows.  The streaming attention's CTAs (9 KB, 16 K registers each) that
+// follow take places beside this kernel's -- two, with the registers its launch bounds leave -- and wait there instead of
+// being started when it ends; the ring still holds most of a CTA's weights.  One new token over 32768 cached ones, us:
+// 43.7 with all of an SM's shared memory, 37.2 with 173 or 193 KB, 36.1 with 145 or 161.
+constexpr int RW_HEADS_SMEM = 161 * 1024;
 constexpr int RW_BARS = 2 * RW_MAX_STAGES + 4;            // full, empty per stage; tmem_full[2], tmem_empty[2]
 constexpr int RW_TAIL = RW_BARS * 8 + 32 + RW_MAX_ROWS * 3 * 4;  // barriers, tmem pointer + abort, 1/rms, key scale, position
 
@@ -77,7 +84,7 @@ __device__ __forceinline__ void umma_kblock(uint32_t d_tmem, uint32_t a_lo, uint
 
 // D_HEAD = 0: a plain product, every column scaled by the row factor and stored.  D_HEAD > 0: key and value heads.
 template <int D_HEAD, int DT>
-__global__ void __launch_bounds__(RW_THREADS, 1)
+__global__ void __launch_bounds__(RW_THREADS, 2)
 kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
                 const __grid_constant__ RowsParams p) {
   constexpr bool HEADS = D_HEAD > 0;
@@ -229,31 +236,39 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
       // STORE_RESIDUAL in the same launch (kvd_decode_step_kv): the first CTA writes the rows it reads into the
       // store slots the host assigned to them
       const bool append = HEADS && p.append_rows != nullptr && block == 0;
+      // R rows of a warp side by side, B loads of each in flight: one round trip for the usual width and up to 8 rows
+      auto take = [&](auto r_c, auto b_c) {
+        constexpr int R = decltype(r_c)::value, B = decltype(b_c)::value;
 #pragma unroll 1
-      for (int g = w8; 4 * g < p.n_rows; g += 8) {
-        const uint4 *src[4];
-        uint4 *dst[4] = {nullptr, nullptr, nullptr, nullptr};
+        for (int g = w8; R * g < p.n_rows; g += 8) {
+          const uint4 *src[R];
+          uint4 *dst[R];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int r = 4 * g + i;
-          src[i] = p.rows + static_cast<size_t>(r < p.n_rows ? r : p.n_rows - 1) * p.row_chunks;
-          // (checking build: the slot lies inside the store)
-          if (append && r < p.n_rows && KVD_BOUNDS_OK(p.append_slot[r] >= 0 && p.append_slot[r] < p.store_slots, p.status))
-            dst[i] = p.append_rows + static_cast<size_t>(p.append_slot[r]) * p.row_chunks;
-        }
-        float ss[4];
-        if (append) warp_rows_sumsq<4, 4, true, DT>(src, dst, p.row_chunks, lane, ss);
-        else warp_rows_sumsq<4, 4, false, DT>(src, dst, p.row_chunks, lane, ss);
-        const float mine = lane == 0 ? ss[0] : lane == 1 ? ss[1] : lane == 2 ? ss[2] : ss[3];
-        const int r = 4 * g + lane;
-        if (lane < 4 && r < p.n_rows) {
-          s_rstd[r] = 1.0f / sqrtf(mine * p.inv_k + p.rms_eps);
-          if (append && KVD_BOUNDS_OK(p.append_slot[r] >= 0 && p.append_slot[r] < p.store_slots, p.status)) {
-            p.append_sumsq[p.append_slot[r]] = mine;
-            p.append_pos[p.append_slot[r]] = p.positions[r];
+          for (int i = 0; i < R; ++i) {
+            const int r = R * g + i;
+            src[i] = p.rows + static_cast<size_t>(r < p.n_rows ? r : p.n_rows - 1) * p.row_chunks;
+            dst[i] = nullptr;
+            // (checking build: the slot lies inside the store)
+            if (append && r < p.n_rows && KVD_BOUNDS_OK(p.append_slot[r] >= 0 && p.append_slot[r] < p.store_slots, p.status))
+              dst[i] = p.append_rows + static_cast<size_t>(p.append_slot[r]) * p.row_chunks;
+          }
+          float ss[R];
+          warp_rows_sumsq<R, B, HEADS, DT>(src, dst, p.row_chunks, lane, ss);
+          float mine = ss[0];
+#pragma unroll
+          for (int i = 1; i < R; ++i) mine = lane == i ? ss[i] : mine;
+          const int r = R * g + lane;
+          if (lane < R && r < p.n_rows) {
+            s_rstd[r] = 1.0f / sqrtf(mine * p.inv_k + p.rms_eps);
+            if (append && KVD_BOUNDS_OK(p.append_slot[r] >= 0 && p.append_slot[r] < p.store_slots, p.status)) {
+              p.append_sumsq[p.append_slot[r]] = mine;
+              p.append_pos[p.append_slot[r]] = p.positions[r];
+            }
           }
         }
-      }
+      };
+      if (p.n_rows <= 8) take(std::integral_constant<int, 1>(), std::integral_constant<int, 10>());
+      else take(std::integral_constant<int, 2>(), std::integral_constant<int, 5>());
     }
     asm volatile("bar.sync 1, 256;" ::: "memory");
     if (warp >= 4 && warp < 8) {
@@ -416,7 +431,8 @@ static kvd_status launch_rows_impl(kvd_ctx *ctx, const CUtensorMap &tmap_w, cons
   const int beyond = RW_MMA_ROWS * 128 - (stage - (p.stage_kb - 1) * p.nr * 128);
   const int slack = beyond > 0 ? beyond : 0;
   const int total = (p.num_k_blocks + p.stage_kb - 1) / p.stage_kb * ((p.n_tiles + ctx->num_sms - 1) / ctx->num_sms);
-  p.stages = (SMEM_MAX - tail - slack) / stage;
+  const int smem = D_HEAD > 0 && p.nr <= RW_FEW_ROWS ? RW_HEADS_SMEM : SMEM_MAX;
+  p.stages = (smem - tail - slack) / stage;
   if (p.stages > RW_MAX_STAGES) p.stages = RW_MAX_STAGES;
   if (p.stages > total) p.stages = total;
   p.tail_off = p.stages * stage + slack;
@@ -496,6 +512,7 @@ kvd_status launch_rows(kvd_ctx *ctx, const LayerState &ls, int k, RowsParams &p,
   if (st != KVD_OK) return st;
   const CUtensorMap &w = ls.tmap_rows[many ? 1 : 0];
   if (!heads) return launch_rows_impl<0, 0>(ctx, w, tmap_x, p, stream);
+  ctx->few_rows_last = true;
   const bool half = ctx->dtype == KVD_DTYPE_F16;
   switch (ctx->desc.d_head) {
     case 64: return half ? launch_rows_impl<64, 1>(ctx, w, tmap_x, p, stream) : launch_rows_impl<64, 0>(ctx, w, tmap_x, p, stream);
