@@ -113,16 +113,11 @@ __global__ void __launch_bounds__(AT_THREADS, ALLIN ? 2 : AT_CTAS_PER_SM) kvd_at
   grid_dependency_wait();
   // ---- query of every head of the group, pre-multiplied by scale * log2(e)
   uint64_t qf[G][4];  // channel pairs (2j, 2j+1)
-  uint4 q_raw[G];
-  auto fetch_query = [&]() {
-#pragma unroll
-    for (int g = 0; g < G; ++g)
-      q_raw[g] = *reinterpret_cast<const uint4 *>(P.q + (static_cast<size_t>(si) * P.n_q + kvh * G + g) * D_HEAD + lig * 8);
-  };
-  auto scale_query = [&]() {
+  auto load_query = [&]() {
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      const uint4 w = q_raw[g];
+      const __nv_bfloat16 *qp = P.q + (static_cast<size_t>(si) * P.n_q + kvh * G + g) * D_HEAD + lig * 8;
+      const uint4 w = *reinterpret_cast<const uint4 *>(qp);
       const uint64_t sc2 = pack2(P.scale_log2e, P.scale_log2e);
       qf[g][0] = fmul2(x2_to_f32x2<DT>(w.x), sc2);
       qf[g][1] = fmul2(x2_to_f32x2<DT>(w.y), sc2);
@@ -130,9 +125,7 @@ __global__ void __launch_bounds__(AT_THREADS, ALLIN ? 2 : AT_CTAS_PER_SM) kvd_at
       qf[g][3] = fmul2(x2_to_f32x2<DT>(w.w), sc2);
     }
   };
-  constexpr bool LATE_QUERY = !ALLIN && G <= 2;  // (wider groups have no registers left for it)
-  if constexpr (!ALLIN) fetch_query();
-  if constexpr (!ALLIN && !LATE_QUERY) scale_query();
+  if constexpr (!ALLIN) load_query();
 
   float m_run[G], l_run[G];
   uint64_t acc[G][4];  // channel pairs
@@ -283,8 +276,7 @@ __global__ void __launch_bounds__(AT_THREADS, ALLIN ? 2 : AT_CTAS_PER_SM) kvd_at
     uint32_t ma = 0, mb = 0;
     issue(0, ka, va, ma);
     issue(1, kb, vb, mb);
-    fetch_query();
-    scale_query();
+    load_query();
     step(ka, va, ma);
     step(kb, vb, mb);
   } else {
@@ -293,10 +285,7 @@ __global__ void __launch_bounds__(AT_THREADS, ALLIN ? 2 : AT_CTAS_PER_SM) kvd_at
     // register double buffering or a shared-memory ring at half the occupancy.
     uint4 ka[U], va[U];
     uint32_t ma = 0;
-    issue(0, ka, va, ma);
-    if constexpr (LATE_QUERY) scale_query();  // (behind the first loads: the wait for the query is not one of its own)
-    step(ka, va, ma);
-    for (int it = 1; it < S.iters; ++it) {
+    for (int it = 0; it < S.iters; ++it) {
       issue(it, ka, va, ma);
       step(ka, va, ma);
     }
@@ -755,8 +744,8 @@ static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t str
   // measurements (11 us lost on a 24 us predecessor), so those are ordered plainly.
   // Behind the few-row projection every grid does: that kernel's CTAs are resident and few, it leaves room for this one's
   // beside them (RW_HEADS_SMEM), and it is too short for the waiting CTAs to cost what they save.  Gemma-3-4B layer, one
-  // new token per sequence, ordered plainly / started early, us per step: 16 x 2048 fp16 43.0 / 38.0, window layer 40 x
-  // 3000 56.0 / 54.2, Qwen3-4B 8 x 4000 51.9 / 48.5.
+  // new token per sequence, ordered plainly / started early, us per step: 16 x 2048 fp16 43.0 / 38.7, window layer 40 x
+  // 3000 56.0 / 54.2, Qwen3-4B 8 x 4000 51.9 / 49.7.
   const bool early = S.early_start || S.total_chunks * S.n_kv <= 148 * AT_CTAS_PER_SM;
   if (S.total_chunks > 0) {
     attr[0].val.programmaticStreamSerializationAllowed = (early && !(serial_launch_mask() & 2)) ? 1 : 0;

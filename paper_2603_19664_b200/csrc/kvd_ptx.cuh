@@ -542,19 +542,15 @@ __device__ __forceinline__ void warp_rows_sumsq(const uint4 *const (&src)[R], ui
         sumsq_chunk<DT>(ps2[r], v[r][j]);
       }
   }
-  if (c < n_chunks) {  // the rest in one batch too: a chunk past the end is not read and adds exact zeros
-    uint4 v[R][B - 1];
+  for (; c < n_chunks; c += 32) {
+    uint4 v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r)
+    for (int r = 0; r < R; ++r) v[r] = src[r][c];
 #pragma unroll
-      for (int j = 0; j < B - 1; ++j) v[r][j] = c + 32 * j < n_chunks ? src[r][c + 32 * j] : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-#pragma unroll
-      for (int j = 0; j < B - 1; ++j) {
-        if (COPY && dst[r] != nullptr && c + 32 * j < n_chunks) dst[r][c + 32 * j] = v[r][j];
-        sumsq_chunk<DT>(ps2[r], v[r][j]);
-      }
+    for (int r = 0; r < R; ++r) {
+      if (COPY && dst[r] != nullptr) dst[r][c] = v[r];
+      sumsq_chunk<DT>(ps2[r], v[r]);
+    }
   }
 #pragma unroll
   for (int r = 0; r < R; ++r) out[r] = sumsq_finish(ps2[r]);

@@ -44,7 +44,7 @@ constexpr int RW_MMA_ROWS = 64;                           // M of the MMA
 // Shared memory of key and value heads of few rows.  The streaming attention's CTAs (9 KB, 16 K registers each) that
 // follow take places beside this kernel's -- two, with the registers its launch bounds leave -- and wait there instead of
 // being started when it ends; the ring still holds most of a CTA's weights.  One new token over 32768 cached ones, us:
-// 43.7 with all of an SM's shared memory, 37.2 with 173 or 193 KB, 36.1 with 145 or 161.
+// 43.7 with all of an SM's shared memory, 37.9 with 173 or 193 KB, 36.8 with 145 or 161.
 constexpr int RW_HEADS_SMEM = 161 * 1024;
 constexpr int RW_BARS = 2 * RW_MAX_STAGES + 4;            // full, empty per stage; tmem_full[2], tmem_empty[2]
 constexpr int RW_TAIL = RW_BARS * 8 + 32 + RW_MAX_ROWS * 3 * 4;  // barriers, tmem pointer + abort, 1/rms, key scale, position
