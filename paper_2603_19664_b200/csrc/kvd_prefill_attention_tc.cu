@@ -89,8 +89,11 @@ __device__ __forceinline__ bool polite_wait(uint32_t bar, uint32_t parity, const
   }
   return true;
 }
-// The same for a whole warp: lane 0 waits, the result is broadcast.
+// The same for a whole warp.  Every lane asks once, and usually that is all: with lane 0 asking alone behind a branch and
+// handing the answer on, a wait for a barrier that had long completed took a softmax warp 200 to 290 clocks.  Otherwise
+// lane 0 waits, and the result is broadcast.
 __device__ __forceinline__ bool polite_warp_wait(uint32_t bar, uint32_t parity, const volatile int *abort_flag, unsigned long long timeout_ns, int lane) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
   int ok = 1;
   if (lane == 0) ok = polite_wait<false>(bar, parity, abort_flag, timeout_ns) ? 1 : 0;
   ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -99,6 +102,13 @@ __device__ __forceinline__ bool polite_warp_wait(uint32_t bar, uint32_t parity, 
 template <bool PAIR>
 __device__ __forceinline__ bool lead_wait(uint32_t bar, uint32_t parity, const volatile int *abort_flag, unsigned long long timeout_ns) {
   return polite_wait<PAIR>(bar, parity, abort_flag, timeout_ns);
+}
+
+// The kernels are programmatic dependents of what precedes them: up to here (barriers, tensor memory) they may run while it
+// ends.  Their own dependents are let in after the allocation, which waits without a limit.
+__device__ __forceinline__ void early_start_point() {
+  grid_launch_dependents();
+  grid_dependency_wait();
 }
 
 // Whether every row of a warp sees every key of a block, without the row's masks (which cost 460 of the 2380 clocks a
@@ -410,6 +420,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1) kvd_prefill_attn_tc_kernel(cons
     }
   }
   __syncthreads();
+  early_start_point();
   // ---- key positions the pair needs: from the smallest first-visible to the largest last-visible of its tokens
   if (tid < NCTA * TOK && pair_tok0 + tid < P.n_rows) {
     const int qp = P.q_pos[pair_tok0 + tid];
@@ -450,7 +461,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1) kvd_prefill_attn_tc_kernel(cons
         uint32_t r[32];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          const uint4 w = valid ? __ldg(qsrc + c * 8 + i) : make_uint4(0u, 0u, 0u, 0u);
+          const uint4 w = valid ? qsrc[c * 8 + i] : make_uint4(0u, 0u, 0u, 0u);
           r[4 * i] = w.x;
           r[4 * i + 1] = w.y;
           r[4 * i + 2] = w.z;
@@ -771,6 +782,7 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
     tmem_relinquish();
   }
   __syncthreads();
+  early_start_point();
   // ---- key positions a tile needs: from the smallest first-visible to the largest last-visible of its tokens
   if (tid < 2 * TOK && cta_tok0 + tid < P.n_rows) {
     const int qp = P.q_pos[cta_tok0 + tid];
@@ -812,7 +824,7 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
       const uint32_t qdst = q_smem + t * Cfg::Q_BYTES + row * 128;
 #pragma unroll
       for (int c = 0; c < D_HEAD / 8; ++c) {
-        const uint4 w = valid ? __ldg(qsrc + c) : make_uint4(0u, 0u, 0u, 0u);
+        const uint4 w = valid ? qsrc[c] : make_uint4(0u, 0u, 0u, 0u);
         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(qdst + (c >> 3) * Cfg::SLAB_Q + (((c & 7) ^ (row & 7)) << 4)), "r"(w.x), "r"(w.y),
                      "r"(w.z), "r"(w.w)
                      : "memory");
@@ -990,6 +1002,551 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
   }
 }
 
+// ------------------------------------------------------------------------------------------------
+// One row tile on two SMs (d_head 128 and 256), for launches whose tiles leave half of the GPU idle: then a tile's walk
+// over its keys is the launch's length.  A cluster of two CTAs shares the tile: of every four key blocks CTA 0 takes the
+// scores and weights of the first two and CTA 1 those of the last two (K blocks are loaded by the CTA that scores them),
+// the weights go to both, and each CTA sums P V of every block over its half of the channels.
+// The bits are those of the kernels above: the same blocks in the same order, an output element still is one
+// accumulator, the reference maximum still passes from block to block, and a part of the row sum (even, odd blocks) still
+// is one chain of additions, handed from one CTA to the other.
+//   TMEM  = [ O : d_head / 2 columns | S_0, S_1 | Q ]
+//   warps = 0-7 softmax (group = block parity), 8 issues S of this CTA's blocks, 9 P V of all blocks, 10 and 11 load K and
+//           V, 12-15 rescale O where a reference maximum moved (the softmax warps of the other CTA cannot do it here).
+//   P     = four blocks of weights in shared memory; the CTA that made a block copies it into the other's
+//           (4 KB per warp, counted on the barrier the product waits on).
+//   m     = a block's reference maxima go to both CTAs (eight slots); the row sums' chains go to the other CTA only.
+// Across the pair everything travels with its own byte count on the receiver's barrier (st.async, bulk copies): nobody
+// waits for a store to be performed.  A barrier that counts bytes is armed by one thread of the receiver.
+// Bound by a softmax warp's chain of latencies: about 3600 clocks for one block of four (scores 450, maximum 280, weights
+// 800 to 1000, six hand-overs).  Gemma-3-4B layer, 837 tokens on 7013: 123 -> 82 us (56 tiles on 112 SMs instead of 56);
+// clock counts led there: K and V gathered by cp.async 136 us, TMA by one warp 100, by one warp each 89.
+template <int D_HEAD>
+struct PsCfg {
+  static constexpr int THREADS = 512, V_COLS = D_HEAD / 2;
+  static constexpr int SLAB_K = PT_KEYS * 128, SLAB_V = PT_KEYS * 128;
+  static constexpr int TILE_K = PT_KEYS * D_HEAD * 2, TILE_V = PT_KEYS * V_COLS * 2;
+  static constexpr int SLOTS_K = D_HEAD == 256 ? 3 : 5, SLOTS_V = D_HEAD == 256 ? 3 : 6, SLOTS = SLOTS_K + SLOTS_V;
+  static constexpr int P_SLOTS = 4, P_BYTES = PT_ROWS * PT_KEYS * 2;
+  static constexpr int M_SLOTS = 8;
+  static constexpr int COL_O = 0, COL_S = D_HEAD / 2, COL_Q = COL_S + 2 * PT_KEYS;
+  static constexpr int COLS = D_HEAD == 256 ? 512 : 256;
+  // full, empty | s_full[2] s_free[2] q_ready o_full | p_ready[4] | pv_done[8] scaled[8] | m[8][4] | chain[2][4] sum[2][4]
+  // (Eight of what a block's maxima run ahead of: they may be seven blocks ahead of the products, and a barrier's phase can
+  // only be told from the one before it.)
+  static constexpr int N_BARS = 2 * SLOTS + 6 + 4 + 16 + 32 + 16;
+  static constexpr int RINGS = SLOTS_K * TILE_K + SLOTS_V * TILE_V;
+  static constexpr int SMEM_BYTES = 1024 + RINGS + P_SLOTS * P_BYTES + N_BARS * 8;
+  static_assert(COL_Q + D_HEAD / 2 <= COLS && SMEM_BYTES + 9 * 1024 + 512 <= 232448, "does not fit");
+};
+
+// Maps of the segments' K and V rows (segment s: 2 s and 2 s + 1), boxes of 64 channels x 64 keys.
+struct PsMaps {
+  CUtensorMap map[2 * KVD_MAX_SEGMENTS];
+};
+
+// A loader warp: n blocks of K (IS_V false) or V of the walk, the t-th of them block_of(t), into the ring of `slots` tiles
+// at `ring`; of V the channels from v_col on.  A block inside one segment is fetched by TMA: the rings are short, and what
+// counts is that a free slot's bytes are under way at once (with 16-byte cp.async from two warps the scores waited for K
+// blocks 83 % of the time, with one warp loading both by TMA still 70 %).  A block across segments, or with positions
+// nobody holds, is gathered.
+template <class Cfg, int D_HEAD, bool IS_V, class BlockOf>
+__device__ __forceinline__ void ps_load_blocks(const PrefillParams &P, const PsMaps &maps, uint32_t ring, uint32_t bar_base, int blk0, int n, int kvh,
+                                               int v_col, const BlockOf &block_of, int lane, volatile int *s_abort, unsigned long long tmo) {
+  constexpr int slots = IS_V ? Cfg::SLOTS_V : Cfg::SLOTS_K, tile = IS_V ? Cfg::TILE_V : Cfg::TILE_K, cols = IS_V ? Cfg::V_COLS : D_HEAD;
+  const int col0 = kvh * D_HEAD + (IS_V ? v_col : 0);
+  bool ok = true;
+  for (int t = 0; t < n; ++t) {
+    const int slot = t % slots;
+    const uint32_t full = bar_base + 8u * ((IS_V ? Cfg::SLOTS_K : 0) + slot), empty = full + 8u * Cfg::SLOTS;
+    if (t >= slots && !polite_warp_wait(empty, ((t / slots) - 1) & 1, s_abort, tmo, lane)) {
+      ok = false;
+      break;
+    }
+    const uint32_t dst = ring + slot * tile;
+    const int pos0 = (blk0 + block_of(t)) * PT_KEYS;
+    int whole = -1;
+#pragma unroll
+    for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg)
+      if (P.first[sg] <= pos0 && pos0 + PT_KEYS <= P.first[sg] + P.len[sg]) whole = sg;
+    if (whole >= 0) {
+      if (elect_one()) {
+        mbar_arrive_expect_tx(full, tile);
+        const CUtensorMap *map = &maps.map[2 * whole + (IS_V ? 1 : 0)];
+#pragma unroll
+        for (int c = 0; c < cols; c += 64) tma_load_2d(dst + (c >> 6) * (PT_KEYS * 128), map, full, col0 + c, pos0 - P.first[whole]);
+      }
+      __syncwarp();
+      continue;
+    }
+#pragma unroll 1
+    for (int i = lane; i < PT_KEYS * (cols / 8); i += 32) {  // 16-byte pieces
+      const int r = i / (cols / 8), c = i % (cols / 8), pos = pos0 + r;
+      const __nv_bfloat16 *src = P.q;
+      bool have = false;
+#pragma unroll
+      for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg) {
+        const int rr = pos - P.first[sg];
+        if (rr >= 0 && rr < P.len[sg]) {
+          src = (IS_V ? P.v[sg] : P.k[sg]) + static_cast<size_t>(rr) * P.stride[sg] + col0 + c * 8;
+          have = true;
+        }
+      }
+      cp_async16(dst + (c >> 3) * (PT_KEYS * 128) + r * 128 + (((c & 7) ^ (r & 7)) << 4), src, have);
+    }
+    cp_async_wait_all();
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(full);
+  }
+  if (!ok) {
+    raise(P.status, STATUS_TIMEOUT, s_abort);
+    // copies may still be in flight: a bounded time that exceeds any load's latency by orders of magnitude
+    const unsigned long long t0 = globaltimer_ns();
+    while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
+  }
+}
+
+template <int D_HEAD, int G, int DT>
+__global__ void __launch_bounds__(PsCfg<D_HEAD>::THREADS, 1)
+    kvd_prefill_attn_split_kernel(const __grid_constant__ PrefillParams P, const __grid_constant__ PsMaps maps) {
+  using Cfg = PsCfg<D_HEAD>;
+  constexpr int TOK = PT_ROWS / G, HALF = D_HEAD / 2;
+  constexpr int SLOTS = Cfg::SLOTS, SLOTS_K = Cfg::SLOTS_K, SLOTS_V = Cfg::SLOTS_V;
+  extern __shared__ uint8_t pt_smem_raw[];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_abort_i, s_lo, s_hi;
+  __shared__ float s_m[Cfg::M_SLOTS][PT_ROWS];                // reference maximum after a block
+  __shared__ __align__(16) uint4 s_chain[2][PT_ROWS];         // a part of the row sum after the other CTA's block
+  __shared__ float s_sum[2][PT_ROWS];                         // the parts, referred to the last maximum
+  volatile int *s_abort = &s_abort_i;
+  const uint32_t ring = (smem_u32(pt_smem_raw) + 1023u) & ~1023u, ring_v = ring + SLOTS_K * Cfg::TILE_K;
+  const uint32_t p_smem = ring + Cfg::RINGS, bar_base = p_smem + Cfg::P_SLOTS * Cfg::P_BYTES;
+  auto bar = [&](int i) { return bar_base + 8u * static_cast<uint32_t>(i); };
+  auto bar_full = [&](int v, int s) { return bar(v * SLOTS_K + s); };
+  auto bar_empty = [&](int v, int s) { return bar(SLOTS + v * SLOTS_K + s); };
+  constexpr int B0 = 2 * SLOTS;
+  auto bar_s_full = [&](int b) { return bar(B0 + b); };
+  auto bar_s_free = [&](int b) { return bar(B0 + 2 + b); };
+  const uint32_t bar_q_ready = bar(B0 + 4), bar_o_full = bar(B0 + 5);
+  auto bar_p_ready = [&](int j) { return bar(B0 + 6 + (j & 3)); };
+  auto bar_pv_done = [&](int j) { return bar(B0 + 10 + (j & 7)); };  // both CTAs' products with the block
+  auto bar_scaled = [&](int j) { return bar(B0 + 18 + (j & 7)); };   // O is ready for the block
+  auto bar_m = [&](int j, int q) { return bar(B0 + 26 + (j & 7) * 4 + q); };
+  auto bar_chain = [&](int g, int q) { return bar(B0 + 58 + g * 4 + q); };
+  auto bar_sum = [&](int g, int q) { return bar(B0 + 66 + g * 4 + q); };
+
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int rank = static_cast<int>(cluster_ctarank());
+  const uint32_t other = static_cast<uint32_t>(rank ^ 1);
+  // start order as above: late tokens first, for every tile all KV heads before the next shorter one
+  const int n_tiles = static_cast<int>(gridDim.x) / (2 * P.n_kv), slot_id = static_cast<int>(blockIdx.x) / 2;
+  const int kvh = slot_id % P.n_kv;
+  const int tok0 = (n_tiles - 1 - slot_id / P.n_kv) * TOK;
+  const unsigned long long tmo = P.timeout_ns;
+  auto owner = [](int j) { return (j >> 1) & 1; };  // the CTA that scores block j
+
+  if (tid == 0) {
+    for (int s = 0; s < SLOTS; ++s) {
+      mbar_init(bar_full(0, s), 1);   // the loader's lane, and the block's bytes where TMA brings them
+      mbar_init(bar_empty(0, s), 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(bar_s_full(b), 1);
+      mbar_init(bar_s_free(b), 4);
+    }
+    mbar_init(bar_q_ready, 8);
+    mbar_init(bar_o_full, 1);
+    for (int s = 0; s < 4; ++s) {
+      mbar_init(bar_p_ready(s), owner(s) == rank ? 4 : 1);  // its four warps here, or the arming thread and 16 KB
+    }
+    for (int s = 0; s < 8; ++s) {
+      mbar_init(bar_pv_done(s), 2);
+      mbar_init(bar_scaled(s), 4);
+    }
+    for (int i = 0; i < 32 + 16; ++i) mbar_init(bar(B0 + 26 + i), 1);
+    fence_mbar_init();
+    s_abort_i = 0;
+    s_lo = INT_MAX;
+    s_hi = -1;
+  }
+  if (warp == 8) {
+    tmem_alloc(smem_u32(&s_tmem), Cfg::COLS);
+    tmem_relinquish();
+  }
+  __syncthreads();
+  early_start_point();
+  if (tid < TOK && tok0 + tid < P.n_rows) {
+    const int qp = P.q_pos[tok0 + tid];
+    int lo = P.window > 0 ? qp - P.window + 1 : 0;
+    lo = lo < P.seg_lo ? P.seg_lo : lo;
+    const int hi = qp < P.seg_hi ? qp : P.seg_hi;
+    if (hi >= lo) {
+      atomicMin(&s_lo, lo);
+      atomicMax(&s_hi, hi);
+    }
+  }
+  tc_fence_before();
+  cluster_sync_all();
+  tc_fence_after();
+  const uint32_t tmem_base = s_tmem;
+  const int blk0 = s_hi >= 0 ? s_lo / PT_KEYS : 0;
+  const int n_blk = s_hi >= 0 ? s_hi / PT_KEYS - blk0 + 1 : 0;
+  const int last4 = (n_blk & 3) - 2 * rank, n_own = (n_blk >> 2) * 2 + (last4 < 0 ? 0 : last4 > 2 ? 2 : last4);  // blocks this CTA scores
+  auto own_block = [&](int t) { return 4 * (t >> 1) + 2 * rank + (t & 1); };
+  auto warp_wait2 = [&](uint32_t b, uint32_t parity) -> bool { return polite_warp_wait(b, parity, s_abort, tmo, lane); };
+  auto m_at = [&](int j, int row) { return smem_u32(&s_m[j & 7][row]); };
+
+  if (warp < 8) {
+    // ------------------------------------------------------------------ softmax and epilogue: thread = MMA row
+    const int wg = warp >> 2, q4 = warp & 3;
+    const int row = q4 * 32 + lane;
+    const int tok = tok0 + row / G, g = row % G;
+    const bool valid = row / G < TOK && tok < P.n_rows;
+    const int qp = valid ? P.q_pos[tok] : -1;
+    const int lo = P.window > 0 ? qp - P.window + 1 : 0;
+    const uint32_t lane_field = static_cast<uint32_t>(q4 * 32) << 16;
+    const size_t row_off = (static_cast<size_t>(valid ? tok : 0) * P.n_q + kvh * G + (valid ? g : 0)) * D_HEAD;
+    if (n_blk > 0) {
+      const uint4 *qsrc = reinterpret_cast<const uint4 *>(P.q + row_off);
+#pragma unroll 1
+      for (int c = wg; c < D_HEAD / 64; c += 2) {
+        uint32_t r[32];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const uint4 w = valid ? qsrc[c * 8 + i] : make_uint4(0u, 0u, 0u, 0u);
+          r[4 * i] = w.x;
+          r[4 * i + 1] = w.y;
+          r[4 * i + 2] = w.z;
+          r[4 * i + 3] = w.w;
+        }
+        tmem_st_x32(tmem_base + lane_field + Cfg::COL_Q + c * 32, r);
+      }
+      tmem_wait_st();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_q_ready);
+    }
+    const uint32_t chain_bar = bar_chain(wg, q4);
+    if (lane == 0) mbar_arrive_expect_tx(chain_bar, 512);
+    uint32_t chain_ph = 0;
+    float m_own = -CUDART_INF_F;
+    uint64_t l2[2] = {0ull, 0ull};
+    bool ok = true, have_part = false;  // have_part: this group took the last block of its parity
+    const uint64_t c2 = pack2(P.scale_log2e, P.scale_log2e), one2 = pack2(1.0f, 1.0f);
+    PtWhole whole_block(valid, lo, qp);
+    for (int j = 2 * rank + wg; j < n_blk; j += 4) {
+      if (!polite_warp_wait(bar_s_full(wg), (j >> 2) & 1, s_abort, tmo, lane)) {
+        raise(P.status, STATUS_TIMEOUT, s_abort);
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t s_col = tmem_base + lane_field + Cfg::COL_S + wg * PT_KEYS;
+      uint32_t s0[32], s1[32];
+      tmem_ld_x32(s_col, s0);
+      tmem_ld_x32(s_col + 32, s1);
+      const bool whole = whole_block(P, (blk0 + j) * PT_KEYS);  // (warp-uniform)
+      unsigned long long vis = ~0ull;
+      if (!whole) vis = pt_visible(P, (blk0 + j) * PT_KEYS, lo, qp);
+      tmem_wait_ld();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_s_free(wg));
+      const float bm = pt_mask_max(s0, s1, whole, vis) * P.scale_log2e;
+      float m_prev = -CUDART_INF_F;
+      if (j > 0) {
+        if (!warp_wait2(bar_m(j - 1, q4), ((j - 1) >> 3) & 1)) {
+          raise(P.status, STATUS_TIMEOUT, s_abort);
+          ok = false;
+          break;
+        }
+        m_prev = s_m[(j - 1) & 7][row];
+      }
+      const float m_new = m_prev == -CUDART_INF_F ? bm : (bm > m_prev + PT_TAU ? bm : m_prev);
+      s_m[j & 7][row] = m_new;
+      st_async_f32(map_to_cta(m_at(j, row), other), map_to_cta(bar_m(j, q4), other), m_new);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_m(j, q4));
+      const float m_use = m_new == -CUDART_INF_F ? 0.f : m_new;
+      // both CTAs' products with the weights that were in this slot have finished
+      if (j >= 4 && !warp_wait2(bar_pv_done(j - 4), ((j - 4) >> 3) & 1)) {
+        raise(P.status, STATUS_TIMEOUT, s_abort);
+        ok = false;
+        break;
+      }
+      const uint64_t nm2 = pack2(-m_use, -m_use);
+      const uint32_t p_slot = p_smem + (j & 3) * Cfg::P_BYTES, prow = p_slot + row * 128;
+      auto weights = [&](uint32_t (&s)[32], int chunk0) {  // in fp32 over the scores, rounded into the slot
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          uint32_t w[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int k = 8 * c + 2 * i;
+            float e0, e1;
+            unpack2(ffma2(pack2(__uint_as_float(s[k]), __uint_as_float(s[k + 1])), c2, nm2), e0, e1);
+            const float p0 = ex2_approx(e0), p1 = ex2_approx(e1);
+            w[i] = pack_out<DT>(p0, p1);
+            s[k] = __float_as_uint(p0);
+            s[k + 1] = __float_as_uint(p1);
+          }
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(prow + (((chunk0 + c) ^ (row & 7)) << 4)), "r"(w[0]), "r"(w[1]), "r"(w[2]),
+                       "r"(w[3])
+                       : "memory");
+        }
+      };
+      weights(s0, 0);
+      weights(s1, 4);
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(bar_p_ready(j));
+        const uint32_t piece = p_slot + q4 * 4096;
+        bulk_copy_to_cta(map_to_cta(piece, other), piece, 4096, map_to_cta(bar_p_ready(j), other));
+      }
+      // the row sum's part: the chain of block j - 2, which the other CTA took, and its reference
+      if (j >= 2) {
+        const uint32_t m_bar = bar_m(j - 2, q4), m_ph = ((j - 2) >> 3) & 1;
+        const bool both = mbar_try_wait(chain_bar, chain_ph) && mbar_try_wait(m_bar, m_ph);
+        if (!__all_sync(0xffffffffu, both) && (!warp_wait2(chain_bar, chain_ph) || !warp_wait2(m_bar, m_ph))) {
+          raise(P.status, STATUS_TIMEOUT, s_abort);
+          ok = false;
+          break;
+        }
+        chain_ph ^= 1u;
+        const uint4 c = s_chain[wg][row];
+        l2[0] = pack2(__uint_as_float(c.x), __uint_as_float(c.y));
+        l2[1] = pack2(__uint_as_float(c.z), __uint_as_float(c.w));
+        m_own = s_m[(j - 2) & 7][row];
+        __syncwarp();
+        if (lane == 0) mbar_arrive_expect_tx(chain_bar, 512);
+      }
+      const float alpha_own = m_own == -CUDART_INF_F ? 1.0f : ex2_approx(m_own - m_use);
+      m_own = m_new;
+      const uint64_t al2 = pack2(alpha_own, alpha_own);
+      l2[0] = fmul2(l2[0], al2);
+      l2[1] = fmul2(l2[1], al2);
+#pragma unroll
+      for (int k = 0; k < 32; k += 2) l2[(k >> 1) & 1] = ffma2(pack2(__uint_as_float(s0[k]), __uint_as_float(s0[k + 1])), one2, l2[(k >> 1) & 1]);
+#pragma unroll
+      for (int k = 0; k < 32; k += 2) l2[(k >> 1) & 1] = ffma2(pack2(__uint_as_float(s1[k]), __uint_as_float(s1[k + 1])), one2, l2[(k >> 1) & 1]);
+      have_part = j + 2 >= n_blk;
+      if (!have_part) {
+        float a0, a1, a2, a3;
+        unpack2(l2[0], a0, a1);
+        unpack2(l2[1], a2, a3);
+        st_async_v4(map_to_cta(smem_u32(&s_chain[wg][row]), other), map_to_cta(chain_bar, other), __float_as_uint(a0), __float_as_uint(a1),
+                    __float_as_uint(a2), __float_as_uint(a3));
+      }
+    }
+    // ---- the row sum: both parts referred to the final maximum, added in group order
+    float l_run = 0.f;
+    if (ok && n_blk > 0) {
+      const int last = n_blk - 1;
+      if (!warp_wait2(bar_m(last, q4), (last >> 3) & 1)) {
+        raise(P.status, STATUS_TIMEOUT, s_abort);
+        ok = false;
+      }
+      if (ok && wg <= last) {
+        if (have_part) {
+          const float m_fin = s_m[last & 7][row], m_use = m_fin == -CUDART_INF_F ? 0.f : m_fin;
+          const float part = pt_row_sum(l2, m_own == -CUDART_INF_F ? 1.0f : ex2_approx(m_own - m_use));
+          s_sum[wg][row] = part;
+          st_async_f32(map_to_cta(smem_u32(&s_sum[wg][row]), other), map_to_cta(bar_sum(wg, q4), other), part);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_sum(wg, q4));
+        } else if (lane == 0) {
+          mbar_arrive_expect_tx(bar_sum(wg, q4), 128);
+        }
+      }
+      if (ok && (!warp_wait2(bar_sum(0, q4), 0) || (last > 0 && !warp_wait2(bar_sum(1, q4), 0)))) {
+        raise(P.status, STATUS_TIMEOUT, s_abort);
+        ok = false;
+      }
+      if (ok) l_run = s_sum[0][row] + (last > 0 ? s_sum[1][row] : 0.f);
+    }
+    // ---- normalise and store this CTA's channels, each group its pieces of 32
+    if (ok && n_blk > 0 && !polite_warp_wait(bar_o_full, 0, s_abort, tmo, lane)) {
+      raise(P.status, STATUS_TIMEOUT, s_abort);
+      ok = false;
+    }
+    if (ok) {
+      tc_fence_after();
+      const float inv = l_run > 0.f ? 1.0f / l_run : 0.f;
+      uint4 *dst = reinterpret_cast<uint4 *>(P.out + row_off + rank * HALF);
+#pragma unroll 1
+      for (int c = wg; c < HALF / 32; c += 2) {
+        uint32_t r[32];
+        if (n_blk > 0) {
+          tmem_ld_x32(tmem_base + lane_field + Cfg::COL_O + c * 32, r);
+          tmem_wait_ld();
+        } else {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) r[i] = 0u;
+        }
+        uint32_t o[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) o[i] = pack_out<DT>(__uint_as_float(r[2 * i]) * inv, __uint_as_float(r[2 * i + 1]) * inv);
+        if (valid) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) dst[c * 4 + i] = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+        }
+      }
+    } else {
+      // copies of this warp may still be on their way into the other CTA (which stays until the barrier below)
+      const unsigned long long t0 = globaltimer_ns();
+      while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
+    }
+  } else if (warp == 8 || warp == 9) {
+    // ------------------------------------------------------------------ MMA issue (one thread per product)
+    constexpr uint32_t IDESC_BASE = (DT == 0 ? umma_idesc_bf16_f32(PT_ROWS, 8) : umma_idesc_f16_f32(PT_ROWS, 8)) & ~(1u << 17);
+    constexpr uint32_t IDESC_S = IDESC_BASE | (static_cast<uint32_t>(PT_KEYS >> 3) << 17);            // N = 64 keys, B K-major
+    constexpr uint32_t IDESC_O = IDESC_BASE | (static_cast<uint32_t>(HALF >> 3) << 17) | (1u << 16);  // N = d_head / 2, B MN-major
+    if (warp == 8 && n_own > 0 && elect_one()) {
+      bool ok = polite_wait<false>(bar_q_ready, 0, s_abort, tmo);
+      tc_fence_after();
+      for (int t = 0; ok && t < n_own; ++t) {
+        const int slot = t % SLOTS_K;
+        if (!polite_wait<false>(bar_full(0, slot), (t / SLOTS_K) & 1, s_abort, tmo) ||
+            (t >= 2 && !polite_wait<false>(bar_s_free(t & 1), ((t - 2) >> 1) & 1, s_abort, tmo))) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t d = tmem_base + Cfg::COL_S + (t & 1) * PT_KEYS;
+        const uint64_t desc0 = umma_smem_desc_sw128(ring + slot * Cfg::TILE_K);
+#pragma unroll
+        for (int ks = 0; ks < D_HEAD / 16; ++ks)
+          umma_f16_ts(d, tmem_base + Cfg::COL_Q + ks * 8, desc0 + (((ks >> 2) * Cfg::SLAB_K + (ks & 3) * 32) >> 4), IDESC_S, ks > 0 ? 1u : 0u);
+        umma_commit(bar_empty(0, slot));
+        umma_commit(bar_s_full(t & 1));
+      }
+      if (!ok) raise(P.status, STATUS_TIMEOUT, s_abort);
+    } else if (warp == 9 && n_blk > 0 && elect_one()) {
+      bool ok = true;
+      for (int s = 0; s < 4; ++s)
+        if (owner(s) != rank) mbar_arrive_expect_tx(bar_p_ready(s), Cfg::P_BYTES);
+      for (int j = 0; j < n_blk; ++j) {
+        const int slot = j % SLOTS_V;
+        if (!polite_wait<false>(bar_scaled(j), (j >> 3) & 1, s_abort, tmo) || !polite_wait<false>(bar_p_ready(j), (j >> 2) & 1, s_abort, tmo) ||
+            !polite_wait<false>(bar_full(1, slot), (j / SLOTS_V) & 1, s_abort, tmo)) {
+          ok = false;
+          break;
+        }
+        if (owner(j) != rank) mbar_arrive_expect_tx(bar_p_ready(j), Cfg::P_BYTES);  // for block j + 4
+        tc_fence_after();
+        const uint64_t desc0 = umma_smem_desc_sw128_mn(ring_v + slot * Cfg::TILE_V, Cfg::SLAB_V);
+        const uint64_t pdesc0 = umma_smem_desc_sw128(p_smem + (j & 3) * Cfg::P_BYTES);
+#pragma unroll
+        for (int ks = 0; ks < PT_KEYS / 16; ++ks)
+          umma_bf16(tmem_base + Cfg::COL_O, pdesc0 + ((ks * 32) >> 4), desc0 + ((ks * 16 * 128) >> 4), IDESC_O, (j > 0 || ks > 0) ? 1u : 0u);
+        umma_commit(bar_empty(1, slot));
+        umma_commit_mask(bar_pv_done(j), 3);
+      }
+      if (ok) umma_commit(bar_o_full);
+      // the other CTA's last commits have arrived here before this one may leave
+      for (int j = n_blk > 4 ? n_blk - 4 : 0; ok && j < n_blk; ++j) ok = polite_wait<true>(bar_pv_done(j), (j >> 3) & 1, s_abort, tmo);
+      if (!ok) raise(P.status, STATUS_TIMEOUT, s_abort);
+    }
+  } else if (warp < 12) {
+    if (warp == 10) ps_load_blocks<Cfg, D_HEAD, false>(P, maps, ring, bar_base, blk0, n_own, kvh, 0, own_block, lane, s_abort, tmo);
+    else ps_load_blocks<Cfg, D_HEAD, true>(P, maps, ring_v, bar_base, blk0, n_blk, kvh, rank * HALF, [](int t) { return t; }, lane, s_abort, tmo);
+  } else {
+    // ------------------------------------------------------------------ O follows the reference maxima
+    const int q4 = warp & 3, row = q4 * 32 + lane;
+    const uint32_t o_col = tmem_base + (static_cast<uint32_t>(q4 * 32) << 16) + Cfg::COL_O;
+    if (lane == 0)
+      for (int j = 0; j < 8; ++j)
+        if (owner(j) != rank) mbar_arrive_expect_tx(bar_m(j, q4), 128);
+    float m_prev = -CUDART_INF_F;
+    for (int j = 0; j < n_blk; ++j) {
+      if (!warp_wait2(bar_m(j, q4), (j >> 3) & 1)) {
+        raise(P.status, STATUS_TIMEOUT, s_abort);
+        break;
+      }
+      if (lane == 0 && owner(j) != rank) mbar_arrive_expect_tx(bar_m(j, q4), 128);  // for block j + 8
+      const float m_new = s_m[j & 7][row], m_use = m_new == -CUDART_INF_F ? 0.f : m_new;
+      const float alpha = m_prev == -CUDART_INF_F ? 1.0f : ex2_approx(m_prev - m_use);
+      m_prev = m_new;
+      if (__any_sync(0xffffffffu, alpha != 1.0f)) {
+        if (!warp_wait2(bar_pv_done(j - 1), ((j - 1) >> 3) & 1)) {
+          raise(P.status, STATUS_TIMEOUT, s_abort);
+          break;
+        }
+        tc_fence_after();
+        pt_rescale<HALF>(o_col, alpha);
+        tc_fence_before();
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_scaled(j));
+    }
+  }
+  // ---- nobody leaves while the other CTA can still write into its shared memory
+  tc_fence_before();
+  cluster_sync_all();
+  if (warp == 8) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, Cfg::COLS);
+  }
+}
+
+template <typename... K, typename... A>
+static kvd_status prefill_launch(kvd_ctx *ctx, void (*kern)(K...), unsigned grid, unsigned threads, size_t smem, unsigned cluster, cudaStream_t stream,
+                                 const A &...args) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(grid, 1, 1);
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = (serial_launch_mask() & 8) ? 0 : 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "launch prefill attention");
+  ctx->launches += 1;
+  return KVD_OK;
+}
+
+template <int D_HEAD, int G>
+static kvd_status prefill_split_launch(kvd_ctx *ctx, const PrefillParams &P, cudaStream_t stream) {
+  using Cfg = PsCfg<D_HEAD>;
+  auto k0 = kvd_prefill_attn_split_kernel<D_HEAD, G, 0>;
+  auto k1 = kvd_prefill_attn_split_kernel<D_HEAD, G, 1>;
+  static bool configured[64] = {};
+  if (!configured[ctx->device & 63]) {
+    cudaError_t e = cudaFuncSetAttribute(k0, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(prefill attention)");
+    configured[ctx->device & 63] = true;
+  }
+  PsMaps maps;
+  memset(&maps, 0, sizeof(maps));
+  for (int i = 0; i < 2 * KVD_MAX_SEGMENTS; ++i) {
+    const int sg = i / 2;
+    if (P.len[sg] < PT_KEYS) continue;  // no block lies inside it
+    cuuint64_t dims[2] = {static_cast<cuuint64_t>(P.n_kv) * D_HEAD, static_cast<cuuint64_t>(P.len[sg])};
+    cuuint64_t strides[1] = {static_cast<cuuint64_t>(P.stride[sg]) * 2};
+    cuuint32_t box[2] = {64, PT_KEYS}, estr[2] = {1, 1};
+    CUresult r = ctx->encode(&maps.map[i], ctx->dtype == 1 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+                             const_cast<__nv_bfloat16 *>(i % 2 ? P.v[sg] : P.k[sg]), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) {
+      ctx->last_error = "cuTensorMapEncodeTiled (segments) failed: " + std::to_string(static_cast<int>(r));
+      return KVD_ERR_CUDA;
+    }
+  }
+  const int tok = PT_ROWS / G;
+  return prefill_launch(ctx, ctx->dtype == 1 ? k1 : k0, 2 * ((P.n_rows + tok - 1) / tok) * P.n_kv, Cfg::THREADS, Cfg::SMEM_BYTES, 2, stream, P, maps);
+}
+
 template <int D_HEAD, int G>
 static kvd_status prefill_dual_launch(kvd_ctx *ctx, const PrefillParams &P, cudaStream_t stream) {
   using Cfg = PdCfg<D_HEAD>;
@@ -1004,12 +1561,7 @@ static kvd_status prefill_dual_launch(kvd_ctx *ctx, const PrefillParams &P, cuda
   }
   const int tok = 2 * (PT_ROWS / G);
   const unsigned grid = static_cast<unsigned>((P.n_rows + tok - 1) / tok * P.n_kv);
-  if (ctx->dtype == 1) k1<<<grid, Cfg::THREADS, Cfg::SMEM_BYTES, stream>>>(P);
-  else k0<<<grid, Cfg::THREADS, Cfg::SMEM_BYTES, stream>>>(P);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "launch prefill attention");
-  ctx->launches += 1;
-  return KVD_OK;
+  return prefill_launch(ctx, ctx->dtype == 1 ? k1 : k0, grid, Cfg::THREADS, Cfg::SMEM_BYTES, 1, stream, P);
 }
 
 template <int D_HEAD, int G, bool PAIR>
@@ -1027,23 +1579,7 @@ static kvd_status prefill_tc_launch(kvd_ctx *ctx, const PrefillParams &P, cudaSt
   const int tok = PT_ROWS / G;
   int tiles = (P.n_rows + tok - 1) / tok;
   if (PAIR) tiles = (tiles + 1) & ~1;  // whole pairs: a CTA whose tile lies past the last row has no rows to store
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3(tiles * P.n_kv, 1, 1);
-  cfg.blockDim = dim3(PT_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = Cfg::SMEM_BYTES;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = PAIR ? 2 : 1;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = ctx->dtype == 1 ? cudaLaunchKernelEx(&cfg, k1, P) : cudaLaunchKernelEx(&cfg, k0, P);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "launch prefill attention");
-  ctx->launches += 1;
-  return KVD_OK;
+  return prefill_launch(ctx, ctx->dtype == 1 ? k1 : k0, tiles * P.n_kv, PT_THREADS, Cfg::SMEM_BYTES, PAIR ? 2 : 1, stream, P);
 }
 
 // Time a launch of CTAs of `tok` tokens would take: a CTA costs `per_cta` + `per_block` for every key block it walks, the
@@ -1086,6 +1622,22 @@ static bool prefill_dual_pays(const kvd_ctx *ctx, const PrefillParams &P, int gr
   return prefill_estimate(ctx, P, 2 * tok, 10.4f, 1.07f) < prefill_estimate(ctx, P, tok, 6.0f, 0.74f);
 }
 
+// One tile on two CTAs: where every tile gets its own pair of SMs (beyond that the pairs would take turns) and the walk is
+// long enough to pay for the second CTA's set-up.  Call alone, us, one tile per CTA or pair of tiles per pair / one tile on
+// two CTAs, Gemma-3-4B layer: 16 tokens 7.5 / 10.9, 16 on 200 (4 blocks) 10.1 / 11.5, 290 13.2 / 12.1, 64 on 400 (8 blocks)
+// 16.5 / 15.7, 64 on 1000 23.9 / 18.6, 600 18.5 / 14.6, 290 on 4000 66.6 / 41.2, 1100 on 4000 (72 tiles) 78.2 / 49.7;
+// Qwen3-4B layer: 150 (3 blocks) 7.8 / 8.3, 64 on 400 11.7 / 10.4, 150 on 1000 18.7 / 15.0, 16 on 4000 49.5 / 31.4.
+// (The positions are on the device; the host assumes the usual call, whose last row sits at the last key.)
+static bool prefill_split_pays(const kvd_ctx *ctx, const PrefillParams &P, int group) {
+  constexpr int LEAST_BLOCKS = 6;
+  const int tok = PT_ROWS / group;
+  const long long tiles = static_cast<long long>((P.n_rows + tok - 1) / tok) * P.n_kv;
+  if (2 * tiles > ctx->num_sms) return false;
+  int first = P.window > 0 ? P.seg_hi - (P.n_rows < tok ? P.n_rows : tok) - P.window + 1 : P.seg_lo;
+  first = first < P.seg_lo ? P.seg_lo : first;
+  return P.seg_hi / PT_KEYS - first / PT_KEYS + 1 >= LEAST_BLOCKS;
+}
+
 template <int D_HEAD>
 static kvd_status prefill_tc_group(kvd_ctx *ctx, const PrefillParams &P, int group, cudaStream_t stream) {
   // pairs where the K/V bytes per block bound the kernel (d_head = 256); at 128 the softmax does, and the hand-overs
@@ -1093,6 +1645,16 @@ static kvd_status prefill_tc_group(kvd_ctx *ctx, const PrefillParams &P, int gro
   static const char *env = getenv("KVD_PREFILL_PAIR");
   const bool pair = D_HEAD >= 128 && (env ? env[0] == '1' : D_HEAD == 256);
   if constexpr (D_HEAD >= 128) {
+    if (prefill_split_pays(ctx, P, group)) {
+      switch (group) {
+        case 1: return prefill_split_launch<D_HEAD, 1>(ctx, P, stream);
+        case 2: return prefill_split_launch<D_HEAD, 2>(ctx, P, stream);
+        case 3: return prefill_split_launch<D_HEAD, 3>(ctx, P, stream);
+        case 4: return prefill_split_launch<D_HEAD, 4>(ctx, P, stream);
+        case 8: return prefill_split_launch<D_HEAD, 8>(ctx, P, stream);
+        default: return KVD_ERR_SHAPE;
+      }
+    }
     if (pair) {
       switch (group) {
         case 1: return prefill_tc_launch<D_HEAD, 1, true>(ctx, P, stream);

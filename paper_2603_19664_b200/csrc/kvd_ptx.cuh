@@ -303,6 +303,30 @@ __device__ __forceinline__ void st_cluster_f32(uint32_t cluster_addr, float v) {
 __device__ __forceinline__ void st_cluster_v4(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
+// Stores into another CTA's shared memory that count their bytes on one of that CTA's barriers (both addresses from
+// map_to_cta): the data and the news of it travel together, and the storing thread waits for nothing.
+__device__ __forceinline__ void st_async_f32(uint32_t cluster_addr, uint32_t cluster_bar, float v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(cluster_addr), "r"(__float_as_uint(v)),
+               "r"(cluster_bar)
+               : "memory");
+}
+__device__ __forceinline__ void st_async_v4(uint32_t cluster_addr, uint32_t cluster_bar, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(cluster_addr), "r"(a),
+               "r"(b), "r"(c), "r"(d), "r"(cluster_bar)
+               : "memory");
+}
+// `bytes` (a multiple of 16, both addresses 16-byte aligned) of this CTA's shared memory into another CTA's.  What the
+// threads wrote there has to be fenced for the async proxy first.
+__device__ __forceinline__ void bulk_copy_to_cta(uint32_t cluster_dst, uint32_t src, uint32_t bytes, uint32_t cluster_bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(cluster_dst), "r"(src),
+               "r"(bytes), "r"(cluster_bar)
+               : "memory");
+}
+// umma_commit, arriving on the barrier at this offset in every CTA of the mask.
+__device__ __forceinline__ void umma_commit_mask(uint32_t bar, uint16_t cta_mask) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"(cta_mask)
+               : "memory");
+}
 // TMEM management and MMA for a pair of CTAs (cta_group::2).  alloc / dealloc / relinquish are
 // executed by the same warp index in both CTAs; the MMA and its commits by one thread of the
 // even-ranked CTA only.
