@@ -1,4 +1,4 @@
-"""ctypes binding of ``libkvd.so`` -- argument marshalling only.
+"""Binding of ``libkvd.so`` -- argument marshalling only (ctypes; the hot calls in C, ``_kvdcall``).
 
 Every function here has the name of the C entry point it calls (``include/kvd.h``) and does nothing
 but convert Python / torch objects to pointers and sizes.  K/V recomputation and attention run
@@ -100,16 +100,23 @@ class KvdError(RuntimeError):
 
 
 _lib: Optional[ctypes.CDLL] = None
+_calls = None  # the C half of the binding: the calls of a decode step without ctypes (csrc/kvd_pycall.c)
+_CALLS = ("kvd_reset_sequence", "kvd_checkpoint_residual", "kvd_recompute_kv", "kvd_recompute_kv_step", "kvd_decode_step_kv",
+          "kvd_decode_attention", "kvd_prefill_attention")
 
 
 def load() -> ctypes.CDLL:
     """Load libkvd.so (built by ``paper_2603_19664_b200.build``); raises if it is missing."""
-    global _lib
+    global _lib, _calls
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
         raise RuntimeError(f"{LIB_PATH} not found: build it with `python -m paper_2603_19664_b200.build` "
                            "(there is no fallback path)")
+    try:
+        from . import _kvdcall
+    except ImportError as e:
+        raise RuntimeError("_kvdcall.so not found or not loadable: build it with `python -m paper_2603_19664_b200.build`") from e
     lib = ctypes.CDLL(LIB_PATH)
     vp, i32, i64, sz = ctypes.c_void_p, ctypes.c_int, ctypes.c_int64, ctypes.c_size_t
     lib.kvd_create.argtypes = [ctypes.POINTER(kvd_model_desc), ctypes.POINTER(vp)]
@@ -245,7 +252,9 @@ def load() -> ctypes.CDLL:
     lib.kvd_scaffold_embed.restype = i32
     lib.kvd_scaffold_argmax.argtypes = [vp, vp, i64, i32, i32, vp, vp]
     lib.kvd_scaffold_argmax.restype = i32
-    _lib = lib
+    for name in _CALLS:
+        _kvdcall.bind(name, ctypes.cast(getattr(lib, name), vp).value)
+    _lib, _calls = lib, _kvdcall
     return lib
 
 
@@ -396,7 +405,11 @@ def kvd_decode_attention_static(n_q_heads: int, n_kv_heads: int, d_head: int, sl
 
 
 class Kvd:
-    """One library context.  Method names mirror the C entry points."""
+    """One library context.  Method names mirror the C entry points.
+
+    The calls of a decode step go through ``_kvdcall``, which marshals plain arguments in C and answers -1, before it has
+    called anything, for all others: those are marshalled here, by ctypes.  A step over 512 tokens of a SmolLM2 layer (four
+    calls, 18.8 us of GPU work): 28.5 us by ctypes alone."""
 
     def __init__(self, desc: kvd_model_desc):
         self._lib = load()
@@ -406,12 +419,13 @@ class Kvd:
         if st != KVD_OK:
             raise KvdError(st, "kvd_create")
         self._h = h
+        self._addr = h.value
         self._keep: List[object] = []  # tensors the context borrows (store arena, workspace)
 
     def close(self) -> None:
         if getattr(self, "_h", None):
             self._lib.kvd_destroy(self._h)
-            self._h = None
+            self._h = self._addr = None
 
     def __del__(self):
         try:
@@ -439,14 +453,20 @@ class Kvd:
                     "kvd_attach_workspace")
 
     def kvd_reset_sequence(self, seq: int) -> None:
-        self._check(self._lib.kvd_reset_sequence(self._h, seq), "kvd_reset_sequence")
+        st = _calls.kvd_reset_sequence(self._addr, seq)
+        if st < 0:
+            st = self._lib.kvd_reset_sequence(self._h, seq)
+        self._check(st, "kvd_reset_sequence")
 
     def kvd_rows_stored(self, layer: int, seq: int) -> int:
         return int(self._lib.kvd_rows_stored(self._h, layer, seq))
 
     def kvd_checkpoint_residual(self, seq: int, layer: int, rows, positions, n: int, stream=None) -> None:
-        self._check(self._lib.kvd_checkpoint_residual(self._h, seq, layer, _ptr(rows), _ptr(positions), n,
-                                                      _stream(stream)), "kvd_checkpoint_residual")
+        stream = _stream(stream)
+        st = _calls.kvd_checkpoint_residual(self._addr, seq, layer, rows, positions, n, stream)
+        if st < 0:
+            st = self._lib.kvd_checkpoint_residual(self._h, seq, layer, _ptr(rows), _ptr(positions), n, stream)
+        self._check(st, "kvd_checkpoint_residual")
 
     def kvd_checkpoint_residual_step(self, layer: int, seqs: Sequence[int], rows, positions, stream=None) -> None:
         arr = (ctypes.c_int32 * max(len(seqs), 1))(*[int(s) for s in seqs])
@@ -455,33 +475,46 @@ class Kvd:
 
     def kvd_recompute_kv(self, layer: int, rows, positions, n: int, k_out, v_out, out_row_stride: int, seq: int = 0,
                          first_row: int = 0, stream=None) -> None:
-        self._check(self._lib.kvd_recompute_kv(self._h, layer, _ptr(rows), _ptr(positions), n, seq, first_row,
-                                               _ptr(k_out), _ptr(v_out), out_row_stride, _stream(stream)),
-                    "kvd_recompute_kv")
+        stream = _stream(stream)
+        st = _calls.kvd_recompute_kv(self._addr, layer, rows, positions, n, k_out, v_out, out_row_stride, seq, first_row, stream)
+        if st < 0:
+            st = self._lib.kvd_recompute_kv(self._h, layer, _ptr(rows), _ptr(positions), n, seq, first_row, _ptr(k_out), _ptr(v_out),
+                                            out_row_stride, stream)
+        self._check(st, "kvd_recompute_kv")
 
     def kvd_recompute_kv_step(self, layer: int, ranges: Sequence[Tuple[int, int, int, object, object]], rows,
                               positions, n_rows: int, k_rows_out, v_rows_out, out_row_stride: int, stream=None) -> None:
         """ranges: (seq, first_row, n, k_out, v_out) per sequence; rows/positions: the new tokens (or None, 0)."""
-        arr = _marshal_ranges(ranges)
-        self._check(self._lib.kvd_recompute_kv_step(self._h, layer, arr, len(ranges), _ptr(rows), _ptr(positions),
-                                                    n_rows, _ptr(k_rows_out), _ptr(v_rows_out), out_row_stride,
-                                                    _stream(stream)), "kvd_recompute_kv_step")
+        stream = _stream(stream)
+        st = _calls.kvd_recompute_kv_step(self._addr, layer, ranges, rows, positions, n_rows, k_rows_out, v_rows_out, out_row_stride, stream)
+        if st < 0:
+            arr = _marshal_ranges(ranges)
+            st = self._lib.kvd_recompute_kv_step(self._h, layer, arr, len(ranges), _ptr(rows), _ptr(positions), n_rows, _ptr(k_rows_out),
+                                                 _ptr(v_rows_out), out_row_stride, stream)
+        self._check(st, "kvd_recompute_kv_step")
 
     def kvd_decode_step_kv(self, layer: int, ranges: Sequence[Tuple[int, int, int, object, object]], out_row_stride: int,
                            rows, positions, n_rows: int, append_seqs: Optional[Sequence[int]], k_rows_out, v_rows_out,
                            rows_out_row_stride: int, stream=None) -> None:
         """ranges as for kvd_recompute_kv_step; append_seqs: the sequence slot each new row is appended to, or None."""
-        arr = _marshal_ranges(ranges)
-        seqs = None if append_seqs is None else (ctypes.c_int32 * max(len(append_seqs), 1))(*[int(x) for x in append_seqs])
-        self._check(self._lib.kvd_decode_step_kv(self._h, layer, arr, len(ranges), out_row_stride, _ptr(rows),
-                                                 _ptr(positions), n_rows, seqs, _ptr(k_rows_out), _ptr(v_rows_out),
-                                                 rows_out_row_stride, _stream(stream)), "kvd_decode_step_kv")
+        stream = _stream(stream)
+        st = _calls.kvd_decode_step_kv(self._addr, layer, ranges, out_row_stride, rows, positions, n_rows, append_seqs, k_rows_out, v_rows_out,
+                                       rows_out_row_stride, stream)
+        if st < 0:
+            arr = _marshal_ranges(ranges)
+            seqs = None if append_seqs is None else (ctypes.c_int32 * max(len(append_seqs), 1))(*[int(x) for x in append_seqs])
+            st = self._lib.kvd_decode_step_kv(self._h, layer, arr, len(ranges), out_row_stride, _ptr(rows), _ptr(positions), n_rows, seqs,
+                                              _ptr(k_rows_out), _ptr(v_rows_out), rows_out_row_stride, stream)
+        self._check(st, "kvd_decode_step_kv")
 
     def kvd_decode_attention(self, layer: int, batch: int, q, q_pos: Sequence[int],
                              segs: Sequence[Sequence[Segment]], scale: float, out, stream=None) -> None:
-        n_segs, pos_arr, seg_arr = _marshal_segments(batch, q_pos, segs)
-        self._check(self._lib.kvd_decode_attention(self._h, layer, batch, _ptr(q), pos_arr, seg_arr, n_segs,
-                                                   float(scale), _ptr(out), _stream(stream)), "kvd_decode_attention")
+        stream = _stream(stream)
+        st = _calls.kvd_decode_attention(self._addr, layer, batch, q, q_pos, segs, scale, out, stream)
+        if st < 0:
+            n_segs, pos_arr, seg_arr = _marshal_segments(batch, q_pos, segs)
+            st = self._lib.kvd_decode_attention(self._h, layer, batch, _ptr(q), pos_arr, seg_arr, n_segs, float(scale), _ptr(out), stream)
+        self._check(st, "kvd_decode_attention")
 
     def kvd_decode_attention_rows(self, layer: int, n_rows: int, q, q_pos: Sequence[int], segs: Sequence[Segment],
                                   scale: float, out, stream=None) -> None:
@@ -495,9 +528,12 @@ class Kvd:
     def kvd_prefill_attention(self, layer: int, n_rows: int, q, q_pos_dev, segs: Sequence[Segment], scale: float, out,
                               stream=None) -> None:
         """Many query rows of one sequence in one launch; q_pos_dev: int32 device tensor [n_rows]."""
-        n_segs, _, seg_arr = _marshal_segments(1, [0], [list(segs)])
-        self._check(self._lib.kvd_prefill_attention(self._h, layer, n_rows, _ptr(q), _ptr(q_pos_dev), seg_arr, n_segs,
-                                                    float(scale), _ptr(out), _stream(stream)), "kvd_prefill_attention")
+        stream = _stream(stream)
+        st = _calls.kvd_prefill_attention(self._addr, layer, n_rows, q, q_pos_dev, segs, scale, out, stream)
+        if st < 0:
+            n_segs, _, seg_arr = _marshal_segments(1, [0], [list(segs)])
+            st = self._lib.kvd_prefill_attention(self._h, layer, n_rows, _ptr(q), _ptr(q_pos_dev), seg_arr, n_segs, float(scale), _ptr(out), stream)
+        self._check(st, "kvd_prefill_attention")
 
     def kvd_decode_attention_recompute(self, layer: int, batch: int, q, q_pos: Sequence[int],
                                        ranges: Sequence[Tuple[int, int, int]], rows, positions, n_rows: int,

@@ -3,7 +3,7 @@
 Compiles every ``csrc/*.cu`` for sm_100a with nvcc into ``libkvd.so`` next to this file.  The CUDA
 runtime is linked statically and the driver API is reached through ``cudaGetDriverEntryPoint``, so
 the library also loads on a machine without a GPU driver (where every entry point that needs a
-device reports an error).
+device reports an error).  ``_kvdcall.so``, beside it, marshals the arguments of the hot calls (csrc/kvd_pycall.c).
 """
 from __future__ import annotations
 
@@ -11,11 +11,13 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libkvd.so")
 LIB_CHECK = os.path.join(HERE, "libkvd_check.so")  # the same sources with -DKVD_CHECK (device-side index tests)
+CALLS = os.path.join(HERE, "_kvdcall.so")  # argument marshalling of the hot calls (csrc/kvd_pycall.c)
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC",
          "--expt-relaxed-constexpr"]
@@ -38,10 +40,22 @@ def needs_build(check: bool = False) -> bool:
     return any(os.path.getmtime(p) > t for p in _deps())
 
 
+def build_calls(force: bool = False) -> str:
+    """Compile the C half of the Python binding (gcc; no CUDA in it)."""
+    src = os.path.join(CSRC, "kvd_pycall.c")
+    deps = [src, os.path.join(os.path.dirname(HERE), "include", "kvd.h")]
+    if force or not os.path.exists(CALLS) or any(os.path.getmtime(p) > os.path.getmtime(CALLS) for p in deps):
+        tmp = CALLS + f".tmp{os.getpid()}"
+        subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-o", tmp, src], check=True)
+        os.replace(tmp, CALLS)
+    return CALLS
+
+
 def build(force: bool = False, verbose: bool = False, check: bool = False) -> str:
     """Compile libkvd.so, or with ``check`` libkvd_check.so: the build whose kernels test the indices they
     derive on the device and report through the status word instead of accessing out of range."""
     LIB = LIB_CHECK if check else globals()["LIB"]
+    build_calls(force)
     if not force and not needs_build(check):
         return LIB
     objdir = os.path.join(HERE, "build", "check") if check else os.path.join(HERE, "build")
