@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1) kvd_prefill_attn_tc_kernel(cons
 // for the scores) about a third of the time.  Here each group has a tile of its own, so nothing is exchanged, a K or V
 // block is loaded once for 256 rows, and each tile's next scores are there before its softmax asks for them.  A CTA
 // takes longer per block than above (1950 against 1550 clocks, for twice the rows), hence only where there are enough
-// of them (prefill_dual_pays).  4096 tokens of a Qwen3-4B layer 207 -> 162 us, 16384 2783 -> 2030 us.
+// of them (prefill_dual_pays).  One / two tiles per CTA, Qwen3-4B layer: 4096 tokens 198 / 151 us.
 //   TMEM = [ O_0, O_1 : d_head columns each | S_00, S_01, S_10, S_11 : 64 columns each (tile, block parity) ]; the
 //          weights of a block overwrite the first half of its scores.  The query tiles are in shared memory.
 //   warps = 0-3 tile 0, 4-7 tile 1, 8 and 9 the products of tiles 0 and 1, 10 and 11 loaders: twelve warps leave a
@@ -1019,8 +1019,9 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
 // Across the pair everything travels with its own byte count on the receiver's barrier (st.async, bulk copies): nobody
 // waits for a store to be performed.  A barrier that counts bytes is armed by one thread of the receiver.
 // Bound by a softmax warp's chain of latencies: about 3600 clocks for one block of four (scores 450, maximum 280, weights
-// 800 to 1000, six hand-overs).  Gemma-3-4B layer, 837 tokens on 7013: 123 -> 82 us (56 tiles on 112 SMs instead of 56);
-// clock counts led there: K and V gathered by cp.async 136 us, TMA by one warp 100, by one warp each 89.
+// 800 to 1000, six hand-overs).  Gemma-3-4B layer, 837 tokens on 7013, call alone: 123 -> 72.5 us (56 tiles on 112 SMs
+// instead of 56).  Clock counts by phase led there: K and V gathered by cp.async 136 us, TMA by one warp 100, by one warp
+// each 89, cheaper waits 81, and the early start.
 template <int D_HEAD>
 struct PsCfg {
   static constexpr int THREADS = 512, V_COLS = D_HEAD / 2;
@@ -1608,11 +1609,12 @@ static float prefill_estimate(const kvd_ctx *ctx, const PrefillParams &P, int to
 
 // Two tiles per CTA (d_head 128) or one.  Two serve more rows per clock but walk a block more slowly, so a call whose
 // longest tiles set its time wants one, and one that keeps every SM busy for several rounds wants two.  Up to one round
-// of single tiles: one.  Beyond four rounds: two.  Between: by estimate; the costs (us) are fitted to 102 launches of 1 to
-// 27 rounds with groups of 1 to 8, windows of 0, 128 and 1024 and 0 to 7000 earlier keys (5 % rms).  One / two tiles per
-// CTA, us: 32 query on 8 KV heads, 600 tokens 14.9 / 21.9, 600 on 7000 176 / 140, 1300 36.1 / 34.0, 2500 93 / 81, 4096
-// 206 / 162; 16 on 8, 1300 23.3 / 32.4, 2500 52.0 / 53.5, 4096 104 / 81; 4 on 1, 8000 99 / 145.  Two tiles whenever there is
-// more than one round, as it was before, cost up to 1.5 times the time.  At d_head 64 the products are too short for two
+// of single tiles: one.  Beyond four rounds: two.  Between: by estimate; the costs (us) were fitted to 102 launches of 1 to
+// 27 rounds with groups of 1 to 8, windows of 0, 128 and 1024 and 0 to 7000 earlier keys (5 % rms), before the waits of
+// both kernels became cheaper; the choices are right for what they cost now.  One / two tiles per CTA, us: 32 query on 8 KV
+// heads, 600 tokens 13.4 / 19.6, 600 on 7000 169 / 134, 1300 33.8 / 31.2, 2500 89 / 75, 4096 198 / 151; 16 on 8, 1300 20.8 /
+// 29.5, 1300 on 4000 106 / 97, 2500 49.0 / 49.6, 4096 101 / 75; 4 on 1, 8000 100 / 140, 8000 on 4000 180 / 205.  Two tiles
+// whenever there is more than one round cost up to 1.5 times the time.  At d_head 64 the products are too short for two
 // tiles: 294 tiles of a SmolLM2 layer 58 / 72 us.
 static bool prefill_dual_pays(const kvd_ctx *ctx, const PrefillParams &P, int group) {
   const int tok = PT_ROWS / group;
