@@ -74,9 +74,10 @@ struct PtCfg {
 
 // A wait of this kernel.  Every SM sub-partition hosts a warp of either softmax group, a loader warp and possibly an MMA
 // thread, and at any time some of them wait: a short sleep between polls leaves the issue slots to the warps that
-// compute (+2 to 7 %).  In a pair
-// the arrivals may come from the partner CTA and publish what its threads wrote to its own shared memory, so the
-// acquire is at cluster scope there.
+// compute (+2 to 7 %).  CLUSTER: the barrier may be completed by the partner CTA, by its threads' arrivals or by bytes that
+// it sends (st.async, bulk copies).  Both release at cluster scope, and only an acquire of that scope synchronises with
+// them.  (A commit of the pair's products needs none: what it announces lies in this CTA's tensor memory or rings and is
+// ordered by tcgen05.fence.)
 template <bool CLUSTER>
 __device__ __forceinline__ bool polite_wait(uint32_t bar, uint32_t parity, const volatile int *abort_flag, unsigned long long timeout_ns) {
   auto done = [&]() { return CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity); };
@@ -92,11 +93,13 @@ __device__ __forceinline__ bool polite_wait(uint32_t bar, uint32_t parity, const
 // The same for a whole warp.  Every lane asks once, and usually that is all: with lane 0 asking alone behind a branch and
 // handing the answer on, a wait for a barrier that had long completed took a softmax warp 200 to 290 clocks.  Otherwise
 // lane 0 waits, and the result is broadcast.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool polite_warp_wait(uint32_t bar, uint32_t parity, const volatile int *abort_flag, unsigned long long timeout_ns, int lane) {
-  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  if (__all_sync(0xffffffffu, CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity))) return true;
   int ok = 1;
-  if (lane == 0) ok = polite_wait<false>(bar, parity, abort_flag, timeout_ns) ? 1 : 0;
+  if (lane == 0) ok = polite_wait<CLUSTER>(bar, parity, abort_flag, timeout_ns) ? 1 : 0;
   ok = __shfl_sync(0xffffffffu, ok, 0);
+  __syncwarp();  // the other lanes' reads follow lane 0's acquire
   return ok != 0;
 }
 template <bool PAIR>
@@ -1195,7 +1198,8 @@ __global__ void __launch_bounds__(PsCfg<D_HEAD>::THREADS, 1)
   const int n_blk = s_hi >= 0 ? s_hi / PT_KEYS - blk0 + 1 : 0;
   const int last4 = (n_blk & 3) - 2 * rank, n_own = (n_blk >> 2) * 2 + (last4 < 0 ? 0 : last4 > 2 ? 2 : last4);  // blocks this CTA scores
   auto own_block = [&](int t) { return 4 * (t >> 1) + 2 * rank + (t & 1); };
-  auto warp_wait2 = [&](uint32_t b, uint32_t parity) -> bool { return polite_warp_wait(b, parity, s_abort, tmo, lane); };
+  // waits on what the other CTA completes, alone or in turn with this one
+  auto peer_wait = [&](uint32_t b, uint32_t parity) -> bool { return polite_warp_wait<true>(b, parity, s_abort, tmo, lane); };
   auto m_at = [&](int j, int row) { return smem_u32(&s_m[j & 7][row]); };
 
   if (warp < 8) {
@@ -1257,7 +1261,7 @@ __global__ void __launch_bounds__(PsCfg<D_HEAD>::THREADS, 1)
       const float bm = pt_mask_max(s0, s1, whole, vis) * P.scale_log2e;
       float m_prev = -CUDART_INF_F;
       if (j > 0) {
-        if (!warp_wait2(bar_m(j - 1, q4), ((j - 1) >> 3) & 1)) {
+        if (!peer_wait(bar_m(j - 1, q4), ((j - 1) >> 3) & 1)) {
           raise(P.status, STATUS_TIMEOUT, s_abort);
           ok = false;
           break;
@@ -1271,7 +1275,7 @@ __global__ void __launch_bounds__(PsCfg<D_HEAD>::THREADS, 1)
       if (lane == 0) mbar_arrive(bar_m(j, q4));
       const float m_use = m_new == -CUDART_INF_F ? 0.f : m_new;
       // both CTAs' products with the weights that were in this slot have finished
-      if (j >= 4 && !warp_wait2(bar_pv_done(j - 4), ((j - 4) >> 3) & 1)) {
+      if (j >= 4 && !peer_wait(bar_pv_done(j - 4), ((j - 4) >> 3) & 1)) {
         raise(P.status, STATUS_TIMEOUT, s_abort);
         ok = false;
         break;
@@ -1309,8 +1313,8 @@ __global__ void __launch_bounds__(PsCfg<D_HEAD>::THREADS, 1)
       // the row sum's part: the chain of block j - 2, which the other CTA took, and its reference
       if (j >= 2) {
         const uint32_t m_bar = bar_m(j - 2, q4), m_ph = ((j - 2) >> 3) & 1;
-        const bool both = mbar_try_wait(chain_bar, chain_ph) && mbar_try_wait(m_bar, m_ph);
-        if (!__all_sync(0xffffffffu, both) && (!warp_wait2(chain_bar, chain_ph) || !warp_wait2(m_bar, m_ph))) {
+        const bool both = mbar_try_wait_cluster(chain_bar, chain_ph) && mbar_try_wait_cluster(m_bar, m_ph);
+        if (!__all_sync(0xffffffffu, both) && (!peer_wait(chain_bar, chain_ph) || !peer_wait(m_bar, m_ph))) {
           raise(P.status, STATUS_TIMEOUT, s_abort);
           ok = false;
           break;
@@ -1345,7 +1349,7 @@ __global__ void __launch_bounds__(PsCfg<D_HEAD>::THREADS, 1)
     float l_run = 0.f;
     if (ok && n_blk > 0) {
       const int last = n_blk - 1;
-      if (!warp_wait2(bar_m(last, q4), (last >> 3) & 1)) {
+      if (!peer_wait(bar_m(last, q4), (last >> 3) & 1)) {
         raise(P.status, STATUS_TIMEOUT, s_abort);
         ok = false;
       }
@@ -1361,7 +1365,7 @@ __global__ void __launch_bounds__(PsCfg<D_HEAD>::THREADS, 1)
           mbar_arrive_expect_tx(bar_sum(wg, q4), 128);
         }
       }
-      if (ok && (!warp_wait2(bar_sum(0, q4), 0) || (last > 0 && !warp_wait2(bar_sum(1, q4), 0)))) {
+      if (ok && (!peer_wait(bar_sum(0, q4), 0) || (last > 0 && !peer_wait(bar_sum(1, q4), 0)))) {
         raise(P.status, STATUS_TIMEOUT, s_abort);
         ok = false;
       }
@@ -1430,7 +1434,7 @@ __global__ void __launch_bounds__(PsCfg<D_HEAD>::THREADS, 1)
         if (owner(s) != rank) mbar_arrive_expect_tx(bar_p_ready(s), Cfg::P_BYTES);
       for (int j = 0; j < n_blk; ++j) {
         const int slot = j % SLOTS_V;
-        if (!polite_wait<false>(bar_scaled(j), (j >> 3) & 1, s_abort, tmo) || !polite_wait<false>(bar_p_ready(j), (j >> 2) & 1, s_abort, tmo) ||
+        if (!polite_wait<false>(bar_scaled(j), (j >> 3) & 1, s_abort, tmo) || !polite_wait<true>(bar_p_ready(j), (j >> 2) & 1, s_abort, tmo) ||
             !polite_wait<false>(bar_full(1, slot), (j / SLOTS_V) & 1, s_abort, tmo)) {
           ok = false;
           break;
@@ -1462,7 +1466,7 @@ __global__ void __launch_bounds__(PsCfg<D_HEAD>::THREADS, 1)
         if (owner(j) != rank) mbar_arrive_expect_tx(bar_m(j, q4), 128);
     float m_prev = -CUDART_INF_F;
     for (int j = 0; j < n_blk; ++j) {
-      if (!warp_wait2(bar_m(j, q4), (j >> 3) & 1)) {
+      if (!peer_wait(bar_m(j, q4), (j >> 3) & 1)) {
         raise(P.status, STATUS_TIMEOUT, s_abort);
         break;
       }
@@ -1471,7 +1475,7 @@ __global__ void __launch_bounds__(PsCfg<D_HEAD>::THREADS, 1)
       const float alpha = m_prev == -CUDART_INF_F ? 1.0f : ex2_approx(m_prev - m_use);
       m_prev = m_new;
       if (__any_sync(0xffffffffu, alpha != 1.0f)) {
-        if (!warp_wait2(bar_pv_done(j - 1), ((j - 1) >> 3) & 1)) {
+        if (!peer_wait(bar_pv_done(j - 1), ((j - 1) >> 3) & 1)) {
           raise(P.status, STATUS_TIMEOUT, s_abort);
           break;
         }

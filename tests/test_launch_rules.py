@@ -86,3 +86,17 @@ def test_kernels_that_derive_store_slots_or_tiles_test_them_in_the_checking_buil
     body = KERNELS["kvd_rows_kernel"][1]
     for index in ("append_slot[r]", "col0"):
         assert re.search(r"KVD_BOUNDS_OK\([^;]*" + re.escape(index), body), index
+
+
+def test_waits_on_what_the_other_cta_completes_acquire_at_cluster_scope():
+    """st.async and bulk copies between the CTAs of a cluster release at cluster scope; a CTA-scope acquire does not
+    synchronise with them, and no run shows that."""
+    body = KERNELS["kvd_prefill_attn_split_kernel"][1]
+    waits = re.findall(r"(\w*wait\w*(?:<\w+>)?)\(\s*(?:bar_(m|chain|sum|pv_done|p_ready)\(|(chain|m)_bar)", body)
+    assert {a or b for _, a, b in waits} == {"m", "chain", "sum", "pv_done", "p_ready"} and len(waits) >= 12
+    assert {f for f, _, _ in waits} <= {"peer_wait", "polite_wait<true>", "mbar_try_wait_cluster"}, waits
+    assert "polite_warp_wait<true>" in body[body.index("auto peer_wait"):].split(";")[0]
+    helper = TEXT["kvd_prefill_attention_tc.cu"]
+    helper = helper[helper.index("bool polite_warp_wait("):]
+    helper = helper[:helper.index("\n}")]
+    assert "CLUSTER ? mbar_try_wait_cluster" in helper and "polite_wait<CLUSTER>" in helper
