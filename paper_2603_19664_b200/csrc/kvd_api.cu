@@ -932,7 +932,7 @@ static kvd_status build_attn_launch(kvd_ctx *ctx, const LayerState &ls, int b0, 
       }
     }
     S.q_pos = q_pos[b];
-    int lo = ls.window > 0 ? S.q_pos - ls.window + 1 : 0;
+    int lo = first_visible(S.q_pos, ls.window);
     if (lo < 0) lo = 0;
     if (min_first > lo) lo = min_first;
     int hi = S.q_pos < max_last ? S.q_pos : max_last;
@@ -1100,7 +1100,7 @@ extern "C" kvd_status kvd_decode_attention_recompute(kvd_ctx *ctx, int layer, in
   for (int b = 0; b < batch; ++b) {
     att[b].q = static_cast<const __nv_bfloat16 *>(q) + static_cast<size_t>(b) * d.n_q_heads * d.d_head;
     att[b].q_pos = q_pos[b];
-    att[b].lo_pos = ls.window > 0 && q_pos[b] - ls.window + 1 > 0 ? q_pos[b] - ls.window + 1 : 0;
+    att[b].lo_pos = first_visible(q_pos[b], ls.window);
     att[b].part_base = L.seq[b].merge_base;
     att[b].reserved = 0;
   }
@@ -1152,7 +1152,7 @@ extern "C" kvd_status kvd_decode_attention_recompute_fp8_rows(kvd_ctx *ctx, int 
     all[b] = ranges[b];
     att[b].q = static_cast<const __nv_bfloat16 *>(q) + static_cast<size_t>(b) * d.n_q_heads * d.d_head;
     att[b].q_pos = q_pos[b];
-    att[b].lo_pos = ls.window > 0 && q_pos[b] - ls.window + 1 > 0 ? q_pos[b] - ls.window + 1 : 0;
+    att[b].lo_pos = first_visible(q_pos[b], ls.window);
     att[b].part_base = L.seq[b].merge_base;
     att[b].reserved = 0;
   }

@@ -145,8 +145,8 @@ __global__ void __launch_bounds__(AT_THREADS, ALLIN ? 2 : AT_CTAS_PER_SM) kvd_at
   int fast_seg = -1;
 #pragma unroll
   for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg)
-    if (chunk_pos0 >= S.first[sg] && chunk_pos0 + chunk_keys <= S.first[sg] + S.len[sg]) fast_seg = sg;
-  const bool fast = fast_seg >= 0 && chunk_pos0 >= S.lo_pos && chunk_pos0 + chunk_keys - 1 <= S.hi_pos;
+    if (segment_holds(S.first[sg], S.len[sg], chunk_pos0, chunk_keys)) fast_seg = sg;
+  const bool fast = fast_seg >= 0 && chunk_pos0 >= S.lo_pos && chunk_keys - 1 <= S.hi_pos - chunk_pos0;
   const __nv_bfloat16 *fk = P.q, *fv = P.q;
   long long fstride = 0;
   if (fast) {
@@ -434,8 +434,8 @@ __global__ void __launch_bounds__(AT_THREADS, AT_CTAS_PER_SM)
   int fast_seg = -1;
 #pragma unroll
   for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg)
-    if (chunk_pos0 >= S.first[sg] && chunk_pos0 + chunk_keys <= S.first[sg] + S.len[sg]) fast_seg = sg;
-  const bool fast = fast_seg >= 0 && chunk_pos0 >= S.lo_pos && chunk_pos0 + chunk_keys - 1 <= S.hi_pos;
+    if (segment_holds(S.first[sg], S.len[sg], chunk_pos0, chunk_keys)) fast_seg = sg;
+  const bool fast = fast_seg >= 0 && chunk_pos0 >= S.lo_pos && chunk_keys - 1 <= S.hi_pos - chunk_pos0;
   const __nv_bfloat16 *fk = P.q, *fv = P.q;
   long long fstride = 0;
   if (fast) {
@@ -948,7 +948,7 @@ extern "C" kvd_status kvd_decode_attention_static(int n_q_heads, int n_kv_heads,
       }
     }
     S.q_pos = q_pos[b];
-    int lo = sliding_window > 0 ? S.q_pos - sliding_window + 1 : 0;
+    int lo = first_visible(S.q_pos, sliding_window);
     if (lo < 0) lo = 0;
     if (min_first > lo) lo = min_first;
     const int hi = S.q_pos < max_last ? S.q_pos : max_last;

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "../../include/kvd.h"
+#include "kvd_positions.h"
 
 namespace kvd {
 

@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(128) kvd_prefill_attn_kernel(const __grid_cons
   // ---- key positions the tile needs: from the smallest first-visible to the largest last-visible of its tokens
   if (tid < TOK && tok0 + tid < P.n_rows) {
     const int qp = P.q_pos[tok0 + tid];
-    int lo = P.window > 0 ? qp - P.window + 1 : 0;
+    int lo = first_visible(qp, P.window);
     lo = lo < P.seg_lo ? P.seg_lo : lo;
     const int hi = qp < P.seg_hi ? qp : P.seg_hi;
     if (hi >= lo) {
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(128) kvd_prefill_attn_kernel(const __grid_cons
   const int r0 = warp * 16 + (lane >> 2), r1 = r0 + 8;
   const int t0 = tok0 + r0 / GP, t1 = tok0 + r1 / GP;
   const int qp0 = t0 < P.n_rows ? P.q_pos[t0] : -1, qp1 = t1 < P.n_rows ? P.q_pos[t1] : -1;
-  const int lo0 = P.window > 0 ? qp0 - P.window + 1 : 0, lo1 = P.window > 0 ? qp1 - P.window + 1 : 0;
+  const int lo0 = first_visible(qp0, P.window), lo1 = first_visible(qp1, P.window);
   __syncthreads();
   const int blk0 = s_hi >= 0 ? s_lo / PF_BLOCK_KEYS : 0, blk1 = s_hi >= 0 ? s_hi / PF_BLOCK_KEYS : -1;
 

@@ -118,39 +118,31 @@ __device__ __forceinline__ void early_start_point() {
 // softmax warp took for a block): the block lies inside one segment and inside the range all the warp's rows see.
 // Rows that are not stored do not count.
 struct PtWhole {
-  int lo, hi;      // the range that every stored row of the warp sees
-  int seg0, seg1;  // [seg0, seg1): the segment the last block was found in
-  __device__ __forceinline__ PtWhole(bool valid, int row_lo, int row_hi) : seg0(0), seg1(0) {
+  int lo, hi;         // the range that every stored row of the warp sees
+  int seg0, seg_len;  // the segment the last block was found in
+  __device__ __forceinline__ PtWhole(bool valid, int row_lo, int row_hi) : seg0(0), seg_len(0) {
     lo = __reduce_max_sync(0xffffffffu, valid ? row_lo : INT_MIN);
     hi = __reduce_min_sync(0xffffffffu, valid ? row_hi : INT_MAX);
   }
   __device__ __forceinline__ bool operator()(const PrefillParams &P, int pos0) {
     if (pos0 < lo || pos0 + PT_KEYS - 1 > hi) return false;
-    if (pos0 < seg0 || pos0 + PT_KEYS > seg1) {
+    if (!segment_holds(seg0, seg_len, pos0, PT_KEYS)) {
 #pragma unroll
       for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg)
-        if (P.first[sg] <= pos0 && pos0 < P.first[sg] + P.len[sg]) {
+        if (segment_holds(P.first[sg], P.len[sg], pos0, 1)) {
           seg0 = P.first[sg];
-          seg1 = P.first[sg] + P.len[sg];
+          seg_len = P.len[sg];
         }
     }
-    return pos0 >= seg0 && pos0 + PT_KEYS <= seg1;
+    return segment_holds(seg0, seg_len, pos0, PT_KEYS);
   }
 };
 // Which keys of the block at pos0 does a row see: present in a segment, in [lo, qp] (bit k = key pos0 + k).
 __device__ __forceinline__ unsigned long long pt_visible(const PrefillParams &P, int pos0, int lo, int qp) {
   unsigned long long vis = 0ull;
 #pragma unroll
-  for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg) {
-    int a = P.first[sg] - pos0, b = P.first[sg] + P.len[sg] - pos0;  // [a, b) of the block's key slots
-    a = a < 0 ? 0 : a;
-    b = b > PT_KEYS ? PT_KEYS : b;
-    if (b > a) vis |= (b - a == 64 ? ~0ull : ((1ull << (b - a)) - 1ull) << a);
-  }
-  int a = lo - pos0, b = qp - pos0 + 1;
-  a = a < 0 ? 0 : a;
-  b = b > PT_KEYS ? PT_KEYS : b;
-  return vis & (b > a ? (b - a == 64 ? ~0ull : ((1ull << (b - a)) - 1ull) << a) : 0ull);
+  for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg) vis |= segment_slots(P.first[sg], P.len[sg], pos0);
+  return vis & visible_slots(lo, qp, pos0);
 }
 // Scores of invisible keys become -inf; the maximum of the 64 in four chains of three-input maxima.
 __device__ __forceinline__ float pt_mask_max(uint32_t (&s0)[32], uint32_t (&s1)[32], bool whole, unsigned long long vis) {
@@ -260,7 +252,7 @@ __device__ __forceinline__ void pt_load_blocks(const PrefillParams &P, uint32_t 
     int whole = -1;
 #pragma unroll
     for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg)
-      if (P.first[sg] <= pos_first && pos_first + ROWS <= P.first[sg] + P.len[sg]) whole = sg;
+      if (segment_holds(P.first[sg], P.len[sg], pos_first, ROWS)) whole = sg;
     if (whole >= 0) {
       const long long stride = P.stride[whole];
       const __nv_bfloat16 *src = (is_v ? P.v[whole] : P.k[whole]) + static_cast<size_t>(pos_first - P.first[whole] + r0) * stride +
@@ -427,7 +419,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1) kvd_prefill_attn_tc_kernel(cons
   // ---- key positions the pair needs: from the smallest first-visible to the largest last-visible of its tokens
   if (tid < NCTA * TOK && pair_tok0 + tid < P.n_rows) {
     const int qp = P.q_pos[pair_tok0 + tid];
-    int lo = P.window > 0 ? qp - P.window + 1 : 0;
+    int lo = first_visible(qp, P.window);
     lo = lo < P.seg_lo ? P.seg_lo : lo;
     const int hi = qp < P.seg_hi ? qp : P.seg_hi;
     if (hi >= lo) {
@@ -453,7 +445,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1) kvd_prefill_attn_tc_kernel(cons
     const int tok = tok0 + row / G, g = row % G;
     const bool valid = row / G < TOK && tok < P.n_rows;
     const int qp = valid ? P.q_pos[tok] : -1;
-    const int lo = P.window > 0 ? qp - P.window + 1 : 0;
+    const int lo = first_visible(qp, P.window);
     const uint32_t lane_field = static_cast<uint32_t>(q4 * 32) << 16;
     const size_t row_off = (static_cast<size_t>(valid ? tok : 0) * P.n_q + kvh * G + (valid ? g : 0)) * D_HEAD;
     if (n_blk > 0) {
@@ -789,7 +781,7 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
   // ---- key positions a tile needs: from the smallest first-visible to the largest last-visible of its tokens
   if (tid < 2 * TOK && cta_tok0 + tid < P.n_rows) {
     const int qp = P.q_pos[cta_tok0 + tid];
-    int lo = P.window > 0 ? qp - P.window + 1 : 0;
+    int lo = first_visible(qp, P.window);
     lo = lo < P.seg_lo ? P.seg_lo : lo;
     const int hi = qp < P.seg_hi ? qp : P.seg_hi;
     if (hi >= lo) {
@@ -816,7 +808,7 @@ __global__ void __launch_bounds__(PdCfg<D_HEAD>::THREADS, 1) kvd_prefill_attn_du
     const int tok = cta_tok0 + t * TOK + row / G, g = row % G;
     const bool valid = row / G < TOK && tok < P.n_rows;
     const int qp = valid ? P.q_pos[tok] : -1;
-    const int lo = P.window > 0 ? qp - P.window + 1 : 0;
+    const int lo = first_visible(qp, P.window);
     const int first_blk = blk0 + tile_skip(t), n = tile_blocks(t);
     const uint32_t lane_field = static_cast<uint32_t>(q4 * 32) << 16;
     const uint32_t o_col = tmem_base + lane_field + t * D_HEAD;
@@ -1072,7 +1064,7 @@ __device__ __forceinline__ void ps_load_blocks(const PrefillParams &P, const PsM
     int whole = -1;
 #pragma unroll
     for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg)
-      if (P.first[sg] <= pos0 && pos0 + PT_KEYS <= P.first[sg] + P.len[sg]) whole = sg;
+      if (segment_holds(P.first[sg], P.len[sg], pos0, PT_KEYS)) whole = sg;
     if (whole >= 0) {
       if (elect_one()) {
         mbar_arrive_expect_tx(full, tile);
@@ -1182,7 +1174,7 @@ __global__ void __launch_bounds__(PsCfg<D_HEAD>::THREADS, 1)
   early_start_point();
   if (tid < TOK && tok0 + tid < P.n_rows) {
     const int qp = P.q_pos[tok0 + tid];
-    int lo = P.window > 0 ? qp - P.window + 1 : 0;
+    int lo = first_visible(qp, P.window);
     lo = lo < P.seg_lo ? P.seg_lo : lo;
     const int hi = qp < P.seg_hi ? qp : P.seg_hi;
     if (hi >= lo) {
@@ -1209,7 +1201,7 @@ __global__ void __launch_bounds__(PsCfg<D_HEAD>::THREADS, 1)
     const int tok = tok0 + row / G, g = row % G;
     const bool valid = row / G < TOK && tok < P.n_rows;
     const int qp = valid ? P.q_pos[tok] : -1;
-    const int lo = P.window > 0 ? qp - P.window + 1 : 0;
+    const int lo = first_visible(qp, P.window);
     const uint32_t lane_field = static_cast<uint32_t>(q4 * 32) << 16;
     const size_t row_off = (static_cast<size_t>(valid ? tok : 0) * P.n_q + kvh * G + (valid ? g : 0)) * D_HEAD;
     if (n_blk > 0) {
@@ -1595,7 +1587,7 @@ static float prefill_estimate(const kvd_ctx *ctx, const PrefillParams &P, int to
   auto cost = [&](int i) {
     const int t0 = (tiles - 1 - i / P.n_kv) * tok, t1 = (t0 + tok < P.n_rows ? t0 + tok : P.n_rows) - 1;
     const int last = P.seg_hi - (P.n_rows - 1 - t1);
-    int first = P.window > 0 ? P.seg_hi - (P.n_rows - 1 - t0) - P.window + 1 : P.seg_lo;
+    int first = first_visible(P.seg_hi - (P.n_rows - 1 - t0), P.window);
     first = first < P.seg_lo ? P.seg_lo : first;
     return per_cta + per_block * static_cast<float>(last >= first ? last / PT_KEYS - first / PT_KEYS + 1 : 0);
   };
@@ -1639,7 +1631,7 @@ static bool prefill_split_pays(const kvd_ctx *ctx, const PrefillParams &P, int g
   const int tok = PT_ROWS / group;
   const long long tiles = static_cast<long long>((P.n_rows + tok - 1) / tok) * P.n_kv;
   if (2 * tiles > ctx->num_sms) return false;
-  int first = P.window > 0 ? P.seg_hi - (P.n_rows < tok ? P.n_rows : tok) - P.window + 1 : P.seg_lo;
+  int first = first_visible(P.seg_hi - (P.n_rows < tok ? P.n_rows : tok), P.window);
   first = first < P.seg_lo ? P.seg_lo : first;
   return P.seg_hi / PT_KEYS - first / PT_KEYS + 1 >= LEAST_BLOCKS;
 }
