@@ -24,9 +24,11 @@
 
 namespace kvd {
 
+// (A coherent load: the kernels are resident while their predecessor writes the new tokens' rows, and the non-coherent form
+// is for memory that nobody writes during the kernel.)
 __device__ __forceinline__ uint4 ldg_stream(const void *p) {
   uint4 r;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
                : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
                : "l"(p));
   return r;

@@ -336,9 +336,9 @@ inline int serial_launch_mask() {
 // (rows, positions, statistics, codes) it therefore reads by plain loads behind grid_dependency_wait(): no __ldg (the
 // non-coherent load is for memory that nobody writes during the kernel), and, in the kernels started by the function
 // below, no __restrict__ on an argument (it permits a load to move above the wait).  __ldg is for tables and weights,
-// which are complete before the first launch that reads them.  (Of older kernels, decode attention still streams K and V,
-// and the fused recompute kernel its queries, by non-coherent loads behind the wait: plain ones measured 80.1 -> 81.0 us
-// for a decode step of 4 x 2048 tokens, 55.0 -> 55.4 for one of 4096.)
+// which are complete before the first launch that reads them.  (Keys, values and queries as well: decode attention's
+// streaming loads cost the same without the non-coherent path, 32768 cached keys 36.7 us per step either way, 16 x 2048
+// 38.6.)
 //
 // Launch of a small kernel that calls grid_dependency_wait() before it touches memory: as a programmatic dependent of
 // its predecessor, so that its launch latency and the predecessor's end overlap (three decoder blocks at batch 1, 35

@@ -795,7 +795,7 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
               if (FUSED && attend) {
 #pragma unroll
                 for (int g = 0; g < NG; ++g) {
-                  const uint4 q0 = __ldg(qh + (g * D_HEAD + c * 16) / 8), q1 = __ldg(qh + (g * D_HEAD + c * 16) / 8 + 1);
+                  const uint4 q0 = qh[(g * D_HEAD + c * 16) / 8], q1 = qh[(g * D_HEAD + c * 16) / 8 + 1];
                   const uint32_t qw[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
 #pragma unroll
                   for (int w = 0; w < 8; ++w) sdot[g] = ffma2(x2_to_f32x2<DT>(o[w]), x2_to_f32x2<DT>(qw[w]), sdot[g]);
@@ -839,8 +839,8 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
               if (FUSED && attend) {
 #pragma unroll
                 for (int g = 0; g < NG; ++g) {
-                  const uint4 a0 = __ldg(qh + (g * D_HEAD + c * 16) / 8), a1 = __ldg(qh + (g * D_HEAD + c * 16) / 8 + 1);
-                  const uint4 b0 = __ldg(qh + (g * D_HEAD + HALF + c * 16) / 8), b1 = __ldg(qh + (g * D_HEAD + HALF + c * 16) / 8 + 1);
+                  const uint4 a0 = qh[(g * D_HEAD + c * 16) / 8], a1 = qh[(g * D_HEAD + c * 16) / 8 + 1];
+                  const uint4 b0 = qh[(g * D_HEAD + HALF + c * 16) / 8], b1 = qh[(g * D_HEAD + HALF + c * 16) / 8 + 1];
                   const uint32_t qa[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
                   const uint32_t qb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll

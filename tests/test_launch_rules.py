@@ -74,6 +74,17 @@ def test_row_statistics_are_plain_loads():
         assert not re.search(r"__ldg\([^)]*(sumsq|J\.scale|positions)", TEXT[f]), f
 
 
+def test_keys_values_and_queries_are_coherent_loads():
+    """Attention is resident while the projection writes the new tokens' keys and values, the recompute kernel while
+    something writes the queries; the non-coherent load is for memory that nobody writes during the kernel."""
+    assert ".nc" not in ALL
+    assert "__ldg" not in TEXT["kvd_attention.cu"]
+    assert not re.search(r"__ldg\(\s*q", TEXT["kvd_recompute.cu"])
+    tables = re.compile(r"__ldg\(\s*(?:src \+ i|p\.w_scale|t_lo \+|t_hi \+|p\.gamma_k \+)")  # rotation tables, prepared weights
+    for f in ("kvd_recompute.cu", "kvd_rows.cu", "kvd_prefill_attention_tc.cu", "kvd_scaffold.cu", "kvd_fp4.cu"):
+        assert len(re.findall(r"__ldg\(", TEXT[f])) == len(tables.findall(TEXT[f])), f
+
+
 def test_the_early_start_threshold_follows_the_device():
     """Which grids leave half of the SMs free is a question to the device, not a literal."""
     text = TEXT["kvd_internal.h"]
