@@ -744,13 +744,15 @@ static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t str
   // Starting early pays for launches of up to one wave (the set-up hides under the predecessor's tail);
   // a many-wave grid whose first CTAs sit on the SMs waiting slowed a short predecessor down in
   // measurements (11 us lost on a 24 us predecessor), so those are ordered plainly.
-  // Behind the few-row projection every grid does: that kernel's CTAs are resident and few, it leaves room for this one's
-  // beside them (RW_HEADS_SMEM), and it is too short for the waiting CTAs to cost what they save.  Gemma-3-4B layer, one
-  // new token per sequence, ordered plainly / started early, us per step: 16 x 2048 fp16 43.0 / 38.7, window layer 40 x
-  // 3000 56.0 / 54.2, Qwen3-4B 8 x 4000 51.9 / 49.7.
-  const bool early = S.early_start || S.total_chunks * S.n_kv <= 148 * AT_CTAS_PER_SM;
+  // Straight behind the few-row projection larger grids do as well: its CTAs are few, and it is too short for the waiting
+  // CTAs to cost what they save.  One new token per sequence, ordered plainly / started early, us per step: Gemma-3-4B layer
+  // 8 x 1000 26.6 / 21.0, 16 x 2048 42.3 / 38.2, 24 x 1000 41.0 / 36.8, 40 x 1024 50.3 / 49.6; Qwen3-4B layer 8 x 2048 36.9 /
+  // 33.6, 16 x 2048 51.5 / 49.5; SmolLM2 layer 17 x 4000 30.7 / 27.2, 64 x 2048 41.1 / 37.3.  Not the tensor-core kernel at
+  // d_head 128 behind more than RW_FEW_ROWS rows, which it slowed down at most sizes (Qwen3-4B layer 17 x 2048 55.3 / 58.3,
+  // 32 x 1000 54.0 / 58.7, 64 x 1024 90.4 / 101.3); there the merge kernel alone starts early.
+  const bool small = S.total_chunks * S.n_kv <= 148 * AT_CTAS_PER_SM;
   if (S.total_chunks > 0) {
-    attr[0].val.programmaticStreamSerializationAllowed = (early && !(serial_launch_mask() & 2)) ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = ((small || S.early_split) && !(serial_launch_mask() & 2)) ? 1 : 0;
     cfg.gridDim = dim3(S.total_chunks * S.n_kv, 1, 1);
     cfg.blockDim = dim3(AT_THREADS, 1, 1);
     if constexpr (G >= 3 && D_HEAD <= 128) {
@@ -770,7 +772,7 @@ static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t str
     }
     if (e != cudaSuccess) return e;
   }
-  attr[0].val.programmaticStreamSerializationAllowed = (early && !(serial_launch_mask() & 4)) ? 1 : 0;
+  attr[0].val.programmaticStreamSerializationAllowed = ((small || S.early_merge) && !(serial_launch_mask() & 4)) ? 1 : 0;
   // as many warps per merge CTA as the longest sequence of the launch has groups of partials
   int max_chunks = 1;
   for (int i = 0; i < S.n_seqs; ++i) max_chunks = S.seq[i].merge_count > max_chunks ? S.seq[i].merge_count : max_chunks;
@@ -788,7 +790,9 @@ static kvd_status launch_attn_impl(kvd_ctx *ctx, const AttnLaunch &L, cudaStream
     static thread_local AttnLaunchT<NSEQ> S;
     static_cast<AttnLaunchHead &>(S) = static_cast<const AttnLaunchHead &>(L);
     for (int i = 0; i < L.n_seqs; ++i) S.seq[i] = L.seq[i];
-    S.early_start = ctx->few_rows_last;
+    // straight behind the projection of the new tokens (attn_launch_pair says why; a second launch of the same call is not)
+    S.early_merge = ctx->few_rows.directly_before(ctx->launches, stream);
+    S.early_split = S.early_merge && !(G >= 3 && D_HEAD == 128 && ctx->few_rows.rows > RW_FEW_ROWS);
     // fp16 contexts (kvd_set_dtype): the same kernels reading and writing fp16
     cudaError_t e = ctx->dtype == 1 ? attn_launch_pair<D_HEAD, G, NSEQ, 1>(S, stream)
                                     : attn_launch_pair<D_HEAD, G, NSEQ, 0>(S, stream);
@@ -992,7 +996,7 @@ extern "C" kvd_status kvd_decode_attention_static(int n_q_heads, int n_kv_heads,
   L.part_o = reinterpret_cast<float *>(scratch + ml_bytes);
   L.status = nullptr;
   L.max_parts = parts;
-  L.early_start = false;
+  L.early_split = L.early_merge = false;
   switch (d_head) {
     case 64: return static_launch_d<64>(L, group, stream);
     case 128: return static_launch_d<128>(L, group, stream);

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "../../include/kvd.h"
+#include "kvd_launch_mark.h"
 #include "kvd_positions.h"
 
 namespace kvd {
@@ -197,7 +198,7 @@ struct AttnLaunchHead {
   float *part_ml;          // [parts][n_q][2]
   int *status;             // device status word (nullptr: none), used by the checking build
   int max_parts;           // slots the partial arrays hold
-  bool early_start;        // the kernels start early whatever the grid
+  bool early_split, early_merge;  // this kernel starts early whatever the grid
 };
 template <int NSEQ>
 struct AttnLaunchT : AttnLaunchHead {
@@ -315,7 +316,7 @@ struct kvd_ctx {
   unsigned long long timeout_ns = 2000000000ull;
   long long *trace = nullptr;
   size_t trace_bytes = 0;
-  bool few_rows_last = false;  // the last K/V projection launched was the few-row kernel's (a hint: it changes no result)
+  kvd::LaunchMark few_rows;  // the last launch of the few-row kernel that made keys and values
   std::string last_error;
   kvd::EncodeTiledFn encode = nullptr;
 };

@@ -946,7 +946,6 @@ static kvd_status launch_impl(kvd_ctx *ctx, const LayerState &ls, const CUtensor
   else le = cudaLaunchKernelEx(&cfg, kern, tmap_store, tmap_rows, tmap_b, tmap_b_part, p, NoFusedParams());
   if (le != cudaSuccess) return cuda_fail(ctx, le, "launch recompute");
   ctx->launches += 1;
-  if (p.k_cols > 0) ctx->few_rows_last = false;
   return KVD_OK;
 }
 

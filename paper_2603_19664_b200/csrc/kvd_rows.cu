@@ -457,6 +457,7 @@ static kvd_status launch_rows_impl(kvd_ctx *ctx, const CUtensorMap &tmap_w, cons
   cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmap_w, tmap_x, p);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "launch rows");
   ctx->launches += 1;
+  if (D_HEAD > 0) ctx->few_rows.set(ctx->launches, stream, p.n_rows);
   return KVD_OK;
 }
 
@@ -512,7 +513,6 @@ kvd_status launch_rows(kvd_ctx *ctx, const LayerState &ls, int k, RowsParams &p,
   if (st != KVD_OK) return st;
   const CUtensorMap &w = ls.tmap_rows[many ? 1 : 0];
   if (!heads) return launch_rows_impl<0, 0>(ctx, w, tmap_x, p, stream);
-  ctx->few_rows_last = true;
   const bool half = ctx->dtype == KVD_DTYPE_F16;
   switch (ctx->desc.d_head) {
     case 64: return half ? launch_rows_impl<64, 1>(ctx, w, tmap_x, p, stream) : launch_rows_impl<64, 0>(ctx, w, tmap_x, p, stream);

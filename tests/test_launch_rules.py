@@ -5,6 +5,7 @@ launch happens to overlap its neighbours in the wrong way.
 """
 import os
 import re
+import subprocess
 
 import pytest
 
@@ -111,3 +112,33 @@ def test_waits_on_what_the_other_cta_completes_acquire_at_cluster_scope():
     helper = helper[helper.index("bool polite_warp_wait("):]
     helper = helper[:helper.index("\n}")]
     assert "CLUSTER ? mbar_try_wait_cluster" in helper and "polite_wait<CLUSTER>" in helper
+
+
+MARK = r"""
+#include "kvd_launch_mark.h"
+using kvd::LaunchMark;
+int main() {
+  LaunchMark m;
+  int s1, s2;
+  if (m.directly_before(0, &s1)) return 1;            // nothing launched yet
+  m.set(7, &s1, 20);
+  if (!m.directly_before(7, &s1) || m.rows != 20) return 2;
+  if (m.directly_before(7, &s2)) return 3;            // another stream
+  if (m.directly_before(8, &s1) || m.directly_before(9, &s1)) return 4;  // another launch in between, or used up
+  m.set(9, &s2, 1);
+  return m.directly_before(9, &s2) ? 0 : 5;
+}
+"""
+
+
+def test_attention_starts_early_only_straight_behind_the_projection(tmp_path):
+    """Grids of several waves start early behind the few-row projection; behind anything else their waiting CTAs take the
+    SMs that a longer kernel needs.  What counts is the context's last launch, on this stream, not the last projection."""
+    (tmp_path / "mark.cpp").write_text(MARK)
+    subprocess.run(["g++", "-std=c++17", "-I", CSRC, "-o", str(tmp_path / "mark"), str(tmp_path / "mark.cpp")], check=True)
+    assert subprocess.run([str(tmp_path / "mark")]).returncode == 0
+    text = TEXT["kvd_attention.cu"]
+    assert "early_merge = ctx->few_rows.directly_before(ctx->launches, stream)" in text and "early_split = S.early_merge &&" in text
+    assert len(re.findall(r"few_rows\.set\(", ALL)) == 1
+    rows = TEXT["kvd_rows.cu"]
+    assert rows.index("ctx->launches += 1") < rows.index("few_rows.set(ctx->launches, stream")
