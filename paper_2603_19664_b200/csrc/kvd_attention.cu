@@ -744,12 +744,13 @@ static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t str
   // Starting early pays for launches of up to one wave (the set-up hides under the predecessor's tail);
   // a many-wave grid whose first CTAs sit on the SMs waiting slowed a short predecessor down in
   // measurements (11 us lost on a 24 us predecessor), so those are ordered plainly.
-  // Straight behind the few-row projection larger grids do as well: its CTAs are few, and it is too short for the waiting
-  // CTAs to cost what they save.  One new token per sequence, ordered plainly / started early, us per step: Gemma-3-4B layer
-  // 8 x 1000 26.6 / 21.0, 16 x 2048 42.3 / 38.2, 24 x 1000 41.0 / 36.8, 40 x 1024 50.3 / 49.6; Qwen3-4B layer 8 x 2048 36.9 /
-  // 33.6, 16 x 2048 51.5 / 49.5; SmolLM2 layer 17 x 4000 30.7 / 27.2, 64 x 2048 41.1 / 37.3.  Not the tensor-core kernel at
-  // d_head 128 behind more than RW_FEW_ROWS rows, which it slowed down at most sizes (Qwen3-4B layer 17 x 2048 55.3 / 58.3,
-  // 32 x 1000 54.0 / 58.7, 64 x 1024 90.4 / 101.3); there the merge kernel alone starts early.
+  // Straight behind the few-row projection larger grids do as well: its CTAs are few, they leave room beside them
+  // (kvd_rows_ring.h), and it is too short for the waiting CTAs to cost what they save.  One new token per sequence, ordered
+  // plainly / started early, us per step: Gemma-3-4B layer 8 x 1000 26.6 / 21.0, 16 x 2048 42.3 / 37.7, 24 x 1000 40.9 / 35.5,
+  // 40 x 1024 49.6 / 45.5, 64 x 2048 111.8 / 106.6; Qwen3-4B layer 8 x 2048 36.9 / 33.6, 16 x 2048 51.5 / 49.6; SmolLM2 layer
+  // 17 x 4000 30.7 / 27.2, 64 x 2048 41.2 / 37.3.  Behind more than RW_FEW_ROWS rows the tensor-core kernel at d_head 128 does
+  // not, only its merge kernel: plainly / both early / merge alone, Qwen3-4B layer, 17 x 1000 36.9 / 42.0 / 36.9, 32 x 1000
+  // 54.0 / 57.2 / 53.3, 64 x 2048 149.2 / 149.1 / 145.8, 17 x 2048 55.4 / 53.0 / 53.2.
   const bool small = S.total_chunks * S.n_kv <= 148 * AT_CTAS_PER_SM;
   if (S.total_chunks > 0) {
     attr[0].val.programmaticStreamSerializationAllowed = ((small || S.early_split) && !(serial_launch_mask() & 2)) ? 1 : 0;

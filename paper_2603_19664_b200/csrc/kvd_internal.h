@@ -15,6 +15,7 @@
 #include "../../include/kvd.h"
 #include "kvd_launch_mark.h"
 #include "kvd_positions.h"
+#include "kvd_rows_ring.h"
 
 namespace kvd {
 
@@ -119,10 +120,7 @@ struct FusedParams {
 struct NoFusedParams {};
 
 // ------------------------------------------------------------------------------ projection of a few rows
-constexpr int RW_MAX_ROWS = RC_INLINE_STAT_ROWS;
-constexpr int RW_FEW_ROWS = 16;
-constexpr int RW_HEAD_TILE = 32;  // columns per CTA of a key or value head
-constexpr int RW_MIN_TILE = 16;   // columns per tile of a plain product, at least
+static_assert(RW_MAX_ROWS == RC_INLINE_STAT_ROWS, "rows of a call whose statistics are taken in the kernel");
 struct RowsParams {
   const uint4 *rows;           // [n_rows][row_chunks]
   const int32_t *positions;    // [n_rows] (heads)

@@ -39,15 +39,6 @@
 namespace kvd {
 
 constexpr int RW_THREADS = 320;
-constexpr int RW_MAX_STAGES = 16;
-constexpr int RW_MMA_ROWS = 64;                           // M of the MMA
-// Shared memory of key and value heads of few rows.  The streaming attention's CTAs (9 KB, 16 K registers each) that
-// follow take places beside this kernel's -- two, with the registers its launch bounds leave -- and wait there instead of
-// being started when it ends; the ring still holds most of a CTA's weights.  One new token over 32768 cached ones, us:
-// 43.7 with all of an SM's shared memory, 37.9 with 173 or 193 KB, 36.8 with 145 or 161.
-constexpr int RW_HEADS_SMEM = 161 * 1024;
-constexpr int RW_BARS = 2 * RW_MAX_STAGES + 4;            // full, empty per stage; tmem_full[2], tmem_empty[2]
-constexpr int RW_TAIL = RW_BARS * 8 + 32 + RW_MAX_ROWS * 3 * 4;  // barriers, tmem pointer + abort, 1/rms, key scale, position
 
 // Four K = 16 steps of one k block: D[64 rows][columns of the tile] += X[64 x 64] W'^T[64 x columns].
 __device__ __forceinline__ void umma_kblock(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
@@ -418,24 +409,16 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
 template <int D_HEAD, int DT>
 static kvd_status launch_rows_impl(kvd_ctx *ctx, const CUtensorMap &tmap_w, const CUtensorMap &tmap_x, RowsParams &p, cudaStream_t stream) {
   auto kern = kvd_rows_kernel<D_HEAD, DT>;
-  constexpr int SMEM_MAX = 232448, CL = D_HEAD > 0 ? D_HEAD / RW_HEAD_TILE : 1;
+  constexpr int CL = D_HEAD > 0 ? D_HEAD / RW_HEAD_TILE : 1;
   static bool configured[64] = {};
   if (!configured[ctx->device & 63]) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, RW_SMEM_MAX);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(rows)");
     configured[ctx->device & 63] = true;
   }
-  const int stage = p.stage_kb * (p.nr + p.tile) * 128;
-  const int tail = RW_TAIL + (D_HEAD > 0 ? p.nr * (D_HEAD + 4) * 4 : 0);
-  // the descriptor of the last stage's last k block spans RW_MMA_ROWS rows from that block's rows on
-  const int beyond = RW_MMA_ROWS * 128 - (stage - (p.stage_kb - 1) * p.nr * 128);
-  const int slack = beyond > 0 ? beyond : 0;
-  const int total = (p.num_k_blocks + p.stage_kb - 1) / p.stage_kb * ((p.n_tiles + ctx->num_sms - 1) / ctx->num_sms);
-  const int smem = D_HEAD > 0 && p.nr <= RW_FEW_ROWS ? RW_HEADS_SMEM : SMEM_MAX;
-  p.stages = (smem - tail - slack) / stage;
-  if (p.stages > RW_MAX_STAGES) p.stages = RW_MAX_STAGES;
-  if (p.stages > total) p.stages = total;
-  p.tail_off = p.stages * stage + slack;
+  const RowsRing ring = rows_ring(p.nr, p.tile, p.stage_kb, D_HEAD, (p.num_k_blocks + p.stage_kb - 1) / p.stage_kb * ((p.n_tiles + ctx->num_sms - 1) / ctx->num_sms));
+  p.stages = ring.stages;
+  p.tail_off = ring.tail_off;
   p.tmem_cols = 64;  // two accumulators; the epilogue reads 32 columns at once
   while (p.tmem_cols < 2 * p.tile) p.tmem_cols *= 2;
   const int grid = D_HEAD > 0 || p.n_tiles < ctx->num_sms ? p.n_tiles : ctx->num_sms;
@@ -443,7 +426,7 @@ static kvd_status launch_rows_impl(kvd_ctx *ctx, const CUtensorMap &tmap_w, cons
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(grid, 1, 1);
   cfg.blockDim = dim3(RW_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = static_cast<size_t>(p.tail_off) + tail;
+  cfg.dynamicSmemBytes = ring.smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -483,15 +466,6 @@ static int rows_tile(const kvd_ctx *ctx, int n_cols) {
   const int t = ((n_cols + rounds * ctx->num_sms - 1) / (rounds * ctx->num_sms) + 7) / 8 * 8;
   return t < RW_MIN_TILE ? RW_MIN_TILE : t;
 }
-// k blocks per stage (a power of two up to 8): stages of 25 to 50 KB.  A stage costs the two single-thread loops some
-// 300 clocks of waits and commits whatever it holds (10240 x 2560, one row: 31, 27 and 23 us with 2, 4 and 8), and the
-// ring needs at least four.  `many`: more than RW_FEW_ROWS rows.
-static int rows_stage_kb(int tile, bool many) {
-  int kb = 8;
-  while (kb > 1 && kb * (tile + (many ? RW_MAX_ROWS : RW_FEW_ROWS)) * 128 > 50 * 1024) kb /= 2;
-  return kb;
-}
-
 kvd_status prepare_rows_map(kvd_ctx *ctx, LayerState &ls, int k, int n_cols, bool heads) {
   ls.rows_tile = heads ? RW_HEAD_TILE : rows_tile(ctx, n_cols);
   kvd_status st = KVD_OK;
