@@ -1639,11 +1639,12 @@ static bool prefill_split_pays(const kvd_ctx *ctx, const PrefillParams &P, int g
 template <int D_HEAD>
 static kvd_status prefill_tc_group(kvd_ctx *ctx, const PrefillParams &P, int group, cudaStream_t stream) {
   // pairs where the K/V bytes per block bound the kernel (d_head = 256); at 128 the softmax does, and the hand-overs
-  // across the pair cost more than the halved traffic returns (measured).  KVD_PREFILL_PAIR=0/1 overrides, for comparisons.
+  // across the pair cost more than the halved traffic returns (measured).  KVD_PREFILL_PAIR=0/1 asks for whole tiles on single
+  // CTAs or pairs in calls of any length, for comparisons.
   static const char *env = getenv("KVD_PREFILL_PAIR");
   const bool pair = D_HEAD >= 128 && (env ? env[0] == '1' : D_HEAD == 256);
   if constexpr (D_HEAD >= 128) {
-    if (prefill_split_pays(ctx, P, group)) {
+    if (!env && prefill_split_pays(ctx, P, group)) {
       switch (group) {
         case 1: return prefill_split_launch<D_HEAD, 1>(ctx, P, stream);
         case 2: return prefill_split_launch<D_HEAD, 2>(ctx, P, stream);

@@ -142,3 +142,10 @@ def test_attention_starts_early_only_straight_behind_the_projection(tmp_path):
     assert len(re.findall(r"few_rows\.set\(", ALL)) == 1
     rows = TEXT["kvd_rows.cu"]
     assert rows.index("ctx->launches += 1") < rows.index("few_rows.set(ctx->launches, stream")
+
+
+def test_the_comparison_switch_reaches_whole_tiles_in_calls_of_any_length():
+    """KVD_PREFILL_PAIR chooses single CTAs or pairs with whole tiles, so a shared tile is taken only where it is not set."""
+    text = TEXT["kvd_prefill_attention_tc.cu"]
+    choice = text[text.index('getenv("KVD_PREFILL_PAIR")'):]
+    assert re.search(r"if \(!env && prefill_split_pays\(", choice)
