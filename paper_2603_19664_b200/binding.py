@@ -116,7 +116,7 @@ def load() -> ctypes.CDLL:
     try:
         from . import _kvdcall
     except ImportError as e:
-        raise RuntimeError("_kvdcall.so not found or not loadable: build it with `python -m paper_2603_19664_b200.build`") from e
+        raise RuntimeError("_kvdcall not found or not loadable: build it with `python -m paper_2603_19664_b200.build`") from e
     lib = ctypes.CDLL(LIB_PATH)
     vp, i32, i64, sz = ctypes.c_void_p, ctypes.c_int, ctypes.c_int64, ctypes.c_size_t
     lib.kvd_create.argtypes = [ctypes.POINTER(kvd_model_desc), ctypes.POINTER(vp)]

@@ -3,7 +3,8 @@
 Compiles every ``csrc/*.cu`` for sm_100a with nvcc into ``libkvd.so`` next to this file.  The CUDA
 runtime is linked statically and the driver API is reached through ``cudaGetDriverEntryPoint``, so
 the library also loads on a machine without a GPU driver (where every entry point that needs a
-device reports an error).  ``_kvdcall.so``, beside it, marshals the arguments of the hot calls (csrc/kvd_pycall.c).
+device reports an error).  ``_kvdcall``, an extension module of the running interpreter, marshals the arguments of the hot
+calls (csrc/kvd_pycall.c).
 """
 from __future__ import annotations
 
@@ -17,7 +18,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libkvd.so")
 LIB_CHECK = os.path.join(HERE, "libkvd_check.so")  # the same sources with -DKVD_CHECK (device-side index tests)
-CALLS = os.path.join(HERE, "_kvdcall.so")  # argument marshalling of the hot calls (csrc/kvd_pycall.c)
+# argument marshalling of the hot calls; named for the interpreter it is built for, which another one does not load
+CALLS = os.path.join(HERE, "_kvdcall" + sysconfig.get_config_var("EXT_SUFFIX"))
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC",
          "--expt-relaxed-constexpr"]
@@ -48,6 +50,9 @@ def build_calls(force: bool = False) -> str:
         tmp = CALLS + f".tmp{os.getpid()}"
         subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-o", tmp, src], check=True)
         os.replace(tmp, CALLS)
+    untagged = os.path.join(HERE, "_kvdcall.so")  # any interpreter would load it
+    if untagged != CALLS and os.path.exists(untagged):
+        os.remove(untagged)
     return CALLS
 
 

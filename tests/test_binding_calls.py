@@ -1,6 +1,8 @@
 """The hot calls marshalled in C (_kvdcall) hand the library what ctypes hands it, and leave every argument that is not
 plain to ctypes: same values, same exceptions (no GPU: callbacks stand in for the library)."""
 import ctypes
+import os
+import sysconfig
 
 import numpy as np
 import pytest
@@ -150,3 +152,10 @@ def test_a_failing_call_and_a_closed_context_raise():
         c.kvd_checkpoint_residual(0, 0, T, T, 1, stream=0)
     with pytest.raises(B.KvdError):
         c.kvd_decode_attention(0, 1, T, [0], [SEGS[0]], 0.0, T, stream=0)
+
+
+def test_the_module_is_named_for_its_interpreter():
+    """It is not built against the limited API: another interpreter in the same tree must not load it."""
+    here = os.path.dirname(B.__file__)
+    assert os.path.basename(B._calls.__file__) == "_kvdcall" + sysconfig.get_config_var("EXT_SUFFIX")
+    assert not os.path.exists(os.path.join(here, "_kvdcall.so"))
