@@ -105,6 +105,13 @@ _CALLS = ("kvd_reset_sequence", "kvd_checkpoint_residual", "kvd_recompute_kv", "
           "kvd_decode_attention", "kvd_prefill_attention")
 
 
+class _NoCalls:
+    """In the place of ``_kvdcall``: every call is left to ctypes."""
+
+    def __getattr__(self, name):
+        return lambda *args: -1
+
+
 def load() -> ctypes.CDLL:
     """Load libkvd.so (built by ``paper_2603_19664_b200.build``); raises if it is missing."""
     global _lib, _calls
@@ -114,9 +121,9 @@ def load() -> ctypes.CDLL:
         raise RuntimeError(f"{LIB_PATH} not found: build it with `python -m paper_2603_19664_b200.build` "
                            "(there is no fallback path)")
     try:
-        from . import _kvdcall
-    except ImportError as e:
-        raise RuntimeError("_kvdcall not found or not loadable: build it with `python -m paper_2603_19664_b200.build`") from e
+        from . import _kvdcall as calls
+    except ImportError:  # not built (no C compiler or no headers of this Python): the same calls, marshalled by ctypes
+        calls = None
     lib = ctypes.CDLL(LIB_PATH)
     vp, i32, i64, sz = ctypes.c_void_p, ctypes.c_int, ctypes.c_int64, ctypes.c_size_t
     lib.kvd_create.argtypes = [ctypes.POINTER(kvd_model_desc), ctypes.POINTER(vp)]
@@ -252,9 +259,9 @@ def load() -> ctypes.CDLL:
     lib.kvd_scaffold_embed.restype = i32
     lib.kvd_scaffold_argmax.argtypes = [vp, vp, i64, i32, i32, vp, vp]
     lib.kvd_scaffold_argmax.restype = i32
-    for name in _CALLS:
-        _kvdcall.bind(name, ctypes.cast(getattr(lib, name), vp).value)
-    _lib, _calls = lib, _kvdcall
+    for name in _CALLS if calls else ():
+        calls.bind(name, ctypes.cast(getattr(lib, name), vp).value)
+    _lib, _calls = lib, calls or _NoCalls()
     return lib
 
 

@@ -60,7 +60,10 @@ def build(force: bool = False, verbose: bool = False, check: bool = False) -> st
     """Compile libkvd.so, or with ``check`` libkvd_check.so: the build whose kernels test the indices they
     derive on the device and report through the status word instead of accessing out of range."""
     LIB = LIB_CHECK if check else globals()["LIB"]
-    build_calls(force)
+    try:
+        build_calls(force)
+    except (OSError, subprocess.CalledProcessError) as e:  # the binding does without it: its calls then cost more host time
+        sys.stderr.write(f"[build] {os.path.basename(CALLS)} not built ({e}): all calls go through ctypes\n")
     if not force and not needs_build(check):
         return LIB
     objdir = os.path.join(HERE, "build", "check") if check else os.path.join(HERE, "build")

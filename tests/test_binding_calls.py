@@ -2,6 +2,8 @@
 plain to ctypes: same values, same exceptions (no GPU: callbacks stand in for the library)."""
 import ctypes
 import os
+import subprocess
+import sys
 import sysconfig
 
 import numpy as np
@@ -159,3 +161,28 @@ def test_the_module_is_named_for_its_interpreter():
     here = os.path.dirname(B.__file__)
     assert os.path.basename(B._calls.__file__) == "_kvdcall" + sysconfig.get_config_var("EXT_SUFFIX")
     assert not os.path.exists(os.path.join(here, "_kvdcall.so"))
+
+
+def test_the_binding_works_without_the_module(fake, monkeypatch):
+    """No C compiler or no Python headers: the library loads, and its calls are marshalled by ctypes."""
+    code = ("import sys; sys.modules['paper_2603_19664_b200._kvdcall'] = None\n"
+            "import paper_2603_19664_b200.binding as B\n"
+            "lib = B.load(); c = B.Kvd.__new__(B.Kvd); c._lib, c._h, c._addr, c._keep = lib, None, None, []\n"
+            "try: c.kvd_reset_sequence(0)\n"
+            "except B.KvdError: print('refused by the library')\n")
+    out = subprocess.run([sys.executable, "-c", code], cwd=os.path.dirname(os.path.dirname(B.__file__)), capture_output=True, text=True, check=True)
+    assert "refused by the library" in out.stdout
+    for call in CALLS:
+        with monkeypatch.context() as m:
+            m.setattr(B, "_calls", B._NoCalls())
+            call(fake)
+    assert len(SEEN) == len(CALLS)
+
+
+def test_a_build_without_a_compiler_goes_on(monkeypatch, tmp_path, capsys):
+    from paper_2603_19664_b200 import build as build_module
+
+    monkeypatch.setattr(build_module, "CALLS", str(tmp_path / "_kvdcall.so"))
+    monkeypatch.setenv("CC", str(tmp_path / "no-such-compiler"))
+    assert os.path.exists(build_module.build())
+    assert "ctypes" in capsys.readouterr().err
