@@ -4,7 +4,8 @@
  * four calls: 8.6 us in Python, 2.9 here).  Every function below takes the arguments of the Kvd method of its name, as they
  * are, behind the context's address, and returns the library's status -- or -1, before anything has been called, if an
  * argument is not of the plain kind it knows (tensors, exact ints in range, lists and tuples): binding.py then marshals the
- * call itself, with whatever conversion or exception that brings.  The library runs without the interpreter lock, as under
+ * call itself, with whatever conversion or exception that brings.  (What is no Exception -- an interrupt, an exit -- is not an
+ * argument's fault and passes through.)  The library runs without the interpreter lock, as under
  * ctypes.
  */
 #define PY_SSIZE_T_CLEAN
@@ -73,7 +74,7 @@ static int as_tensor(PyObject *o, void **out, int optional) {
   if (o == Py_None || PyLong_Check(o)) return 0;
   r = PyObject_CallMethodNoArgs(o, s_data_ptr);
   if (r == NULL) {
-    PyErr_Clear();
+    if (PyErr_ExceptionMatches(PyExc_Exception)) PyErr_Clear();
     return 0;
   }
   ok = as_handle(r, out) && r != Py_None;
@@ -177,7 +178,7 @@ static int as_segments(PyObject *const *lists, Py_ssize_t rows, kvd_kv_segment *
   return 1;
 }
 
-#define UNUSUAL return PyLong_FromLong(-1)
+#define UNUSUAL return PyErr_Occurred() ? NULL : PyLong_FromLong(-1)
 #define CALL(expr)                    \
   do {                                \
     kvd_status st_;                   \

@@ -147,6 +147,22 @@ def test_what_was_refused_is_refused(fake, monkeypatch, call, error):
     assert not SEEN
 
 
+def test_an_interrupt_inside_an_argument_is_not_swallowed(fake):
+    class Interrupted:
+        calls = 0
+
+        def data_ptr(self):
+            self.calls += 1
+            if self.calls == 1:
+                raise KeyboardInterrupt
+            return 0
+
+    for call in (lambda c, t: c.kvd_checkpoint_residual(1, 2, t, T, 7), lambda c, t: c.kvd_decode_attention(0, 1, T, [4], [[(t, T, 64, 0, 5)]], 0.0, T)):
+        with pytest.raises(KeyboardInterrupt):
+            call(fake, Interrupted())
+    assert not SEEN
+
+
 def test_a_failing_call_and_a_closed_context_raise():
     c = B.Kvd.__new__(B.Kvd)
     c._lib, c._h, c._addr, c._keep = LIB, None, None, []
