@@ -22,12 +22,20 @@ def _span(start, opening, closing):
     return i
 
 
-# name -> (arguments, body) of every kernel
+# name -> (arguments, body) of every kernel; a device function that holds the two calls of an early start is written out
+HELPERS = {}
+for m in re.finditer(r"__device__ __forceinline__ void (\w+)\(\) \{", ALL):
+    body = ALL[m.end():_span(m.end(), "{", "}") - 1]
+    if "grid_dependency_wait" in body or "grid_launch_dependents" in body:
+        HELPERS[m.group(1)] = body
 KERNELS = {}
 for m in re.finditer(r"__global__ void\s+(?:__launch_bounds__\((?:[^()]|\([^()]*\))*\)\s*)?(\w+)\s*\(", ALL):
     args_end = _span(m.end(), "(", ")")
     body = ALL.index("{", args_end) + 1
-    KERNELS[m.group(1)] = (ALL[m.end():args_end], ALL[body:_span(body, "{", "}")])
+    text = ALL[body:_span(body, "{", "}")]
+    for name, helper in HELPERS.items():
+        text = text.replace(name + "();", helper)
+    KERNELS[m.group(1)] = (ALL[m.end():args_end], text)
 
 
 @pytest.mark.parametrize("name", sorted(k for k, (_, b) in KERNELS.items() if "tmem_alloc" in b and "grid_launch_dependents" in b))
@@ -39,8 +47,21 @@ def test_dependents_start_only_after_tensor_memory_is_allocated(name):
     assert alloc < start and re.search(r"__syncthreads\(\)|cluster_sync_all\(\)", body[alloc:start])
 
 
-def test_both_projection_kernels_are_covered():
-    assert all("tmem_alloc" in KERNELS[k][1] and "grid_launch_dependents" in KERNELS[k][1] for k in ("kvd_rows_kernel", "kvd_recompute_kernel"))
+PREFILL = ["kvd_prefill_attn_tc_kernel", "kvd_prefill_attn_dual_kernel", "kvd_prefill_attn_split_kernel"]
+
+
+def test_every_kernel_with_tensor_memory_is_covered():
+    early = {k for k, (_, b) in KERNELS.items() if "tmem_alloc" in b}
+    assert early == {"kvd_rows_kernel", "kvd_recompute_kernel", *PREFILL}
+    assert all("grid_launch_dependents" in KERNELS[k][1] and "grid_dependency_wait" in KERNELS[k][1] for k in early)
+
+
+@pytest.mark.parametrize("name", PREFILL + ["kvd_attn_split_kernel", "kvd_attn_split_mma_kernel", "kvd_attn_merge_kernel"])
+def test_attention_reads_nothing_of_its_predecessor_before_the_wait(name):
+    args, body = KERNELS[name]
+    assert "__restrict__" not in args and "__ldg" not in body
+    before = body[:body.index("grid_dependency_wait();")]
+    assert not re.search(r"P\.(q|q_pos|k|v|out|part_o|part_ml|status)\b", before)
 
 
 def test_few_row_producer_waits_for_its_last_copies_on_every_path():
