@@ -71,6 +71,33 @@ def test_rows_follow_the_oracle_and_do_not_depend_on_each_other(shape):
     ctx.close()
 
 
+@pytest.mark.parametrize("shape,n", [(GEMMA3_4B_GLOBAL, 1250), (GEMMA3_4B_LOCAL, 1250), (QWEN3_4B, 330), (QWEN3_4B, 1200)], ids=lambda v: getattr(v, "name", str(v)))
+def test_rows_of_calls_of_many_tiles_follow_the_oracle(shape, n):
+    """75 tiles and more: a tile is one CTA's (or a pair of tiles a pair's), where fewer would be shared by two; with keys
+    missing between segments, rows without a key and rows past the last one."""
+    T = 1300
+    ctx, _ = open_layer(shape, max_tokens=4096)
+    kdim = shape.n_kv_heads * shape.d_head
+    assert -(-n // (128 // (shape.n_q_heads // shape.n_kv_heads))) * shape.n_kv_heads >= 75
+    K, V = make_kv(shape, T, seed=25)
+    first, cut1, cut2 = 5, 300, 310
+    seg_bits = [(K[first:cut1], V[first:cut1], first), (K[cut2:T - 1], V[cut2:T - 1], cut2), (K[T - 1:], V[T - 1:], T - 1)]
+    kd = [(dev(k), dev(v)) for k, v, _ in seg_bits]
+    segs = [(kd[i][0], kd[i][1], kdim, seg_bits[i][2], seg_bits[i][0].shape[0]) for i in range(3)]
+    rng = np.random.default_rng(26)
+    special = [0, 4, 5, 63, 64, 299, 300, 305, 309, 310, 639, 640, T - 1, T + 50]
+    q_pos = np.sort(np.concatenate([special, rng.integers(0, T, n - len(special))]))
+    q_bits = make_query(shape, n, seed=27)
+    out = torch.full((n, shape.n_q_heads, shape.d_head), 9.0, dtype=torch.bfloat16, device="cuda")
+    ctx.kvd_prefill_attention(0, n, dev(q_bits), torch.from_numpy(q_pos.astype(np.int32)).cuda(), segs, 0.0, out)
+    assert ctx.kvd_poll_status() == kvd.KVD_OK
+    empty = np.flatnonzero(q_pos < first)
+    assert len(empty) >= 2 and bool((out[torch.from_numpy(empty).cuda()] == 0).all())
+    sample = sorted(set([int(np.flatnonzero(q_pos == p)[0]) for p in special if p >= first] + rng.choice(np.flatnonzero(q_pos >= first), 14, replace=False).tolist()))
+    attn_check(host_f64(out[torch.tensor(sample).cuda()]), oracle_rows(shape, q_bits, q_pos, seg_bits, sample))
+    ctx.close()
+
+
 def test_causal_prefill_of_consecutive_tokens_and_rows_without_keys():
     shape = GEMMA3_4B_GLOBAL
     ctx, _ = open_layer(shape, max_tokens=2048)

@@ -2,9 +2,9 @@
 is shared by two CTAs.  A row's bits do not depend on that: they equal those of the same rows inside a call of more tiles
 than that, which takes whole tiles, and (in the other file) follow the oracle.
 
-Walks of 6 to 13 blocks and of 79 (every remainder of the four blocks the CTAs take turns by, and many rounds of every
+Walks of 0 to 13 blocks and of 79 (every remainder of the four blocks the CTAs take turns by, and many rounds of every
 ring), growing scores (the reference maximum moves, the accumulated output is rescaled), blocks across a gap between
-segments, windows, every group size, tiles with empty rows, rows without a key, fp16.
+segments, windows, every group size, one tile to 74, tiles with empty rows, rows without a key, rows past the call, fp16.
 """
 import pytest
 import torch
@@ -37,11 +37,22 @@ def test_a_shared_tile_has_the_bits_of_a_whole_one(n_q, n_kv, d_head, window, dt
         pos = torch.arange(keys - n, keys, dtype=torch.int32, device="cuda")
         pos[1] = 1  # sees no key
         long_pos = torch.cat((pos, torch.randint(3, keys, (whole - n,), generator=g, device="cuda").to(torch.int32)))
-        out, ref = torch.full_like(q[:n], 9.0), torch.zeros_like(q[:whole])
+        ref = torch.zeros_like(q[:whole])
         c.kvd_prefill_attention(0, whole, q, long_pos, segs, 0.0, ref)
         for rows in {n, 1, min(n, 37)}:
+            out = torch.full_like(q[:n + 1], 9.0)
             c.kvd_prefill_attention(0, rows, q, pos, segs, 0.0, out)
-            assert torch.equal(out[:rows], ref[:rows]), (keys, rows)
-        assert bool((out[1] == 0).all()) and bool(torch.isfinite(out.float()).all())
+            assert torch.equal(out[:rows], ref[:rows]) and bool((out[rows:] == 9).all()), (keys, rows)
+        assert bool((ref[1] == 0).all()) and bool(torch.isfinite(ref.float()).all())
+    # as many tiles as are shared, each with a walk of its own: from no block (rows in front of the first key) and one to all
+    for keys, first in ((700, 3), (T - 20, 3)):
+        n = 74 // n_kv * (128 // group) - 3
+        segs = [(k, v, kdim, first, keys // 2), (k[keys // 2:], v[keys // 2:], kdim, first + keys // 2 + 17, keys - keys // 2)]
+        pos = (torch.arange(n, device="cuda") * (keys + 25) // n).to(torch.int32)
+        more = torch.full((128 // group * (148 // n_kv + 1) - n,), keys, dtype=torch.int32, device="cuda")
+        ref, out = torch.zeros_like(q[:n + len(more)]), torch.full_like(q[:n + 1], 9.0)
+        c.kvd_prefill_attention(0, n + len(more), q, torch.cat((pos, more)), segs, 0.0, ref)
+        c.kvd_prefill_attention(0, n, q, pos, segs, 0.0, out)
+        assert torch.equal(out[:n], ref[:n]) and bool((out[n] == 9).all()) and bool((out[0] == 0).all()), keys
     assert c.kvd_poll_status() == kvd.KVD_OK
     c.close()
