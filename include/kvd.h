@@ -376,7 +376,9 @@ kvd_status kvd_decode_attention_rows(kvd_ctx *ctx, int layer, int n_rows, const 
  * position; the softmax weights are rounded to the element type before the second product (fp32 accumulation); a
  * row's weights are taken against a reference that follows its maximum in steps (it moves when a block exceeds it by
  * 2^8), which changes rounding, not the softmax.  Both products run as tcgen05.mma with scores and output in tensor
- * memory (CTA pairs at d_head 256); KVD_ERR_TIMEOUT from kvd_poll_status if an in-kernel wait ran out.
+ * memory.  How tiles of 128 rows go to CTAs changes no bit: at d_head 128 and 256 a tile is shared by two CTAs where tiles
+ * are few and the walk over the keys is long; otherwise pairs of CTAs share keys and values at 256, long calls put two tiles
+ * on a CTA at 128, and the rest take one each.  KVD_ERR_TIMEOUT from kvd_poll_status if an in-kernel wait ran out.
  * A row's result depends on that row, its position and the keys alone -- not on n_rows, on the row's index or on the
  * other rows of the call -- so a token attended alone and the same token inside a long call give the same bits.
  * They are NOT the bits of kvd_decode_attention / kvd_decode_attention_rows (another split of the keys): same

@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(AT_THREADS, ALLIN ? 2 : AT_CTAS_PER_SM) kvd_at
 #pragma unroll
   for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg)
     if (segment_holds(S.first[sg], S.len[sg], chunk_pos0, chunk_keys)) fast_seg = sg;
-  const bool fast = fast_seg >= 0 && chunk_pos0 >= S.lo_pos && chunk_keys - 1 <= S.hi_pos - chunk_pos0;
+  const bool fast = fast_seg >= 0 && chunk_pos0 >= S.lo_pos && ends_by(chunk_pos0, chunk_keys, S.hi_pos);
   const __nv_bfloat16 *fk = P.q, *fv = P.q;
   long long fstride = 0;
   if (fast) {
@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(AT_THREADS, AT_CTAS_PER_SM)
 #pragma unroll
   for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg)
     if (segment_holds(S.first[sg], S.len[sg], chunk_pos0, chunk_keys)) fast_seg = sg;
-  const bool fast = fast_seg >= 0 && chunk_pos0 >= S.lo_pos && chunk_keys - 1 <= S.hi_pos - chunk_pos0;
+  const bool fast = fast_seg >= 0 && chunk_pos0 >= S.lo_pos && ends_by(chunk_pos0, chunk_keys, S.hi_pos);
   const __nv_bfloat16 *fk = P.q, *fv = P.q;
   long long fstride = 0;
   if (fast) {
