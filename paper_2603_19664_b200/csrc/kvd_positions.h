@@ -13,13 +13,12 @@ namespace kvd {
 // First key position that a query at qp sees (window > 0: the last `window` positions up to its own).
 KVD_HD int first_visible(int qp, int window) { return window > 0 && qp >= window ? qp - window + 1 : 0; }
 
-// Whether the positions pos .. pos + n - 1 all lie inside the segment first .. first + len - 1, which ends at the largest int
-// or before it (0 <= first, len, n).  (With this form and the next, decode attention is as fast as with the sum of pos and n,
-// which can overflow: FP8 step over 4096 rows 35.4 us.  With pos - first <= len - n, or with unsigned sums, it took 35.6.)
-KVD_HD bool segment_holds(int first, int len, int pos, int n) { return first <= pos && n <= first + len - pos; }
-// Whether the last of them, pos + n - 1, is at most `last`, a position that a segment may hold (0 <= pos, last; last + 1 is an
-// int; 0 < n).
-KVD_HD bool ends_by(int pos, int n, int last) { return n <= last - pos + 1; }
+// Whether the positions pos .. pos + n - 1 all lie inside the segment first .. first + len - 1 (which ends before the largest
+// int; 0 <= n).  (64-bit sums: decode attention is as fast with them as with sums that overflow, an FP8 step over 4096 rows 35.2
+// us; with differences, or unsigned sums, it took 35.5.)
+KVD_HD bool segment_holds(int first, int len, int pos, int n) { return first <= pos && static_cast<long long>(pos) + n <= first + len; }
+// Whether the last of them, pos + n - 1, is at most `last`.
+KVD_HD bool ends_by(int pos, int n, int last) { return static_cast<long long>(pos) + n - 1 <= last; }
 
 // Of the 64 positions from pos0 on, those in [a, b) counted from pos0, as bits.
 KVD_HD unsigned long long slots64(int a, int b) {

@@ -40,7 +40,7 @@ int main() {
       }
     for (int last : at)
       for (int n : {1, 32, 64, 128})
-        if (last >= 0 && last < INT_MAX && ends_by(pos0, n, last) != (static_cast<int64_t>(pos0) + n - 1 <= last)) return 5;
+        if (ends_by(pos0, n, last) != (static_cast<int64_t>(pos0) + n - 1 <= last)) return 5;
     for (int lo : at)
       for (int qp : at) {
         if (lo < 0) continue;
