@@ -68,6 +68,50 @@ __device__ __forceinline__ float reduce8_transposed(const float (&v)[8], int lig
   return w1;
 }
 
+// Where the keys of one warp iteration (a run of n <= 32) lie.  A chunk inside one segment and inside the visible range
+// (the common case) has addresses linear in the position; of any other chunk each run is asked for by itself, and only a
+// run that crosses an edge is looked up key by key, one key per lane.  The choice is uniform over the warp and does not
+// change which keys are read.  (Before, each lane went through the segments for each of its keys: 900 keys of three
+// sequences, Gemma-3-4B layer, 6.6 -> 4.8 us, a step's attention over 701 keys 5.9 -> 3.5.)
+struct KeyRun {
+  const __nv_bfloat16 *k, *v;  // row of the run's first key, at the KV head (linear runs)
+  long long stride;
+  bool linear;
+};
+__device__ __forceinline__ int after(int pos, int n) { return static_cast<int>(static_cast<unsigned>(pos) + static_cast<unsigned>(n)); }
+__device__ __forceinline__ KeyRun key_run(const AttnSeq &S, int pos, int n, size_t head_el) {
+  int at = -1;
+#pragma unroll
+  for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg)
+    if (segment_holds(S.first[sg], S.len[sg], pos, n)) at = sg;
+  KeyRun r = {nullptr, nullptr, 0, at >= 0 && pos >= S.lo_pos && ends_by(pos, n, S.hi_pos)};
+  if (r.linear) {
+    r.stride = S.stride[at];
+    const size_t off = static_cast<size_t>(pos - S.first[at]) * r.stride + head_el;
+    r.k = S.k[at] + off;
+    r.v = S.v[at] + off;
+  }
+  return r;
+}
+// Rows of the key at one position, null when the query does not see it or nobody holds it.
+__device__ __forceinline__ void key_rows(const AttnSeq &S, int pos, size_t head_el, const __nv_bfloat16 *&k, const __nv_bfloat16 *&v) {
+  k = v = nullptr;
+  if (pos >= S.lo_pos && pos <= S.hi_pos) {
+#pragma unroll
+    for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg) {
+      const int r = pos - S.first[sg];
+      if (r >= 0 && r < S.len[sg]) {
+        const size_t off = static_cast<size_t>(r) * S.stride[sg] + head_el;
+        k = S.k[sg] + off;
+        v = S.v[sg] + off;
+      }
+    }
+  }
+}
+__device__ __forceinline__ const __nv_bfloat16 *lane_ptr(const __nv_bfloat16 *p, int src) {
+  return reinterpret_cast<const __nv_bfloat16 *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(p), src));
+}
+
 // DT: element type of q, K, V and the output (0 = bf16, 1 = fp16; kvd_set_dtype).
 // ALLIN: for launches of at most two CTAs per SM whose chunks are two iterations long (a single sequence of
 // a few thousand keys), where nothing else on the SM hides a load's latency: the loads of both iterations are
@@ -141,59 +185,32 @@ __global__ void __launch_bounds__(AT_THREADS, ALLIN ? 2 : AT_CTAS_PER_SM) kvd_at
 
   const size_t head_off = static_cast<size_t>(kvh) * D_HEAD + lig * 8;
 
-  // Whole chunk inside one segment and inside the visible range (the common case): addresses are
-  // linear in the position.  Otherwise every key is looked up in the segment list.  The choice is
-  // uniform over the CTA and does not change which keys are read or in which order.
-  int fast_seg = -1;
-#pragma unroll
-  for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg)
-    if (segment_holds(S.first[sg], S.len[sg], chunk_pos0, chunk_keys)) fast_seg = sg;
-  const bool fast = fast_seg >= 0 && chunk_pos0 >= S.lo_pos && ends_by(chunk_pos0, chunk_keys, S.hi_pos);
-  const __nv_bfloat16 *fk = P.q, *fv = P.q;
-  long long fstride = 0;
-  if (fast) {
-    fstride = S.stride[fast_seg];
-    const size_t off = static_cast<size_t>(chunk_pos0 - S.first[fast_seg]) * fstride + head_off;
-    fk = S.k[fast_seg] + off;
-    fv = S.v[fast_seg] + off;
-  }
-
   // issue the 16 loads of one iteration (8 keys, 8 values) for this lane group
-  auto issue = [&](int it, uint4 (&kr)[U], uint4 (&vr)[U], uint32_t &vmask) {
-    const int rel0 = ((it * AT_WARPS + warp) * KPL + grp) * U;  // first of this group's 8 positions
-    if (fast) {
-      const __nv_bfloat16 *kp = fk + static_cast<size_t>(rel0) * fstride;
-      const __nv_bfloat16 *vp = fv + static_cast<size_t>(rel0) * fstride;
+  const KeyRun whole = key_run(S, chunk_pos0, chunk_keys, head_off);
+  auto issue_linear = [&](int it, uint4 (&kr)[U], uint4 (&vr)[U], uint32_t &vmask) {
+    const size_t rel0 = static_cast<size_t>(((it * AT_WARPS + warp) * KPL + grp) * U);
+    const __nv_bfloat16 *kp = whole.k + rel0 * whole.stride;
+    const __nv_bfloat16 *vp = whole.v + rel0 * whole.stride;
 #pragma unroll
-      for (int u = 0; u < U; ++u) kr[u] = ldg_stream(kp + u * fstride);
+    for (int u = 0; u < U; ++u) kr[u] = ldg_stream(kp + u * whole.stride);
 #pragma unroll
-      for (int u = 0; u < U; ++u) vr[u] = ldg_stream(vp + u * fstride);
-      vmask = 0xFFu;
-    } else {
-      // masked keys are not loaded: they read as zeros and score -inf
-      vmask = 0;
+    for (int u = 0; u < U; ++u) vr[u] = ldg_stream(vp + u * whole.stride);
+    vmask = 0xFFu;
+  };
+  // masked keys are not loaded: they read as zeros and score -inf.  Lane l looks up key l of the warp's iteration.
+  auto issue_any = [&](int it, uint4 (&kr)[U], uint4 (&vr)[U], uint32_t &vmask) {
+    const int pos0 = after(chunk_pos0, (it * AT_WARPS + warp) * KPL * U);
+    const __nv_bfloat16 *kl = nullptr, *vl = nullptr;
+    if (lane < KPL * U) key_rows(S, after(pos0, lane), head_off - lig * 8, kl, vl);
+    vmask = (__ballot_sync(0xffffffffu, kl != nullptr) >> (grp * U)) & 0xFFu;
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int pos = chunk_pos0 + rel0 + u;
-        const __nv_bfloat16 *kp = nullptr, *vp = nullptr;
-        if (pos >= S.lo_pos && pos <= S.hi_pos) {
-#pragma unroll
-          for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg) {
-            const int r = pos - S.first[sg];
-            if (r >= 0 && r < S.len[sg]) {
-              const size_t off = static_cast<size_t>(r) * S.stride[sg] + head_off;
-              kp = S.k[sg] + off;
-              vp = S.v[sg] + off;
-              vmask |= 1u << u;
-            }
-          }
-        }
-        kr[u] = make_uint4(0u, 0u, 0u, 0u);
-        vr[u] = make_uint4(0u, 0u, 0u, 0u);
-        if (kp != nullptr) {
-          kr[u] = ldg_stream(kp);
-          vr[u] = ldg_stream(vp);
-        }
+    for (int u = 0; u < U; ++u) {
+      const __nv_bfloat16 *kp = lane_ptr(kl, grp * U + u) + lig * 8, *vp = lane_ptr(vl, grp * U + u) + lig * 8;
+      kr[u] = make_uint4(0u, 0u, 0u, 0u);
+      vr[u] = make_uint4(0u, 0u, 0u, 0u);
+      if ((vmask >> u) & 1u) {
+        kr[u] = ldg_stream(kp);
+        vr[u] = ldg_stream(vp);
       }
     }
   };
@@ -276,19 +293,26 @@ __global__ void __launch_bounds__(AT_THREADS, ALLIN ? 2 : AT_CTAS_PER_SM) kvd_at
     // both iterations' loads, then the query, then the arithmetic in the usual order
     uint4 ka[U], va[U], kb[U], vb[U];
     uint32_t ma = 0, mb = 0;
-    issue(0, ka, va, ma);
-    issue(1, kb, vb, mb);
+    if (whole.linear) {
+      issue_linear(0, ka, va, ma);
+      issue_linear(1, kb, vb, mb);
+    } else {
+      issue_any(0, ka, va, ma);
+      issue_any(1, kb, vb, mb);
+    }
     load_query();
     step(ka, va, ma);
     step(kb, vb, mb);
   } else {
     // One buffer of loads per iteration; latency is hidden by the other 15 warps resident on the SM
     // (the kernel is capped at 128 registers so that four CTAs fit), which measured faster than
-    // register double buffering or a shared-memory ring at half the occupancy.
+    // register double buffering or the other kernel's shared-memory ring (16 x 2048 keys of a Gemma-3-4B layer 26.0 us,
+    // with the ring 30.8: two query heads per key leave registers enough, and its rings leave the L1 too small for loads).
     uint4 ka[U], va[U];
     uint32_t ma = 0;
     for (int it = 0; it < S.iters; ++it) {
-      issue(it, ka, va, ma);
+      if (whole.linear) issue_linear(it, ka, va, ma);
+      else issue_any(it, ka, va, ma);
       step(ka, va, ma);
     }
   }
@@ -352,6 +376,16 @@ __global__ void __launch_bounds__(AT_THREADS, ALLIN ? 2 : AT_CTAS_PER_SM) kvd_at
 // to bf16 for the second product (fp32 sums), as the scores' softmax weights are in any tensor-core
 // attention; the partials have the same format as those of the kernel above and go to the same merge.
 // Chunking, the position -> (chunk, warp, block) assignment and the masking rules are identical.
+//
+// K and V pass through a ring of shared memory that every warp has to itself: a piece is the K or the V of one warp
+// iteration (4 KB whatever the head size), fetched by 16-byte asynchronous copies, which need no registers.  Held in
+// registers, beside the accumulators, the 16 loads of an iteration spilled and were waited for in turns, and nothing was on its
+// way while a warp computed.  Three pieces per warp and four CTAs per SM, so that 12 KB per warp are always in flight, or four
+// pieces (a whole chunk of two iterations, one round trip to memory) where the grid has at most three CTAs for an SM.  The
+// kernel alone, us, registers / ring: Qwen3-4B layer, one sequence of 1500 keys 11.2 / 6.0, 8 x 2000 20.8 / 16.0, 40 x 1000
+// 42.9 / 36, 64 x 3000 176 / 140 (5.6 TB/s), one of 30000 29.8 / 22.1; SmolLM2 layer 8 x 2000 8.3 / 5.0.  Four pieces at three
+// CTAs per SM for every grid: 8 x 2000 18.8, one of 30000 28.0, SmolLM2 40 x 3000 24.2 against 20.7.
+constexpr int AT_PIECE = 4096;
 template <int DT>
 __device__ __forceinline__ void mma_x16_m16n8k16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                                  uint32_t b0, uint32_t b1) {
@@ -378,8 +412,8 @@ __device__ __forceinline__ void mma_x16_m16n8k8(float (&c)[4], uint32_t a0, uint
                  : "r"(a0), "r"(a1), "r"(b0));
 }
 
-template <int D_HEAD, int G, int NSEQ, int DT = 0>
-__global__ void __launch_bounds__(AT_THREADS, AT_CTAS_PER_SM)
+template <int D_HEAD, int G, int NSEQ, int DT = 0, int SLOTS = 3>
+__global__ void __launch_bounds__(AT_THREADS, SLOTS == 3 ? AT_CTAS_PER_SM : 3)
     kvd_attn_split_mma_kernel(const __grid_constant__ AttnLaunchT<NSEQ> P) {
   static_assert(G >= 1 && G <= 8 && D_HEAD <= 128, "query heads are the 8 columns of the second product");
   constexpr int LPK = D_HEAD / 8, KPL = 32 / LPK;
@@ -388,9 +422,9 @@ __global__ void __launch_bounds__(AT_THREADS, AT_CTAS_PER_SM)
   constexpr int KP = D_HEAD / 32;             // 16-byte pieces of a key row per thread (first product)
   constexpr int VP = D_HEAD / 64;             // 16-byte pieces of a value row per thread (second product)
   constexpr int MB = D_HEAD / 16;             // 16-channel blocks of the output
-  __shared__ float s_o[AT_WARPS][G][D_HEAD];
-  __shared__ float s_m[AT_WARPS][G];
-  __shared__ float s_l[AT_WARPS][G];
+  constexpr int ROW = D_HEAD * 2;             // bytes of a key's row, [WARP_KEYS][ROW] is a piece
+  static_assert(WARP_KEYS * ROW == AT_PIECE && G * D_HEAD * 4 <= SLOTS * AT_PIECE && WARP_KEYS <= 32, "a piece, a warp's partial in its ring's place");
+  extern __shared__ __align__(16) uint8_t at_ring[];  // the warps' rings
   grid_launch_dependents();
 
   int si = 0;
@@ -411,8 +445,52 @@ __global__ void __launch_bounds__(AT_THREADS, AT_CTAS_PER_SM)
   const int t = lane & 3;    // fragment pair index
   const int chunk_keys = WARP_KEYS * AT_WARPS * S.iters;
   const int chunk_pos0 = S.chunk0_pos + chunk * chunk_keys;
+  const size_t head_el = static_cast<size_t>(kvh) * D_HEAD;
+  const KeyRun whole = key_run(S, chunk_pos0, chunk_keys, head_el);
 
   grid_dependency_wait();
+  // ---- pieces come in by whole rows (lane group grp's LPK lanes fetch row KPL u + grp) and are read as fragments: chunk c
+  // (16 bytes) of row r of a piece of keys lies at c ^ 4 (r & 1), of values at c ^ 2 (r / 2 & 3), so that the eight lanes
+  // that a shared-memory access serves at a time meet different banks (rows g8 of keys, rows 2 t and 2 t + 1 of values)
+  uint8_t *ring = at_ring + warp * (SLOTS * AT_PIECE);
+  const uint32_t ring_addr = smem_u32(ring);
+  const int grp = lane / LPK, lig = lane % LPK;
+  // fetch piece i (K of iteration i / 2 where i is even, else V); visible: its keys that are, as bits
+  auto fetch = [&](int i, uint32_t &visible) {
+    const int it = i >> 1, run0 = (it * AT_WARPS + warp) * WARP_KEYS;
+    if (it < S.iters) {
+      const uint32_t dst = ring_addr + (i % SLOTS) * AT_PIECE;
+      auto place = [&](int u) {
+        const int r = KPL * u + grp;
+        return dst + r * ROW + ((lig ^ ((i & 1) ? ((r >> 1) & 3) * 2 : (r & 1) * 4)) << 4);
+      };
+      const KeyRun run = whole.linear ? whole : key_run(S, after(chunk_pos0, run0), WARP_KEYS, head_el);
+      if (run.linear) {
+        const __nv_bfloat16 *src = ((i & 1) ? run.v : run.k) + static_cast<size_t>((whole.linear ? run0 : 0) + grp) * run.stride + lig * 8;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) cp_async16(place(u), src + u * KPL * run.stride, true);
+        visible = ~0u;
+      } else {
+        // masked keys are not loaded: they read as zeros and score -inf.  Lane l looks up key l of the run.
+        const __nv_bfloat16 *kl = nullptr, *vl = nullptr;
+        if (lane < WARP_KEYS) key_rows(S, after(chunk_pos0, run0 + lane), head_el, kl, vl);
+        visible = __ballot_sync(0xffffffffu, kl != nullptr);
+        if (visible != 0u) {  // (a run that nothing is seen of takes no part)
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const __nv_bfloat16 *src = lane_ptr((i & 1) ? vl : kl, KPL * u + grp);
+            cp_async16(place(u), src ? src + lig * 8 : P.q, src != nullptr);
+          }
+        }
+      }
+    }
+    cp_async_commit();  // (an empty group past the end: the waits below count groups)
+  };
+  uint32_t vis = 0, vnext = 0, vafter = 0, vlast = 0;
+  fetch(0, vis);
+  fetch(1, vis);
+  fetch(2, vnext);
+  if constexpr (SLOTS == 4) fetch(3, vlast);
   // ---- query rows as A fragments: thread (g8, t) holds channels [32 j + 8 t, 32 j + 8 t + 8) of head g8
   uint32_t qa[KP][4];
 #pragma unroll
@@ -432,79 +510,35 @@ __global__ void __launch_bounds__(AT_THREADS, AT_CTAS_PER_SM)
 #pragma unroll
     for (int r = 0; r < 4; ++r) oacc[mb][r] = 0.f;
 
-  const size_t head_el = static_cast<size_t>(kvh) * D_HEAD;
-  int fast_seg = -1;
-#pragma unroll
-  for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg)
-    if (segment_holds(S.first[sg], S.len[sg], chunk_pos0, chunk_keys)) fast_seg = sg;
-  const bool fast = fast_seg >= 0 && chunk_pos0 >= S.lo_pos && ends_by(chunk_pos0, chunk_keys, S.hi_pos);
-  const __nv_bfloat16 *fk = P.q, *fv = P.q;
-  long long fstride = 0;
-  if (fast) {
-    fstride = S.stride[fast_seg];
-    const size_t off = static_cast<size_t>(chunk_pos0 - S.first[fast_seg]) * fstride + head_el;
-    fk = S.k[fast_seg] + off;
-    fv = S.v[fast_seg] + off;
-  }
-  // row pointers (K, V) of the key at chunk-relative position rel, or null when it is not visible
-  auto locate = [&](int rel, const __nv_bfloat16 *&kp, const __nv_bfloat16 *&vp) {
-    kp = vp = nullptr;
-    if (fast) {
-      kp = fk + static_cast<size_t>(rel) * fstride;
-      vp = fv + static_cast<size_t>(rel) * fstride;
-      return;
-    }
-    const int pos = chunk_pos0 + rel;
-    if (pos >= S.lo_pos && pos <= S.hi_pos) {
-#pragma unroll
-      for (int sg = 0; sg < KVD_MAX_SEGMENTS; ++sg) {
-        const int r = pos - S.first[sg];
-        if (r >= 0 && r < S.len[sg]) {
-          const size_t off = static_cast<size_t>(r) * S.stride[sg] + head_el;
-          kp = S.k[sg] + off;
-          vp = S.v[sg] + off;
-        }
-      }
-    }
-  };
-
+#pragma unroll 1
   for (int it = 0; it < S.iters; ++it) {
-    const int rel0 = (it * AT_WARPS + warp) * WARP_KEYS;
-    // ---- all loads of the iteration: per block, the key row of key g8 (first product) and the value
-    // rows of keys 2t and 2t+1 (second product); invisible keys read as zeros
-    uint4 kr[NBLK][KP], vr[NBLK][2][VP];
-    uint32_t vmask = 0;  // bit 2b + i: key 8b + 2t + i is visible
+    cp_async_wait_group<SLOTS - 1>();
+    __syncwarp();  // (the other lanes' copies)
+    // ---- scores of the iteration's keys for (up to) 8 heads, one block of 8 keys after the other
+    float sc[NBLK][4];
+    const uint8_t *kp = ring + (2 * it) % SLOTS * AT_PIECE;
 #pragma unroll
     for (int b = 0; b < NBLK; ++b) {
-      const __nv_bfloat16 *kp, *vp_unused, *kp_unused, *vp0, *vp1;
-      locate(rel0 + 8 * b + g8, kp, vp_unused);
-      locate(rel0 + 8 * b + 2 * t, kp_unused, vp0);
-      locate(rel0 + 8 * b + 2 * t + 1, kp_unused, vp1);
 #pragma unroll
-      for (int j = 0; j < KP; ++j)
-        kr[b][j] = kp ? ldg_stream(kp + 32 * j + 8 * t) : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-      for (int i = 0; i < VP; ++i) {
-        vr[b][0][i] = vp0 ? ldg_stream(vp0 + 64 * i + 8 * g8) : make_uint4(0u, 0u, 0u, 0u);
-        vr[b][1][i] = vp1 ? ldg_stream(vp1 + 64 * i + 8 * g8) : make_uint4(0u, 0u, 0u, 0u);
-      }
-      vmask |= (vp0 ? 1u : 0u) << (2 * b);
-      vmask |= (vp1 ? 1u : 0u) << (2 * b + 1);
-    }
-    if (!__any_sync(0xffffffffu, vmask != 0u)) continue;  // nothing visible in this warp's keys
-
-#pragma unroll
-    for (int b = 0; b < NBLK; ++b) {
-      // ---- scores of 8 keys for (up to) 8 heads
-      float sc[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int r = 0; r < 4; ++r) sc[b][r] = 0.f;
 #pragma unroll
       for (int j = 0; j < KP; ++j) {
-        mma_x16_m16n8k16<DT>(sc, qa[j][0], 0u, qa[j][1], 0u, kr[b][j].x, kr[b][j].y);
-        mma_x16_m16n8k16<DT>(sc, qa[j][2], 0u, qa[j][3], 0u, kr[b][j].z, kr[b][j].w);
+        const uint4 kr = *reinterpret_cast<const uint4 *>(kp + (8 * b + g8) * ROW + (((4 * j + t) ^ ((g8 & 1) * 4)) << 4));
+        mma_x16_m16n8k16<DT>(sc[b], qa[j][0], 0u, qa[j][1], 0u, kr.x, kr.y);
+        mma_x16_m16n8k16<DT>(sc[b], qa[j][2], 0u, qa[j][3], 0u, kr.z, kr.w);
       }
+    }
+    __syncwarp();  // every lane has read the piece that the next copies replace
+    fetch(2 * it + SLOTS, SLOTS == 3 ? vlast : vafter);  // V of the next iteration, or K of the one after it
+    cp_async_wait_group<SLOTS - 1>();
+    __syncwarp();
+    const uint8_t *vp = ring + (2 * it + 1) % SLOTS * AT_PIECE;
+    if (vis != 0u) {  // (uniform; nothing to add otherwise)
+#pragma unroll
+    for (int b = 0; b < NBLK; ++b) {
       // thread (g8, t): head g8, keys 2t and 2t+1 of the block
-      const float s0 = ((vmask >> (2 * b)) & 1u) ? sc[0] * P.scale_log2e : -CUDART_INF_F;
-      const float s1 = ((vmask >> (2 * b + 1)) & 1u) ? sc[1] * P.scale_log2e : -CUDART_INF_F;
+      const float s0 = ((vis >> (8 * b + 2 * t)) & 1u) ? sc[b][0] * P.scale_log2e : -CUDART_INF_F;
+      const float s1 = ((vis >> (8 * b + 2 * t + 1)) & 1u) ? sc[b][1] * P.scale_log2e : -CUDART_INF_F;
       float bmax = fmaxf(s0, s1);
       bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, 1));
       bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, 2));
@@ -531,8 +565,9 @@ __global__ void __launch_bounds__(AT_THREADS, AT_CTAS_PER_SM)
       // from keys 2t (low half) and 2t+1 (high half)
 #pragma unroll
       for (int i = 0; i < VP; ++i) {
-        const uint32_t v0[4] = {vr[b][0][i].x, vr[b][0][i].y, vr[b][0][i].z, vr[b][0][i].w};
-        const uint32_t v1[4] = {vr[b][1][i].x, vr[b][1][i].y, vr[b][1][i].z, vr[b][1][i].w};
+        const uint8_t *v01 = vp + (8 * b + 2 * t) * ROW + (((8 * i + g8) ^ (2 * t)) << 4);  // (rows 2t and 2t+1 swizzle alike)
+        const uint4 w0 = *reinterpret_cast<const uint4 *>(v01), w1 = *reinterpret_cast<const uint4 *>(v01 + ROW);
+        const uint32_t v0[4] = {w0.x, w0.y, w0.z, w0.w}, v1[4] = {w1.x, w1.y, w1.z, w1.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const uint32_t a0 = __byte_perm(v0[e], v1[e], 0x5410);  // channel 2e of both keys
@@ -541,7 +576,17 @@ __global__ void __launch_bounds__(AT_THREADS, AT_CTAS_PER_SM)
         }
       }
     }
+    }
+    __syncwarp();
+    vis = vnext;
+    if constexpr (SLOTS == 4) vnext = vafter;
+    fetch(2 * it + 1 + SLOTS, SLOTS == 3 ? vnext : vlast);
   }
+  cp_async_wait_all();  // (empty groups)
+  // (maximum and sum lie behind the head's outputs: with nothing beside the rings, four CTAs fit the 196 KB split of an SM's
+  // memory and leave 60 KB of L1 instead of 28: 16 x 2000, Qwen3-4B layer, 43.7 -> 41.7 us for the call)
+  auto out_of = [&](int w, int g) { return reinterpret_cast<float *>(at_ring + w * (SLOTS * AT_PIECE)) + g * (D_HEAD + 2); };
+  __syncwarp();
 
   // ---- one partial per warp into shared memory, then the CTA's partial as in the kernel above
   {
@@ -549,8 +594,8 @@ __global__ void __launch_bounds__(AT_THREADS, AT_CTAS_PER_SM)
     l += __shfl_xor_sync(0xffffffffu, l, 1);
     l += __shfl_xor_sync(0xffffffffu, l, 2);
     if (t == 0 && g8 < G) {
-      s_m[warp][g8] = m_run;
-      s_l[warp][g8] = l;
+      out_of(warp, g8)[D_HEAD] = m_run;
+      out_of(warp, g8)[D_HEAD + 1] = l;
     }
 #pragma unroll
     for (int mb = 0; mb < MB; ++mb) {
@@ -558,7 +603,7 @@ __global__ void __launch_bounds__(AT_THREADS, AT_CTAS_PER_SM)
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
         const int head = 2 * t + (r & 1);
-        if (head < G) s_o[warp][head][ch + (r >> 1)] = oacc[mb][r];
+        if (head < G) out_of(warp, head)[ch + (r >> 1)] = oacc[mb][r];
       }
     }
   }
@@ -568,14 +613,14 @@ __global__ void __launch_bounds__(AT_THREADS, AT_CTAS_PER_SM)
     const int g = idx / D_HEAD, c = idx % D_HEAD;
     float M = -CUDART_INF_F;
 #pragma unroll
-    for (int pp = 0; pp < AT_WARPS; ++pp) M = fmaxf(M, s_m[pp][g]);
+    for (int pp = 0; pp < AT_WARPS; ++pp) M = fmaxf(M, out_of(pp, g)[D_HEAD]);
     const float Mu = (M == -CUDART_INF_F) ? 0.f : M;
     float o = 0.f, l = 0.f;
 #pragma unroll
     for (int pp = 0; pp < AT_WARPS; ++pp) {
-      const float w = exp2f(s_m[pp][g] - Mu);
-      o = fmaf(w, s_o[pp][g][c], o);
-      l = fmaf(w, s_l[pp][g], l);
+      const float w = exp2f(out_of(pp, g)[D_HEAD] - Mu);
+      o = fmaf(w, out_of(pp, g)[c], o);
+      l = fmaf(w, out_of(pp, g)[D_HEAD + 1], l);
     }
     const size_t hq = pidx * P.n_q + kvh * G + g;
     if (!KVD_BOUNDS_OK(pidx < static_cast<size_t>(P.max_parts), P.status)) continue;  // checking build: the partial's slot
@@ -715,7 +760,12 @@ static cudaError_t attn_configure() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (!done[dev & 63]) {
-    if constexpr (!(G >= 3 && D_HEAD <= 128)) {
+    if constexpr (G >= 3 && D_HEAD <= 128) {
+      e = cudaFuncSetAttribute(kvd_attn_split_mma_kernel<D_HEAD, G, NSEQ, DT, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_WARPS * 3 * AT_PIECE);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kvd_attn_split_mma_kernel<D_HEAD, G, NSEQ, DT, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_WARPS * 4 * AT_PIECE);
+      if (e != cudaSuccess) return e;
+    } else {
       e = cudaFuncSetAttribute(kvd_attn_split_kernel<D_HEAD, G, NSEQ, DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                AttnSmem<D_HEAD, G>::BYTES);
       if (e != cudaSuccess) return e;
@@ -757,8 +807,10 @@ static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t str
     cfg.gridDim = dim3(S.total_chunks * S.n_kv, 1, 1);
     cfg.blockDim = dim3(AT_THREADS, 1, 1);
     if constexpr (G >= 3 && D_HEAD <= 128) {
-      cfg.dynamicSmemBytes = 0;
-      e = cudaLaunchKernelEx(&cfg, kvd_attn_split_mma_kernel<D_HEAD, G, NSEQ, DT>, S);
+      const bool few = S.total_chunks * S.n_kv <= 148 * 3;  // all of the grid at once with four pieces per warp
+      cfg.dynamicSmemBytes = AT_WARPS * (few ? 4 : 3) * AT_PIECE;
+      if (few) e = cudaLaunchKernelEx(&cfg, kvd_attn_split_mma_kernel<D_HEAD, G, NSEQ, DT, 4>, S);
+      else e = cudaLaunchKernelEx(&cfg, kvd_attn_split_mma_kernel<D_HEAD, G, NSEQ, DT, 3>, S);
     } else {
       cfg.dynamicSmemBytes = AttnSmem<D_HEAD, G>::BYTES;
       // at most two CTAs per SM, every chunk two iterations long: the variant that issues all loads at once
