@@ -638,23 +638,27 @@ __global__ void __launch_bounds__(AT_THREADS, SLOTS == 3 ? AT_CTAS_PER_SM : 3)
 // which the streaming CTAs would spend idle on their SM; the kernel boundary costs about as much
 // once per step and needs no counters.  A sequence without a visible key gets zeros.
 //
-// One CTA per (sequence, KV head, slice of 64 channels).  Warp w merges the w-th group of consecutive
+// One CTA per (sequence, KV head, GH of its G query heads, slice of 64 channels).  Warp w merges the w-th group of consecutive
 // partials of its head group, each lane owning two channels of every head: a partial costs a lane 4*G
 // registers, a group is as many partials as fit 64 registers (attn_merge_group(G)), all fetched at
 // once, so a warp's work is one round trip to the L2; the warp results are added in warp order.  The
 // launch has as many warps per CTA as its longest sequence has groups (at most 16; beyond that a warp
 // takes several groups, 16 apart); a shorter sequence leaves the extra warps idle, so its summation
 // order depends on its own chunk count only.
-template <int D_HEAD, int G, int NSEQ, int DT = 0>
+template <int D_HEAD, int G, int NSEQ, int DT, int GH>
 __global__ void __launch_bounds__(AT_MERGE_THREADS)
     kvd_attn_merge_kernel(const __grid_constant__ AttnLaunchT<NSEQ> P) {
   constexpr int SLICES = D_HEAD / AT_MERGE_SLICE;
   constexpr int PF = attn_merge_group(G);
-  __shared__ float s_o[AT_MERGE_WARPS][G][AT_MERGE_SLICE];
-  __shared__ float s_l[AT_MERGE_WARPS][G];
+  // of every warp of the CTA: outputs [GH][AT_MERGE_SLICE] and sums [GH] (as much as the launch's warps need: the kernel's
+  // loads in flight pass through the L1, which shared memory is taken from: 64 x 3000 keys of a Qwen3-4B layer 15.8 -> 12.5 us,
+  // 40 x 1000 7.3 -> 5.2)
+  extern __shared__ float at_merge_smem[];
+  float (*s_o)[GH][AT_MERGE_SLICE] = reinterpret_cast<float (*)[GH][AT_MERGE_SLICE]>(at_merge_smem);
+  float (*s_l)[GH] = reinterpret_cast<float (*)[GH]>(at_merge_smem + blockDim.x / 32 * GH * AT_MERGE_SLICE);
   const int slice = blockIdx.x % SLICES;
   const int head_slot = blockIdx.x / SLICES;
-  const int si = head_slot / P.n_kv, kvh = head_slot % P.n_kv;
+  const int si = head_slot / (P.n_q / GH), head0 = head_slot % (P.n_q / GH) * GH;  // sequence, first query head
   const AttnSeq &S = P.seq[si];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   grid_launch_dependents();
@@ -666,19 +670,19 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
   const int count = KVD_BOUNDS_OK(S.merge_base >= 0 && S.merge_base + S.merge_count <= P.max_parts, P.status) ? S.merge_count : 0;
   const int n_groups = (count + PF - 1) / PF;
   const int warps_used = n_groups < AT_MERGE_WARPS ? n_groups : AT_MERGE_WARPS;
-  const float *ml0 = P.part_ml + (static_cast<size_t>(S.merge_base) * P.n_q + kvh * G) * 2;
-  const float *po0 = P.part_o + (static_cast<size_t>(S.merge_base) * P.n_q + kvh * G) * D_HEAD +
+  const float *ml0 = P.part_ml + (static_cast<size_t>(S.merge_base) * P.n_q + head0) * 2;
+  const float *po0 = P.part_o + (static_cast<size_t>(S.merge_base) * P.n_q + head0) * D_HEAD +
                      slice * AT_MERGE_SLICE + lane * 2;
   const size_t ml_stride = static_cast<size_t>(P.n_q) * 2, po_stride = static_cast<size_t>(P.n_q) * D_HEAD;
   if (warp < warps_used) {
-    float2 vbuf[PF][G], mlbuf[PF][G];
+    float2 vbuf[PF][GH], mlbuf[PF][GH];
     // (a partial past the end re-reads the last one and is skipped below: no branch between the loads)
     auto fetch_group = [&](int grp) {
 #pragma unroll
       for (int i = 0; i < PF; ++i) {
         const int ch = grp * PF + i < count ? grp * PF + i : count - 1;
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
+        for (int g = 0; g < GH; ++g) {
           mlbuf[i][g] = __ldcg(reinterpret_cast<const float2 *>(ml0 + ch * ml_stride + g * 2));
           vbuf[i][g] = __ldcg(reinterpret_cast<const float2 *>(po0 + ch * po_stride + g * D_HEAD));
         }
@@ -687,9 +691,9 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
     fetch_group(warp);
     // the maximum of each head over all partials: lanes over partials (the first 256 loaded before
     // any is used), then shuffles -- every warp by itself, no block barrier
-    float Mu[G];
+    float Mu[GH];
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
+    for (int g = 0; g < GH; ++g) {
       float mv[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
@@ -702,10 +706,10 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
       for (int msk = 16; msk >= 1; msk >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, msk));
       Mu[g] = (mx == -CUDART_INF_F) ? 0.f : mx;
     }
-    float2 o[G];
-    float l[G];
+    float2 o[GH];
+    float l[GH];
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
+    for (int g = 0; g < GH; ++g) {
       l[g] = 0.f;
       o[g] = make_float2(0.f, 0.f);
     }
@@ -715,7 +719,7 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
       for (int i = 0; i < PF; ++i) {
         if (grp * PF + i < count) {
 #pragma unroll
-          for (int g = 0; g < G; ++g) {
+          for (int g = 0; g < GH; ++g) {
             const float w = exp2f(mlbuf[i][g].x - Mu[g]);
             l[g] = fmaf(w, mlbuf[i][g].y, l[g]);
             o[g].x = fmaf(w, vbuf[i][g].x, o[g].x);
@@ -725,7 +729,7 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
       }
     }
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
+    for (int g = 0; g < GH; ++g) {
       if (lane == 0) s_l[warp][g] = l[g];
       s_o[warp][g][lane * 2] = o[g].x;
       s_o[warp][g][lane * 2 + 1] = o[g].y;
@@ -733,7 +737,7 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
   }
   __syncthreads();
   // the warp sums are added in warp order
-  for (int idx = threadIdx.x; idx < G * AT_MERGE_SLICE; idx += blockDim.x) {
+  for (int idx = threadIdx.x; idx < GH * AT_MERGE_SLICE; idx += blockDim.x) {
     const int g = idx / AT_MERGE_SLICE, c = idx % AT_MERGE_SLICE;
     float ov = 0.f, lv = 0.f;
     for (int w = 0; w < warps_used; ++w) {
@@ -741,7 +745,7 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
       lv += s_l[w][g];
     }
     const float r = lv > 0.f ? ov / lv : 0.f;
-    const size_t oi = (static_cast<size_t>(si) * P.n_q + kvh * G + g) * D_HEAD + slice * AT_MERGE_SLICE + c;
+    const size_t oi = (static_cast<size_t>(si) * P.n_q + head0 + g) * D_HEAD + slice * AT_MERGE_SLICE + c;
     if constexpr (DT == 0) P.out[oi] = __float2bfloat16_rn(r);
     else reinterpret_cast<__half *>(P.out)[oi] = __float2half_rn(r);
   }
@@ -831,10 +835,21 @@ static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t str
   for (int i = 0; i < S.n_seqs; ++i) max_chunks = S.seq[i].merge_count > max_chunks ? S.seq[i].merge_count : max_chunks;
   int merge_warps = (max_chunks + attn_merge_group(G) - 1) / attn_merge_group(G);
   if (merge_warps > AT_MERGE_WARPS) merge_warps = AT_MERGE_WARPS;
-  cfg.gridDim = dim3(S.n_seqs * S.n_kv * (D_HEAD / AT_MERGE_SLICE), 1, 1);
   cfg.blockDim = dim3(32 * merge_warps, 1, 1);
-  cfg.dynamicSmemBytes = 0;
-  return cudaLaunchKernelEx(&cfg, kvd_attn_merge_kernel<D_HEAD, G, NSEQ, DT>, S);
+  auto merge = [&](auto kern, int heads) {
+    cfg.gridDim = dim3(S.n_seqs * (S.n_q / heads) * (D_HEAD / AT_MERGE_SLICE), 1, 1);
+    cfg.dynamicSmemBytes = merge_warps * heads * (AT_MERGE_SLICE + 1) * sizeof(float);
+    return cudaLaunchKernelEx(&cfg, kern, S);
+  };
+  // A CTA per query head as long as the SMs hold all of their warps at once: a CTA of a whole group issues G times the loads
+  // from one SM while most SMs have no CTA.  us, group / head: SmolLM2 step 3.4 / 1.9, Qwen3-4B layer 1 x 30000 7.0 / 5.1, 8 x 2000
+  // 4.7 / 3.4, 32 x 500 5.5 / 3.7, Gemma-3-4B layer 4 x 2048 4.5 / 3.6, 1 x 32768 4.7 / 3.8; beyond one wave the group's is ahead:
+  // Gemma 64 x 1000 3.6 / 4.3, Qwen 64 x 3000 12.9 / 13.3.
+  if constexpr (G > 1) {
+    if (S.n_seqs * S.n_q * (D_HEAD / AT_MERGE_SLICE) * merge_warps <= 148 * AT_MERGE_WARPS)
+      return merge(kvd_attn_merge_kernel<D_HEAD, G, NSEQ, DT, 1>, 1);
+  }
+  return merge(kvd_attn_merge_kernel<D_HEAD, G, NSEQ, DT, G>, G);
 }
 
 template <int D_HEAD, int G, int NSEQ>
