@@ -56,6 +56,20 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
+// Whether that phase has completed, asked without waiting: for a thread that has work of its own to issue while the answer
+// is on its way.
+__device__ __forceinline__ uint32_t mbar_test_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok;
+}
+
 // Bounded wait: returns false when `timeout_ns` elapsed or another thread of the CTA raised the
 // abort flag.  Never spins forever.  The slow path (timer, abort flag) is kept out of line so that
 // a wait on a barrier that has already completed costs one try_wait.

@@ -18,7 +18,8 @@
 // Measured (B200, one bf16 row, time of the launch alone): 2560 -> 262144 columns 323 us with the 256-row tiles, 197 us
 // here (6.8 TB/s of weights); 2560 -> 20480 43 and 23.5 us; 10240 -> 2560 54 and 20.7 us; 2560 -> 2048 20 and 10.7 us; K and
 // V of a Gemma-3-4B layer 25.6 and 12.9 us.  Short products are bound by launch, first-load latency and, where K is
-// long, by the chain of K / 16 dependent MMAs (24 clocks each).  The operands the other way round (weights as the M
+// long, by the chain of K / 16 dependent MMAs (24 clocks each alone; 36 in this kernel before the issuer asked for a stage
+// ahead of its end, 27 since: in a chain of launches 10240 -> 2560 15.3 -> 13.3 us, with 24 rows 22.7 -> 20.0).  The operands the other way round (weights as the M
 // of the MMA, 64 columns per CTA) measured 282, 38 and 44 us: too few CTAs for the narrow products.
 //
 // Weights never change after they were prepared, so the loads of the first stages are issued before the
@@ -181,7 +182,7 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
       const uint32_t idesc = DT == 1 ? umma_idesc_f16_f32(RW_MMA_ROWS, tile) : umma_idesc_bf16_f32(RW_MMA_ROWS, tile);
       constexpr uint32_t desc_hi = (1024u >> 4) | (1u << 14) | (2u << 29);  // as in kvd_recompute.cu
       int s = 0;
-      uint32_t ph = 0;
+      uint32_t ph = 0, ready = 0;  // ready: stage s is known to have landed
       bool ok = true;
       for (int t = 0; ok && t < my_tiles; ++t) {
         const int a = t & 1;
@@ -193,25 +194,31 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
         const uint32_t d = tmem_base + a * (p.tmem_cols / 2);
         int left = p.num_k_blocks;
         for (int k = 0; k < steps; ++k) {
-          if (!mbar_wait(bar_full(s), ph, s_abort, tmo)) {
+          if (!ready && !mbar_wait(bar_full(s), ph, s_abort, tmo)) {
             raise(p.status, STATUS_TIMEOUT, s_abort);
             ok = false;
             break;
           }
           tc_fence_after();
-          uint32_t xa = ((ring + s * stage_bytes) >> 4) | (1u << 16), wb = ((ring + s * stage_bytes + w_off) >> 4) | (1u << 16);
-          const int n = left < kbs ? left : kbs;
-          for (int b = 0; b < n; ++b) {
-            umma_kblock(d, xa, wb, desc_hi, idesc, (k | b) != 0 ? 1u : 0u);
-            xa += x_kb >> 4;
-            wb += w_kb >> 4;
-          }
-          left -= n;
-          umma_commit(bar_empty(s));
+          const uint32_t xa = ((ring + s * stage_bytes) >> 4) | (1u << 16), wb = ((ring + s * stage_bytes + w_off) >> 4) | (1u << 16);
+          const uint32_t x_step = x_kb >> 4, w_step = w_kb >> 4, empty = bar_empty(s);
           if (++s == stages) {
             s = 0;
             ph ^= 1u;
           }
+          const int n = left < kbs ? left : kbs;
+          umma_kblock(d, xa, wb, desc_hi, idesc, k != 0 ? 1u : 0u);
+          // The tensor cores hold few MMAs ahead of the one they work on, and a barrier answers late beside their reads of
+          // shared memory: asked for between two stages, the next one's state cost 250 clocks of idle tensor cores.
+          ready = mbar_test_wait(bar_full(s), ph);
+          if (n == 8) {
+#pragma unroll
+            for (int b = 1; b < 8; ++b) umma_kblock(d, xa + b * x_step, wb + b * w_step, desc_hi, idesc, 1u);
+          } else {
+            for (int b = 1; b < n; ++b) umma_kblock(d, xa + b * x_step, wb + b * w_step, desc_hi, idesc, 1u);
+          }
+          left -= n;
+          umma_commit(empty);
         }
         if (ok) umma_commit(bar_tmem_full(a));
       }
