@@ -27,9 +27,12 @@
 //
 // Warps: 0 producer (one lane), 1 MMA issuer (one lane) and tensor-memory owner, 2-9 row statistics, of these
 // 4-7 the epilogue.  Plain products walk over tiles (two accumulators); key/value projections
-// have one 32-column tile per CTA, the d_head / 32 CTAs of a head form a cluster and exchange their accumulators,
-// because the key norm runs over the whole head in one fixed order and the half-split rotation pairs columns of
-// different tiles.
+// have one 32-column tile per CTA, the d_head / 32 CTAs of a head form a cluster and exchange their accumulators where
+// the key norm runs over the whole head in one fixed order or the half-split rotation pairs columns of different tiles.
+// What the end of a CTA waits for is latency: the columns travel by st.async, 16 bytes a lane, and count on the receiver's
+// barrier; two lanes take a row's norm; positions, rotation and scale of the keys are fetched while the products run.  (One
+// thread per row storing to every CTA, a cluster barrier, then the norm, then the tables: 2.6 us behind the last product;
+// one row of a Gemma-3-4B layer in a chain 6.5 -> 5.6 us, three 6.2 -> 5.5.)
 #include <string.h>
 
 #include <type_traits>
@@ -96,18 +99,49 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
   volatile int *s_abort = reinterpret_cast<volatile int *>(s_tmem + 1);
   float *s_rstd = reinterpret_cast<float *>(s_tmem + 8);
   float *s_kscale = s_rstd + RW_MAX_ROWS;
-  int *s_pos = reinterpret_cast<int *>(s_kscale + RW_MAX_ROWS);
-  float *s_y = reinterpret_cast<float *>(s_pos + RW_MAX_ROWS);  // heads: accumulators of the whole head, [row][LD]
+  float *s_y = s_kscale + RW_MAX_ROWS;  // heads: accumulators of the whole head, [row][LD]
   const uint32_t ring = smem_u32(rw_smem), bar_base = smem_u32(bars);
   auto bar_full = [&](int s) { return bar_base + 8u * s; };
   auto bar_empty = [&](int s) { return bar_base + 8u * (RW_MAX_STAGES + s); };
   auto bar_tmem_full = [&](int a) { return bar_base + 8u * (2 * RW_MAX_STAGES + a); };
   auto bar_tmem_empty = [&](int a) { return bar_base + 8u * (2 * RW_MAX_STAGES + 2 + a); };
+  const uint32_t bar_head = bar_base + 8u * (2 * RW_MAX_STAGES + 4);  // keys: the other CTAs' columns of the head
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const unsigned long long tmo = p.timeout_ns;
   const int steps = (p.num_k_blocks + kbs - 1) / kbs;  // stages of a tile
   const int block = static_cast<int>(blockIdx.x), blocks = static_cast<int>(gridDim.x);
   const int my_tiles = (p.n_tiles - block + blocks - 1) / blocks;
+  const int head_col = block * RW_HEAD_TILE;     // heads: the CTA's first column
+  const bool key = HEADS && head_col < p.k_cols;
+  const bool exchange = key && (p.qk_norm || p.rope_half);  // what it makes of its columns depends on other CTAs' columns
+  // heads: the last part's row of this thread (half a warp per row) and what the rotation of its two columns takes, fetched
+  // by warps 2 to 9 while the products run
+  const int last_row = 2 * ((warp + 8) % 10) + (lane >> 4), head_c = head_col % (HEADS ? D_HEAD : 1) + 2 * (lane & 15);
+  struct Turn {
+    float cs[2], sn[2], ga[2], gb[2];
+  } turn = {};
+  auto position = [&](int r) {
+    const int pos = p.positions[r];
+    if (pos >= 0 && pos < p.max_pos) return pos;
+    atomicOr(p.status, STATUS_POSITION);
+    return pos < 0 ? 0 : p.max_pos - 1;
+  };
+  auto fetch_turn = [&](int pos) {
+    if constexpr (HEADS) {
+      constexpr int HALF = D_HEAD / 2;
+      const float2 *t_hi = p.rope_hi + static_cast<size_t>(pos >> ROPE_LO_BITS) * HALF;
+      const float2 *t_lo = p.rope_lo + (pos & (ROPE_LO_SIZE - 1));
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int i = p.rope_half ? (head_c + j) % HALF : head_c / 2;  // pair (i, i + HALF), or the columns' own
+        const float2 h = __ldg(t_hi + i), l = __ldg(t_lo + i * ROPE_LO_SIZE);
+        turn.cs[j] = fmaf(h.x, l.x, -h.y * l.y);
+        turn.sn[j] = fmaf(h.y, l.x, h.x * l.y);
+        turn.ga[j] = p.gamma_k ? __ldg(p.gamma_k + (p.rope_half ? i : head_c)) : 1.0f;
+        turn.gb[j] = p.gamma_k ? __ldg(p.gamma_k + (p.rope_half ? i + HALF : head_c + 1)) : 1.0f;
+      }
+    }
+  };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) {
@@ -119,7 +153,9 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
       mbar_init(bar_tmem_empty(a), 4);  // one arrival per epilogue warp
     }
     *s_abort = 0;
+    if (HEADS) mbar_init(bar_head, 1);
     fence_mbar_init();
+    if (exchange) mbar_arrive_expect_tx(bar_head, (CL - 1) * p.n_rows * RW_HEAD_TILE * 4);
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(s_tmem), p.tmem_cols);
@@ -269,6 +305,7 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
       else take(std::integral_constant<int, 2>(), std::integral_constant<int, 5>());
     }
     asm volatile("bar.sync 1, 256;" ::: "memory");
+    if (key && last_row < p.n_rows) fetch_turn(position(last_row));
     if (warp >= 4 && warp < 8) {
       // ---------------------------------------------------------------- epilogue
       // (M = 64: rows 16 q .. 16 q + 15 are lanes 0-15 of tensor memory quarter q)
@@ -291,15 +328,19 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
             uint32_t v[RW_HEAD_TILE];
             tmem_ld_x32(acc, v);
             tmem_wait_ld();
+            float *mine = s_y + static_cast<int>(rank) * RW_HEAD_TILE;
             if (valid) {
-              float *dst = s_y + row * LD + static_cast<int>(rank) * RW_HEAD_TILE;
 #pragma unroll
-              for (int j = 0; j < RW_HEAD_TILE; j += 4) {
-                *reinterpret_cast<uint4 *>(dst + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-                if (col0 < p.k_cols) {  // keys: the whole head goes to each of its CTAs
-#pragma unroll
-                  for (uint32_t q = 1; q < CL; ++q)
-                    st_cluster_v4(map_to_cta(smem_u32(dst + j), (rank + q) % CL), v[j], v[j + 1], v[j + 2], v[j + 3]);
+              for (int j = 0; j < RW_HEAD_TILE; j += 4) *reinterpret_cast<uint4 *>(mine + row * LD + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+            }
+            if (exchange) {  // keys: the whole head goes to each of its CTAs, (CL - 1) x 8 pieces of 16 bytes a row
+              __syncwarp();
+              for (int i = lane; i < static_cast<int>(CL - 1) * 8; i += 32) {
+                const uint32_t to = (rank + 1 + i / 8) % CL, bar = map_to_cta(bar_head, to);
+                for (int r = quarter * 16; r < p.n_rows && r < quarter * 16 + 16; ++r) {
+                  const float *src = mine + r * LD + i % 8 * 4;
+                  const uint4 y = *reinterpret_cast<const uint4 *>(src);
+                  st_async_v4(map_to_cta(smem_u32(src), to), bar, y.x, y.y, y.z, y.w);
                 }
               }
             }
@@ -332,84 +373,84 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
   }
   __syncwarp();
   tc_fence_before();
-  if (CL > 1) cluster_sync_all();
-  else __syncthreads();
+  __syncthreads();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, p.tmem_cols);
   }
   if constexpr (HEADS) {
     // ------------------------------------------------------------------ key norm, rotation, stores: all warps
-    if (*s_abort != 0) return;
+    // (No CTA leaves before every CTA of the head has sent its columns, and each waits for those it is sent, also behind
+    // an abort: nothing arrives in the shared memory of a CTA that is gone.)
+    cluster_arrive_relaxed();
+    if (exchange) {
+      int ok = 1;
+      if (lane == 0) {
+        const unsigned long long t0 = globaltimer_ns();
+        while (!mbar_try_wait_cluster(bar_head, 0))
+          if (globaltimer_ns() - t0 > tmo) {
+            ok = 0;
+            break;
+          }
+      }
+      if (!__shfl_sync(0xffffffffu, ok, 0)) raise(p.status, STATUS_TIMEOUT, s_abort);
+      __syncwarp();
+    }
     constexpr int HALF = D_HEAD / 2;
-    const int col0 = block * RW_HEAD_TILE;
-    const bool key = col0 < p.k_cols;
-    if (threadIdx.x < p.n_rows) {
-      const int r = threadIdx.x;
+    // two lanes per row: four chains (columns j mod 4) in ascending order, two-wide: the order of the recompute kernel
+    if (warp * 16 < p.n_rows) {
+      const int r = threadIdx.x / 2 < p.n_rows ? threadIdx.x / 2 : p.n_rows - 1, half = threadIdx.x & 1;
       const float rstd = s_rstd[r];
       float kscale = rstd;
       if (key && p.qk_norm) {
-        // four chains (columns j mod 4) in ascending order, two-wide: the order of the recompute kernel
-        uint64_t ss2[2] = {0ull, 0ull};
+        uint64_t ss2 = 0ull;
         const uint64_t rstd2 = pack2(rstd, rstd);
-#pragma unroll 8
-        for (int c = 0; c < D_HEAD; c += 4) {
-          const float4 y = *reinterpret_cast<const float4 *>(s_y + r * LD + c);
-          const uint64_t v0 = fmul2(pack2(y.x, y.y), rstd2), v1 = fmul2(pack2(y.z, y.w), rstd2);
-          ss2[0] = ffma2(v0, v0, ss2[0]);
-          ss2[1] = ffma2(v1, v1, ss2[1]);
+#pragma unroll 16
+        for (int c = 2 * half; c < D_HEAD; c += 4) {
+          const float2 y = *reinterpret_cast<const float2 *>(s_y + r * LD + c);
+          const uint64_t v = fmul2(pack2(y.x, y.y), rstd2);
+          ss2 = ffma2(v, v, ss2);
         }
-        float s0, s1, s2, s3;
-        unpack2(ss2[0], s0, s1);
-        unpack2(ss2[1], s2, s3);
-        const float ss = (s0 + s1) + (s2 + s3);
+        float s0, s1;
+        unpack2(ss2, s0, s1);
+        const float mine = s0 + s1, ss = mine + __shfl_xor_sync(0xffffffffu, mine, 1);
         kscale = rstd * (1.0f / sqrtf(ss * (1.0f / D_HEAD) + p.qk_eps));
       }
-      int pos = p.positions[r];
-      if (pos < 0 || pos >= p.max_pos) {
-        atomicOr(p.status, STATUS_POSITION);
-        pos = pos < 0 ? 0 : p.max_pos - 1;
-      }
       s_kscale[r] = kscale;
-      s_pos[r] = pos;
     }
     __syncthreads();
-    const int c = col0 % D_HEAD + 2 * (lane & 15);  // this lane's two columns of the head; half a warp per row
-    for (int r = 2 * warp + (lane >> 4); r < p.n_rows; r += 2 * (RW_THREADS / 32)) {
+    const bool whole = *s_abort == 0;
+    for (int r = last_row; whole && r < p.n_rows; r += 2 * (RW_THREADS / 32)) {
       // (checking build: this CTA's columns lie inside the key or the value heads)
-      if (!KVD_BOUNDS_OK(col0 + RW_HEAD_TILE <= (key ? p.k_cols : p.n_cols) && r < RW_MAX_ROWS, p.status)) continue;
+      if (!KVD_BOUNDS_OK(head_col + RW_HEAD_TILE <= (key ? p.k_cols : p.n_cols) && r < RW_MAX_ROWS, p.status)) continue;
       const float *y = s_y + r * LD;
       const float ks = s_kscale[r];
+      const int c = head_c;
       uint32_t o;
       if (!key) {
         o = pack_out<DT>(y[c] * ks, y[c + 1] * ks);
       } else {
-        const int pos = s_pos[r];
-        const float2 *t_hi = p.rope_hi + static_cast<size_t>(pos >> ROPE_LO_BITS) * HALF;
-        const float2 *t_lo = p.rope_lo + (pos & (ROPE_LO_SIZE - 1));
-        auto gamma = [&](int i) { return p.gamma_k ? __ldg(p.gamma_k + i) : 1.0f; };
+        if (warp < 2 || r != last_row) fetch_turn(position(r));
         if (!p.rope_half) {
-          const float2 h = __ldg(t_hi + c / 2), l = __ldg(t_lo + c / 2 * ROPE_LO_SIZE);
-          const float cs = fmaf(h.x, l.x, -h.y * l.y), sn = fmaf(h.y, l.x, h.x * l.y);
-          const float a = y[c] * ks * gamma(c), b = y[c + 1] * ks * gamma(c + 1);
-          o = pack_out<DT>(fmaf(a, cs, -b * sn), fmaf(a, sn, b * cs));
+          const float a = y[c] * ks * turn.ga[0], b = y[c + 1] * ks * turn.gb[0];
+          o = pack_out<DT>(fmaf(a, turn.cs[0], -b * turn.sn[0]), fmaf(a, turn.sn[0], b * turn.cs[0]));
         } else {
           float v[2];
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
             const int i = (c + j) % HALF;  // pair (i, i + HALF)
-            const float2 h = __ldg(t_hi + i), l = __ldg(t_lo + i * ROPE_LO_SIZE);
-            const float cs = fmaf(h.x, l.x, -h.y * l.y), sn = fmaf(h.y, l.x, h.x * l.y);
-            const float a = y[i] * ks * gamma(i), b = y[i + HALF] * ks * gamma(i + HALF);
-            v[j] = c < HALF ? fmaf(a, cs, -b * sn) : fmaf(a, sn, b * cs);
+            const float a = y[i] * ks * turn.ga[j], b = y[i + HALF] * ks * turn.gb[j];
+            v[j] = c < HALF ? fmaf(a, turn.cs[j], -b * turn.sn[j]) : fmaf(a, turn.sn[j], b * turn.cs[j]);
           }
           o = pack_out<DT>(v[0], v[1]);
         }
       }
-      __nv_bfloat16 *dst = (key ? p.k_out + (col0 / D_HEAD) * D_HEAD : p.v_out + (col0 - p.k_cols) / D_HEAD * D_HEAD) +
+      __nv_bfloat16 *dst = (key ? p.k_out + (head_col / D_HEAD) * D_HEAD : p.v_out + (head_col - p.k_cols) / D_HEAD * D_HEAD) +
                            static_cast<size_t>(r) * p.out_stride + c;
       *reinterpret_cast<uint32_t *>(dst) = o;
     }
+    __syncwarp();
+    cluster_wait();
   }
 }
 

@@ -9,8 +9,8 @@ constexpr int RW_HEAD_TILE = 32;  // columns per CTA of a key or value head
 constexpr int RW_MIN_TILE = 16;   // columns per tile of a plain product, at least
 constexpr int RW_MMA_ROWS = 64;   // M of the MMA
 constexpr int RW_MAX_STAGES = 16;
-constexpr int RW_BARS = 2 * RW_MAX_STAGES + 4;                   // full, empty per stage; tmem_full[2], tmem_empty[2]
-constexpr int RW_TAIL = RW_BARS * 8 + 32 + RW_MAX_ROWS * 3 * 4;  // barriers, tmem pointer + abort, 1/rms, key scale, position
+constexpr int RW_BARS = 2 * RW_MAX_STAGES + 6;                   // full, empty per stage; tmem_full[2], tmem_empty[2], head, (16-byte multiple)
+constexpr int RW_TAIL = RW_BARS * 8 + 32 + RW_MAX_ROWS * 2 * 4;  // barriers, tmem pointer + abort, 1/rms, key scale
 constexpr int RW_SMEM_MAX = 232448;
 // Key and value heads leave an SM room for two CTAs of the streaming attention behind them (9 to 18 KB and 16 K registers
 // each; the kernel's launch bounds leave the registers), which take their places beside a CTA of this kernel and wait there
