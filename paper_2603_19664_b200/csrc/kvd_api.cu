@@ -909,6 +909,7 @@ static kvd_status build_attn_launch(kvd_ctx *ctx, const LayerState &ls, int b0, 
                                     void *out, const int *pre_parts, AttnLaunch &L) {
   const kvd_model_desc &d = ctx->desc;
   int parts = 0, slots = 0;
+  L.tail = pre_parts != nullptr;
   for (int i = 0; i < nb; ++i) {
     const int b = b0 + i;
     AttnSeq &S = L.seq[i];
@@ -949,6 +950,7 @@ static kvd_status build_attn_launch(kvd_ctx *ctx, const LayerState &ls, int b0, 
       const int ck = attn_chunk_keys(d.d_head, S.iters);
       S.chunk0_pos = lo / ck * ck;
       S.n_chunks = hi / ck - lo / ck + 1;
+      L.tail = L.tail && hi - lo < AT_TAIL_KEYS;
     }
     const int pre = pre_parts ? pre_parts[b] : 0;
     S.merge_base = slots;
@@ -956,6 +958,21 @@ static kvd_status build_attn_launch(kvd_ctx *ctx, const LayerState &ls, int b0, 
     S.merge_count = pre + S.n_chunks;
     slots += S.merge_count;
     parts += S.n_chunks;
+  }
+  // Behind a fused recompute a handful of live keys (the new token's, as a rule) is no streaming launch: the merge kernel
+  // takes them beside the partials it fetches.  FP8 step with a streaming launch for the one key / without, us: Gemma-3-4B layer,
+  // 4096 rows 31.0 / 27.3, Qwen3-4B layer 4 x 2000 59 / 55.5.  (Every key there is a round of shuffles in one warp; a sequence
+  // with more than AT_TAIL_KEYS sends the whole launch through the streaming kernel.)
+  L.tail = L.tail && parts > 0;
+  if (L.tail) {
+    parts = slots = 0;
+    for (int i = 0; i < nb; ++i) {
+      AttnSeq &S = L.seq[i];
+      S.n_chunks = S.part_base = 0;
+      S.merge_base = S.slot_base = slots;
+      S.merge_count = pre_parts[b0 + i];
+      slots += S.merge_count;
+    }
   }
   if (slots > ctx->max_parts) return KVD_ERR_CAPACITY;
   const float sc = scale > 0.f ? scale : 1.0f / sqrtf(static_cast<float>(d.d_head));

@@ -18,6 +18,7 @@
 #include <string.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "kvd_internal.h"
 #include "kvd_ptx.cuh"
@@ -645,10 +646,14 @@ __global__ void __launch_bounds__(AT_THREADS, SLOTS == 3 ? AT_CTAS_PER_SM : 3)
 // launch has as many warps per CTA as its longest sequence has groups (at most 16; beyond that a warp
 // takes several groups, 16 apart); a shorter sequence leaves the extra warps idle, so its summation
 // order depends on its own chunk count only.
-template <int D_HEAD, int G, int NSEQ, int DT, int GH>
+//
+// TAIL (behind a fused recompute with a few live keys): one more warp attends the sequence's live keys, of which there are
+// AT_TAIL_KEYS at most, while the others fetch their partials; the two are put together at the end.
+template <int D_HEAD, int G, int NSEQ, int DT, int GH, bool TAIL>
 __global__ void __launch_bounds__(AT_MERGE_THREADS)
     kvd_attn_merge_kernel(const __grid_constant__ AttnLaunchT<NSEQ> P) {
   constexpr int SLICES = D_HEAD / AT_MERGE_SLICE;
+  constexpr int MAX_WARPS = AT_MERGE_WARPS - (TAIL ? 1 : 0);
   constexpr int PF = attn_merge_group(G);
   // of every warp of the CTA: outputs [GH][AT_MERGE_SLICE] and sums [GH] (as much as the launch's warps need: the kernel's
   // loads in flight pass through the L1, which shared memory is taken from: 64 x 3000 keys of a Qwen3-4B layer 15.8 -> 12.5 us,
@@ -656,6 +661,7 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
   extern __shared__ float at_merge_smem[];
   float (*s_o)[GH][AT_MERGE_SLICE] = reinterpret_cast<float (*)[GH][AT_MERGE_SLICE]>(at_merge_smem);
   float (*s_l)[GH] = reinterpret_cast<float (*)[GH]>(at_merge_smem + blockDim.x / 32 * GH * AT_MERGE_SLICE);
+  float *s_max = at_merge_smem + blockDim.x / 32 * GH * (AT_MERGE_SLICE + 1);  // TAIL: maxima of the partials [GH], of the keys [GH]
   const int slice = blockIdx.x % SLICES;
   const int head_slot = blockIdx.x / SLICES;
   const int si = head_slot / (P.n_q / GH), head0 = head_slot % (P.n_q / GH) * GH;  // sequence, first query head
@@ -669,7 +675,7 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
   // (checking build: the slots to merge lie inside the partial arrays; otherwise nothing is merged)
   const int count = KVD_BOUNDS_OK(S.merge_base >= 0 && S.merge_base + S.merge_count <= P.max_parts, P.status) ? S.merge_count : 0;
   const int n_groups = (count + PF - 1) / PF;
-  const int warps_used = n_groups < AT_MERGE_WARPS ? n_groups : AT_MERGE_WARPS;
+  const int warps_used = n_groups < MAX_WARPS ? n_groups : MAX_WARPS;
   const float *ml0 = P.part_ml + (static_cast<size_t>(S.merge_base) * P.n_q + head0) * 2;
   const float *po0 = P.part_o + (static_cast<size_t>(S.merge_base) * P.n_q + head0) * D_HEAD +
                      slice * AT_MERGE_SLICE + lane * 2;
@@ -705,6 +711,7 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
 #pragma unroll
       for (int msk = 16; msk >= 1; msk >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, msk));
       Mu[g] = (mx == -CUDART_INF_F) ? 0.f : mx;
+      if (TAIL && warp == 0 && lane == 0) s_max[g] = mx;
     }
     float2 o[GH];
     float l[GH];
@@ -713,7 +720,7 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
       l[g] = 0.f;
       o[g] = make_float2(0.f, 0.f);
     }
-    for (int grp = warp; grp < n_groups; grp += AT_MERGE_WARPS) {
+    for (int grp = warp; grp < n_groups; grp += MAX_WARPS) {
       if (grp != warp) fetch_group(grp);
 #pragma unroll
       for (int i = 0; i < PF; ++i) {
@@ -735,6 +742,75 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
       s_o[warp][g][lane * 2 + 1] = o[g].y;
     }
   }
+  const int tail_warp = static_cast<int>(blockDim.x / 32) - 1;
+  if constexpr (TAIL) {
+    if (warp == tail_warp) {
+      constexpr int EPL = D_HEAD / 32, W = EPL / 4;  // channels per lane, 8-byte words of them
+      const int n_keys = S.hi_pos - S.lo_pos + 1;    // (not positive where no live key is visible)
+      const __nv_bfloat16 *kl = nullptr, *vl = nullptr;
+      if (lane < n_keys) key_rows(S, S.lo_pos + lane, static_cast<size_t>(head0 / G) * D_HEAD, kl, vl);
+      const uint32_t held = __ballot_sync(0xffffffffu, kl != nullptr);
+      uint2 kr[AT_TAIL_KEYS][W];
+      uint32_t vr[AT_TAIL_KEYS];
+#pragma unroll
+      for (int j = 0; j < AT_TAIL_KEYS; ++j) {
+        const __nv_bfloat16 *kp = lane_ptr(kl, j) + lane * EPL, *vp = lane_ptr(vl, j) + slice * AT_MERGE_SLICE + lane * 2;
+        vr[j] = 0u;
+#pragma unroll
+        for (int w = 0; w < W; ++w) kr[j][w] = make_uint2(0u, 0u);
+        if ((held >> j) & 1u) {
+#pragma unroll
+          for (int w = 0; w < W; ++w) kr[j][w] = __ldcg(reinterpret_cast<const uint2 *>(kp) + w);
+          vr[j] = __ldcg(reinterpret_cast<const uint32_t *>(vp));
+        }
+      }
+#pragma unroll
+      for (int g = 0; g < GH; ++g) {
+        const uint2 *qp = reinterpret_cast<const uint2 *>(P.q + (static_cast<size_t>(si) * P.n_q + head0 + g) * D_HEAD + lane * EPL);
+        float sc[AT_TAIL_KEYS], mx = -CUDART_INF_F;
+        uint2 qw[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) qw[w] = __ldcg(qp + w);
+#pragma unroll
+        for (int j = 0; j < AT_TAIL_KEYS; ++j) {
+          sc[j] = -CUDART_INF_F;
+          if ((held >> j) & 1u) {
+            uint64_t dot = 0ull;
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+              dot = ffma2(x2_to_f32x2<DT>(qw[w].x), x2_to_f32x2<DT>(kr[j][w].x), dot);
+              dot = ffma2(x2_to_f32x2<DT>(qw[w].y), x2_to_f32x2<DT>(kr[j][w].y), dot);
+            }
+            float even, odd;
+            unpack2(dot, even, odd);
+            float t = even + odd;
+#pragma unroll
+            for (int msk = 16; msk >= 1; msk >>= 1) t += __shfl_xor_sync(0xffffffffu, t, msk);
+            sc[j] = t * P.scale_log2e;
+            mx = fmaxf(mx, sc[j]);
+          }
+        }
+        float l = 0.f;
+        uint64_t o = 0ull;
+#pragma unroll
+        for (int j = 0; j < AT_TAIL_KEYS; ++j)
+          if ((held >> j) & 1u) {
+            const float w = exp2f(sc[j] - mx);
+            l += w;
+            o = ffma2(pack2(w, w), x2_to_f32x2<DT>(vr[j]), o);
+          }
+        float o0, o1;
+        unpack2(o, o0, o1);
+        if (lane == 0) {
+          s_max[GH + g] = mx;
+          s_l[warp][g] = l;
+          if (warps_used == 0) s_max[g] = -CUDART_INF_F;
+        }
+        s_o[warp][g][lane * 2] = o0;
+        s_o[warp][g][lane * 2 + 1] = o1;
+      }
+    }
+  }
   __syncthreads();
   // the warp sums are added in warp order
   for (int idx = threadIdx.x; idx < GH * AT_MERGE_SLICE; idx += blockDim.x) {
@@ -743,6 +819,12 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
     for (int w = 0; w < warps_used; ++w) {
       ov += s_o[w][g][c];
       lv += s_l[w][g];
+    }
+    if constexpr (TAIL) {
+      const float mp = s_max[g], mk = s_max[GH + g], mt = fmaxf(mp, mk);
+      const float wp = mp == -CUDART_INF_F ? 0.f : exp2f(mp - mt), wk = mk == -CUDART_INF_F ? 0.f : exp2f(mk - mt);
+      ov = ov * wp + s_o[tail_warp][g][c] * wk;
+      lv = lv * wp + s_l[tail_warp][g] * wk;
     }
     const float r = lv > 0.f ? ov / lv : 0.f;
     const size_t oi = (static_cast<size_t>(si) * P.n_q + head0 + g) * D_HEAD + slice * AT_MERGE_SLICE + c;
@@ -834,12 +916,23 @@ static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t str
   int max_chunks = 1;
   for (int i = 0; i < S.n_seqs; ++i) max_chunks = S.seq[i].merge_count > max_chunks ? S.seq[i].merge_count : max_chunks;
   int merge_warps = (max_chunks + attn_merge_group(G) - 1) / attn_merge_group(G);
-  if (merge_warps > AT_MERGE_WARPS) merge_warps = AT_MERGE_WARPS;
+  // (the heads the fused recompute exists for)
+  constexpr bool TAILS = (D_HEAD == 256 && G <= 2) || (D_HEAD == 128 && (G <= 2 || G == 4));
+  const int most = AT_MERGE_WARPS - (S.tail ? 1 : 0);
+  if (merge_warps > most) merge_warps = most;
+  if (S.tail) merge_warps += 1;
   cfg.blockDim = dim3(32 * merge_warps, 1, 1);
   auto merge = [&](auto kern, int heads) {
     cfg.gridDim = dim3(S.n_seqs * (S.n_q / heads) * (D_HEAD / AT_MERGE_SLICE), 1, 1);
-    cfg.dynamicSmemBytes = merge_warps * heads * (AT_MERGE_SLICE + 1) * sizeof(float);
+    cfg.dynamicSmemBytes = (merge_warps * (AT_MERGE_SLICE + 1) + 2) * heads * sizeof(float);
     return cudaLaunchKernelEx(&cfg, kern, S);
+  };
+  auto merge_by = [&](auto heads_c) {
+    constexpr int GH = decltype(heads_c)::value;
+    if constexpr (TAILS) {
+      if (S.tail) return merge(kvd_attn_merge_kernel<D_HEAD, G, NSEQ, DT, GH, true>, GH);
+    }
+    return merge(kvd_attn_merge_kernel<D_HEAD, G, NSEQ, DT, GH, false>, GH);
   };
   // A CTA per query head as long as the SMs hold all of their warps at once: a CTA of a whole group issues G times the loads
   // from one SM while most SMs have no CTA.  us, group / head: SmolLM2 step 3.4 / 1.9, Qwen3-4B layer 1 x 30000 7.0 / 5.1, 8 x 2000
@@ -847,9 +940,9 @@ static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t str
   // Gemma 64 x 1000 3.6 / 4.3, Qwen 64 x 3000 12.9 / 13.3.
   if constexpr (G > 1) {
     if (S.n_seqs * S.n_q * (D_HEAD / AT_MERGE_SLICE) * merge_warps <= 148 * AT_MERGE_WARPS)
-      return merge(kvd_attn_merge_kernel<D_HEAD, G, NSEQ, DT, 1>, 1);
+      return merge_by(std::integral_constant<int, 1>());
   }
-  return merge(kvd_attn_merge_kernel<D_HEAD, G, NSEQ, DT, G>, G);
+  return merge_by(std::integral_constant<int, G>());
 }
 
 template <int D_HEAD, int G, int NSEQ>
@@ -1064,7 +1157,7 @@ extern "C" kvd_status kvd_decode_attention_static(int n_q_heads, int n_kv_heads,
   L.part_o = reinterpret_cast<float *>(scratch + ml_bytes);
   L.status = nullptr;
   L.max_parts = parts;
-  L.early_split = L.early_merge = false;
+  L.early_split = L.early_merge = L.tail = false;
   switch (d_head) {
     case 64: return static_launch_d<64>(L, group, stream);
     case 128: return static_launch_d<128>(L, group, stream);

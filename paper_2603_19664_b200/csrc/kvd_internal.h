@@ -158,6 +158,7 @@ constexpr int AT_CTAS_PER_SM = 4;      // 128 registers per thread
 constexpr int AT_MERGE_THREADS = 640;  // merge kernel: at most 20 warps (102 registers each)
 constexpr int AT_MERGE_WARPS = 20;
 constexpr int AT_MERGE_SLICE = 64;     // channels per merge CTA
+constexpr int AT_TAIL_KEYS = 8;        // live keys per sequence that the merge kernel takes itself, behind a fused recompute
 // partials one warp of the merge kernel fetches at once: 4*G registers each, 64 registers in all
 constexpr int attn_merge_group(int g) { return 16 / g >= 1 ? 16 / g : 1; }
 constexpr int AT_UNROLL = 8;          // keys per lane group per iteration
@@ -197,6 +198,7 @@ struct AttnLaunchHead {
   int *status;             // device status word (nullptr: none), used by the checking build
   int max_parts;           // slots the partial arrays hold
   bool early_split, early_merge;  // this kernel starts early whatever the grid
+  bool tail;               // the merge kernel attends the live keys itself (at most AT_TAIL_KEYS per sequence)
 };
 template <int NSEQ>
 struct AttnLaunchT : AttnLaunchHead {
