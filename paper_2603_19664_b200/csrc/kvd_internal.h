@@ -44,6 +44,7 @@ constexpr int RC_INLINE_STAT_ROWS = 64;
 constexpr int RC_TRACE_TILES = 8;    // tiles per CTA recorded when a trace buffer is attached
 constexpr int RC_TRACE_FIELDS = 16;  // int64 slots per (CTA, tile); see kvd_set_trace
 constexpr int RC_THREADS = 320;  // warp 2 TMA, warp 3 MMA, warps 0,1,8,9 row statistics, warps 4-7 epilogue
+constexpr int RC_THREADS_8 = 384;  // with two epilogue groups: warps 0,1 row statistics, 4-7 and 8-11 epilogue (168 registers, as with 320)
 
 // store slots of the rows of kvd_checkpoint_residual_step (one new row per sequence of a batch)
 struct CkptSlots {

@@ -47,6 +47,12 @@
 //           channels, the MMA kind is f8f6f4; the scales ride in the per-row factor of the epilogue.
 //           Combines with FG > 0 (kvd_decode_attention_recompute_fp8).
 //   DT = 1  fp16 rows, weights and outputs (kvd_set_dtype), plain variant only.
+//   EPI = 8 two epilogue groups (warps 4-7 and 8-11; rows' statistics by warps 0 and 1): launches whose key tiles' epilogues
+//           nothing overlaps, and the fused FP8 variant, whose main loop is shorter than they are.  Groups take the heads of
+//           a tile in turns, or half of the columns where it has one head (both add up the key norm, for the same bits), in
+//           the fused variant half of the rows of a value tile.  us, one / two groups: 837 rows of a Gemma-3-4B layer 24.9 /
+//           22.5; FP8 step 4096 rows 24.2 / 22.9, Qwen3-4B layer 4 x 2000 48.4 / 44.3.  Beyond two tiles per cluster of
+//           bf16 rows the other warps' instructions cost 1 to 2 %: one group there.
 #include <math_constants.h>
 #include <string.h>
 
@@ -67,7 +73,7 @@ namespace kvd {
 // epilogues are exposed (one tile per cluster; the FP8 variant, whose main loop is shorter than that
 // epilogue; the fused variant, which has given a stage away already) take LOSM, the others the seventh
 // stage.  The arithmetic is the same either way.
-template <int BLOCK_N, int D_HEAD, int FG = 0, bool LOSM = false>
+template <int BLOCK_N, int D_HEAD, int FG = 0, bool LOSM = false, int EPI = 4>
 struct RcCfg {
   static constexpr bool FUSED = FG > 0;
   static_assert(!FUSED || LOSM, "the fused variant keeps the low table in shared memory");
@@ -79,13 +85,14 @@ struct RcCfg {
   static constexpr int TMEM_COLS = 2 * BLOCK_N;
   // barriers: full[S] (used in the even CTA), empty[S], tmem_full[2], tmem_empty[2], stats_full[2], rstd_free[2]
   // + stats_x (the four statistics warps among themselves); fused: + scores[2] (both CTAs' epilogue
-  // threads), epi (the four epilogue warps among themselves)
-  static constexpr int NUM_BARS = 2 * STAGES + 9 + (FUSED ? 3 : 0);
+  // threads), epi (the epilogue warps among themselves), half[2] (what the second epilogue group hands to the first)
+  static constexpr int NUM_BARS = 2 * STAGES + 9 + (FUSED ? 5 : 0);
   static constexpr int BAR_BYTES = (NUM_BARS * 8 + 15) / 16 * 16;
   // fused: scores / weights [2 units][heads of the tile x FG][256 rows of the pair], 1/rms of the 256 rows
-  // [2 units][256], partial sums of the weights [heads x FG][4 warps]
+  // [2 units][256], partial sums of the weights [heads x FG][EPI warps]
   static constexpr int GT = (BLOCK_N / D_HEAD) * (FUSED ? FG : 0);
-  static constexpr int FUSED_BYTES = FUSED ? (2 * GT * 256 + 2 * 256 + GT * 4) * 4 : 0;
+  // with two epilogue groups also what the second hands over: score parts of a split head, sums over its rows [FG][128] each
+  static constexpr int FUSED_BYTES = FUSED ? (2 * GT * 256 + 2 * 256 + GT * EPI + (EPI == 8 ? 2 * FG * 128 : 0)) * 4 : 0;
   static constexpr int LO_BYTES = LOSM ? (D_HEAD / 2) * ROPE_LO_SIZE * 8 : 0;
   static constexpr int TAIL_BYTES = BAR_BYTES + 16 /*tmem ptr, abort*/ + 2 * RC_BLOCK_M * 4 /*rstd*/ + 256 * 4 /*gamma_k*/ + FUSED_BYTES + LO_BYTES;
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + TAIL_BYTES;  // the base must be 1024-byte aligned
@@ -169,13 +176,13 @@ KVD_DEFINE_UMMA_KBLOCK(umma_kblock_pair_tf32, "tf32")  // fp32 operands read as 
 // weights; a k block is then 128 channels in the same 128-byte rows, the MMA kind f8f6f4, and the rows'
 // and the matrix's quantisation scales ride in the per-row factor that the statistics warps hand over).
 // DT = 1: fp16 rows, weights and outputs instead of bf16 (plain variant only).
-template <int BLOCK_N, int D_HEAD, bool TRACE, int FG, int EB = 2, bool LOSM = (FG > 0), int DT = 0>
-__global__ void __launch_bounds__(RC_THREADS, 1)
+template <int BLOCK_N, int D_HEAD, bool TRACE, int FG, int EB = 2, bool LOSM = (FG > 0), int DT = 0, int EPI = 4>
+__global__ void __launch_bounds__(EPI == 8 ? RC_THREADS_8 : RC_THREADS, 1)
 kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __grid_constant__ CUtensorMap tmap_rows,
                      const __grid_constant__ CUtensorMap tmap_b, const __grid_constant__ CUtensorMap tmap_b_part,
                      const __grid_constant__ RecomputeParams p,
                      const __grid_constant__ std::conditional_t<(FG > 0), FusedParams, NoFusedParams> f) {
-  using Cfg = RcCfg<BLOCK_N, D_HEAD, FG, LOSM>;
+  using Cfg = RcCfg<BLOCK_N, D_HEAD, FG, LOSM, EPI>;
   constexpr int STAGES = Cfg::STAGES;
   constexpr bool FUSED = FG > 0;
   static_assert(DT == 0 || (DT == 1 && EB == 2) || (DT == 2 && EB == 4 && FG == 0),
@@ -183,6 +190,10 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
   constexpr int EW = DT == 2 ? 2 : 1;  // 16-bit units per output element (output pointers count 16-bit units)
   constexpr int KB_ELEMS = RC_BLOCK_K * 2 / EB;  // channels per k block
   static_assert(BLOCK_N % D_HEAD == 0, "a tile must hold whole heads");
+  constexpr int SW = EPI == 8 ? 2 : 4, SR = 4 / SW;  // statistics warps, rows of a thread of theirs
+  constexpr int GROUPS = EPI / 4;  // epilogue groups: heads in turns, or where a tile has one head half of its columns each
+  constexpr bool SPLIT_HEAD = GROUPS == 2 && BLOCK_N == D_HEAD;
+  constexpr uint32_t SCORERS = SPLIT_HEAD || GROUPS == 1 ? 256 : 512;
 
   extern __shared__ __align__(1024) uint8_t smem[];
   // the 128-byte swizzle pattern is anchored at 1024-byte boundaries; there is no slack to realign
@@ -198,9 +209,10 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
   float *s_gamma_k = s_rstd + 2 * RC_BLOCK_M;
   float *s_sc = s_gamma_k + 256;                 // fused: [2][GT][256]
   float *s_rall = s_sc + 2 * Cfg::GT * 256;      // fused: [2][256]
-  float *s_lsum = s_rall + 2 * 256;              // fused: [GT][4]
+  float *s_lsum = s_rall + 2 * 256;              // fused: [GT][EPI]
+  float *s_half = s_lsum + Cfg::GT * EPI;        // fused, two epilogue groups: [2][FG][128]
   // LOSM: the low rotation table [pair][16], behind whatever precedes it in this variant's tail
-  float2 *s_lo = reinterpret_cast<float2 *>(FUSED ? s_lsum + Cfg::GT * 4 : s_gamma_k + 256);
+  float2 *s_lo = reinterpret_cast<float2 *>(FUSED ? s_half + (EPI == 8 ? 2 * FG * 128 : 0) : s_gamma_k + 256);
 
   const uint32_t smem_base = smem_u32(smem);
   const uint32_t bar_base = smem_u32(bars);
@@ -213,6 +225,7 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
   const uint32_t bar_stats_x = bar_base + 8u * (2 * STAGES + 8);
   auto bar_scores = [&](int u) { return bar_base + 8u * (2 * STAGES + 9 + u); };  // fused only
   const uint32_t bar_epi = bar_base + 8u * (2 * STAGES + 11);                       // fused only
+  auto bar_half = [&](int i) { return bar_base + 8u * (2 * STAGES + 12 + i); };     // fused, two epilogue groups
   const uint32_t cta_rank = cluster_ctarank();  // 0: issues the MMAs, 1: its partner
   const int cluster_id = static_cast<int>(blockIdx.x >> 1);
   const int num_clusters = static_cast<int>(gridDim.x >> 1);
@@ -289,15 +302,15 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(bar_tmem_full(a), 1);
-      mbar_init(bar_tmem_empty(a), 8);           // one arrival per epilogue warp of both CTAs
-      mbar_init(bar_stats_full(a), RC_BLOCK_M);  // one arrival per statistics thread
-      mbar_init(bar_rstd_free(a), 4);            // one arrival per local epilogue warp
+      mbar_init(bar_tmem_empty(a), 2 * EPI);     // one arrival per epilogue warp of both CTAs
+      mbar_init(bar_stats_full(a), 32 * SW);     // one arrival per statistics thread
+      mbar_init(bar_rstd_free(a), EPI);          // one arrival per local epilogue warp
     }
-    mbar_init(bar_stats_x, 4);  // one arrival per statistics warp
+    mbar_init(bar_stats_x, SW);  // one arrival per statistics warp
     if (FUSED) {
-      mbar_init(bar_scores(0), 256);  // one arrival per epilogue thread of both CTAs
-      mbar_init(bar_scores(1), 256);
-      mbar_init(bar_epi, 4);          // one arrival per local epilogue warp
+      for (int u = 0; u < 2; ++u) mbar_init(bar_scores(u), SCORERS);  // one arrival per thread of both CTAs that makes scores
+      mbar_init(bar_epi, EPI);        // one arrival per local epilogue warp
+      for (int i = 0; i < 2; ++i) mbar_init(bar_half(i), 4);  // one arrival per warp of the second group
     }
     *s_abort = 0;
     fence_mbar_init();
@@ -311,7 +324,7 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
     // (written at kvd_set_layer time: may be read before the dependency wait below)
     const uint4 *src = reinterpret_cast<const uint4 *>(p.rope_lo);
     uint4 *dstl = reinterpret_cast<uint4 *>(s_lo);
-    for (int i = threadIdx.x; i < Cfg::LO_BYTES / 16; i += RC_THREADS) dstl[i] = __ldg(src + i);
+    for (int i = threadIdx.x; i < Cfg::LO_BYTES / 16; i += blockDim.x) dstl[i] = __ldg(src + i);
   }
   if (warp == 3) {
     tmem_alloc_pair(smem_u32(s_tmem), Cfg::TMEM_COLS);
@@ -471,15 +484,14 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
         }
       }
     }
-  } else if (warp < 2 || warp >= 8) {
+  } else if (warp < 2 || (EPI == 4 && warp >= 8)) {
     // ------------------------------------------------------------------ row statistics (Eq. 2)
-    const int w4 = warp < 2 ? warp : warp - 6;  // warps 0, 1, 8, 9 -> rows 32 * w4 .. 32 * w4 + 31
-    const int row = w4 * 32 + lane;
+    const int w4 = warp < 2 ? warp : warp - 6;  // warps 0, 1, 8, 9 -> rows 32 * SR * w4 + 32 * i + lane
     int a = 0;
     uint32_t aph = 0;
     int job, m0, n0_, width_;
     bool first_of_unit;
-    float rstd_row = 0.f;  // of this thread's row, kept for the other tiles of the unit
+    float rstd_row[SR] = {};  // of this thread's rows, kept for the other tiles of the unit
     uint32_t xph = 0;      // phase of the statistics warps' own barrier
     for (int ti = 0; tile_at(ti, job, m0, n0_, width_, first_of_unit); ++ti) {
       const long long st0 = TRACE ? clock64() : 0;
@@ -495,12 +507,16 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
         if (J.sumsq != nullptr) {
           // checkpointed rows (or caller rows whose statistics a kernel of their own took): the sum of
           // squares is read back
-          const float sum = row < n_here ? J.sumsq[m0 + row] : 0.f;
-          rstd_row = 1.0f / sqrtf(sum * p.inv_d_hidden + p.rms_eps);
-          // FP8 rows: the accumulator is a sum of code products; row scale and matrix scale go with 1/rms
-          if (EB == 1) rstd_row *= (row < n_here ? J.scale[m0 + row] : 0.f) * __ldg(p.w_scale);
+          // (FP8 rows: the accumulator is a sum of code products; row scale and matrix scale go with 1/rms)
+#pragma unroll
+          for (int i = 0; i < SR; ++i) {
+            const int row = (w4 * SR + i) * 32 + lane;
+            const float sum = row < n_here ? J.sumsq[m0 + row] : 0.f;
+            rstd_row[i] = 1.0f / sqrtf(sum * p.inv_d_hidden + p.rms_eps);
+            if (EB == 1) rstd_row[i] *= (row < n_here ? J.scale[m0 + row] : 0.f) * __ldg(p.w_scale);
+          }
         } else {
-          // a few caller rows: the four warps share them in groups of four rows (group g -> warp g % 4),
+          // a few caller rows: the warps share them in groups of four rows (group g -> warp g % SW),
           // leave 1/rms in s_rstd[a] and meet on a barrier before every thread picks up its own row.
           // Rows past the end of the job read the job's last row instead (no branch inside a group).
           const uint4 *base = reinterpret_cast<const uint4 *>(p.ext_rows) + static_cast<size_t>(m0) * p.row_chunks;
@@ -508,7 +524,7 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
           // (with their positions and statistics) into the store slots the host assigned to them
           const bool append = p.append_n > 0 && n0_ == 0;
 #pragma unroll 1
-          for (int g = w4; g < 32 && 4 * g < n_here; g += 4) {
+          for (int g = w4; g < 32 && 4 * g < n_here; g += SW) {
             const uint4 *src[4];
             uint4 *dst[4] = {nullptr, nullptr, nullptr, nullptr};
 #pragma unroll
@@ -538,10 +554,15 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
             break;
           }
           xph ^= 1u;
-          rstd_row = row < n_here ? s_rstd[a * RC_BLOCK_M + row] : 0.f;
+#pragma unroll
+          for (int i = 0; i < SR; ++i) {
+            const int row = (w4 * SR + i) * 32 + lane;
+            rstd_row[i] = row < n_here ? s_rstd[a * RC_BLOCK_M + row] : 0.f;
+          }
         }
       }
-      s_rstd[a * RC_BLOCK_M + row] = rstd_row;
+#pragma unroll
+      for (int i = 0; i < SR; ++i) s_rstd[a * RC_BLOCK_M + (w4 * SR + i) * 32 + lane] = rstd_row[i];
       mbar_arrive(bar_stats_full(a));
       if (TRACE && threadIdx.x == 0) {
         trace_put<TRACE>(p.trace, ti, 8, 0);
@@ -552,16 +573,17 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
         aph ^= 1u;
       }
     }
-  } else if (warp >= 4 && warp < 8) {
+  } else if (warp >= 4) {
     // ------------------------------------------------------------------ epilogue
     const int quarter = warp & 3;  // TMEM lanes [32*quarter, 32*quarter + 32) belong to this warp
+    const int part = GROUPS == 2 && warp >= 8 ? 1 : 0;  // of the two epilogue groups
     const int row = quarter * 32 + lane;
     const uint32_t lane_field = static_cast<uint32_t>(quarter * 32) << 16;
     constexpr int HALF = D_HEAD / 2;
     constexpr int NG = FUSED ? FG : 1;
     int a = 0;
     uint32_t aph = 0;
-    uint32_t sph[2] = {0u, 0u}, eph = 0;  // fused: phases of the score barriers and of the epilogue warps' barrier
+    uint32_t sph[2] = {0u, 0u}, eph = 0, hph[2] = {0u, 0u};  // fused: phases of the score, epilogue and hand-over barriers
     int job, m0, n0, width;
     bool first_of_unit;
     for (int ti = 0; tile_at(ti, job, m0, n0, width, first_of_unit); ++ti) {
@@ -613,9 +635,9 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
         // 256 rows.  out[ch] = sum_r w[r] * acc[ch][r] with w[r] = exp2(score[r] - max) / rms(x_r).
         constexpr int GT = Cfg::GT;
         constexpr int WPH = D_HEAD >= 128 ? 4 : D_HEAD / 32;  // local epilogue warps that share a head
-        constexpr int RPW = 256 / WPH;                          // rows whose weights each of them makes
+        constexpr int RPW = 256 / (WPH * GROUPS);               // rows whose weights each of them makes
         const int ch = static_cast<int>(cta_rank) * RC_BLOCK_M + row;
-        const int hh = ch / D_HEAD, cih = ch % D_HEAD, wi = quarter % WPH;
+        const int hh = ch / D_HEAD, cih = ch % D_HEAD, wi = quarter % WPH + part * WPH;
         float *sc = s_sc + (ubuf * GT + hh * NG) * 256;
         const float *ra = s_rall + ubuf * 256;
         auto epi_sync = [&]() -> bool {
@@ -657,7 +679,7 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
           }
 #pragma unroll
           for (int msk = 16; msk >= 1; msk >>= 1) lp += __shfl_xor_sync(0xffffffffu, lp, msk);
-          if (lane == 0) s_lsum[(hh * NG + g) * 4 + wi] = lp;
+          if (lane == 0) s_lsum[(hh * NG + g) * EPI + wi] = lp;
         }
         if (!epi_sync()) {
           raise(p.status, STATUS_TIMEOUT, s_abort);
@@ -667,7 +689,7 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
         for (int g = 0; g < NG; ++g) {
           float l = 0.f;
 #pragma unroll
-          for (int w = 0; w < WPH; ++w) l += s_lsum[(hh * NG + g) * 4 + w];
+          for (int w = 0; w < WPH * GROUPS; ++w) l += s_lsum[(hh * NG + g) * EPI + w];
           lsum[g] = l;
           o[g] = 0.f;
         }
@@ -675,7 +697,7 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
         // their weight is zero, but 0 * NaN is not, so those columns are skipped or zeroed
         const int nvalid = J.n - (m0 - static_cast<int>(cta_rank) * RC_BLOCK_M);
 #pragma unroll 1
-        for (int c8 = 0; c8 < 8 && c8 * 32 < nvalid; ++c8) {
+        for (int c8 = part * (8 / GROUPS); c8 < (part + 1) * (8 / GROUPS) && c8 * 32 < nvalid; ++c8) {
           uint32_t r[32];
           tmem_ld_x32(acc + c8 * 32, r);
           tmem_wait_ld();
@@ -696,7 +718,25 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
             }
           }
         }
+        if constexpr (GROUPS == 2) {  // the second group's half of the rows
+          float *hand = s_half + NG * 128;
+          if (part == 1) {
+#pragma unroll
+            for (int g = 0; g < NG; ++g) hand[g * 128 + row] = o[g];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_half(1));
+          } else {
+            if (!warp_wait(bar_half(1), hph[1], s_abort, tmo, lane)) {
+              raise(p.status, STATUS_TIMEOUT, s_abort);
+              break;
+            }
+#pragma unroll
+            for (int g = 0; g < NG; ++g) o[g] += hand[g * 128 + row];
+          }
+          hph[1] ^= 1u;
+        }
         if constexpr (FUSED) {
+          if (part == 0) {
           const size_t slot = static_cast<size_t>(part_base) + (m0 - static_cast<int>(cta_rank) * RC_BLOCK_M) / (2 * RC_BLOCK_M);
           const int kvh = (n0 - p.k_cols) / D_HEAD + hh;
 #pragma unroll
@@ -705,18 +745,21 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
             f.part_o[qh * D_HEAD + cih] = o[g];
             if (cih == 0) *reinterpret_cast<float2 *>(f.part_ml + qh * 2) = make_float2(mx[g], lsum[g]);
           }
+          }
         }
       } else {
 
+      // (two groups: the heads of a tile in turns; a single head, whole or a part of a value head, by halves of its columns)
 #pragma unroll 1
-      for (int hh = 0; hh * D_HEAD < width; ++hh) {
+      for (int hh = width > D_HEAD ? part : 0; hh * D_HEAD < width; hh += width > D_HEAD ? GROUPS : 1) {
         const int col0 = n0 + hh * D_HEAD;  // first fused column of this head (or of this part of a value head)
         const uint32_t tcol = acc + hh * D_HEAD;
         if (col0 >= p.k_cols) {
           // ---- value head (Eq. 14): scale by 1/rms and store
           __nv_bfloat16 *dst = J.v_out + (static_cast<size_t>(m) * out_stride + (col0 - p.k_cols)) * EW;
+          const int n32 = (width < D_HEAD ? width : D_HEAD) / 32, whole_head = GROUPS == 1 || width > D_HEAD;
 #pragma unroll 1
-          for (int c = 0; c < (width < D_HEAD ? width : D_HEAD) / 32; ++c) {
+          for (int c = whole_head ? 0 : part * (n32 / 2); c < (whole_head ? n32 : (part + 1) * (n32 / 2)); ++c) {
             uint32_t r[32];
             tmem_ld_x32(tcol + c * 32, r);
             tmem_wait_ld();
@@ -761,17 +804,19 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
             const float ss = (s0 + s1) + (s2 + s3);
             kscale = rstd * (1.0f / sqrtf(ss * (1.0f / D_HEAD) + p.qk_eps));
           }
+          const bool halves = GROUPS == 2 && width <= D_HEAD;
           if (p.rope_style == KVD_ROPE_INTERLEAVED) {
             constexpr int NC = D_HEAD / 16;  // 16 columns = 8 rotation pairs per step
+            const int c0 = halves ? part * (NC / 2) : 0, c1 = halves ? c0 + NC / 2 : NC;
             float4 hn[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) hn[j] = t_hi[j];
+            for (int j = 0; j < 4; ++j) hn[j] = t_hi[c0 * 4 + j];
 #pragma unroll 1
-            for (int c = 0; c < NC; ++c) {
+            for (int c = c0; c < c1; ++c) {
               float4 h[4];
 #pragma unroll
               for (int j = 0; j < 4; ++j) h[j] = hn[j];
-              const int cn = c + 1 < NC ? c + 1 : c;  // prefetch the next step's table entries
+              const int cn = c + 1 < c1 ? c + 1 : c;  // prefetch the next step's table entries
 #pragma unroll
               for (int j = 0; j < 4; ++j) hn[j] = t_hi[cn * 4 + j];
               uint32_t r[16];
@@ -806,15 +851,16 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
             }
           } else {
             constexpr int NC = HALF / 16;  // 16 pairs (i, i + HALF) per step
+            const int c0 = halves ? part * (NC / 2) : 0, c1 = halves ? c0 + NC / 2 : NC;
             float4 hn[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) hn[j] = t_hi[j];
+            for (int j = 0; j < 8; ++j) hn[j] = t_hi[c0 * 8 + j];
 #pragma unroll 1
-            for (int c = 0; c < NC; ++c) {
+            for (int c = c0; c < c1; ++c) {
               float4 h[8];
 #pragma unroll
               for (int j = 0; j < 8; ++j) h[j] = hn[j];
-              const int cn = c + 1 < NC ? c + 1 : c;
+              const int cn = c + 1 < c1 ? c + 1 : c;
 #pragma unroll
               for (int j = 0; j < 8; ++j) hn[j] = t_hi[cn * 8 + j];
               uint32_t ra[16], rb[16];
@@ -858,20 +904,44 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
           if (FUSED && attend) {
             // the scores of this row (log2 units, -inf when the query does not see the key) go to both
             // CTAs of the pair: the value tile's epilogue needs those of all 256 rows
+            float sv[NG];
 #pragma unroll
             for (int g = 0; g < NG; ++g) {
               float lo, hi;
               unpack2(sdot[g], lo, hi);
-              float sv = (lo + hi) * f_scale;
-              if (!visible) sv = -CUDART_INF_F;
-              float *dstp = s_sc + (ubuf * Cfg::GT + hh * NG + g) * 256 + static_cast<int>(cta_rank) * RC_BLOCK_M + row;
-              *dstp = sv;
-              st_cluster_f32(map_to_cta(smem_u32(dstp), cta_rank ^ 1u), sv);
+              sv[g] = lo + hi;
+            }
+            if constexpr (SPLIT_HEAD) {  // the second group's half of the channels
+              if (part == 1) {
+#pragma unroll
+                for (int g = 0; g < NG; ++g) s_half[g * 128 + row] = sv[g];
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_half(0));
+              } else {
+                if (!warp_wait(bar_half(0), hph[0], s_abort, tmo, lane)) {
+                  raise(p.status, STATUS_TIMEOUT, s_abort);
+                  ok = false;
+                  break;
+                }
+#pragma unroll
+                for (int g = 0; g < NG; ++g) sv[g] += s_half[g * 128 + row];
+              }
+              hph[0] ^= 1u;
+            }
+            if (!SPLIT_HEAD || part == 0) {
+#pragma unroll
+              for (int g = 0; g < NG; ++g) {
+                const float sg = visible ? sv[g] * f_scale : -CUDART_INF_F;
+                float *dstp = s_sc + (ubuf * Cfg::GT + hh * NG + g) * 256 + static_cast<int>(cta_rank) * RC_BLOCK_M + row;
+                *dstp = sg;
+                st_cluster_f32(map_to_cta(smem_u32(dstp), cta_rank ^ 1u), sg);
+              }
             }
           }
         }
       }
-      if (FUSED && attend) {
+      if (!ok) break;
+      if (FUSED && attend && (!SPLIT_HEAD || part == 0)) {
         // 1/rms of the row, then "this thread's scores are in place" to both CTAs (a release at cluster
         // scope: the partner's value-tile epilogue reads what was just stored into its shared memory)
         float *rp = s_rall + ubuf * 256 + static_cast<int>(cta_rank) * RC_BLOCK_M + row;
@@ -912,12 +982,12 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
 }
 
 // ------------------------------------------------------------------------------ host launcher
-template <int BLOCK_N, int D_HEAD, bool TRACE, int FG, int EB = 2, bool LOSM = (FG > 0), int DT = 0>
+template <int BLOCK_N, int D_HEAD, bool TRACE, int FG, int EB = 2, bool LOSM = (FG > 0), int DT = 0, int EPI = 4>
 static kvd_status launch_impl(kvd_ctx *ctx, const LayerState &ls, const CUtensorMap &tmap_store,
                               const CUtensorMap &tmap_rows, const RecomputeParams &p, const FusedParams *fp,
                               cudaStream_t stream) {
-  using Cfg = RcCfg<BLOCK_N, D_HEAD, FG, LOSM>;
-  auto kern = kvd_recompute_kernel<BLOCK_N, D_HEAD, TRACE, FG, EB, LOSM, DT>;
+  using Cfg = RcCfg<BLOCK_N, D_HEAD, FG, LOSM, EPI>;
+  auto kern = kvd_recompute_kernel<BLOCK_N, D_HEAD, TRACE, FG, EB, LOSM, DT, EPI>;
   const CUtensorMap &tmap_b = EB == 1 ? ls.tmap_b8 : ls.tmap_b;
   const CUtensorMap &tmap_b_part = EB == 1 || p.parts <= 1 ? tmap_b : ls.tmap_b_part[p.parts == 2 ? 0 : 1];
   static bool configured[64] = {};
@@ -929,7 +999,7 @@ static kvd_status launch_impl(kvd_ctx *ctx, const LayerState &ls, const CUtensor
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(2 * p.clusters, 1, 1);
-  cfg.blockDim = dim3(RC_THREADS, 1, 1);
+  cfg.blockDim = dim3(EPI == 8 ? RC_THREADS_8 : RC_THREADS, 1, 1);
   cfg.dynamicSmemBytes = Cfg::SMEM_BYTES;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
@@ -958,9 +1028,9 @@ static kvd_status launch_sel(kvd_ctx *ctx, const LayerState &ls, const CUtensorM
     if (ctx->dtype == 1) return launch_impl<BLOCK_N, D_HEAD, false, 0, 2, true, 1>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
     if (ctx->dtype == 2) return launch_impl<BLOCK_N, D_HEAD, false, 0, 4, true, 2>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
     if (p.trace != nullptr) return launch_impl<BLOCK_N, D_HEAD, true, 0>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
-    // one tile per cluster at most: every key tile's epilogue is exposed -> the low table from shared memory
+    // one tile per cluster at most: every key tile's epilogue is exposed -> the low table from shared memory, two groups
     if (p.whole_tiles + (p.num_m_blocks * p.num_n_blocks - p.whole_tiles) * p.parts <= ctx->num_sms / 2)
-      return launch_impl<BLOCK_N, D_HEAD, false, 0, 2, true>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
+      return launch_impl<BLOCK_N, D_HEAD, false, 0, 2, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
   }
   // the fused variant on fp16 rows, weights, queries and outputs (same tiles, MMA kind f16 with fp16 operands)
   if constexpr (FG > 0) {
@@ -1035,11 +1105,11 @@ kvd_status launch_recompute_fused(kvd_ctx *ctx, const LayerState &ls, const CUte
   if (ctx->block_n != 256 || p.k_cols % 256 != 0) return KVD_ERR_UNSUPPORTED;
   if (eb == 1) {  // rows and weights as E4M3 codes (the FP8 store)
     if (dh == 256 && g == 2 && p.trace != nullptr) return launch_impl<256, 256, true, 2, 1>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
-    if (dh == 256 && g == 2) return launch_impl<256, 256, false, 2, 1>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
-    if (dh == 256 && g == 1) return launch_impl<256, 256, false, 1, 1>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
-    if (dh == 128 && g == 4) return launch_impl<256, 128, false, 4, 1>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
-    if (dh == 128 && g == 2) return launch_impl<256, 128, false, 2, 1>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
-    if (dh == 128 && g == 1) return launch_impl<256, 128, false, 1, 1>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
+    if (dh == 256 && g == 2) return launch_impl<256, 256, false, 2, 1, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
+    if (dh == 256 && g == 1) return launch_impl<256, 256, false, 1, 1, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
+    if (dh == 128 && g == 4) return launch_impl<256, 128, false, 4, 1, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
+    if (dh == 128 && g == 2) return launch_impl<256, 128, false, 2, 1, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
+    if (dh == 128 && g == 1) return launch_impl<256, 128, false, 1, 1, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
     return KVD_ERR_UNSUPPORTED;
   }
   if (dh == 256 && g == 2) return launch_sel<256, 256, 2>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
