@@ -114,6 +114,7 @@ __device__ __forceinline__ void trace_put(long long *trace, int tile_iter, int f
 // the partner CTA wrote.
 __device__ __forceinline__ bool warp_wait_cluster(uint32_t bar, uint32_t parity, const volatile int *abort_flag,
                                                   unsigned long long timeout_ns, int lane) {
+  if (__all_sync(0xffffffffu, mbar_try_wait_cluster(bar, parity))) return true;
   int ok = 1;
   if (lane == 0 && !mbar_try_wait_cluster(bar, parity)) {
     const unsigned long long t0 = globaltimer_ns();
@@ -625,6 +626,9 @@ kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __gri
       // in place of 16: 3 x 1000 rows of a Gemma-3-4B layer 30.2 -> 27.2 us, 2600 rows 29.9 -> 28.0, 4 x 2048 61.9 -> 59.2, FP8 step
       // 22.9 -> 21.8.  (The next step's columns asked for while one is rotated: 27.2 -> 28.4.)
       if (n0 < p.k_cols && (lane & 15) * 16 < HALF) touch(reinterpret_cast<const char *>(t_hi) + (lane & 15) * 128);
+      // (fused: likewise the queries that the rotated keys meet, 512 bytes of a tile's heads per query of a group: FP8 step, Qwen3-4B
+      // layer 4 x 2000, 51.9 -> 50.7 us, Gemma-3-4B layer 4096 rows 26.55 -> 26.3)
+      if (FUSED && attend && first_of_unit && lane < 4 * NG) touch(reinterpret_cast<const char *>(qrow + static_cast<size_t>(n0) * NG) + lane * 128);
       // warp-uniform outcome: tcgen05.ld below is an aligned instruction
       if (!warp_wait(bar_tmem_full(a), aph, s_abort, tmo, lane) || !warp_wait(bar_stats_full(a), aph, s_abort, tmo, lane)) {
         raise(p.status, STATUS_TIMEOUT, s_abort);
