@@ -959,6 +959,7 @@ static kvd_status build_attn_launch(kvd_ctx *ctx, const LayerState &ls, int b0, 
     slots += S.merge_count;
     parts += S.n_chunks;
   }
+  if (slots > ctx->max_parts) return KVD_ERR_CAPACITY;  // (also where the merge kernel takes live keys below: what is refused does not hang on it)
   // Behind a fused recompute a handful of live keys (the new token's, as a rule) is no streaming launch: the merge kernel
   // takes them beside the partials it fetches.  FP8 step with a streaming launch for the one key / without, us: Gemma-3-4B layer,
   // 4096 rows 31.0 / 27.3, Qwen3-4B layer 4 x 2000 59 / 55.5.  (Every key there is a round of shuffles in one warp; a sequence
@@ -974,7 +975,6 @@ static kvd_status build_attn_launch(kvd_ctx *ctx, const LayerState &ls, int b0, 
       slots += S.merge_count;
     }
   }
-  if (slots > ctx->max_parts) return KVD_ERR_CAPACITY;
   const float sc = scale > 0.f ? scale : 1.0f / sqrtf(static_cast<float>(d.d_head));
   L.n_seqs = nb;
   L.total_chunks = parts;
