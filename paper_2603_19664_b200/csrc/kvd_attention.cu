@@ -369,9 +369,9 @@ __global__ void __launch_bounds__(AT_THREADS, ALLIN ? 2 : AT_CTAS_PER_SM) kvd_at
 // so the two products run on the tensor cores with the query heads padded to a 16-row tile:
 //     S (16 heads x 8 keys)         = Q (16 x d_head) * K^T            mma.m16n8k16, d_head/16 per 8 keys
 //     O^T (d_head x 8 heads)       += V^T (d_head x 8 keys) * P^T      mma.m16n8k8,  d_head/16 per 8 keys
-// Operands come straight from global memory with the same 16-byte loads: a contraction does not care
-// which channel (or key) sits in which slot as long as both operands agree, so each thread loads
-// contiguous 16-byte pieces and uses them as the fragment registers the instruction wants -- K pieces
+// Operands are read from shared memory in contiguous 16-byte pieces: a contraction does not care which
+// channel (or key) sits in which slot as long as both operands agree, so each thread
+// uses its pieces as the fragment registers the instruction wants -- K pieces
 // as B fragments of the first product (the query is loaded the same way), pairs of V pieces of two
 // neighbouring keys, interleaved with two byte permutes, as A fragments of the second.  P is rounded
 // to bf16 for the second product (fp32 sums), as the scores' softmax weights are in any tensor-core

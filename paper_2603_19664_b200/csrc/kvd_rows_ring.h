@@ -12,8 +12,8 @@ constexpr int RW_MAX_STAGES = 16;
 constexpr int RW_BARS = 2 * RW_MAX_STAGES + 6;                   // full, empty per stage; tmem_full[2], tmem_empty[2], head, (16-byte multiple)
 constexpr int RW_TAIL = RW_BARS * 8 + 32 + RW_MAX_ROWS * 2 * 4;  // barriers, tmem pointer + abort, 1/rms, key scale
 constexpr int RW_SMEM_MAX = 232448;
-// Key and value heads leave an SM room for two CTAs of the streaming attention behind them (9 to 18 KB and 16 K registers
-// each; the kernel's launch bounds leave the registers), which take their places beside a CTA of this kernel and wait there
+// Key and value heads leave an SM room for two CTAs of the fp32 streaming attention behind them (9 to 18 KB and 16 K registers
+// each, the tensor-core kernel's 48 KB fit once up to RW_FEW_ROWS rows; the kernel's launch bounds leave the registers), which take their places beside a CTA of this kernel and wait there
 // instead of being started when it ends.  Up to RW_FEW_ROWS rows three stages of 8 k blocks do that: projection alone / step
 // with attention, us, two, three, four stages and all of an SM's shared memory: Gemma-3-4B layer 1 x 8192 8.8 / 22.3, 7.6 /
 // 21.1, 7.4 / 21.4, 7.4 / 24.0; 16 x 2048 8.3 / 38.3, 7.6 / 37.7, -, 7.7 / 40.0; Qwen3-4B layer 8 x 2048 -, 7.1 / 33.6, 7.2 /
