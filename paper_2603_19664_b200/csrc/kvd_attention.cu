@@ -792,10 +792,11 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
         }
         float l = 0.f;
         uint64_t o = 0ull;
+        const float m_use = (mx == -CUDART_INF_F) ? 0.f : mx;  // (keys that all score minus infinity weigh nothing)
 #pragma unroll
         for (int j = 0; j < AT_TAIL_KEYS; ++j)
           if ((held >> j) & 1u) {
-            const float w = exp2f(sc[j] - mx);
+            const float w = exp2f(sc[j] - m_use);
             l += w;
             o = ffma2(pack2(w, w), x2_to_f32x2<DT>(vr[j]), o);
           }

@@ -2,9 +2,12 @@
 of a streaming launch: around that limit, ragged batches, and windows that hide some or all of the recomputed keys.  Against
 the oracle and the two-call path, with the tolerance of the other fused tests."""
 import dataclasses
+import math
 
 import pytest
+import torch
 
+import paper_2603_19664_b200 as kvd
 from kvd_synth import GEMMA3_4B_GLOBAL, GEMMA3_4B_LOCAL, QWEN3_4B
 from test_gpu_fused import attn_check, run_case
 
@@ -25,3 +28,87 @@ def test_windows_over_the_live_keys(window):
     fused, two, ref = run_case(shape, [290, 513], 3, seed=window)
     attn_check(fused, ref, "fused vs oracle")
     attn_check(fused, two, "fused vs two-call")
+
+
+class Step:
+    """Fused steps over one small layer.  Sequence b: n_old[b] rows of the store at positions 0 .. n_old[b] - 1, live keys at
+    n_old[b] + live[b][i] (ascending; a gap begins another segment), the query at the last of all.  kind: bf16, f16 or fp8."""
+    D = 256
+
+    def __init__(self, layer, n_old, live, kind="bf16", rope=kvd.KVD_ROPE_INTERLEAVED, seed=0):
+        self.nq, self.nkv, self.dh = layer
+        self.n_old, self.live, self.kind, self.kdim = n_old, live, kind, layer[1] * layer[2]
+        self.dt, B = torch.float16 if kind == "f16" else torch.bfloat16, len(n_old)
+        self.desc = kvd.make_desc(1, self.D, *layer, 1e-6, True, 1e-6, rope, B, max(n_old) + 64, B)
+        self.c = kvd.Kvd(self.desc)
+        if kind == "f16":
+            self.c.kvd_set_dtype(1)
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        draw = lambda *s: torch.randn(s, generator=g, device="cuda").to(self.dt)  # noqa: E731
+        self.c.kvd_set_layer(0, draw(self.D, 2 * self.kdim) * self.D ** -0.5, 1 + 0.1 * draw(self.D), 1 + 0.1 * draw(self.dh), 1e4, 0)
+        self.c.kvd_attach_workspace(torch.empty(kvd.kvd_workspace_bytes(self.desc), dtype=torch.uint8, device="cuda"))
+        fp8 = kind == "fp8"
+        arena = torch.empty((kvd.kvd_store_bytes_fp8 if fp8 else kvd.kvd_store_bytes)(self.desc, 1), dtype=torch.uint8, device="cuda")
+        (self.c.kvd_attach_store_fp8 if fp8 else self.c.kvd_attach_store)(arena, 1)
+        self.q, self.k, self.v = draw(B, self.nq, self.dh), [draw(len(p), self.nkv, self.dh) for p in live], [draw(len(p), self.nkv, self.dh) for p in live]
+        self.rebuilt = []
+        for b, n in enumerate(n_old):
+            x, pos = draw(max(n, 1), self.D), torch.arange(max(n, 1), dtype=torch.int32, device="cuda")
+            kb, vb = (torch.empty((n, self.nkv, self.dh), dtype=self.dt, device="cuda") for _ in range(2))
+            if n:
+                (self.c.kvd_checkpoint_residual_fp8 if fp8 else self.c.kvd_checkpoint_residual)(b, 0, x, pos, n)
+                if fp8:
+                    self.c.kvd_recompute_kv_fp8(0, [(b, 0, n, kb, vb)], self.kdim)
+                else:
+                    self.c.kvd_recompute_kv(0, None, None, n, kb, vb, self.kdim, seq=b, first_row=0)
+            self.rebuilt.append((kb, vb))
+
+    def run(self, seqs=None):
+        """Output rows of a call over these sequences (all of them)."""
+        seqs = list(range(len(self.n_old))) if seqs is None else seqs
+        segs, q_pos = [], []
+        for b in seqs:
+            p, row = self.live[b], []
+            for i in range(len(p)):
+                if i == 0 or p[i] != p[i - 1] + 1:
+                    row.append([self.k[b][i:], self.v[b][i:], self.kdim, self.n_old[b] + p[i], 0])
+                row[-1][4] += 1
+            segs.append([tuple(s) for s in row])
+            q_pos.append(self.n_old[b] + p[-1] if p else max(self.n_old[b] - 1, 0))
+        q, ranges = self.q[seqs].contiguous(), [(b, 0, self.n_old[b]) for b in seqs]
+        out = torch.full_like(q, 9.0)
+        if self.kind == "fp8":
+            self.c.kvd_decode_attention_recompute_fp8(0, len(seqs), q, q_pos, ranges, [], self.kdim, segs, 0.0, out)
+        else:
+            self.c.kvd_decode_attention_recompute(0, len(seqs), q, q_pos, ranges, None, None, 0, None, None, self.kdim, segs, 0.0, out)
+        assert self.c.kvd_poll_status() == kvd.KVD_OK
+        return out
+
+    def check(self, out):
+        """Softmax attention in 64 bits over the keys and values that the library rebuilds (rounded to 16 bits) and the live
+        ones; a key that scores minus infinity weighs nothing.  Tolerance of the other attention tests."""
+        for b, row in enumerate(out):
+            k, v = (torch.cat((a, l)).double().repeat_interleave(self.nq // self.nkv, 1) for a, l in zip(self.rebuilt[b], (self.k[b], self.v[b])))
+            score = torch.einsum("hd,nhd->hn", self.q[b].double(), k) / math.sqrt(self.dh)
+            weight = torch.exp(score - score.amax(1, keepdim=True).clamp(min=-1e30))
+            total = weight.sum(1, keepdim=True)
+            want = torch.einsum("hn,nhd->hd", weight / torch.where(total > 0, total, 1.0), v)
+            err = (row.double() - want).abs()
+            assert err.norm() <= 1e-2 * want.norm() and err.max() <= 1e-2 * want.abs().max(), b
+
+
+GROUPS = {"2-256": (4, 2, 256), "1-256": (2, 2, 256), "4-128": (8, 2, 128), "2-128": (4, 2, 128), "1-128": (2, 2, 128)}  # all that the fused kernel exists for
+
+
+@pytest.mark.parametrize("kind", ["bf16", "f16", "fp8"])
+@pytest.mark.parametrize("layer", ["2-256", "4-128"])
+@pytest.mark.parametrize("n_old,live,lost", [
+    (300, [0], [0]), (300, [0, 1, 2], [0, 1, 2]), (300, [0, 1, 2], [1]), (700, list(range(8)), list(range(8))),
+    (300, list(range(9)), list(range(9))), (0, [0, 1], [0, 1])])  # (nine: through the streaming kernel; none rebuilt: zeros)
+def test_live_keys_that_score_minus_infinity(kind, layer, n_old, live, lost):
+    """An overflowed key (16-bit stores of keys overflow to infinity) weighs nothing, also where it is the only live one."""
+    s = Step(GROUPS[layer], [n_old], [live], kind)
+    s.q[:, :, 5] = s.q[:, :, 5].abs() + 0.5
+    for i in lost:
+        s.k[0][i, 0, 5] = -math.inf  # for the first KV head's queries
+    s.check(s.run())
