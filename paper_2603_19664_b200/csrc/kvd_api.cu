@@ -908,8 +908,8 @@ static kvd_status build_attn_launch(kvd_ctx *ctx, const LayerState &ls, int b0, 
                                     const int32_t *q_pos, const kvd_kv_segment *segs, int n_segs, float scale,
                                     void *out, const int *pre_parts, AttnLaunch &L) {
   const kvd_model_desc &d = ctx->desc;
-  int parts = 0, slots = 0;
-  L.tail = pre_parts != nullptr;
+  int parts = 0, slots = 0, streamed_slots = 0;
+  L.tail = false;
   for (int i = 0; i < nb; ++i) {
     const int b = b0 + i;
     AttnSeq &S = L.seq[i];
@@ -940,6 +940,8 @@ static kvd_status build_attn_launch(kvd_ctx *ctx, const LayerState &ls, int b0, 
     S.lo_pos = lo;
     S.hi_pos = hi;
     S.part_base = parts;
+    const int pre = pre_parts ? pre_parts[b] : 0;
+    streamed_slots += pre;
     if (max_last < 0 || hi < lo) {
       S.n_chunks = 0;
       S.iters = 1;
@@ -950,31 +952,24 @@ static kvd_status build_attn_launch(kvd_ctx *ctx, const LayerState &ls, int b0, 
       const int ck = attn_chunk_keys(d.d_head, S.iters);
       S.chunk0_pos = lo / ck * ck;
       S.n_chunks = hi / ck - lo / ck + 1;
-      L.tail = L.tail && hi - lo < AT_TAIL_KEYS;
+      streamed_slots += S.n_chunks;
+      // Behind a fused recompute a handful of live keys (the new token's, as a rule) is no work for the streaming kernel: the
+      // merge kernel takes them beside the partials it fetches (attn_tail).  FP8 step with a streaming launch for the one key /
+      // without, us: Gemma-3-4B layer, 4096 rows 31.0 / 27.3, Qwen3-4B layer 4 x 2000 59 / 55.5.  (Every key there is a round
+      // of shuffles in one warp.)  Each sequence by itself: what attends it does not depend on its neighbours.
+      if (pre_parts && hi - lo < AT_TAIL_KEYS) {
+        S.n_chunks = 0;
+        L.tail = true;
+      }
     }
-    const int pre = pre_parts ? pre_parts[b] : 0;
     S.merge_base = slots;
     S.slot_base = slots + pre;
     S.merge_count = pre + S.n_chunks;
     slots += S.merge_count;
     parts += S.n_chunks;
   }
-  if (slots > ctx->max_parts) return KVD_ERR_CAPACITY;  // (also where the merge kernel takes live keys below: what is refused does not hang on it)
-  // Behind a fused recompute a handful of live keys (the new token's, as a rule) is no streaming launch: the merge kernel
-  // takes them beside the partials it fetches.  FP8 step with a streaming launch for the one key / without, us: Gemma-3-4B layer,
-  // 4096 rows 31.0 / 27.3, Qwen3-4B layer 4 x 2000 59 / 55.5.  (Every key there is a round of shuffles in one warp; a sequence
-  // with more than AT_TAIL_KEYS sends the whole launch through the streaming kernel.)
-  L.tail = L.tail && parts > 0;
-  if (L.tail) {
-    parts = slots = 0;
-    for (int i = 0; i < nb; ++i) {
-      AttnSeq &S = L.seq[i];
-      S.n_chunks = S.part_base = 0;
-      S.merge_base = S.slot_base = slots;
-      S.merge_count = pre_parts[b0 + i];
-      slots += S.merge_count;
-    }
-  }
+  // (counted as if all live keys were streamed: what is refused does not hang on which kernel takes them)
+  if (streamed_slots > ctx->max_parts) return KVD_ERR_CAPACITY;
   const float sc = scale > 0.f ? scale : 1.0f / sqrtf(static_cast<float>(d.d_head));
   L.n_seqs = nb;
   L.total_chunks = parts;

@@ -643,17 +643,17 @@ __global__ void __launch_bounds__(AT_THREADS, SLOTS == 3 ? AT_CTAS_PER_SM : 3)
 // partials of its head group, each lane owning two channels of every head: a partial costs a lane 4*G
 // registers, a group is as many partials as fit 64 registers (attn_merge_group(G)), all fetched at
 // once, so a warp's work is one round trip to the L2; the warp results are added in warp order.  The
-// launch has as many warps per CTA as its longest sequence has groups (at most 16; beyond that a warp
-// takes several groups, 16 apart); a shorter sequence leaves the extra warps idle, so its summation
+// launch has as many warps per CTA as its longest sequence has groups (at most AT_MERGE_WARPS; beyond that a warp
+// takes several groups, that many apart); a shorter sequence leaves the extra warps idle, so its summation
 // order depends on its own chunk count only.
 //
-// TAIL (behind a fused recompute with a few live keys): one more warp attends the sequence's live keys, of which there are
-// AT_TAIL_KEYS at most, while the others fetch their partials; the two are put together at the end.
+// TAIL (behind a fused recompute, where a sequence has a few live keys): the last warp attends the live keys of such a
+// sequence, of which there are AT_TAIL_KEYS at most, while the others (one fewer at most) fetch its partials; the two are put
+// together at the end.  A sequence without such keys is merged as in the other launches, by all warps.
 template <int D_HEAD, int G, int NSEQ, int DT, int GH, bool TAIL>
 __global__ void __launch_bounds__(AT_MERGE_THREADS)
     kvd_attn_merge_kernel(const __grid_constant__ AttnLaunchT<NSEQ> P) {
   constexpr int SLICES = D_HEAD / AT_MERGE_SLICE;
-  constexpr int MAX_WARPS = AT_MERGE_WARPS - (TAIL ? 1 : 0);
   constexpr int PF = attn_merge_group(G);
   // of every warp of the CTA: outputs [GH][AT_MERGE_SLICE] and sums [GH] (as much as the launch's warps need: the kernel's
   // loads in flight pass through the L1, which shared memory is taken from: 64 x 3000 keys of a Qwen3-4B layer 15.8 -> 12.5 us,
@@ -666,6 +666,8 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
   const int head_slot = blockIdx.x / SLICES;
   const int si = head_slot / (P.n_q / GH), head0 = head_slot % (P.n_q / GH) * GH;  // sequence, first query head
   const AttnSeq &S = P.seq[si];
+  const bool tail = TAIL && attn_tail(S);
+  const int max_warps = AT_MERGE_WARPS - (tail ? 1 : 0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   grid_launch_dependents();
   // wait until the preceding grid in the stream (the streaming kernel) has completed and its
@@ -675,7 +677,7 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
   // (checking build: the slots to merge lie inside the partial arrays; otherwise nothing is merged)
   const int count = KVD_BOUNDS_OK(S.merge_base >= 0 && S.merge_base + S.merge_count <= P.max_parts, P.status) ? S.merge_count : 0;
   const int n_groups = (count + PF - 1) / PF;
-  const int warps_used = n_groups < MAX_WARPS ? n_groups : MAX_WARPS;
+  const int warps_used = n_groups < max_warps ? n_groups : max_warps;
   const float *ml0 = P.part_ml + (static_cast<size_t>(S.merge_base) * P.n_q + head0) * 2;
   const float *po0 = P.part_o + (static_cast<size_t>(S.merge_base) * P.n_q + head0) * D_HEAD +
                      slice * AT_MERGE_SLICE + lane * 2;
@@ -711,7 +713,7 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
 #pragma unroll
       for (int msk = 16; msk >= 1; msk >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, msk));
       Mu[g] = (mx == -CUDART_INF_F) ? 0.f : mx;
-      if (TAIL && warp == 0 && lane == 0) s_max[g] = mx;
+      if (tail && warp == 0 && lane == 0) s_max[g] = mx;
     }
     float2 o[GH];
     float l[GH];
@@ -720,7 +722,7 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
       l[g] = 0.f;
       o[g] = make_float2(0.f, 0.f);
     }
-    for (int grp = warp; grp < n_groups; grp += MAX_WARPS) {
+    for (int grp = warp; grp < n_groups; grp += max_warps) {
       if (grp != warp) fetch_group(grp);
 #pragma unroll
       for (int i = 0; i < PF; ++i) {
@@ -744,9 +746,9 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
   }
   const int tail_warp = static_cast<int>(blockDim.x / 32) - 1;
   if constexpr (TAIL) {
-    if (warp == tail_warp) {
+    if (tail && warp == tail_warp) {
       constexpr int EPL = D_HEAD / 32, W = EPL / 4;  // channels per lane, 8-byte words of them
-      const int n_keys = S.hi_pos - S.lo_pos + 1;    // (not positive where no live key is visible)
+      const int n_keys = S.hi_pos - S.lo_pos + 1;
       const __nv_bfloat16 *kl = nullptr, *vl = nullptr;
       if (lane < n_keys) key_rows(S, S.lo_pos + lane, static_cast<size_t>(head0 / G) * D_HEAD, kl, vl);
       const uint32_t held = __ballot_sync(0xffffffffu, kl != nullptr);
@@ -821,7 +823,7 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
       ov += s_o[w][g][c];
       lv += s_l[w][g];
     }
-    if constexpr (TAIL) {
+    if (tail) {
       const float mp = s_max[g], mk = s_max[GH + g], mt = fmaxf(mp, mk);
       const float wp = mp == -CUDART_INF_F ? 0.f : exp2f(mp - mt), wk = mk == -CUDART_INF_F ? 0.f : exp2f(mk - mt);
       ov = ov * wp + s_o[tail_warp][g][c] * wk;
@@ -914,14 +916,15 @@ static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t str
   }
   attr[0].val.programmaticStreamSerializationAllowed = ((small || S.early_merge) && !(serial_launch_mask() & 4)) ? 1 : 0;
   // as many warps per merge CTA as the longest sequence of the launch has groups of partials
-  int max_chunks = 1;
-  for (int i = 0; i < S.n_seqs; ++i) max_chunks = S.seq[i].merge_count > max_chunks ? S.seq[i].merge_count : max_chunks;
-  int merge_warps = (max_chunks + attn_merge_group(G) - 1) / attn_merge_group(G);
+  int merge_warps = 1;
+  for (int i = 0; i < S.n_seqs; ++i) {
+    const int own = S.tail && attn_tail(S.seq[i]) ? 1 : 0, most = AT_MERGE_WARPS - own;  // (a warp for live keys)
+    const int groups = (S.seq[i].merge_count + attn_merge_group(G) - 1) / attn_merge_group(G);
+    const int warps = (groups < most ? groups : most) + own;
+    merge_warps = warps > merge_warps ? warps : merge_warps;
+  }
   // (the heads the fused recompute exists for)
   constexpr bool TAILS = (D_HEAD == 256 && G <= 2) || (D_HEAD == 128 && (G <= 2 || G == 4));
-  const int most = AT_MERGE_WARPS - (S.tail ? 1 : 0);
-  if (merge_warps > most) merge_warps = most;
-  if (S.tail) merge_warps += 1;
   cfg.blockDim = dim3(32 * merge_warps, 1, 1);
   auto merge = [&](auto kern, int heads) {
     cfg.gridDim = dim3(S.n_seqs * (S.n_q / heads) * (D_HEAD / AT_MERGE_SLICE), 1, 1);

@@ -183,6 +183,9 @@ struct AttnSeq {
   int merge_count;  // streaming kernel's chunks, preceded by partials of the fused recompute kernel if any
 };
 
+// Live keys that the merge kernel attends itself: visible, and not cut into chunks.
+__host__ __device__ inline bool attn_tail(const AttnSeq &S) { return S.n_chunks == 0 && S.hi_pos >= S.lo_pos; }
+
 // Launch-wide fields, followed by the per-sequence descriptors.  The kernel takes the variant whose
 // array is just large enough (AttnLaunchT<4> for small batches: a 10 KB parameter block costs
 // microseconds to launch).
@@ -199,7 +202,7 @@ struct AttnLaunchHead {
   int *status;             // device status word (nullptr: none), used by the checking build
   int max_parts;           // slots the partial arrays hold
   bool early_split, early_merge;  // this kernel starts early whatever the grid
-  bool tail;               // the merge kernel attends the live keys itself (at most AT_TAIL_KEYS per sequence)
+  bool tail;               // there is a sequence whose live keys the merge kernel attends itself (attn_tail)
 };
 template <int NSEQ>
 struct AttnLaunchT : AttnLaunchHead {

@@ -112,3 +112,28 @@ def test_live_keys_that_score_minus_infinity(kind, layer, n_old, live, lost):
     for i in lost:
         s.k[0][i, 0, 5] = -math.inf  # for the first KV head's queries
     s.check(s.run())
+
+
+WIDE = {"2-256": (8, 4, 256), "4-128": (16, 4, 128)}  # (with 64 sequences more warps than the SMs hold at once: a merge CTA per KV head)
+FEW, EIGHT, NINE = [0], list(range(8)), list(range(9))
+
+
+@pytest.mark.parametrize("kind", ["bf16", "f16", "fp8"])
+@pytest.mark.parametrize("layer", WIDE)
+@pytest.mark.parametrize("n_old,live", [
+    ([300, 300, 513], [FEW, NINE, EIGHT]),                                    # the streaming kernel takes the second one's
+    ([20000, 300, 20300], [FEW, [], NINE]),                                   # more groups of partials than a merge CTA has warps
+    ([260 + b for b in range(64)], [(FEW, EIGHT, NINE, [])[b % 4] for b in range(64)])], ids=["3", "long", "64"])
+def test_a_sequence_gets_the_same_bits_alone_and_among_others(kind, layer, n_old, live):
+    s = Step(WIDE[layer], n_old, live, kind)
+    out = s.run()
+    s.check(out)
+    for b in range(min(len(n_old), 8)):
+        assert torch.equal(s.run([b])[0], out[b]), b
+        assert torch.equal(s.run([b, (b + 1) % len(n_old)])[0], out[b]), b
+    before = s.c.kvd_launch_count()
+    s.run([b for b, p in enumerate(live) if len(p) <= 8])
+    assert s.c.kvd_launch_count() - before == 2  # (recompute, merge)
+    before = s.c.kvd_launch_count()
+    s.run()
+    assert s.c.kvd_launch_count() - before == 3
