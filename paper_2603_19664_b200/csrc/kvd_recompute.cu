@@ -1044,6 +1044,8 @@ static kvd_status launch_sel(kvd_ctx *ctx, const LayerState &ls, const CUtensorM
     if (ctx->dtype == 1 && exposed) return launch_impl<BLOCK_N, D_HEAD, false, 0, 2, true, 1, 8>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
     if (ctx->dtype == 1) return launch_impl<BLOCK_N, D_HEAD, false, 0, 2, true, 1>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
     if (ctx->dtype == 2) return launch_impl<BLOCK_N, D_HEAD, false, 0, 4, true, 2>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
+    // (traced: the same two kernels)
+    if (p.trace != nullptr && exposed) return launch_impl<BLOCK_N, D_HEAD, true, 0, 2, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
     if (p.trace != nullptr) return launch_impl<BLOCK_N, D_HEAD, true, 0>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
     // one tile per cluster at most: every key tile's epilogue is exposed -> the low table from shared memory, two groups
     if (exposed) return launch_impl<BLOCK_N, D_HEAD, false, 0, 2, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
@@ -1120,7 +1122,7 @@ kvd_status launch_recompute_fused(kvd_ctx *ctx, const LayerState &ls, const CUte
   const int dh = ctx->desc.d_head, g = ctx->desc.n_q_heads / ctx->desc.n_kv_heads;
   if (ctx->block_n != 256 || p.k_cols % 256 != 0) return KVD_ERR_UNSUPPORTED;
   if (eb == 1) {  // rows and weights as E4M3 codes (the FP8 store)
-    if (dh == 256 && g == 2 && p.trace != nullptr) return launch_impl<256, 256, true, 2, 1>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
+    if (dh == 256 && g == 2 && p.trace != nullptr) return launch_impl<256, 256, true, 2, 1, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
     if (dh == 256 && g == 2) return launch_impl<256, 256, false, 2, 1, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
     if (dh == 256 && g == 1) return launch_impl<256, 256, false, 1, 1, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);
     if (dh == 128 && g == 4) return launch_impl<256, 128, false, 4, 1, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, &fp, stream);

@@ -5,6 +5,7 @@ import torch
 import paper_2603_19664_b200 as kvd
 from kvd_synth import GEMMA3_4B_GLOBAL, QWEN3_4B, make_residuals
 from gpu_util import dev, open_layer
+from test_gpu_fused_tail import Step
 
 pytestmark = pytest.mark.gpu
 
@@ -65,3 +66,18 @@ def test_a_traced_call_of_few_rows(dtype):
     assert bool((trace[0, 0, 7] > trace[0, 0, 6])) == (dtype == 0) and bool((trace[32:] == 0).all())
     assert ctx.kvd_poll_status() == kvd.KVD_OK
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [1, 300, 2560, 40000])
+def test_a_traced_fused_call_has_the_bits_of_an_untraced_one(n):
+    s = Step((4, 2, 256), [n], [[0]], "fp8")
+    out = s.run()
+    words = kvd.kvd_trace_bytes(s.desc, (n + 255) // 256, 2) // 8
+    trace = torch.zeros((words,), dtype=torch.int64, device="cuda")
+    s.c.kvd_set_trace(trace)
+    traced = s.run()
+    s.c.kvd_set_trace(None)
+    assert torch.equal(out, traced)
+    t = trace.view(-1, 8, 16)
+    assert bool((t[:, 0, 7] > t[:, 0, 6]).all())  # every CTA recorded its first tile's epilogue
+    s.c.close()
