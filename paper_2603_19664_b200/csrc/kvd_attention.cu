@@ -883,16 +883,15 @@ static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t str
   // Starting early pays for launches of up to one wave (the set-up hides under the predecessor's tail);
   // a many-wave grid whose first CTAs sit on the SMs waiting slowed a short predecessor down in
   // measurements (11 us lost on a 24 us predecessor), so those are ordered plainly.
-  // Straight behind the few-row projection larger grids do as well: its CTAs are few, they leave room beside them
-  // (kvd_rows_ring.h), and it is too short for the waiting CTAs to cost what they save.  One new token per sequence, ordered
-  // plainly / started early, us per step: Gemma-3-4B layer 8 x 1000 26.6 / 21.0, 16 x 2048 42.3 / 37.7, 24 x 1000 40.9 / 35.5,
-  // 40 x 1024 49.6 / 45.5, 64 x 2048 111.8 / 106.6; Qwen3-4B layer 8 x 2048 36.9 / 33.6, 16 x 2048 51.5 / 49.6; SmolLM2 layer
-  // 17 x 4000 30.7 / 27.2, 64 x 2048 41.2 / 37.3.  Behind more than RW_FEW_ROWS rows the tensor-core kernel at d_head 128 does
-  // not, only its merge kernel: plainly / both early / merge alone, Qwen3-4B layer, 17 x 1000 36.9 / 42.0 / 36.9, 32 x 1000
-  // 54.0 / 57.2 / 53.3, 64 x 2048 149.2 / 149.1 / 145.8, 17 x 2048 55.4 / 53.0 / 53.2.
+  // Straight behind the few-row projection larger grids do as well: its CTAs are few, they leave room beside them or SMs of
+  // their own (kvd_rows_ring.h), and it is too short for the waiting CTAs to cost what they save.  One new token per sequence,
+  // ordered plainly / started early, us per step: Gemma-3-4B layer 16 x 2048 42.1 / 37.8, 24 x 1000 37.0 / 32.6, 40 x 1024 50.6 /
+  // 46.5, 64 x 2048 111.1 / 107.0; Qwen3-4B layer 8 x 2048 30.8 / 26.1, 16 x 2048 45.2 / 41.3, 17 x 1000 33.0 / 28.5, 17 x 2048
+  // 48.2 / 43.9, 32 x 1000 48.2 / 44.8, 64 x 1000 76.1 / 71.9, 64 x 2048 124.7 / 119.3; SmolLM2 layer 16 x 4000 25.5 / 20.9, 17 x
+  // 4000 26.8 / 22.6, 64 x 2048 41.0 / 36.6; 32 query heads on 4 of 128, 32 x 2000 54.5 / 48.7.
   const bool small = S.total_chunks * S.n_kv <= 148 * AT_CTAS_PER_SM;
   if (S.total_chunks > 0) {
-    attr[0].val.programmaticStreamSerializationAllowed = ((small || S.early_split) && !(serial_launch_mask() & 2)) ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = ((small || S.early) && !(serial_launch_mask() & 2)) ? 1 : 0;
     cfg.gridDim = dim3(S.total_chunks * S.n_kv, 1, 1);
     cfg.blockDim = dim3(AT_THREADS, 1, 1);
     if constexpr (G >= 3 && D_HEAD <= 128) {
@@ -914,7 +913,7 @@ static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t str
     }
     if (e != cudaSuccess) return e;
   }
-  attr[0].val.programmaticStreamSerializationAllowed = ((small || S.early_merge) && !(serial_launch_mask() & 4)) ? 1 : 0;
+  attr[0].val.programmaticStreamSerializationAllowed = ((small || S.early) && !(serial_launch_mask() & 4)) ? 1 : 0;
   // as many warps per merge CTA as the longest sequence of the launch has groups of partials
   int merge_warps = 1;
   for (int i = 0; i < S.n_seqs; ++i) {
@@ -956,8 +955,7 @@ static kvd_status launch_attn_impl(kvd_ctx *ctx, const AttnLaunch &L, cudaStream
     static_cast<AttnLaunchHead &>(S) = static_cast<const AttnLaunchHead &>(L);
     for (int i = 0; i < L.n_seqs; ++i) S.seq[i] = L.seq[i];
     // straight behind the projection of the new tokens (attn_launch_pair says why; a second launch of the same call is not)
-    S.early_merge = ctx->few_rows.directly_before(ctx->launches, stream);
-    S.early_split = S.early_merge && !(G >= 3 && D_HEAD == 128 && ctx->few_rows.rows > RW_FEW_ROWS);
+    S.early = ctx->few_rows.directly_before(ctx->launches, stream);
     // fp16 contexts (kvd_set_dtype): the same kernels reading and writing fp16
     cudaError_t e = ctx->dtype == 1 ? attn_launch_pair<D_HEAD, G, NSEQ, 1>(S, stream)
                                     : attn_launch_pair<D_HEAD, G, NSEQ, 0>(S, stream);
@@ -1161,7 +1159,7 @@ extern "C" kvd_status kvd_decode_attention_static(int n_q_heads, int n_kv_heads,
   L.part_o = reinterpret_cast<float *>(scratch + ml_bytes);
   L.status = nullptr;
   L.max_parts = parts;
-  L.early_split = L.early_merge = L.tail = false;
+  L.early = L.tail = false;
   switch (d_head) {
     case 64: return static_launch_d<64>(L, group, stream);
     case 128: return static_launch_d<128>(L, group, stream);

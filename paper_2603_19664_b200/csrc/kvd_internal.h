@@ -201,7 +201,7 @@ struct AttnLaunchHead {
   float *part_ml;          // [parts][n_q][2]
   int *status;             // device status word (nullptr: none), used by the checking build
   int max_parts;           // slots the partial arrays hold
-  bool early_split, early_merge;  // this kernel starts early whatever the grid
+  bool early;              // both kernels start early whatever their grids
   bool tail;               // there is a sequence whose live keys the merge kernel attends itself (attn_tail)
 };
 template <int NSEQ>

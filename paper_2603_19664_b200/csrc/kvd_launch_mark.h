@@ -9,11 +9,9 @@ namespace kvd {
 struct LaunchMark {
   uint64_t at = ~0ull;           // launches of the context, the marked one included
   const void *stream = nullptr;
-  int rows = 0;                  // that the marked launch took
-  void set(uint64_t launches, const void *s, int n_rows) {
+  void set(uint64_t launches, const void *s) {
     at = launches;
     stream = s;
-    rows = n_rows;
   }
   bool directly_before(uint64_t launches, const void *s) const { return at == launches && stream == s; }
 };

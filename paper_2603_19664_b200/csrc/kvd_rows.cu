@@ -488,7 +488,7 @@ static kvd_status launch_rows_impl(kvd_ctx *ctx, const CUtensorMap &tmap_w, cons
   cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmap_w, tmap_x, p);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "launch rows");
   ctx->launches += 1;
-  if (D_HEAD > 0) ctx->few_rows.set(ctx->launches, stream, p.n_rows);
+  if (D_HEAD > 0) ctx->few_rows.set(ctx->launches, stream);
   return KVD_OK;
 }
 

@@ -13,8 +13,10 @@ constexpr int RW_BARS = 2 * RW_MAX_STAGES + 6;                   // full, empty 
 constexpr int RW_TAIL = RW_BARS * 8 + 32 + RW_MAX_ROWS * 2 * 4;  // barriers, tmem pointer + abort, 1/rms, key scale
 constexpr int RW_SMEM_MAX = 232448;
 // Key and value heads leave an SM room for two CTAs of the fp32 streaming attention behind them (9 to 18 KB and 16 K registers
-// each, the tensor-core kernel's 48 KB fit once up to RW_FEW_ROWS rows; the kernel's launch bounds leave the registers), which take their places beside a CTA of this kernel and wait there
-// instead of being started when it ends.  Up to RW_FEW_ROWS rows three stages of 8 k blocks do that: projection alone / step
+// each; the kernel's launch bounds leave the registers), or up to RW_FEW_ROWS rows for one of the tensor-core streaming
+// attention (48 KB, 64 in small grids), which take their places beside a CTA of this kernel and wait there
+// instead of being started when it ends.  (Beyond RW_FEW_ROWS rows the tensor-core kernel's find the SMs that have no CTA of
+// this kernel: 12 to 64 have one.)  Up to RW_FEW_ROWS rows three stages of 8 k blocks do that: projection alone / step
 // with attention, us, two, three, four stages and all of an SM's shared memory: Gemma-3-4B layer 1 x 8192 8.8 / 22.3, 7.6 /
 // 21.1, 7.4 / 21.4, 7.4 / 24.0; 16 x 2048 8.3 / 38.3, 7.6 / 37.7, -, 7.7 / 40.0; Qwen3-4B layer 8 x 2048 -, 7.1 / 33.6, 7.2 /
 // 34.4, 7.2 / 41.0; 16 rows of a 5120-wide layer alone 12.2, 10.9, -, 10.9.  (Stages of 4 and 6 k blocks cost the projection

@@ -142,11 +142,11 @@ int main() {
   LaunchMark m;
   int s1, s2;
   if (m.directly_before(0, &s1)) return 1;            // nothing launched yet
-  m.set(7, &s1, 20);
-  if (!m.directly_before(7, &s1) || m.rows != 20) return 2;
+  m.set(7, &s1);
+  if (!m.directly_before(7, &s1)) return 2;
   if (m.directly_before(7, &s2)) return 3;            // another stream
   if (m.directly_before(8, &s1) || m.directly_before(9, &s1)) return 4;  // another launch in between, or used up
-  m.set(9, &s2, 1);
+  m.set(9, &s2);
   return m.directly_before(9, &s2) ? 0 : 5;
 }
 """
@@ -159,7 +159,8 @@ def test_attention_starts_early_only_straight_behind_the_projection(tmp_path):
     subprocess.run(["g++", "-std=c++17", "-I", CSRC, "-o", str(tmp_path / "mark"), str(tmp_path / "mark.cpp")], check=True)
     assert subprocess.run([str(tmp_path / "mark")]).returncode == 0
     text = TEXT["kvd_attention.cu"]
-    assert "early_merge = ctx->few_rows.directly_before(ctx->launches, stream)" in text and "early_split = S.early_merge &&" in text
+    assert "S.early = ctx->few_rows.directly_before(ctx->launches, stream);" in text
+    assert len(re.findall(r"small \|\| S\.early\)", text)) == 2  # both kernels, whatever the rows and the head size
     assert len(re.findall(r"few_rows\.set\(", ALL)) == 1
     rows = TEXT["kvd_rows.cu"]
     assert rows.index("ctx->launches += 1") < rows.index("few_rows.set(ctx->launches, stream")

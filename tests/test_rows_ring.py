@@ -1,5 +1,5 @@
-"""The ring of the few-row projection kernel (csrc/kvd_rows_ring.h): stages, and room for two streaming attention CTAs beside a
-CTA that makes keys and values, over all row counts, head sizes and product shapes."""
+"""The ring of the few-row projection kernel (csrc/kvd_rows_ring.h): stages, and room for two streaming attention CTAs (of the
+tensor-core kernel: one, up to 16 rows) beside a CTA that makes keys and values, over all row counts, head sizes and product shapes."""
 import os
 import subprocess
 
@@ -19,6 +19,8 @@ int main() {
         if (r.stages < (steps < least ? steps : least) || r.stages > steps || r.stages > RW_MAX_STAGES) return 1;
         const int attention = d_head == 64 ? 12672 : d_head == 128 ? 16640 : 16512;  // up to four query heads per KV head
         if (r.smem + 1024 + 2 * (attention + 1024) > 228 * 1024) return 2;
+        // the tensor-core streaming kernel's CTAs (heads of 64 and 128): four warps' rings of up to four pieces
+        if (!many && d_head <= 128 && r.smem + 1024 + 4 * 4 * 4096 + 1024 > 228 * 1024) return 5;
       }
     for (int tile = RW_MIN_TILE; tile <= 256; tile += 8)
       for (int total = 1; total <= 400; total += 7) {
