@@ -1039,16 +1039,23 @@ static kvd_status launch_sel(kvd_ctx *ctx, const LayerState &ls, const CUtensorM
                              const CUtensorMap &tmap_rows, const RecomputeParams &p, const FusedParams *fp,
                              cudaStream_t stream) {
   if constexpr (FG == 0) {
-    // fp16 and fp32 contexts: low table in shared memory for all launch sizes
+    // One tile per cluster at most: every key tile's epilogue is exposed -> the low table from shared memory (fp16 and fp32
+    // contexts: for all launch sizes), two groups.  Where they split a single head of half-split pairs, whose steps are as long
+    // with one group, what the second costs in norm and statistics is more than it saves (Gemma-3-4B layer with such
+    // pairs, one / two groups, us: 200 rows 21.5 / 21.9, 512 22.1 / 22.4, 800 22.6 / 23.2): one group.
     const bool exposed = p.whole_tiles + (p.num_m_blocks * p.num_n_blocks - p.whole_tiles) * p.parts <= ctx->num_sms / 2;
-    if (ctx->dtype == 1 && exposed) return launch_impl<BLOCK_N, D_HEAD, false, 0, 2, true, 1, 8>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
+    const bool two = exposed && !(D_HEAD == 256 && p.rope_style == KVD_ROPE_HALF);
+    if (ctx->dtype == 1 && two) return launch_impl<BLOCK_N, D_HEAD, false, 0, 2, true, 1, 8>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
     if (ctx->dtype == 1) return launch_impl<BLOCK_N, D_HEAD, false, 0, 2, true, 1>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
     if (ctx->dtype == 2) return launch_impl<BLOCK_N, D_HEAD, false, 0, 4, true, 2>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
-    // (traced: the same two kernels)
-    if (p.trace != nullptr && exposed) return launch_impl<BLOCK_N, D_HEAD, true, 0, 2, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
-    if (p.trace != nullptr) return launch_impl<BLOCK_N, D_HEAD, true, 0>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
-    // one tile per cluster at most: every key tile's epilogue is exposed -> the low table from shared memory, two groups
-    if (exposed) return launch_impl<BLOCK_N, D_HEAD, false, 0, 2, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
+    const bool traced = p.trace != nullptr;  // (the same kernels)
+    if (two && traced) return launch_impl<BLOCK_N, D_HEAD, true, 0, 2, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
+    if (two) return launch_impl<BLOCK_N, D_HEAD, false, 0, 2, true, 0, 8>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
+    if constexpr (D_HEAD == 256) {
+      if (exposed && traced) return launch_impl<BLOCK_N, D_HEAD, true, 0, 2, true>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
+      if (exposed) return launch_impl<BLOCK_N, D_HEAD, false, 0, 2, true>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
+    }
+    if (traced) return launch_impl<BLOCK_N, D_HEAD, true, 0>(ctx, ls, tmap_store, tmap_rows, p, fp, stream);
   }
   // the fused variant on fp16 rows, weights, queries and outputs (same tiles, MMA kind f16 with fp16 operands)
   if constexpr (FG > 0) {

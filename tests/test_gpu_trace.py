@@ -1,18 +1,21 @@
 """The trace buffer of kvd_set_trace: a launch that does not fit it records nothing, one that fits stays inside it."""
+import dataclasses
+
 import pytest
 import torch
 
 import paper_2603_19664_b200 as kvd
-from kvd_synth import GEMMA3_4B_GLOBAL, QWEN3_4B, make_residuals
+from kvd_synth import GEMMA3_4B_GLOBAL, QWEN3_4B, ROPE_HALF, make_residuals
 from gpu_util import dev, open_layer
 from test_gpu_fused_tail import Step
 
 pytestmark = pytest.mark.gpu
 
 WORDS = 8 * 16  # int64 slots per CTA
+GEMMA_HALF = dataclasses.replace(GEMMA3_4B_GLOBAL, name="gemma3-4b-half-split", rope_style=ROPE_HALF)  # (another kernel in short launches)
 
 
-@pytest.mark.parametrize("shape", [QWEN3_4B, GEMMA3_4B_GLOBAL], ids=lambda s: s.name)
+@pytest.mark.parametrize("shape", [QWEN3_4B, GEMMA3_4B_GLOBAL, GEMMA_HALF], ids=lambda s: s.name)
 @pytest.mark.parametrize("n", [65, 200, 256, 300, 2560])
 def test_trace_stays_inside_its_buffer(shape, n):
     kdim = shape.n_kv_heads * shape.d_head
