@@ -383,19 +383,21 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
     // (No CTA leaves before every CTA of the head has sent its columns, and each waits for those it is sent, also behind
     // an abort: nothing arrives in the shared memory of a CTA that is gone.)
     cluster_arrive_relaxed();
-    if (exchange) {
+    auto columns_within = [&](unsigned long long limit_ns) -> bool {
       int ok = 1;
       if (lane == 0) {
         const unsigned long long t0 = globaltimer_ns();
         while (!mbar_try_wait_cluster(bar_head, 0))
-          if (globaltimer_ns() - t0 > tmo) {
+          if (globaltimer_ns() - t0 > limit_ns) {
             ok = 0;
             break;
           }
       }
-      if (!__shfl_sync(0xffffffffu, ok, 0)) raise(p.status, STATUS_TIMEOUT, s_abort);
-      __syncwarp();
-    }
+      return __shfl_sync(0xffffffffu, ok, 0) != 0;
+    };
+    const bool got = !exchange || columns_within(tmo);
+    if (!got) raise(p.status, STATUS_TIMEOUT, s_abort);
+    __syncwarp();
     constexpr int HALF = D_HEAD / 2;
     // two lanes per row: four chains (columns j mod 4) in ascending order, two-wide: the order of the recompute kernel
     if (warp * 16 < p.n_rows) {
@@ -451,6 +453,9 @@ kvd_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
     }
     __syncwarp();
     cluster_wait();
+    // Every CTA has sent by now what it sends, but its arrival does not say that it has landed: a CTA that has not seen all
+    // columns stays for as long as that could take.
+    if (!got) columns_within(200000ull);
   }
 }
 

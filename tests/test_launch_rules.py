@@ -75,6 +75,16 @@ def test_few_row_producer_waits_for_its_last_copies_on_every_path():
     assert "if (" not in between  # the wait hangs on no condition
 
 
+def test_a_few_row_cta_outlives_the_columns_it_is_sent():
+    """What another CTA of the head sends must not land in the shared memory of whatever runs there next.  Each CTA waits
+    for it; one that gave up leaves behind the cluster barrier (all have sent) and a second wait (it has landed)."""
+    body = KERNELS["kvd_rows_kernel"][1]
+    tail = body[body.index("cluster_arrive_relaxed();"):]
+    assert re.search(r"mbar_try_wait_cluster\(bar_head, 0\)", tail[:tail.index("const bool got = !exchange || columns_within(tmo);")])
+    assert "return;" not in tail
+    assert re.fullmatch(r"\s*if \(!got\) columns_within\(\d+ull\);\s*\}\s*\}\s*", tail[tail.index("cluster_wait();") + 15:])
+
+
 SMALL = sorted(set(re.findall(r"launch_dependent\((?:ctx, )?(kvd_\w+)", ALL)))
 
 
