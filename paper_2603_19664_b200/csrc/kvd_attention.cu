@@ -836,19 +836,20 @@ __global__ void __launch_bounds__(AT_MERGE_THREADS)
   }
 }
 
-// dynamic shared memory of the kernel and its one-time opt-in (sizes above 48 KB need it)
+// dynamic shared memory of the kernel and its one-time opt-in (sizes above 48 KB need it); the device's SMs
 template <int D_HEAD, int G>
 struct AttnSmem {
   static constexpr int NPART = AT_WARPS * (32 / (D_HEAD / 8));
   static constexpr int BYTES = NPART * G * (D_HEAD + 2) * 4;
 };
 template <int D_HEAD, int G, int NSEQ, int DT>
-static cudaError_t attn_configure() {
-  static bool done[64] = {};
+static cudaError_t attn_configure(int *num_sms) {
+  static std::atomic<int> sms[64] = {};  // 0: not configured yet
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (!done[dev & 63]) {
+  *num_sms = sms[dev & 63].load(std::memory_order_acquire);
+  if (*num_sms == 0) {
     if constexpr (G >= 3 && D_HEAD <= 128) {
       e = cudaFuncSetAttribute(kvd_attn_split_mma_kernel<D_HEAD, G, NSEQ, DT, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_WARPS * 3 * AT_PIECE);
       if (e == cudaSuccess)
@@ -864,14 +865,17 @@ static cudaError_t attn_configure() {
         if (e != cudaSuccess) return e;
       }
     }
-    done[dev & 63] = true;
+    e = cudaDeviceGetAttribute(num_sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    sms[dev & 63].store(*num_sms, std::memory_order_release);
   }
   return cudaSuccess;
 }
 // the two launches of a decode step: stream + partials, then merge
 template <int D_HEAD, int G, int NSEQ, int DT = 0>
 static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t stream) {
-  cudaError_t e = attn_configure<D_HEAD, G, NSEQ, DT>();
+  int num_sms = 0;
+  cudaError_t e = attn_configure<D_HEAD, G, NSEQ, DT>(&num_sms);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
@@ -889,20 +893,20 @@ static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t str
   // 46.5, 64 x 2048 111.1 / 107.0; Qwen3-4B layer 8 x 2048 30.8 / 26.1, 16 x 2048 45.2 / 41.3, 17 x 1000 33.0 / 28.5, 17 x 2048
   // 48.2 / 43.9, 32 x 1000 48.2 / 44.8, 64 x 1000 76.1 / 71.9, 64 x 2048 124.7 / 119.3; SmolLM2 layer 16 x 4000 25.5 / 20.9, 17 x
   // 4000 26.8 / 22.6, 64 x 2048 41.0 / 36.6; 32 query heads on 4 of 128, 32 x 2000 54.5 / 48.7.
-  const bool small = S.total_chunks * S.n_kv <= 148 * AT_CTAS_PER_SM;
+  const bool small = S.total_chunks * S.n_kv <= num_sms * AT_CTAS_PER_SM;
   if (S.total_chunks > 0) {
     attr[0].val.programmaticStreamSerializationAllowed = ((small || S.early) && !(serial_launch_mask() & 2)) ? 1 : 0;
     cfg.gridDim = dim3(S.total_chunks * S.n_kv, 1, 1);
     cfg.blockDim = dim3(AT_THREADS, 1, 1);
     if constexpr (G >= 3 && D_HEAD <= 128) {
-      const bool few = S.total_chunks * S.n_kv <= 148 * 3;  // all of the grid at once with four pieces per warp
+      const bool few = S.total_chunks * S.n_kv <= num_sms * 3;  // all of the grid at once with four pieces per warp
       cfg.dynamicSmemBytes = AT_WARPS * (few ? 4 : 3) * AT_PIECE;
       if (few) e = cudaLaunchKernelEx(&cfg, kvd_attn_split_mma_kernel<D_HEAD, G, NSEQ, DT, 4>, S);
       else e = cudaLaunchKernelEx(&cfg, kvd_attn_split_mma_kernel<D_HEAD, G, NSEQ, DT, 3>, S);
     } else {
       cfg.dynamicSmemBytes = AttnSmem<D_HEAD, G>::BYTES;
       // at most two CTAs per SM, every chunk two iterations long: the variant that issues all loads at once
-      bool allin = G <= 2 && S.total_chunks * S.n_kv <= 148 * 2;
+      bool allin = G <= 2 && S.total_chunks * S.n_kv <= num_sms * 2;
       for (int i = 0; i < S.n_seqs; ++i) allin = allin && (S.seq[i].n_chunks == 0 || S.seq[i].iters == 2);
       if constexpr (G <= 2) {
         if (allin) e = cudaLaunchKernelEx(&cfg, kvd_attn_split_kernel<D_HEAD, G, NSEQ, DT, true>, S);
@@ -942,7 +946,7 @@ static cudaError_t attn_launch_pair(const AttnLaunchT<NSEQ> &S, cudaStream_t str
   // 4.7 / 3.4, 32 x 500 5.5 / 3.7, Gemma-3-4B layer 4 x 2048 4.5 / 3.6, 1 x 32768 4.7 / 3.8; beyond one wave the group's is ahead:
   // Gemma 64 x 1000 3.6 / 4.3, Qwen 64 x 3000 12.9 / 13.3.
   if constexpr (G > 1) {
-    if (S.n_seqs * S.n_q * (D_HEAD / AT_MERGE_SLICE) * merge_warps <= 148 * AT_MERGE_WARPS)
+    if (S.n_seqs * S.n_q * (D_HEAD / AT_MERGE_SLICE) * merge_warps <= num_sms * AT_MERGE_WARPS)
       return merge_by(std::integral_constant<int, 1>());
   }
   return merge_by(std::integral_constant<int, G>());

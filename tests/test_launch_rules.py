@@ -125,6 +125,13 @@ def test_the_early_start_threshold_follows_the_device():
     assert "ctx->num_sms" in fn and not re.search(r"grid\.x\s*[<>]=?\s*\d", fn)
 
 
+def test_attention_launches_ask_the_device_for_its_sms():
+    text = TEXT["kvd_attention.cu"]
+    launch = text[text.index("static cudaError_t attn_launch_pair("):]
+    launch = launch[:launch.index("\n}")]
+    assert not re.search(r"\b148\b", launch) and len(re.findall(r"<= num_sms \*", launch)) == 4
+
+
 def test_kernels_that_derive_store_slots_or_tiles_test_them_in_the_checking_build():
     body = KERNELS["kvd_rows_kernel"][1]
     for index in ("append_slot[r]", "col0"):
