@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(AT_THREADS, SLOTS == 3 ? AT_CTAS_PER_SM : 3)
   constexpr int VP = D_HEAD / 64;             // 16-byte pieces of a value row per thread (second product)
   constexpr int MB = D_HEAD / 16;             // 16-channel blocks of the output
   constexpr int ROW = D_HEAD * 2;             // bytes of a key's row, [WARP_KEYS][ROW] is a piece
-  static_assert(WARP_KEYS * ROW == AT_PIECE && G * D_HEAD * 4 <= SLOTS * AT_PIECE && WARP_KEYS <= 32, "a piece, a warp's partial in its ring's place");
+  static_assert(WARP_KEYS * ROW == AT_PIECE && G * (D_HEAD + 2) * 4 <= SLOTS * AT_PIECE && WARP_KEYS <= 32, "a piece, a warp's partial in its ring's place");
   extern __shared__ __align__(16) uint8_t at_ring[];  // the warps' rings
   grid_launch_dependents();
 

@@ -317,9 +317,6 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
 __device__ __forceinline__ void st_cluster_f32(uint32_t cluster_addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
 }
-__device__ __forceinline__ void st_cluster_v4(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
 // Stores into another CTA's shared memory that count their bytes on one of that CTA's barriers (both addresses from
 // map_to_cta): the data and the news of it travel together, and the storing thread waits for nothing.
 __device__ __forceinline__ void st_async_f32(uint32_t cluster_addr, uint32_t cluster_bar, float v) {

@@ -46,13 +46,13 @@
 //   EB = 1  FP8 checkpoints (kvd_recompute_kv_fp8): rows and weights are E4M3 codes, a k block is 128
 //           channels, the MMA kind is f8f6f4; the scales ride in the per-row factor of the epilogue.
 //           Combines with FG > 0 (kvd_decode_attention_recompute_fp8).
-//   DT = 1  fp16 rows, weights and outputs (kvd_set_dtype), plain variant only.
+//   DT = 1  fp16 rows, weights and outputs (kvd_set_dtype); DT = 2 fp32 (TF32 products), plain variant only.
 //   EPI = 8 two epilogue groups (warps 4-7 and 8-11; rows' statistics by warps 0 and 1): launches whose key tiles' epilogues
 //           nothing overlaps, and the fused FP8 variant, whose main loop is shorter than they are.  Groups take the heads of
 //           a tile in turns, or half of the columns where it has one head (both add up the key norm, for the same bits), in
 //           the fused variant half of the rows of a value tile.  us, one / two groups: 837 rows of a Gemma-3-4B layer 24.9 /
-//           22.5; FP8 step 4096 rows 24.2 / 22.9, Qwen3-4B layer 4 x 2000 48.4 / 44.3.  Beyond two tiles per cluster of
-//           bf16 rows the other warps' instructions cost 1 to 2 %: one group there.
+//           22.5; FP8 step 4096 rows 24.2 / 22.9, Qwen3-4B layer 4 x 2000 48.4 / 44.3.  Beyond one tile per cluster of
+//           bf16 or fp16 rows the other warps' instructions cost 1 to 2 %: one group there (launch_sel).
 #include <math_constants.h>
 #include <string.h>
 
@@ -84,7 +84,7 @@ struct RcCfg {
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int TMEM_COLS = 2 * BLOCK_N;
   // barriers: full[S] (used in the even CTA), empty[S], tmem_full[2], tmem_empty[2], stats_full[2], rstd_free[2]
-  // + stats_x (the four statistics warps among themselves); fused: + scores[2] (both CTAs' epilogue
+  // + stats_x (the statistics warps among themselves); fused: + scores[2] (both CTAs' epilogue
   // threads), epi (the epilogue warps among themselves), half[2] (what the second epilogue group hands to the first)
   static constexpr int NUM_BARS = 2 * STAGES + 9 + (FUSED ? 5 : 0);
   static constexpr int BAR_BYTES = (NUM_BARS * 8 + 15) / 16 * 16;
@@ -181,7 +181,7 @@ KVD_DEFINE_UMMA_KBLOCK(umma_kblock_pair_tf32, "tf32")  // fp32 operands read as 
 // EB = bytes per operand element: 2 = bf16 rows and weights, 1 = the FP8 variant (E4M3 codes of rows and
 // weights; a k block is then 128 channels in the same 128-byte rows, the MMA kind f8f6f4, and the rows'
 // and the matrix's quantisation scales ride in the per-row factor that the statistics warps hand over).
-// DT = 1: fp16 rows, weights and outputs instead of bf16 (plain variant only).
+// DT = 1: fp16 rows, weights and outputs instead of bf16; DT = 2: fp32 (plain variant only).
 template <int BLOCK_N, int D_HEAD, bool TRACE, int FG, int EB = 2, bool LOSM = (FG > 0), int DT = 0, int EPI = 4>
 __global__ void __launch_bounds__(EPI == 8 ? RC_THREADS_8 : RC_THREADS, 1)
 kvd_recompute_kernel(const __grid_constant__ CUtensorMap tmap_store, const __grid_constant__ CUtensorMap tmap_rows,
