@@ -406,7 +406,9 @@ kvd_status kvd_prefill_attention(kvd_ctx *ctx, int layer, int n_rows, const void
  *   The current token can be folded into the recomputed part: its row is checkpointed like every token's, so
  *   ranges[b] may end with it (n counts it) while `rows` still makes its K_t, V_t for a window that keeps them;
  *   when no live segment is left (n_segs == 0 or all lengths 0) the live-segment launch is skipped.
- * Three launches (recompute+attend, live segments, merge), two without live segments.  The fused form pays
+ * Two launches (recompute+attend, merge) where no sequence has more than eight visible live positions -- the merge kernel
+ * attends those itself -- and three (live segments in between) otherwise.  A sequence's result does not depend on the
+ * other sequences of the call.  The fused form pays
  * where the recompute volume is large (kvd_fused_recompute_pays); below that the two-call sequence
  * kvd_recompute_kv_step + kvd_decode_attention is faster, because a unit of work here is a key tile AND a
  * value tile on one SM pair, where the plain kernel gives every tile its own.  KVD_ERR_UNSUPPORTED, with nothing launched,
