@@ -1,6 +1,7 @@
-"""The fused recompute call with a handful of live keys, which the merge kernel attends itself (at most 8 per sequence) instead
-of a streaming launch: around that limit, ragged batches, and windows that hide some or all of the recomputed keys.  Against
-the oracle and the two-call path, with the tolerance of the other fused tests."""
+"""The fused recompute calls with a handful of live keys, which the merge kernel attends itself (at most 8 per sequence) instead
+of a streaming launch: around that limit, ragged and mixed batches, gaps, windows that hide some or all of the recomputed keys,
+keys that score minus infinity, and every head form of the fused kernel with both rotations.  Against the oracle or softmax
+attention in 64 bits, with the tolerance of the other fused tests, and for the same bits alone and among others."""
 import dataclasses
 import math
 
@@ -137,3 +138,25 @@ def test_a_sequence_gets_the_same_bits_alone_and_among_others(kind, layer, n_old
     before = s.c.kvd_launch_count()
     s.run()
     assert s.c.kvd_launch_count() - before == 3
+
+
+@pytest.mark.parametrize("rope", [kvd.KVD_ROPE_INTERLEAVED, kvd.KVD_ROPE_HALF], ids=["pairs", "half-split"])
+@pytest.mark.parametrize("kind", ["bf16", "f16", "fp8"])
+@pytest.mark.parametrize("layer", GROUPS)
+def test_every_head_form_with_both_rotations_and_gaps_between_live_keys(layer, kind, rope):
+    s = Step(GROUPS[layer], [700, 300, 1, 513], [[0, 2, 3, 7], EIGHT, [4], [0, 1, 2, 5, 6, 7, 12, 13]], kind, rope, seed=3)
+    s.check(s.run())
+
+
+@pytest.mark.parametrize("kind", ["bf16", "f16", "fp8"])
+@pytest.mark.parametrize("layer", WIDE)
+@pytest.mark.parametrize("batch", [16, 64])  # a merge CTA per query head, per KV head
+def test_batches_whose_live_keys_the_merge_kernel_takes(batch, layer, kind):
+    s = Step(WIDE[layer], [260 + 3 * b for b in range(batch)], [list(range(1 + b % 8)) for b in range(batch)], kind, seed=batch)
+    nq, _, dh = WIDE[layer]
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert (batch * nq * (dh // 64) * 2 > 20 * sms) == (batch == 64)  # (one warp for partials, one for live keys)
+    before = s.c.kvd_launch_count()
+    out = s.run()
+    assert s.c.kvd_launch_count() - before == 2
+    s.check(out)
