@@ -60,7 +60,7 @@ def test_checking_build_reports_and_passes_the_parity_suites():
     env = dict(os.environ, KVD_LIBRARY="check")
     r = subprocess.run([sys.executable, "-c", SELFTEST], cwd=ROOT, env=env, capture_output=True, text=True, timeout=900)
     assert r.returncode == 0 and "checking build ok" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
-    files = ["tests/test_gpu_recompute.py", "tests/test_gpu_attention.py", "tests/test_gpu_fused.py", "tests/test_gpu_fp8.py",
+    files = ["tests/test_gpu_recompute.py", "tests/test_gpu_attention.py", "tests/test_gpu_fused.py", "tests/test_gpu_fused_tail.py", "tests/test_gpu_fp8.py",
              "tests/test_gpu_scaffold.py", "tests/test_gpu_rows.py"]
     r = subprocess.run([sys.executable, "-m", "pytest", "-x", "-q", "-m", "gpu", "-p", "no:cacheprovider", *files], cwd=ROOT,
                        env=env, capture_output=True, text=True, timeout=1800)

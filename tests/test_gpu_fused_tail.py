@@ -115,6 +115,22 @@ def test_live_keys_that_score_minus_infinity(kind, layer, n_old, live, lost):
     s.check(s.run())
 
 
+@pytest.mark.parametrize("value", [math.nan, math.inf])
+@pytest.mark.parametrize("kind", ["bf16", "f16"])
+@pytest.mark.parametrize("layer", ["2-256", "4-128"])
+@pytest.mark.parametrize("live", [[0], [0, 1, 2], list(range(9))])
+def test_live_keys_that_score_nan_or_plus_infinity_give_what_the_two_calls_give(live, layer, kind, value):
+    s = Step(GROUPS[layer], [300], [live], kind)
+    s.q[:, :, 5] = s.q[:, :, 5].abs() + 0.5
+    s.k[0][0, 0, 5] = value
+    out, two = s.run(), torch.full_like(s.q, 9.0)
+    segs = [(*s.rebuilt[0], s.kdim, 0, 300), (s.k[0], s.v[0], s.kdim, 300, len(live))]
+    s.c.kvd_decode_attention(0, 1, s.q, [300 + live[-1]], [segs], 0.0, two)
+    heads = s.nq // s.nkv  # of the first KV head
+    assert torch.equal(out[:, :heads], two[:, :heads]) and s.c.kvd_poll_status() == kvd.KVD_OK
+    attn_check(out[:, heads:].double().cpu().numpy(), two[:, heads:].double().cpu().numpy())
+
+
 WIDE = {"2-256": (8, 4, 256), "4-128": (16, 4, 128)}  # (with 64 sequences more warps than the SMs hold at once: a merge CTA per KV head)
 FEW, EIGHT, NINE = [0], list(range(8)), list(range(9))
 
